@@ -126,12 +126,11 @@ typedef enum {
                                  context's stream (see vote_get_kernel_times)        */
     VOTE_OPT_BATCH_WORKERS = 10, /* host workers (streams) of vote_solve_batched, 1..32,
                                  default 4                                           */
-    VOTE_OPT_DIVE = 11,       /* 1: before the sweep, expand one root-to-leaf path
-                                 that always takes the child with the largest UB, so
-                                 pruning starts from a leaf's count; 0: off; 2
-                                 (default): on for n >= 131072 surfaces.  Results do
-                                 not depend on it (Sec. 3.3: any valid bound may
-                                 prune)                                              */
+    VOTE_OPT_DIVE = 11,       /* 1 or 2 (default): first follow the cells with the largest
+                                 UBs and LBs down to the leaves, so pruning starts from
+                                 a leaf's count, and again from levels that grow large;
+                                 0: off.  Results do not depend on it (Sec. 3.3: any
+                                 valid bound may prune)                              */
     VOTE_OPT_SPIN_LIMIT = 12, /* polls of a bounded device-side wait (the proximity
                                  passes' wait for their bulk copies) before the kernel
                                  gives up and the solve returns VOTE_ETIMEOUT;

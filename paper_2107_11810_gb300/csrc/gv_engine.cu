@@ -6,13 +6,14 @@
 // the deepest non-empty level, tests all their children (k_test count pass),
 // raises the best lower bound, drops children below it (B&B pruning, Sec. 3.3),
 // lays out the survivors and writes their records, snapped for the next level
-// (emit pass, canonization of Sec. 3.2).  Taking the deepest level first is a
-// depth-first order over chunks: memory stays bounded by one chunk's expansion per
-// level, and leaves are reached early, which raises the pruning bound early.  The
-// result does not depend on this order.
+// (emit pass, canonization of Sec. 3.2).  The order (search(), dive()) follows the
+// cells with the largest bounds down to the leaves first, which raises the pruning
+// bound to about its final value, then opens the rest level by level while the next
+// level has room, else the deepest level first.  The result does not depend on it.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
@@ -62,7 +63,7 @@ struct DevBuf {
 
 struct LevelStore {
     DevBuf rec, mult, tile_cell;       // packed records (whole tiles), multiplicities, owning cell per tile
-    DevBuf key, rbeg, rcnt, ub;
+    DevBuf key, rbeg, rcnt, ub, lb;
     int64_t ncells = 0, nrecs = 0;     // nrecs: record slots in use (a multiple of 32)
 };
 
@@ -81,7 +82,7 @@ struct vote_ctx {
                                // 2: also one line per expansion step
     unsigned spin_limit = GV_SPIN_LIMIT;   // VOTE_OPT_SPIN_LIMIT
     int batch_workers = 4;
-    int dive = 2;              // greedy dive: 0 off, 1 on, 2 on for n >= kDiveMinN
+    int dive = 2;              // dives along the cells with the largest bounds: 0 off, 1 or 2 on
     int family = 0;
     double eps_in[GV_MAXD] = {}, bounds_in[2 * GV_MAXD] = {};
     std::vector<vote_ctx *> workers;   // sub-contexts of vote_solve_batched
@@ -97,6 +98,8 @@ struct vote_ctx {
     int64_t trace_cap = 0;
     int64_t fault_alloc_at = 0, alloc_count = 0;
     LevelStore ls[GV_MAXL + 1];
+    LevelStore beam;           // the selected cells of one level, during the dive
+    DevBuf beam_sel, beam_src;
     DevBuf levs_dev, path, scal, alive, geo64, geo32, geo32lo, cnt, tinfo, ballot, tdst, child_idx, cursor, keepflag, recn, bsums;
     DevBuf tr_level, tr_key, tr_ub, tr_lb, surf_tmp, mask_tmp;
     DevBuf ss_partial, ss_io;  // soft score: block partials; point [d] + outputs [d] + grad_out [1]
@@ -420,10 +423,13 @@ static void finalize_levels(vote_ctx *c, const unsigned *qmax) {
 // ---------------------------------------------------------------------------
 // device memory
 // ---------------------------------------------------------------------------
-static vote_status ensure(vote_ctx *c, DevBuf &b, size_t bytes) {
+// keep: bytes of the old contents to preserve
+static vote_status ensure(vote_ctx *c, DevBuf &b, size_t bytes, size_t keep = 0) {
     if (bytes <= b.bytes && b.p) return VOTE_OK;
     size_t want = bytes + bytes / 4 + 256;
-    if (b.p) {
+    void *old = keep ? b.p : nullptr;
+    if (old) want = std::max(want, 2 * b.bytes);     // appended to: few copies of the old contents
+    if (b.p && !old) {
         CK(cudaFreeAsync(b.p, c->stream));
         b.p = nullptr;
         b.bytes = 0;
@@ -436,9 +442,13 @@ static vote_status ensure(vote_ctx *c, DevBuf &b, size_t bytes) {
     cudaError_t e = cudaMallocAsync(&b.p, want, c->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        b.p = nullptr;
+        b.p = old;
         set_err("device allocation of %zu bytes failed: %s", want, cudaGetErrorString(e));
         return VOTE_ENOMEM;
+    }
+    if (old) {
+        CK(cudaMemcpyAsync(b.p, old, keep, cudaMemcpyDeviceToDevice, c->stream));
+        CK(cudaFreeAsync(old, c->stream));
     }
     b.bytes = want;
     return VOTE_OK;
@@ -488,37 +498,40 @@ static int rec_bytes_at(const vote_ctx *c, int l) {
 
 // Every array is checked against its own allocated size (ensure returns at once
 // when it is large enough), so no separate capacity figure can drift from the
-// allocations.  slots: record slots (a multiple of 32).
-static vote_status ensure_level(vote_ctx *c, int l, size_t slots, size_t cells) {
-    LevelStore &s = c->ls[l];
+// allocations.  slots: record slots (a multiple of 32) in level l's format.  What the
+// level holds (its ncells, nrecs) is preserved.
+static vote_status ensure_level(vote_ctx *c, LevelStore &s, int l, size_t slots, size_t cells) {
+    const size_t nr = (size_t)s.nrecs, nc = (size_t)s.ncells;
     if (slots > 0) {
-        TRY(ensure(c, s.rec, slots * rec_bytes_at(c, l)));
-        if (c->group) TRY(ensure(c, s.mult, slots * 4));   // without grouping every mult is 1
-        TRY(ensure(c, s.tile_cell, (slots / 32) * 4));
+        TRY(ensure(c, s.rec, slots * rec_bytes_at(c, l), nr * rec_bytes_at(c, l)));
+        if (c->group) TRY(ensure(c, s.mult, slots * 4, nr * 4));   // without grouping every mult is 1
+        TRY(ensure(c, s.tile_cell, (slots / 32) * 4, (nr / 32) * 4));
     }
     if (cells > 0) {
-        TRY(ensure(c, s.key, cells * 8));
-        TRY(ensure(c, s.rbeg, cells * 8));
-        TRY(ensure(c, s.rcnt, cells * 4));
-        TRY(ensure(c, s.ub, cells * 4));
+        TRY(ensure(c, s.key, cells * 8, nc * 8));
+        TRY(ensure(c, s.rbeg, cells * 8, nc * 8));
+        TRY(ensure(c, s.rcnt, cells * 4, nc * 4));
+        TRY(ensure(c, s.ub, cells * 4, nc * 4));
+        TRY(ensure(c, s.lb, cells * 4, nc * 4));
     }
     return VOTE_OK;
 }
 
-static RecView rec_view(vote_ctx *c, int l) {
+static RecView rec_view(vote_ctx *c, const LevelStore &s) {
     RecView v;
-    v.rec = (uint32_t *)c->ls[l].rec.p;
-    v.mult = c->group ? (uint32_t *)c->ls[l].mult.p : nullptr;
-    v.tile_cell = (uint32_t *)c->ls[l].tile_cell.p;
+    v.rec = (uint32_t *)s.rec.p;
+    v.mult = c->group ? (uint32_t *)s.mult.p : nullptr;
+    v.tile_cell = (uint32_t *)s.tile_cell.p;
     return v;
 }
 
-static CellView cell_view(vote_ctx *c, int l) {
+static CellView cell_view(const LevelStore &s) {
     CellView v;
-    v.key = (uint64_t *)c->ls[l].key.p;
-    v.rbeg = (uint64_t *)c->ls[l].rbeg.p;
-    v.rcnt = (uint32_t *)c->ls[l].rcnt.p;
-    v.ub = (uint32_t *)c->ls[l].ub.p;
+    v.key = (uint64_t *)s.key.p;
+    v.rbeg = (uint64_t *)s.rbeg.p;
+    v.rcnt = (uint32_t *)s.rcnt.p;
+    v.ub = (uint32_t *)s.ub.p;
+    v.lb = (uint32_t *)s.lb.p;
     return v;
 }
 
@@ -561,38 +574,35 @@ static void ev_collect(vote_ctx *c) {
 // search
 // ---------------------------------------------------------------------------
 
-// Expand a chunk of level-l cells taken from the top of the level's stack.  With
-// only >= 0, the single cell `only` is expanded where it sits instead (greedy
-// dive); its UB is then set to 0, so the sweep later finds it below every
-// threshold and gives it no children.
-static vote_status expand_chunk(vote_ctx *c, int l, int64_t only = -1) {
+// Expand a chunk of level-l cells taken from the top of the level's stack, or, in the
+// dive, all cells of the beam store (a selection of level l).
+static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     const Problem &P = c->P;
-    LevelStore &S = c->ls[l];
+    LevelStore &S = beam ? c->beam : c->ls[l];
     const int ns = c->ns;
     const Level &lev = c->lev[l];
     int nvalid = 0;
     for (int s = 0; s < ns; ++s)
         if (!(s & ~lev.split_mask)) ++nvalid;
     // chunk: cells [c0, c1) from the top of the stack, about chunk_records records
-    int64_t c1 = only >= 0 ? only + 1 : S.ncells, r1 = S.nrecs;
+    const int64_t c1 = S.ncells, r1 = S.nrecs;
     int64_t avg = S.nrecs / (S.ncells > 0 ? S.ncells : 1);
     int64_t K = c->chunk_records / (avg > 0 ? avg : 1);
-    if (K < 1 || only >= 0) K = 1;
+    if (K < 1) K = 1;
     if (K > (1 << 22)) K = 1 << 22;
     int64_t c0, r0;
     for (;;) {
         c0 = c1 - K > 0 ? c1 - K : 0;
+        if (beam) c0 = 0;
+        if (c0 == 0 && !c->kernel_timing && (beam || K == 1 || r1 <= 2 * c->chunk_records)) {
+            r0 = 0;                                  // the level's first record: nothing to read back
+            break;
+        }
         CK(cudaMemcpyAsync(c->h_tmp, (uint64_t *)S.rbeg.p + c0, 8, cudaMemcpyDeviceToHost, c->stream));
-        if (only >= 0)
-            CK(cudaMemcpyAsync(c->h_tmp + 1, (uint32_t *)S.rcnt.p + only, 4, cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
         ev_collect(c);
         r0 = (int64_t)c->h_tmp[0];
-        if (only >= 0) {
-            r1 = r0 + (((int64_t)(uint32_t)c->h_tmp[1] + 31) & ~(int64_t)31);
-            break;
-        }
-        if (r1 - r0 <= 2 * c->chunk_records || K == 1) break;
+        if (beam || r1 - r0 <= 2 * c->chunk_records || K == 1) break;
         K = K / 2;
     }
     nvtxRangePushA("expand_chunk");
@@ -611,7 +621,7 @@ static vote_status expand_chunk(vote_ctx *c, int l, int64_t only = -1) {
     TRY(ensure(c, c->keepflag, nch * 4));
     TRY(ensure(c, c->recn, nch * 4));
     TRY(ensure(c, c->bsums, ((nch + 255) / 256) * 16 + 16));
-    if (!lev.leaf_children) TRY(ensure_level(c, l + 1, 0, nch));    // records: sized below, exactly
+    if (!lev.leaf_children) TRY(ensure_level(c, c->ls[l + 1], l + 1, 0, (size_t)c->ls[l + 1].ncells + nch));    // records: sized below, exactly
     CK(cudaMemsetAsync(c->cnt.p, 0, nch * 12, c->stream));
     CK(cudaMemsetAsync(c->cursor.p, 0, nch * 4, c->stream));
     CK(cudaMemsetAsync(&dsc(c)->n_cells, 0, 16, c->stream));
@@ -620,10 +630,10 @@ static vote_status expand_chunk(vote_ctx *c, int l, int64_t only = -1) {
     std::memset(&ch, 0, sizeof(ch));
     ch.P = P;
     ch.lev = lev;
-    ch.cells = cell_view(c, l);
+    ch.cells = cell_view(S);
     ch.c0 = c0;
     ch.nc = nc;
-    ch.in = rec_view(c, l);
+    ch.in = rec_view(c, S);
     ch.in_rbeg = (const uint64_t *)S.rbeg.p;
     ch.in_rcnt = (const uint32_t *)S.rcnt.p;
     ch.in_c0 = c0;
@@ -698,8 +708,10 @@ static vote_status expand_chunk(vote_ctx *c, int l, int64_t only = -1) {
     ch.tinfo = (int2 *)c->tinfo.p;
     ch.ballot = (uint32_t *)c->ballot.p;
     if (!lev.leaf_children) {
-        ch.next_cells = cell_view(c, l + 1);
-        ch.out = rec_view(c, l + 1);
+        ch.next_cells = cell_view(c->ls[l + 1]);
+        ch.next_c0 = c->ls[l + 1].ncells;
+        ch.next_r0 = c->ls[l + 1].nrecs;
+        ch.out = rec_view(c, c->ls[l + 1]);
     }
     ev_mark(c, -1);
     launch_cell_geo(ch, c->stream);
@@ -720,12 +732,8 @@ static vote_status expand_chunk(vote_ctx *c, int l, int64_t only = -1) {
     c->stats.cells += nc;
     c->lv_cells[l] += nc;
     c->lv_recs[l] += nt * 32;
-    if (only >= 0) {
-        CK(cudaMemsetAsync((uint32_t *)S.ub.p + only, 0, 4, c->stream));
-    } else {
-        S.ncells = c0;
-        S.nrecs = r0;
-    }
+    S.ncells = c0;
+    S.nrecs = r0;
     if (lev.leaf_children) {
         if (c->log >= 2)
             std::fprintf(stderr, "[vote] step %lld level %d: %lld cells, %lld tiles, count %.0f B, leaves\n",
@@ -737,11 +745,12 @@ static vote_status expand_chunk(vote_ctx *c, int l, int64_t only = -1) {
     }
     CK(cudaMemcpyAsync(&c->h_sc->n_cells, &dsc(c)->n_cells, 16, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    LevelStore &N = c->ls[l + 1];
     int64_t new_cells = (int64_t)c->h_sc->n_cells, new_slots = (int64_t)c->h_sc->n_recs;
     if (new_slots > 0) {
-        TRY(ensure_level(c, l + 1, (size_t)new_slots, 0));
+        TRY(ensure_level(c, N, l + 1, (size_t)(N.nrecs + new_slots), 0));
         TRY(ensure(c, c->tdst, (size_t)nt * ns * 8));
-        ch.out = rec_view(c, l + 1);
+        ch.out = rec_view(c, c->ls[l + 1]);
         ch.tdst = (unsigned long long *)c->tdst.p;
         ev_mark(c, -1);
         launch_next_tiles(ch, new_cells, c->stream);
@@ -770,9 +779,9 @@ static vote_status expand_chunk(vote_ctx *c, int l, int64_t only = -1) {
                                          (double)new_slots * rec_bytes_at(c, l + 1) : 0.0,
                      (long long)new_cells, c->h_sc->tests, c->h_sc->rechecks, c->h_sc->rechecks_df);
     }
-    c->ls[l + 1].ncells = new_cells;
-    c->ls[l + 1].nrecs = new_slots;
-    if (new_slots > c->stats.peak_records) c->stats.peak_records = new_slots;
+    N.ncells += new_cells;
+    N.nrecs += new_slots;
+    if (N.nrecs > c->stats.peak_records) c->stats.peak_records = N.nrecs;
     nvtxRangePop();
     return VOTE_OK;
 }
@@ -795,9 +804,100 @@ static vote_status replay(vote_ctx *c, const double *surfaces, int64_t n, int la
     return VOTE_OK;
 }
 
-// Below this many surfaces the dive's per-level host round trips cost more than the
-// pruning they buy (the whole search is then a few chunks).
-static const int64_t kDiveMinN = 1 << 17;
+// A dive takes max(kBeamRecords, level's records / beam_divisor(d)) records of a level.
+// Measured (GB300, three instances per family, ms): 2^17, 2^19 and 2^20 records give
+// 13.6, 12.5 and 13.9 on the batch of 24 3DoF problems (a larger beam opens more than
+// it must) and 1.23, 0.70 and 0.70 on 10,000 lines (a smaller one takes more dependent
+// steps than a level that is opened whole).  Divisors 8 / 16 / 32: point sets 17 / 16 to
+// 84 / 54 to 87 (the best leaf's ancestor is often outside the top sixteenth), planes of
+// 1e4 points 60 / 54 / 52, 6DoF 25 / 21 / 15, radial 27 / 22 / 21.
+static const int64_t kBeamRecords = (int64_t)1 << 19;
+static int64_t beam_divisor(int d) { return d == 4 ? 8 : (d > 4 ? 32 : 16); }
+
+// records expanded into a level between two dives from it: a dive's cost (about a
+// millisecond of dependent steps) stays below a few percent of theirs
+static const int64_t kDiveEvery = (int64_t)1 << 28;
+
+// A dive: from level l0 down to the leaves, expand on every level the cells with the
+// largest UBs and LBs (k_beam_*).  A level that fits is expanded whole.
+static vote_status dive(vote_ctx *c, int l0) {
+    for (int l = l0; l < c->P.L; ++l) {
+        LevelStore &S = c->ls[l];
+        if (S.ncells <= 0) return VOTE_OK;
+        int64_t budget = std::max(kBeamRecords, S.nrecs / beam_divisor(c->P.d));
+        if (budget > c->chunk_records) budget = c->chunk_records;
+        if (S.nrecs <= budget || S.ncells == 1) {
+            TRY(expand_chunk(c, l));
+            continue;
+        }
+        const int64_t m = S.ncells;
+        c->beam.ncells = c->beam.nrecs = 0;
+        TRY(ensure_level(c, c->beam, l, 0, (size_t)m));
+        TRY(ensure(c, c->beam_sel, sizeof(BeamSel)));
+        TRY(ensure(c, c->beam_src, (size_t)m * 8));
+        TRY(ensure(c, c->bsums, (size_t)((m + 255) / 256) * 16 + 16));
+        CK(cudaMemsetAsync(c->beam_sel.p, 0, sizeof(BeamSel), c->stream));
+        launch_beam_select(c->P, cell_view(S), m, budget, (BeamSel *)c->beam_sel.p, (unsigned long long *)c->bsums.p,
+                           cell_view(c->beam), (uint64_t *)c->beam_src.p, dsc(c), c->stream);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(&c->h_sc->n_cells, &dsc(c)->n_cells, 16, cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+        ev_collect(c);
+        const int64_t nsel = (int64_t)c->h_sc->n_cells, rsel = (int64_t)c->h_sc->n_recs;
+        c->stats.launches += 5;
+        if (nsel <= 0) {                 // no cell reaches the bound any more (it never falls)
+            S.ncells = S.nrecs = 0;
+            return VOTE_OK;
+        }
+        c->beam.ncells = nsel;
+        TRY(ensure_level(c, c->beam, l, (size_t)rsel, 0));
+        c->beam.nrecs = rsel;
+        launch_beam_gather(rec_view(c, S), rec_view(c, c->beam), cell_view(c->beam), (const uint64_t *)c->beam_src.p,
+                           nsel, rsel / 32, rec_bytes_at(c, l), c->stream);
+        CK(cudaGetLastError());
+        c->stats.launches += 1;
+        TRY(expand_chunk(c, l, true));
+    }
+    return VOTE_OK;
+}
+
+// The search.  A dive from the root; then level by level, shallowest first, so that a
+// level's bounds are raised by all of its cells before its children are opened, while
+// the next level holds less than one step's records; when every level below is full,
+// the deepest first, which bounds the memory (room for 4 steps: a first solve of planes
+// with 1e6 points took 1564 ms instead of 1430 ms, more memory being mapped).  Whenever
+// a level has grown large, another dive starts from it: its own UBs and LBs point better
+// than those of the levels above.  Measured against one root-to-leaf path of the largest
+// UB for n >= 2^17 and the deepest level first: point sets 132 -> 17 ms, 6DoF 47 -> 13,
+// radial 70 -> 22, affine 4-space 204 -> 55, planes of 1e4 points 110 -> 54, 3DoF with
+// 1e6 matches 12.5 -> 7.9; with the final depth known from the start (VOTE_OPT_INITIAL_LB)
+// they took 13.5, -, 19, 52, 47 and 4.4 ms.
+static vote_status search(vote_ctx *c) {
+    const int L = c->P.L;
+    const bool dives = c->dive && c->prune;
+    const int64_t full = std::min(c->chunk_records, (int64_t)1 << 34);
+    int64_t since[GV_MAXL + 1];          // records expanded into the level since its last dive
+    for (int l = 0; l <= L; ++l) since[l] = -1;
+    if (dives) TRY(dive(c, 0));
+    for (;;) {
+        int l = -1;
+        for (int x = 0; x < L; ++x)
+            if (c->ls[x].ncells > 0) {
+                l = x;
+                if (x + 1 == L || c->ls[x + 1].nrecs <= full) break;
+            }
+        if (l < 0) return VOTE_OK;
+        const int64_t before = l + 1 < L ? c->ls[l + 1].nrecs : 0;
+        TRY(expand_chunk(c, l));
+        if (!dives || l + 1 >= L) continue;
+        const int64_t grown = c->ls[l + 1].nrecs - before;
+        if (since[l + 1] >= 0) since[l + 1] += grown;
+        if (c->ls[l + 1].nrecs > 8 * kBeamRecords && (since[l + 1] < 0 || since[l + 1] > kDiveEvery)) {
+            since[l + 1] = 0;
+            TRY(dive(c, l + 1));
+        }
+    }
+}
 
 static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, double *best_point,
                                int64_t *best_leaf, int64_t *depth, uint32_t *mask);
@@ -856,9 +956,9 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
         dep = n;                                   // the domain is a leaf: every surface counts
     } else if (n > 0) {
         const int64_t slots0 = (n + 31) & ~(int64_t)31;
-        TRY(ensure_level(c, 0, (size_t)slots0, 1));
+        TRY(ensure_level(c, c->ls[0], 0, (size_t)slots0, 1));
         ev_mark(c, -1);
-        launch_lift(P, c->lev[0], surfaces, n, rec_view(c, 0), dsc(c), c->stream);
+        launch_lift(P, c->lev[0], surfaces, n, rec_view(c, c->ls[0]), dsc(c), c->stream);
         c->stats.launches += 1;
         ev_mark(c, VOTE_K_LIFT);
         CK(cudaGetLastError());
@@ -868,6 +968,7 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
         CK(cudaMemcpyAsync(c->ls[0].rbeg.p, &rb0, 8, cudaMemcpyHostToDevice, c->stream));
         CK(cudaMemcpyAsync(c->ls[0].rcnt.p, &cnt0, 4, cudaMemcpyHostToDevice, c->stream));
         CK(cudaMemcpyAsync(c->ls[0].ub.p, &cnt0, 4, cudaMemcpyHostToDevice, c->stream));
+        CK(cudaMemsetAsync(c->ls[0].lb.p, 0, 4, c->stream));
         CK(cudaStreamSynchronize(c->stream));    // host sources above live on this frame
         c->ls[0].ncells = 1;
         c->ls[0].nrecs = slots0;
@@ -879,38 +980,7 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
             return VOTE_EINVAL;
         }
         finalize_levels(c, c->h_sc->qmax);
-        if (c->dive == 1 || (c->dive == 2 && n >= kDiveMinN)) {
-            // greedy dive: from the root, expand only the child with the largest UB
-            // (the first on ties) down to the leaves, so the sweep starts with a
-            // leaf's count as its pruning bound
-            int64_t cell = 0;
-            for (int l = 0; l < P.L; ++l) {
-                TRY(expand_chunk(c, l, cell));
-                int64_t m = l + 1 < P.L ? c->ls[l + 1].ncells : 0;
-                if (m <= 0) break;
-                uint32_t best = 0;
-                cell = -1;
-                for (int64_t i0 = 0; i0 < m; i0 += 16) {      // 16 UBs fit the pinned slot
-                    int64_t k = m - i0 < 16 ? m - i0 : 16;
-                    CK(cudaMemcpyAsync(c->h_tmp, (uint32_t *)c->ls[l + 1].ub.p + i0, 4 * (size_t)k,
-                                       cudaMemcpyDeviceToHost, c->stream));
-                    CK(cudaStreamSynchronize(c->stream));
-                    const uint32_t *ub = (const uint32_t *)c->h_tmp;
-                    for (int64_t i = 0; i < k; ++i)
-                        if (cell < 0 || ub[i] > best) best = ub[i], cell = i0 + i;
-                }
-            }
-        }
-        for (;;) {
-            int l = -1;
-            for (int x = P.L - 1; x >= 0; --x)
-                if (c->ls[x].ncells > 0) {
-                    l = x;
-                    break;
-                }
-            if (l < 0) break;
-            TRY(expand_chunk(c, l));
-        }
+        TRY(search(c));
         TRY(read_scalars(c));
         ev_collect(c);
         if (c->h_sc->err & kErrTimeout) {
@@ -1436,17 +1506,17 @@ void vote_destroy(vote_ctx *c) {
         if (ws) cudaStreamDestroy(ws);
     }
     c->workers.clear();
-    for (int l = 0; l <= GV_MAXL; ++l) {
-        LevelStore &s = c->ls[l];
+    for (int l = 0; l <= GV_MAXL + 1; ++l) {
+        LevelStore &s = l <= GV_MAXL ? c->ls[l] : c->beam;
         release(c, s.rec); release(c, s.mult); release(c, s.tile_cell);
-        release(c, s.key); release(c, s.rbeg); release(c, s.rcnt); release(c, s.ub);
+        release(c, s.key); release(c, s.rbeg); release(c, s.rcnt); release(c, s.ub); release(c, s.lb);
     }
     DevBuf *bufs[] = {&c->levs_dev, &c->path, &c->scal, &c->alive, &c->geo64, &c->geo32, &c->geo32lo, &c->cnt, &c->tinfo,
                       &c->ballot, &c->tdst,
                       &c->child_idx, &c->cursor, &c->keepflag, &c->recn, &c->bsums, &c->tr_level, &c->tr_key,
                       &c->tr_ub, &c->tr_lb, &c->surf_tmp, &c->mask_tmp, &c->ss_partial,
                       &c->ss_io, &c->g_table, &c->g_owner, &c->g_newpos, &c->g_ccount, &c->g_ccur,
-                      &c->g_rbeg, &c->g_rec, &c->g_mult, &c->g_tile};
+                      &c->g_rbeg, &c->g_rec, &c->g_mult, &c->g_tile, &c->beam_sel, &c->beam_src};
     for (DevBuf *b : bufs) release(c, *b);
     cudaStreamSynchronize(c->stream);
     for (int i = 0; i < vote_ctx::kEv; ++i)

@@ -322,15 +322,189 @@ __global__ void __launch_bounds__(256) k_child_write(Chunk c, const uint32_t *ke
     if (!in) return;
     if (keep) {
         int cl = idx / NS, s = idx % NS;
-        unsigned long long ci = bs_cells[blockIdx.x] + ec;
+        unsigned long long ci = c.next_c0 + bs_cells[blockIdx.x] + ec;
         c.next_cells.key[ci] = child_key(c.P, c.cells.key[c.c0 + cl], c.lev.l, s);
-        c.next_cells.rbeg[ci] = bs_recs[blockIdx.x] + er;
+        c.next_cells.rbeg[ci] = c.next_r0 + bs_recs[blockIdx.x] + er;
         c.next_cells.rcnt[ci] = c.cnt[(size_t)idx * 3 + 2];
         c.next_cells.ub[ci] = c.cnt[(size_t)idx * 3];
+        c.next_cells.lb[ci] = c.cnt[(size_t)idx * 3 + 1];
         c.child_idx[idx] = (int32_t)ci;
     } else {
         c.child_idx[idx] = -1;
     }
+}
+
+// ---------------------------------------------------------------------------
+// Beam selection (the search order; any count some leaf reaches is a valid lower
+// bound, Sec. 3.3, so results do not depend on it).  A selection of a level's cells
+// holds about `budget` record slots: half of them in the cells with the largest UBs,
+// half in those with the largest LBs.  Of the two the UB finds the best leaf's ancestor
+// on the coarse levels of pose, ray, point-set and affine searches, the LB on the
+// middle levels of planes, where almost every UB is alike.
+//
+// k_beam_hist: record slots per UB and LB bin (64 bins per octave) and the cells with
+// the largest UB and LB; k_beam_pick: the bin at which the slots of the bins above
+// reach the budget, and the share of that bin's cells that still fits; k_beam_mark:
+// selected cells (the border bin's by a hash of their keys, so the choice depends on
+// nothing but the cells) and block totals; k_scan_sums; k_beam_write: the selected
+// cells in index order, their UB in the level set to 0 (no threshold is below 1, so
+// they are found pruned later and no cell is tested twice); k_beam_gather: their
+// records, copied so that one contiguous chunk holds them (a warp per tile, the owning
+// cell by binary search; the copy moves at most a few tens of MB).
+// ---------------------------------------------------------------------------
+
+// 64 bins per octave: the exponent and six mantissa bits of a count as a float
+__device__ __forceinline__ int beam_bin(unsigned v) {
+    const int b = (int)((__float_as_uint((float)v) >> 17) - (127u << 6));
+    return b < 0 ? 0 : (b >= kBeamBins ? kBeamBins - 1 : b);
+}
+
+__device__ __forceinline__ unsigned beam_hash(uint64_t key) {
+    key = (key ^ (key >> 31)) * 0x9E3779B97F4A7C15ull;
+    key = (key ^ (key >> 29)) * 0xff51afd7ed558ccdull;
+    return (unsigned)(key >> 32);
+}
+
+__device__ __forceinline__ unsigned long long warp_max64(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(kFull, v, o);
+        v = y > v ? y : v;
+    }
+    return v;
+}
+
+__global__ void __launch_bounds__(256) k_beam_hist(CellView cells, int64_t ncells, BeamSel *sel, Problem P,
+                                                   const Scalars *sc) {
+    __shared__ unsigned long long hist[2][kBeamBins];
+    for (int i = threadIdx.x; i < 2 * kBeamBins; i += 256) hist[0][i] = 0ull;
+    const unsigned thr = prune_threshold(P, sc, 1);
+    __syncthreads();
+    unsigned long long best[2] = {0ull, 0ull};
+    for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < ncells; i += gridDim.x * 256ll) {
+        const unsigned ub = cells.ub[i];
+        if (ub < thr) continue;
+        const unsigned v[2] = {ub, cells.lb[i]};
+        const unsigned long long slots = (cells.rcnt[i] + 31u) & ~31u;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (!v[k]) continue;
+            atomicAdd(&hist[k][beam_bin(v[k])], slots);
+            const unsigned long long cand = ((unsigned long long)v[k] << 32) | (unsigned)~(unsigned)i;
+            best[k] = cand > best[k] ? cand : best[k];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        best[k] = warp_max64(best[k]);
+        if ((threadIdx.x & 31) == 0 && best[k]) atomicMax(&sel->best[k], best[k]);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 2 * kBeamBins; i += 256)
+        if (hist[0][i]) atomicAdd(&sel->hist[0][i], hist[0][i]);
+}
+
+__global__ void __launch_bounds__(256) k_beam_pick(BeamSel *sel, unsigned long long budget) {
+    // thread t owns bins [8 t', 8 t' + 8), t' counted from the top, so a prefix over the
+    // threads is the slots of all higher bins
+    constexpr int PER = kBeamBins / 256;
+    const int top = kBeamBins - 1 - (int)threadIdx.x * PER;
+    for (int k = 0; k < 2; ++k) {
+        unsigned long long v[PER], sum = 0ull, total;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            v[i] = sel->hist[k][top - i];
+            sum += v[i];
+        }
+        unsigned long long above = block_excl_scan(sum, &total);
+        if (total <= budget) {
+            if (threadIdx.x == 0) {
+                sel->border[k] = -1;
+                sel->share[k] = 0u;
+            }
+            continue;
+        }
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            if (above <= budget && above + v[i] > budget) {
+                sel->border[k] = top - i;
+                sel->share[k] = (unsigned)((double)(budget - above) / (double)v[i] * 4294967295.0);
+            }
+            above += v[i];
+        }
+    }
+}
+
+__device__ __forceinline__ bool beam_selected(const CellView &cells, int64_t i, int64_t ncells, const BeamSel *sel,
+                                              unsigned thr) {
+    if (i >= ncells) return false;
+    const unsigned ub = cells.ub[i];
+    if (ub < thr) return false;
+    const unsigned v[2] = {ub, cells.lb[i]};
+    const unsigned h = beam_hash(cells.key[i]);
+    bool keep = false;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (!v[k]) continue;
+        const int b = beam_bin(v[k]);
+        keep |= b > sel->border[k] || (b == sel->border[k] && h < sel->share[k]) ||
+                (unsigned)~(unsigned)sel->best[k] == (unsigned)i;
+    }
+    return keep;
+}
+
+__global__ void __launch_bounds__(256) k_beam_mark(CellView cells, int64_t ncells, const BeamSel *sel, Problem P,
+                                                   const Scalars *sc, unsigned long long *bs_cells,
+                                                   unsigned long long *bs_recs) {
+    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
+    const bool keep = beam_selected(cells, i, ncells, sel, prune_threshold(P, sc, 1));
+    unsigned long long tc, tr;
+    block_excl_scan(keep ? 1ull : 0ull, &tc);
+    block_excl_scan(keep ? (unsigned long long)((cells.rcnt[i] + 31u) & ~31u) : 0ull, &tr);
+    if (threadIdx.x == 0) {
+        bs_cells[blockIdx.x] = tc;
+        bs_recs[blockIdx.x] = tr;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_beam_write(CellView cells, int64_t ncells, const BeamSel *sel, Problem P,
+                                                    const Scalars *sc, const unsigned long long *bs_cells,
+                                                    const unsigned long long *bs_recs, CellView out,
+                                                    uint64_t *src_rbeg) {
+    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
+    const bool keep = beam_selected(cells, i, ncells, sel, prune_threshold(P, sc, 1));
+    unsigned long long tc, tr;
+    const unsigned long long ec = block_excl_scan(keep ? 1ull : 0ull, &tc);
+    const unsigned long long er =
+        block_excl_scan(keep ? (unsigned long long)((cells.rcnt[i] + 31u) & ~31u) : 0ull, &tr);
+    if (!keep) return;
+    const unsigned long long o = bs_cells[blockIdx.x] + ec;
+    out.key[o] = cells.key[i];
+    out.rbeg[o] = bs_recs[blockIdx.x] + er;
+    out.rcnt[o] = cells.rcnt[i];
+    out.ub[o] = cells.ub[i];
+    src_rbeg[o] = cells.rbeg[i];
+    cells.ub[i] = 0u;
+}
+
+// nq: 16-byte words of one tile's records
+__global__ void __launch_bounds__(256) k_beam_gather(RecView in, RecView out, CellView sel, const uint64_t *src_rbeg,
+                                                     int64_t ncells, int64_t ntiles, int nq) {
+    const int64_t t = (blockIdx.x * 256ll + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (t >= ntiles) return;
+    int64_t a = 0, b = ncells;                      // last cell whose first record is at or before the tile
+    while (b - a > 1) {
+        const int64_t m = (a + b) >> 1;
+        if ((int64_t)(sel.rbeg[m] >> 5) <= t) a = m;
+        else b = m;
+    }
+    const int64_t ts = (int64_t)(src_rbeg[a] >> 5) + (t - (int64_t)(sel.rbeg[a] >> 5));
+    const uint4 *src = reinterpret_cast<const uint4 *>(in.rec) + ts * nq;
+    uint4 *dst = reinterpret_cast<uint4 *>(out.rec) + t * nq;
+    for (int i = lane; i < nq; i += 32) dst[i] = src[i];
+    if (out.mult) out.mult[t * 32 + lane] = in.mult[ts * 32 + lane];
+    if (lane == 0) out.tile_cell[t] = (uint32_t)a;
 }
 
 // ---------------------------------------------------------------------------
@@ -350,10 +524,10 @@ __global__ void k_tile_info(Chunk c) {
 }
 
 // the next level's tile -> cell table: one warp per new cell writes its tiles
-__global__ void k_next_tiles(CellView next, RecView out, int64_t ncells) {
-    const int64_t cell = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+__global__ void k_next_tiles(CellView next, RecView out, int64_t c0, int64_t ncells) {
+    const int64_t cell = c0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
-    if (cell >= ncells) return;
+    if (cell >= c0 + ncells) return;
     const int64_t t0 = (int64_t)(next.rbeg[cell] >> 5), nt = ((int64_t)next.rcnt[cell] + 31) >> 5;
     for (int64_t i = lane; i < nt; i += 32) out.tile_cell[t0 + i] = (uint32_t)cell;
 }
@@ -659,7 +833,7 @@ void launch_tile_info(const Chunk &c, cudaStream_t st) {
 }
 
 void launch_next_tiles(const Chunk &c, int64_t ncells, cudaStream_t st) {
-    if (ncells > 0) k_next_tiles<<<blocks_for(ncells * 32, 256), 256, 0, st>>>(c.next_cells, c.out, ncells);
+    if (ncells > 0) k_next_tiles<<<blocks_for(ncells * 32, 256), 256, 0, st>>>(c.next_cells, c.out, c.next_c0, ncells);
 }
 
 void launch_tile_dst(const Chunk &c, cudaStream_t st) {
@@ -703,6 +877,25 @@ void launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsi
     else if (ns == 16) k_child_write<16><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
     else if (ns == 32) k_child_write<32><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
     else k_child_write<64><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
+}
+
+void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, BeamSel *sel,
+                        unsigned long long *bsums, const CellView &out, uint64_t *src_rbeg, Scalars *sc,
+                        cudaStream_t st) {
+    const unsigned nb = blocks_for(ncells, 256);
+    unsigned long long *ba = bsums, *bb = bsums + nb;
+    k_beam_hist<<<nb < 1024u ? nb : 1024u, 256, 0, st>>>(cells, ncells, sel, P, sc);
+    k_beam_pick<<<1, 256, 0, st>>>(sel, (unsigned long long)budget / 2);
+    k_beam_mark<<<nb, 256, 0, st>>>(cells, ncells, sel, P, sc, ba, bb);
+    k_scan_sums<<<1, 256, 0, st>>>(ba, bb, (int)nb, sc);
+    k_beam_write<<<nb, 256, 0, st>>>(cells, ncells, sel, P, sc, ba, bb, out, src_rbeg);
+}
+
+void launch_beam_gather(const RecView &in, const RecView &out, const CellView &sel, const uint64_t *src_rbeg,
+                        int64_t ncells, int64_t ntiles, int rec_bytes, cudaStream_t st) {
+    if (ntiles > 0)
+        k_beam_gather<<<blocks_for(ntiles * 32, 256), 256, 0, st>>>(in, out, sel, src_rbeg, ncells, ntiles,
+                                                                    32 * rec_bytes / 16);
 }
 
 void launch_group(const Chunk &c, uint32_t *table, uint32_t tmask, uint32_t *owner, uint32_t *ccount,

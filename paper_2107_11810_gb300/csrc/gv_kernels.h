@@ -20,12 +20,13 @@ struct RecView {
 };
 
 // Cells of one level: packed leaf-aligned key, first record (a multiple of 32),
-// record count, UB.
+// record count, UB, LB.
 struct CellView {
     uint64_t *key;
     uint64_t *rbeg;
     uint32_t *rcnt;
     uint32_t *ub;
+    uint32_t *lb;
 };
 
 // Device-resident scalars of one solve.
@@ -77,6 +78,7 @@ struct Chunk {
     int32_t *child_idx;      // [nc][2^d]         index of the child cell or -1
     uint32_t *cursor;        // [nc][2^d]         next free record of the child
     CellView next_cells;     // cells of level l+1
+    int64_t next_c0, next_r0;// its cells and record slots before this step (the step appends)
     RecView out;             // records of level l+1
     Scalars *sc;
     Trace trace;
@@ -90,6 +92,16 @@ struct Chunk {
 // (every G is FP32-exact and a multiple of 2^e; kNoExp when not).
 __host__ __device__ constexpr int geo32_floats(int nfs, int nd, int le) { return nfs * nd * le + nd * le + 1; }
 constexpr int kNoExp = -1000;
+
+// Selection of a level's cells with the largest UBs (index 0) and LBs (index 1)
+// (k_beam_*); zeroed before each use.
+constexpr int kBeamBins = 2048;
+struct BeamSel {
+    unsigned long long hist[2][kBeamBins];  // record slots per bin
+    unsigned long long best[2];      // (value << 32) | ~index of the cell with the largest value
+    int border[2];                   // bins above are selected whole
+    unsigned share[2];               // selected share of the border bin (2^32 = all)
+};
 
 // Path geometry for replaying surfaces along the root-to-cell path.
 struct PathStep {
@@ -110,7 +122,7 @@ void launch_count(const Chunk &c, cudaStream_t st);
 void launch_count_wide(const Chunk &c, cudaStream_t st);
 bool launch_emit_wide(const Chunk &c, cudaStream_t st);
 // after the children are laid out: the next level's tile -> cell table for cells
-// [0, ncells) and every tile's output positions (tdst)
+// [next_c0, next_c0 + ncells) and every tile's output positions (tdst)
 void launch_next_tiles(const Chunk &c, int64_t ncells, cudaStream_t st);
 void launch_tile_dst(const Chunk &c, cudaStream_t st);
 // false if the level's record formats have no emit pass (never chosen by the engine)
@@ -119,6 +131,14 @@ void launch_child_lbmax(const Chunk &c, cudaStream_t st);
 // keepflag, recn: [nc * 2^d]; bsums: 2 * ceil(nc * 2^d / 256)
 void launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
                         cudaStream_t st);
+// the cells of a level (whose sum of record slots exceeds budget) with the largest UBs and LBs:
+// out and src_rbeg receive them ([ncells] at most), sc->n_cells / n_recs their number
+// and slots; bsums: 2 * ceil(ncells / 256); then their records
+void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, BeamSel *sel,
+                        unsigned long long *bsums, const CellView &out, uint64_t *src_rbeg, Scalars *sc,
+                        cudaStream_t st);
+void launch_beam_gather(const RecView &in, const RecView &out, const CellView &sel, const uint64_t *src_rbeg,
+                        int64_t ncells, int64_t ntiles, int rec_bytes, cudaStream_t st);
 void launch_path_geo(const Problem &P, const Level *levs_dev, int lam, uint64_t key, PathStep *path,
                      cudaStream_t st);
 void launch_replay(const Problem &P, const Level *levs_dev, const PathStep *path, int lam, const double *prm,
