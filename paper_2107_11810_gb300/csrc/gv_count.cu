@@ -1,344 +1,192 @@
 // gv_count.cu -- count pass of the proximity test (Algorithm 2's per-sub-box
-// selection with the surface-box test of Sec. 3.2): for every record of a chunk and
-// every child of its cell, the UB test (|residual| <= eps + cell radius + Lipschitz
-// term + accumulated canonization error) and the LB test (|residual| <= eps -
-// accumulated error); per child the multiplicity sums UB, LB and the number of
-// UB-passing records; per tile and child the ballot of UB-passing lanes, which the
-// emit pass uses to write the child records.
+// selection with the surface-box test of Sec. 3.2) for families with at most 8
+// children: for every record of a chunk and every child of its cell, the UB test
+// (|residual| <= eps + cell radius + Lipschitz term + accumulated canonization error)
+// and, where lower bounds are wanted, the LB test (|residual| <= eps - accumulated
+// error); per tile and child the ballot of passing lanes.  Counts and output positions
+// come from the ballots (k_tile_scan); undecided records are queued for the FP64
+// definition (k_recheck).
 //
-// FP32 screen + FP64 recheck: the decisions are taken in FP32 in units of the snap
-// step; a lane whose comparison falls inside the screen's error band re-evaluates
-// its record with the exact FP64 definition, and its counts and ballot bits are
-// corrected (a rare path).  Plain FP64 mode evaluates every record exactly.
+// The pass is bound by instruction issue (its records take a tenth of the DRAM rate), so
+// it is built for few instructions per (tile, child): only children that exist are
+// tested (a kernel per split mask); residuals, shifts and squared comparisons of two
+// children go through the packed FP32 operations; a decision costs half a packed
+// multiply-add, one compare and one ballot, and the band of a record is checked once,
+// from the smallest |y^2 - R^2| of its children.  Records are read with plain coalesced
+// loads one tile ahead, so nothing waits at a block barrier.
 #include "gv_tile.cuh"
 
 namespace gv {
 
-#ifndef GV_MINBLOCKS_COUNT
-#define GV_MINBLOCKS_COUNT 3
-#endif
-
-// Shared memory of one block: two buffers of one group (kBlockTiles tiles) of
-// records and tile information.
-template <int NW>
-constexpr size_t count_smem_bytes() {
-    return 2 * (size_t)kBlockTiles * 32 * NW * 4 + 2 * (size_t)kBlockTiles * sizeof(int2);
+template <int N>
+__device__ __forceinline__ void store_row(uint32_t *p, const unsigned *v) {
+    if constexpr (N == 2) {
+        *reinterpret_cast<uint2 *>(p) = make_uint2(v[0], v[1]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) *reinterpret_cast<uint4 *>(p + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    }
 }
 
-// A persistent block takes a contiguous range of groups of kBlockTiles tiles;
-// while one group is tested, the next one's records and tile information are
-// copied into the other buffer (bulk copies completing on an mbarrier).  Warp w
-// tests tiles w * kTW .. w * kTW + kTW - 1 of each group.
-template <int FAM, bool Q16, int PREC, bool WEIGHTED>
-__global__ void __launch_bounds__(256, GV_MINBLOCKS_COUNT) k_count(const __grid_constant__ Chunk c) {
+// KF: free coordinates that split, DM: dependent coordinates that split (bit mask).
+// Each warp takes a contiguous range of the chunk's tiles (runs of tiles of one cell
+// stay together: the cell's coefficients are spread from one register per lane only
+// when the cell changes).
+template <int FAM, bool Q16, int KF, int DM, bool LB>
+__global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk c) {
     using F = Fam<FAM>;
-    constexpr int NS = 1 << F::D, NFS = 1 << F::K, ND = F::ND, LE = F::LE, NFP = F::NFP;
-    constexpr int NW = rec_words(NFP, Q16);
-    constexpr int RW = 32 * NW;                             // words per tile
-    constexpr int GT = kBlockTiles;
-    constexpr int NCW = (NS + 3) / 4;                      // byte-packed counter words
-    constexpr int GF = geo32_floats(NFS, ND, LE);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int ND = F::ND, LE = F::LE, NFS = 1 << KF, NS = NFS * dep_slots(DM);
+    constexpr int NW = rec_words(F::NFP, Q16), NG = NFS * ND * LE;
+    static_assert(NG <= 32 && NS >= 2 && NS <= 8, "coefficients of a cell fit one register per lane");
+    const int lane = threadIdx.x & 31;
     const Level &lev = c.lev;
-    const int smask = lev.split_mask;
-    extern __shared__ __align__(128) uint32_t s_dyn[];
-    uint32_t *s_rec = s_dyn;                                              // [2][GT * RW]
-    int2 *s_ti = reinterpret_cast<int2 *>(s_dyn + 2 * GT * RW);           // [2][GT]
-    __shared__ __align__(8) uint64_t s_bar[2];
-
     const int64_t nt = c.t1 - c.t0;
-    const int64_t ng = (nt + GT - 1) / GT;
-    const int64_t g0 = (int64_t)blockIdx.x * ng / gridDim.x, g1 = (int64_t)(blockIdx.x + 1) * ng / gridDim.x;
-    if (threadIdx.x == 0) {
-        mbar_init(&s_bar[0], 1);
-        mbar_init(&s_bar[1], 1);
-        mbar_init_fence();
-    }
-    __syncthreads();
-    // thread 0: copy group g into buffer (g - g0) & 1
-    auto issue = [&](int64_t g) {
-        const int b = (int)((g - g0) & 1);
-        const int64_t ta = g * GT;                                        // chunk-relative first tile
-        const int ntl = (int)((ta + GT < nt ? ta + GT : nt) - ta);
-        const unsigned rbytes = (unsigned)ntl * RW * 4;
-        const unsigned ibytes = (unsigned)((ntl + 1) & ~1) * (unsigned)sizeof(int2);   // 16-byte multiple
-        mbar_expect_tx(&s_bar[b], rbytes + ibytes);
-        bulk_load(s_rec + b * GT * RW, c.in.rec + (c.t0 + ta) * RW, rbytes, &s_bar[b]);
-        bulk_load(s_ti + b * GT, c.tinfo + ta, ibytes, &s_bar[b]);
-    };
-    if (threadIdx.x == 0 && g0 < g1) issue(g0);
-
-    // dependent shifts and lower-bound radii of this level (steps)
-    float hs[ND], Lc[ND];
+    const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
+    float hs[ND], negL2[ND];
 #pragma unroll
     for (int j = 0; j < ND; ++j) {
-        hs[j] = ((smask >> (F::K + j)) & 1) ? lev.Hs[j] : 0.0f;
-        Lc[j] = lev.Lc[j];
+        hs[j] = lev.Hs[j];
+        negL2[j] = -lev.Lc[j] * lev.Lc[j];
     }
-    unsigned nvslot = 0;
+    const float *gp = c.geo32 + (lane < NG ? lane : 0);
+    auto load_g = [&](int cell) { return __ldg(gp + (size_t)(cell < 0 ? 0 : cell) * c.gf); };
+    int run = -1;
+    float G[NG];
 #pragma unroll
-    for (int s = 0; s < NS; ++s) nvslot += !(s & ~smask);
-
-    // counts of the current run of tiles of one cell
-    unsigned pu[NCW], pl[NCW];
-    unsigned wu[WEIGHTED ? NS : 1], wl[WEIGHTED ? NS : 1], wn[WEIGHTED ? NS : 1];
-#pragma unroll
-    for (int x = 0; x < NCW; ++x) pu[x] = pl[x] = 0u;
-#pragma unroll
-    for (int s = 0; s < (WEIGHTED ? NS : 1); ++s) wu[s] = wl[s] = wn[s] = 0u;
-    int run = -1;                 // chunk-local cell of the run
-    float G[GF];
-#pragma unroll
-    for (int i = 0; i < GF; ++i) G[i] = 0.0f;
-    unsigned ntest = 0, nrechk = 0, nrec = 0;
-
-    // lane x < 3 NS accumulates counter x / NS (UB, LB, records) of child slot x % NS
-    // for the current run; the byte-packed per-lane counters are drained into it
-    // every kTW tiles (before a byte could carry) and it goes to the cell's global
-    // counters when the run ends
-    unsigned acc = 0;
-    auto drain = [&]() {
-        if constexpr (!WEIGHTED) {
-            unsigned au[NCW], al[NCW];
-#pragma unroll
-            for (int x = 0; x < NCW; ++x) {
-                au[x] = __reduce_add_sync(kFull, pu[x]);
-                al[x] = __reduce_add_sync(kFull, pl[x]);
-                pu[x] = pl[x] = 0u;
-            }
-            const int s = lane % NS, kind = lane / NS;
-            unsigned word = kind == 1 ? al[0] : au[0];
-#pragma unroll
-            for (int x = 1; x < NCW; ++x)
-                if ((s >> 2) == x) word = kind == 1 ? al[x] : au[x];
-            if (lane < 3 * NS) acc += (word >> (8 * (s & 3))) & 255u;
-        } else {
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-                if (lane == s) acc += wu[s];
-                if (lane == NS + s) acc += wl[s];
-                if (lane == 2 * NS + s) acc += wn[s];
-                wu[s] = wl[s] = wn[s] = 0u;
-            }
-        }
-    };
-    auto flush = [&]() {
-        if (run < 0) return;
-        drain();
-        if (lane < 3 * NS && acc) atomicAdd(c.cnt + ((size_t)run * NS + lane % NS) * 3 + lane / NS, acc);
-        acc = 0;
-    };
-
-    int64_t gfail = -1;                                             // group whose copy did not arrive
+    for (int i = 0; i < NG; ++i) G[i] = 0.0f;
+    unsigned nrec = 0;
+    if (ta < tb) {
+        // one tile ahead: records and the lane's coefficient; tile information two ahead
+        int2 ti1 = c.tinfo[ta], ti2 = c.tinfo[ta + 1 < tb ? ta + 1 : ta];
+        uint32_t w1[NW];
+        load_words<NW>(c.in.rec, (c.t0 + ta) * 32 + lane, w1);
+        float g1 = load_g(ti1.x);
 #pragma unroll 1
-    for (int64_t g = g0; g < g1; ++g) {
-        const int b = (int)((g - g0) & 1);
-        if (threadIdx.x == 0 && g + 1 < g1) issue(g + 1);
-        const bool ok = mbar_wait(&s_bar[b], (unsigned)(((g - g0) >> 1) & 1), c.spin, &c.sc->err);
-        if (__syncthreads_or(!ok)) {                                // uniform: a copy did not arrive
-            gfail = g;
-            break;
-        }
-#pragma unroll 1
-        for (int k = 0; k < kTW; ++k) {
-            const int lt = warp * kTW + k;                          // tile within the group
-            const int64_t tile = c.t0 + g * GT + lt;
-            if (tile >= c.t1) break;                                // uniform
-            const int2 ti = s_ti[b * GT + lt];
-            const int cl = ti.x;
-            if (cl < 0) continue;                                   // uniform: the cell was pruned
-            if (cl != run) {                                        // uniform: a new cell
-                flush();
-                run = cl;
-                if (PREC == 1) {
-                    const float *gp = c.geo32 + (size_t)cl * GF;
-#pragma unroll
-                    for (int i = 0; i < GF; ++i) G[i] = __ldg(gp + i);
-                }
-            }
+        for (int64_t tt = ta; tt < tb; ++tt) {
+            const int2 ti = ti1;
+            const float g = g1;
             uint32_t w[NW];
 #pragma unroll
-            for (int i = 0; i < NW; ++i) w[i] = s_rec[b * GT * RW + lt * RW + lane * NW + i];
-            const int nvalid = ti.y;
-            const bool act = lane < nvalid;
-            const int64_t r = tile * 32 + lane;
-            ntest += (unsigned)nvalid * nvslot;
+            for (int i = 0; i < NW; ++i) w[i] = w1[i];
+            if (tt + 1 < tb) {
+                ti1 = ti2;
+                load_words<NW>(c.in.rec, (c.t0 + tt + 1) * 32 + lane, w1);
+                g1 = load_g(ti1.x);
+                if (tt + 2 < tb) ti2 = c.tinfo[tt + 2];
+            }
+            if (ti.x < 0) continue;                                 // uniform: the cell was pruned
+            if (ti.x != run) {                                      // uniform: a new cell
+                run = ti.x;
+#pragma unroll
+                for (int i = 0; i < NG; ++i) G[i] = __shfl_sync(kFull, g, i);
+            }
+            const int nvalid = ti.y & 63;
             nrec += (unsigned)nvalid;
-            const uint32_t mult = WEIGHTED ? (act ? c.in.mult[r] : 0u) : 1u;
-            const double *g64 = c.geo64 + (size_t)cl * NFS * F::NB;
-            unsigned bw[NS];                 // the tile's ballot per child slot
+            float qf[ND], qt[LE], R[ND], negR2[ND], near[ND], nearL[ND];
 #pragma unroll
-            for (int s = 0; s < NS; ++s) bw[s] = 0u;
-            bool uns = false;
-            if constexpr (PREC == 1) {
-                float qf[ND], qt[LE], R[ND], M[ND], Rlo[ND], Rhi[ND], Llo[ND], Lhi[ND];
+            for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
 #pragma unroll
-                for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
+            for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
+            F::radius32(lev, qt, R);
 #pragma unroll
-                for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
-                F::radius32(lev, qt, R);
-                magnitudes<FAM>(qf, qt, G + NFS * ND * LE, hs, M);
+            for (int j = 0; j < ND; ++j) {
+                negR2[j] = -R[j] * R[j];
+                near[j] = nearL[j] = 3.0e38f;
+            }
+            // a lane without a record fails every test (its residual is out of reach)
+            if (lane >= nvalid) qf[0] = 1.0e15f;
+            float u[ND][NFS];
 #pragma unroll
-                for (int j = 0; j < ND; ++j) {
-                    const float e = kBandTest * (M[j] + R[j]);
-                    Rlo[j] = R[j] - e;
-                    Rhi[j] = R[j] + e;
-                    Llo[j] = Lc[j] - e;
-                    Lhi[j] = Lc[j] + e;
-                }
-                // a lane without a record fails every test (its residual is out of reach)
-                if (!act) qf[0] = 1.0e30f;
+            for (int j = 0; j < ND; ++j) {
+                if constexpr (NFS >= 2) {
 #pragma unroll
-                for (int fs = 0; fs < NFS; ++fs) {
-                    float u[ND];
-                    partial32<FAM>(qf, qt, G, fs, u);
+                    for (int f = 0; f < NFS; f += 2) {
+                        f2 v = f2_make(qf[j], qf[j]);
 #pragma unroll
-                    for (int ds = 0; ds < (1 << ND); ++ds) {
-                        // every slot is tested, also those of coordinates that no longer
-                        // split: their counts and ballots are never read, and testing them
-                        // costs less than branching around them
-                        const int s = fs | (ds << F::K);
-                        bool ub, lb;
-                        screen<FAM>(ds, u, hs, Rlo, Rhi, Llo, Lhi, ub, lb, uns);
-                        const unsigned bb = __ballot_sync(kFull, ub);
-                        bw[s] = bb;
-                        if constexpr (!WEIGHTED) {
-                            if (ub) pu[s >> 2] += 1u << (8 * (s & 3));
-                            if (lb) pl[s >> 2] += 1u << (8 * (s & 3));
-                        } else {
-                            wu[s] += __reduce_add_sync(kFull, ub ? mult : 0u);
-                            wl[s] += __reduce_add_sync(kFull, lb ? mult : 0u);
-                            wn[s] += __popc(bb);
-                        }
+                        for (int m = 0; m < LE; ++m)
+                            if (F::uses(j, m))
+                                v = f2_fma(f2_make(qt[m], qt[m]),
+                                           f2_make(G[(f * ND + j) * LE + m], G[((f + 1) * ND + j) * LE + m]), v);
+                        f2_get(v, u[j][f], u[j][f + 1]);
                     }
+                } else {
+                    float v = qf[j];
+#pragma unroll
+                    for (int m = 0; m < LE; ++m)
+                        if (F::uses(j, m)) v = __fmaf_rn(qt[m], G[j * LE + m], v);
+                    u[j][0] = v;
                 }
-                const unsigned unsb = __ballot_sync(kFull, act && uns);
-                if (unsb) {
-                    // rare: the lanes whose screen was unsure take the FP64 definition; the
-                    // difference to what was counted is added directly to the cell's counters
-                    unsigned m64u = 0;
-                    if ((unsb >> lane) & 1) {
-                        unsigned m32u = 0, m32l = 0;
-#pragma unroll
-                        for (int fs = 0; fs < NFS; ++fs) {
-                            float u[ND];
-                            partial32<FAM>(qf, qt, G, fs, u);
-#pragma unroll
-                            for (int ds = 0; ds < (1 << ND); ++ds) {
-                                const int s = fs | (ds << F::K);
-                                bool ub, lb, un = false;
-                                screen<FAM>(ds, u, hs, Rlo, Rhi, Llo, Lhi, ub, lb, un);
-                                m32u |= (unsigned)ub << s;
-                                m32l |= (unsigned)lb << s;
-                            }
-                        }
-                        const uint2 m64 = eval64_words<FAM, Q16>(&c.P, &c.lev, rec_words_of<NW>(w), g64);
-                        m64u = m64.x;
-                        nrechk += nvslot;
-                        const unsigned valid = (1u << NS) - 1u;
-                        for (unsigned d = ((m32u ^ m64.x) | (m32l ^ m64.y)) & valid; d; d &= d - 1) {
-                            int s = __ffs(d) - 1;
-                            int du = (int)((m64.x >> s) & 1) - (int)((m32u >> s) & 1);
-                            int dl = (int)((m64.y >> s) & 1) - (int)((m32l >> s) & 1);
-                            uint32_t *bc = c.cnt + ((size_t)cl * NS + s) * 3;
-                            if (du) {
-                                atomicAdd(bc, (unsigned)(du * (int)mult));
-                                atomicAdd(bc + 2, (unsigned)du);
-                            }
-                            if (dl) atomicAdd(bc + 1, (unsigned)(dl * (int)mult));
-                        }
-                    }
-#pragma unroll
-                    for (int s = 0; s < NS; ++s)
-                        bw[s] = (bw[s] & ~unsb) | __ballot_sync(kFull, ((unsb >> lane) & 1) && ((m64u >> s) & 1));
-                }
-            } else {
-                // plain FP64: every record by the definition
-                uint2 m64 = make_uint2(0u, 0u);
-                if (act) m64 = eval64_words<FAM, Q16>(&c.P, &c.lev, rec_words_of<NW>(w), g64);
+            }
+            unsigned bu[NS], bl[NS];
+            test_children<ND, NFS, DM, LB>(u, hs, negR2, negL2, near, nearL, bu, bl);
+            const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
+            const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, negR2, near, nearL)) & act;
+            if (unsb) {                                             // rare: left to the definition
 #pragma unroll
                 for (int s = 0; s < NS; ++s) {
-                    bool ub = (m64.x >> s) & 1, lb = (m64.y >> s) & 1;
-                    const unsigned bb = __ballot_sync(kFull, ub);
-                    bw[s] = bb;
-                    if constexpr (!WEIGHTED) {
-                        if (ub) pu[s >> 2] += 1u << (8 * (s & 3));
-                        if (lb) pl[s >> 2] += 1u << (8 * (s & 3));
-                    } else {
-                        wu[s] += __reduce_add_sync(kFull, ub ? mult : 0u);
-                        wl[s] += __reduce_add_sync(kFull, lb ? mult : 0u);
-                        wn[s] += __popc(bb);
-                    }
+                    bu[s] &= ~unsb;
+                    bl[s] &= ~unsb;
                 }
+                if (lane == 0) c.uns[atomicAdd(&c.sc->n_uns, 1u)] = make_uint2((unsigned)tt, unsb);
             }
-            // the tile's ballots, one word per child slot (0 for slots that do not exist)
             if (lane == 0) {
-                uint4 *bp = reinterpret_cast<uint4 *>(c.ballot + (size_t)(tile - c.t0) * NS);
-#pragma unroll
-                for (int q = 0; q < NS / 4; ++q) bp[q] = make_uint4(bw[4 * q], bw[4 * q + 1], bw[4 * q + 2], bw[4 * q + 3]);
+                store_row<NS>(c.ballot + (size_t)tt * NS, bu);
+                if constexpr (LB) store_row<NS>(c.lballot + (size_t)tt * NS, bl);
             }
         }
-        // a warp's byte counters gain at most 32 per tile and group: drain them before
-        // they could carry
-        if (!WEIGHTED) drain();
-        __syncthreads();                                            // buffer b is free again
     }
-    if (gfail >= 0 && threadIdx.x == 0) {
-        // the copies of groups gfail and gfail + 1 (no later one was issued) may still
-        // be in flight: wait for them, bounded, before the block's shared memory is
-        // released
-        const int64_t ge = gfail + 2 < g1 ? gfail + 2 : g1;
-        for (int64_t g = gfail; g < ge; ++g) {
-            const int b = (int)((g - g0) & 1);
-            if (!mbar_wait(&s_bar[b], (unsigned)(((g - g0) >> 1) & 1), GV_SPIN_LIMIT, &c.sc->err)) break;
-        }
-    }
-    flush();
-    ntest = __reduce_add_sync(kFull, lane == 0 ? ntest : 0u);
-    nrec = __reduce_add_sync(kFull, lane == 0 ? nrec : 0u);
-    nrechk = __reduce_add_sync(kFull, nrechk);
-    if (lane == 0) {
-        if (ntest) atomicAdd(&c.sc->tests, (unsigned long long)ntest);
-        if (nrec) atomicAdd(&c.sc->records, (unsigned long long)nrec);
-        if (nrechk) atomicAdd(&c.sc->rechecks, (unsigned long long)nrechk);
+    if (lane == 0 && nrec) {
+        atomicAdd(&c.sc->records, (unsigned long long)nrec);
+        atomicAdd(&c.sc->tests, (unsigned long long)nrec * NS);
     }
 }
 
-#define GV_DISPATCH(fam, CALL)                                                   \
-    switch (fam) {                                                               \
-    case FAM_LINE2D: { constexpr int FAMV = FAM_LINE2D; CALL; } break;           \
-    case FAM_PLANE3D_SPH: { constexpr int FAMV = FAM_PLANE3D_SPH; CALL; } break; \
-    case FAM_POSE3DOF: { constexpr int FAMV = FAM_POSE3DOF; CALL; } break;       \
-    case FAM_RAYS3D: { constexpr int FAMV = FAM_RAYS3D; CALL; } break;           \
-    default: break;                                                              \
+// a persistent grid: as many blocks as are resident (4 per SM), fewer when there are not
+// two tiles per warp
+template <int FAM, bool Q16, int KF, int DM>
+static void launch_kd(const Chunk &c, cudaStream_t st) {
+    if constexpr (KF <= Fam<FAM>::K && DM < (1 << Fam<FAM>::ND) && (KF || DM)) {
+        const int64_t nt = c.t1 - c.t0;
+        const int64_t want = (int64_t)sm_count() * 4, need = (nt + 15) / 16;
+        const unsigned g = (unsigned)(want < need ? want : need);
+        if (c.lb) k_count<FAM, Q16, KF, DM, true><<<g, 256, 0, st>>>(c);
+        else k_count<FAM, Q16, KF, DM, false><<<g, 256, 0, st>>>(c);
     }
+}
 
-// Persistent grid: as many blocks as fit on the device at once (kernel occupancy
-// at the shared memory the records take), at most one per group.
+template <int FAM, bool Q16>
+static void launch_fam(const Chunk &c, cudaStream_t st) {
+    switch (c.kf * 4 + c.dm) {
+    case 1: launch_kd<FAM, Q16, 0, 1>(c, st); break;
+    case 2: launch_kd<FAM, Q16, 0, 2>(c, st); break;
+    case 3: launch_kd<FAM, Q16, 0, 3>(c, st); break;
+    case 4: launch_kd<FAM, Q16, 1, 0>(c, st); break;
+    case 5: launch_kd<FAM, Q16, 1, 1>(c, st); break;
+    case 6: launch_kd<FAM, Q16, 1, 2>(c, st); break;
+    case 7: launch_kd<FAM, Q16, 1, 3>(c, st); break;
+    case 8: launch_kd<FAM, Q16, 2, 0>(c, st); break;
+    case 9: launch_kd<FAM, Q16, 2, 1>(c, st); break;
+    default: break;
+    }
+}
 
 void launch_count(const Chunk &c, cudaStream_t st) {
-    const int64_t nt = c.t1 - c.t0;
-    if (nt <= 0) return;
-    if (c.P.d > 3) {
-        launch_count_wide(c, st);
-        return;
-    }
-    const int64_t ng = (nt + kBlockTiles - 1) / kBlockTiles;
-    const bool w = c.in.mult != nullptr;
-#define GV_COUNT(Q16, PREC)                                                                                   \
-    {                                                                                                          \
-        constexpr int NW = rec_words(Fam<FAMV>::NFP, Q16);                                                     \
-        if (w) launch_persistent((const void *)k_count<FAMV, Q16, PREC, true>, count_smem_bytes<NW>(), ng, c, st);          \
-        else launch_persistent((const void *)k_count<FAMV, Q16, PREC, false>, count_smem_bytes<NW>(), ng, c, st);           \
-    }
-    if (c.precision == 0) {
-        GV_DISPATCH(c.P.fam, GV_COUNT(false, 0));
-    } else if (c.lev.q16) {
-        GV_DISPATCH(c.P.fam, GV_COUNT(true, 1));
-    } else {
-        GV_DISPATCH(c.P.fam, GV_COUNT(false, 1));
+    if (c.t1 <= c.t0) return;
+    if (c.precision == 0) return launch_count_exact(c, st);
+    if (c.P.d > 3) return launch_count_wide(c, st);
+#define GV_COUNT(FAMV)                                  \
+    if (c.lev.q16) launch_fam<FAMV, true>(c, st);       \
+    else launch_fam<FAMV, false>(c, st)
+    switch (c.P.fam) {
+    case FAM_LINE2D: GV_COUNT(FAM_LINE2D); break;
+    case FAM_PLANE3D_SPH: GV_COUNT(FAM_PLANE3D_SPH); break;
+    case FAM_POSE3DOF: GV_COUNT(FAM_POSE3DOF); break;
+    case FAM_RAYS3D: GV_COUNT(FAM_RAYS3D); break;
+    default: break;
     }
 #undef GV_COUNT
+    launch_recheck(c, st);
 }
 
 }  // namespace gv

@@ -58,7 +58,9 @@ struct Level {                 // tests of the children of a level-l cell
     float lam_c[4];            // family-specific scale of the Lipschitz term (see Fam::radius32)
     float rho2;                // family-specific ratio of essential steps (planes: (s_t,z / s_t,x)^2)
     float Lc[GV_MAXD];         // eps_j - A1_j (lower-bound radius)
-    // set per solve, once the input's parameter ranges are known
+    // set per solve, once the input's parameter ranges are known: the screen's band
+    float kappa[GV_MAXD];      // undecided by the radius: |y^2 - R^2| < kappa R^2
+    float bandL[GV_MAXD], bandL0[GV_MAXD];  // undecided by the lower-bound radius: | |y| - Lc | < bandL R + bandL0
     float qt_max[GV_MAXT];     // bound on |q_t,m| of this level's records
     int q16;                   // this level's records hold 16-bit fields
     int q16_next;              // the next level's records hold 16-bit fields
@@ -150,6 +152,18 @@ __device__ __forceinline__ int64_t cell_coord(const Problem &P, uint64_t key, in
 
 __device__ __forceinline__ double cell_center(const Problem &P, const double *h, int j, int64_t i) {
     return dadd(P.lo[j], dmul((double)(2 * i + 1), h[j]));
+}
+
+// the low bits of s spread over the set bits of mask (a child slot's coordinate bits)
+__device__ __forceinline__ int expand_bits(int s, int mask) {
+    int r = 0;
+#pragma unroll
+    for (int j = 0; j < GV_MAXD; ++j)
+        if ((mask >> j) & 1) {
+            r |= (s & 1) << j;
+            s >>= 1;
+        }
+    return r;
 }
 
 __device__ __forceinline__ uint64_t child_key(const Problem &P, uint64_t key, int l, int slot) {
@@ -605,10 +619,17 @@ template <> struct Fam<FAM_RADIAL5DOF> {
 // coefficients rounded once from FP64, so |y - y_exact| <= 10 u M_j (u = 2^-24; the
 // FP64 definition's own error is below 2^-48 M_j); the FP32 radius (at most three
 // approximate square roots of at most 4 ulp, a few multiply-adds, constants rounded
-// once) is within 13 u R of the exact radius.
+// once) is within 13 u R of the exact radius.  Squaring both adds at most 2 u R^2.
 // A comparison of |y| with R (or with the lower-bound radius) is decided in FP32
 // only when it clears kBandTest (M_j + R); a snap only when y is kBandSnap M_j away
 // from a rounding tie: both about twice the bound.
+// The count pass bounds M_j by kMagPerRadius R_j on every level below the root: such a
+// record passed the UB test one level up, so |q_f| is at most that radius, which with
+// half-widths and Lipschitz terms twice this level's, a re-snapped t (its change moves
+// the radius by less than eps) and the snap's half step is at most 3 R; |H| <= R; and
+// sum |q_t| Gmax is at most twice the Lipschitz term of R (|q_x| + |q_y| <= sqrt(2)
+// |q_xy| and the like), 2 R.  The root's records take the input's largest fields.
+constexpr float kMagPerRadius = 7.0f;
 constexpr float kU32 = 5.9604645e-08f;
 constexpr float kBandTest = 24.0f * kU32;
 constexpr float kBandSnap = 12.0f * kU32;

@@ -71,7 +71,6 @@ struct vote_ctx {
     Problem P;
     Level lev[GV_MAXL];
     double h_leaf[GV_MAXD];
-    int ns = 0;                // 2^d child slots
     int device = 0;
     cudaStream_t stream = 0;
     int precision = 1, prune = 1, group = 0;
@@ -100,7 +99,8 @@ struct vote_ctx {
     LevelStore ls[GV_MAXL + 1];
     LevelStore beam;           // the selected cells of one level, during the dive
     DevBuf beam_sel, beam_src;
-    DevBuf levs_dev, path, scal, alive, geo64, geo32, geo32lo, cnt, tinfo, ballot, tdst, child_idx, cursor, keepflag, recn, bsums;
+    DevBuf levs_dev, path, scal, alive, geo64, geo32, geo32lo, cnt, tinfo, ballot, lballot, uns, off, cbase, child_idx;
+    DevBuf keepflag, recn, bsums;
     DevBuf tr_level, tr_key, tr_ub, tr_lb, surf_tmp, mask_tmp;
     DevBuf ss_partial, ss_io;  // soft score: block partials; point [d] + outputs [d] + grad_out [1]
     DevBuf g_table, g_owner, g_newpos, g_ccount, g_ccur, g_rbeg, g_rec, g_mult, g_tile;
@@ -394,7 +394,8 @@ static void finalize_levels(vote_ctx *c, const unsigned *qmax) {
     double rprev[GV_MAXD] = {};
     for (int l = 0; l < P.L; ++l) {
         Level &v = c->lev[l];
-        double T[GV_MAXT], lam[GV_MAXD * GV_MAXD], qtb[GV_MAXT];
+        double T[GV_MAXT], lam[GV_MAXD * GV_MAXD], qtb[GV_MAXT], sigma[GV_MAXT];
+        family_sigma(P.fam, v.h, sigma);
         bool fits = c->precision == 1 && l >= 1;
         for (int m = 0; m < P.le; ++m) {
             double ratio = v.s_t[m] / c->lev[0].s_t[m];                 // a power of two >= 1
@@ -409,6 +410,18 @@ static void finalize_levels(vote_ctx *c, const unsigned *qmax) {
             for (int i = 0; i < P.k; ++i) R += lam[j * P.k + i] * v.h1[i];
             R = (R + v.A1[j]) * 1.001;
             double qfb = l == 0 ? (double)qmax[j] + 1.0 : std::ceil(rprev[j] / P.s_f[j]) + 1.0;
+            // the screen's band (kBandTest (M + R), and M + Lc for the lower bound), as a
+            // multiple of the record's radius: M <= mag R
+            double mag = kMagPerRadius;
+            if (l == 0) {
+                double M = qfb + v.Hs[j];
+                for (int m = 0; m < P.le; ++m) M += qtb[m] * v.gscale[j][m] * sigma[m];
+                mag = M / v.rc0[j];
+            }
+            const double bandR = 1.01 * kBandTest * (mag + 1.0);
+            v.kappa[j] = (float)(1.01 * bandR * (2.0 + bandR));
+            v.bandL[j] = (float)(1.01 * kBandTest * mag);
+            v.bandL0[j] = (float)(1.01 * kBandTest) * v.Lc[j];
             fits &= qfb <= 32000.0;
             rprev[j] = R;
         }
@@ -579,11 +592,14 @@ static void ev_collect(vote_ctx *c) {
 static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     const Problem &P = c->P;
     LevelStore &S = beam ? c->beam : c->ls[l];
-    const int ns = c->ns;
     const Level &lev = c->lev[l];
-    int nvalid = 0;
-    for (int s = 0; s < ns; ++s)
-        if (!(s & ~lev.split_mask)) ++nvalid;
+    int kf = 0, dm = lev.split_mask >> P.k, lns = 0;
+    for (int j = 0; j < P.d; ++j) {
+        const int split = (lev.split_mask >> j) & 1;
+        lns += split;
+        if (j < P.k) kf += split;
+    }
+    const int ns = 1 << lns, nfs = 1 << kf;
     // chunk: cells [c0, c1) from the top of the stack, about chunk_records records
     const int64_t c1 = S.ncells, r1 = S.nrecs;
     int64_t avg = S.nrecs / (S.ncells > 0 ? S.ncells : 1);
@@ -607,24 +623,22 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     }
     nvtxRangePushA("expand_chunk");
     const int nc = (int)(c1 - c0);
-    const int nfs = 1 << P.k;
     const int NB = family_nb(P.fam);
     const int gf = geo32_floats(nfs, P.nd, P.le);
     const size_t nch = (size_t)nc * ns;
+    const size_t cnt_arrays = c->group ? 3 : 2;
     TRY(ensure(c, c->alive, nc));
     TRY(ensure(c, c->geo64, (size_t)nc * nfs * NB * 8));
     TRY(ensure(c, c->geo32, (size_t)nc * gf * 4));
     TRY(ensure(c, c->geo32lo, (size_t)nc * nfs * P.nd * P.le * 4));
-    TRY(ensure(c, c->cnt, nch * 12));
+    TRY(ensure(c, c->cnt, nch * 4 * cnt_arrays));
     TRY(ensure(c, c->child_idx, nch * 4));
-    TRY(ensure(c, c->cursor, nch * 4));
+    TRY(ensure(c, c->cbase, nch * 8));
     TRY(ensure(c, c->keepflag, nch * 4));
     TRY(ensure(c, c->recn, nch * 4));
     TRY(ensure(c, c->bsums, ((nch + 255) / 256) * 16 + 16));
-    if (!lev.leaf_children) TRY(ensure_level(c, c->ls[l + 1], l + 1, 0, (size_t)c->ls[l + 1].ncells + nch));    // records: sized below, exactly
-    CK(cudaMemsetAsync(c->cnt.p, 0, nch * 12, c->stream));
-    CK(cudaMemsetAsync(c->cursor.p, 0, nch * 4, c->stream));
-    CK(cudaMemsetAsync(&dsc(c)->n_cells, 0, 16, c->stream));
+    if (!lev.leaf_children) TRY(ensure_level(c, c->ls[l + 1], l + 1, 0, (size_t)c->ls[l + 1].ncells + nch));
+    CK(cudaMemsetAsync(c->cnt.p, 0, nch * 4 * cnt_arrays, c->stream));
 
     Chunk ch;
     std::memset(&ch, 0, sizeof(ch));
@@ -633,6 +647,12 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     ch.cells = cell_view(S);
     ch.c0 = c0;
     ch.nc = nc;
+    ch.ns = ns;
+    ch.lns = lns;
+    ch.nfs = nfs;
+    ch.kf = kf;
+    ch.dm = dm;
+    ch.gf = gf;
     ch.in = rec_view(c, S);
     ch.in_rbeg = (const uint64_t *)S.rbeg.p;
     ch.in_rcnt = (const uint32_t *)S.rcnt.p;
@@ -643,9 +663,11 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     ch.geo64 = (double *)c->geo64.p;
     ch.geo32 = (float *)c->geo32.p;
     ch.geo32lo = (float *)c->geo32lo.p;
-    ch.cnt = (uint32_t *)c->cnt.p;
+    ch.crec = (uint32_t *)c->cnt.p;
+    ch.clb = ch.crec + nch;
+    ch.cub = c->group ? ch.crec + 2 * nch : ch.crec;
     ch.child_idx = (int32_t *)c->child_idx.p;
-    ch.cursor = (uint32_t *)c->cursor.p;
+    ch.cbase = (unsigned long long *)c->cbase.p;
     ch.sc = dsc(c);
     if (c->trace_cap > 0) {
         ch.trace.cap = (unsigned long long)c->trace_cap;
@@ -656,6 +678,8 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     }
     ch.prune = c->prune;
     ch.precision = c->precision;
+    // leaves need no lower bound: their own counts are one
+    ch.lb = !lev.leaf_children || c->trace_cap > 0;
     ch.spin = c->spin_limit;
 
     const int rb = rec_bytes_at(c, l);
@@ -703,10 +727,17 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
         ch.t1 = gs / 32;
     }
     const int64_t nt = ch.t1 - ch.t0;
-    TRY(ensure(c, c->tinfo, (size_t)(nt > 0 ? nt : 1) * 8 + 16));
-    TRY(ensure(c, c->ballot, (size_t)(nt > 0 ? nt : 1) * ns * 4));
+    const size_t ntp = (size_t)(nt > 0 ? nt : 1);
+    TRY(ensure(c, c->tinfo, ntp * 8));
+    TRY(ensure(c, c->ballot, ntp * ns * 4 + 16));      // bulk copies round up to 16 bytes
+    TRY(ensure(c, c->off, ntp * ns * 4 + 16));
+    if (ch.lb) TRY(ensure(c, c->lballot, ntp * ns * 4));
+    if (c->precision == 1) TRY(ensure(c, c->uns, ntp * 8));
     ch.tinfo = (int2 *)c->tinfo.p;
     ch.ballot = (uint32_t *)c->ballot.p;
+    ch.lballot = (uint32_t *)c->lballot.p;
+    ch.uns = (uint2 *)c->uns.p;
+    ch.off = (uint32_t *)c->off.p;
     if (!lev.leaf_children) {
         ch.next_cells = cell_view(c->ls[l + 1]);
         ch.next_c0 = c->ls[l + 1].ncells;
@@ -719,7 +750,7 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     ev_mark(c, VOTE_K_CELL_GEO);
     launch_count(ch, c->stream);
     ev_mark(c, VOTE_K_TEST_COUNT);
-    launch_child_lbmax(ch, c->stream);
+    launch_tile_scan(ch, c->stream);
     launch_child_alloc(ch, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p, (unsigned long long *)c->bsums.p,
                        c->stream);
     ev_mark(c, VOTE_K_CHILDREN);
@@ -728,7 +759,7 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     c->kbytes[VOTE_K_CELL_GEO] += (double)nc * (8 + 4);
     CK(cudaGetLastError());
     c->stats.chunks++;
-    c->stats.launches += lev.leaf_children ? 5 : 7;
+    c->stats.launches += (lev.leaf_children ? 5 : 7) + (c->precision == 1);
     c->stats.cells += nc;
     c->lv_cells[l] += nc;
     c->lv_recs[l] += nt * 32;
@@ -739,7 +770,7 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
             std::fprintf(stderr, "[vote] step %lld level %d: %lld cells, %lld tiles, count %.0f B, leaves\n",
                          (long long)c->stats.chunks - 1, l, (long long)nc, (long long)nt,
                          (double)nt * 32 * rb + (double)nt * ns * 4);
-        c->stats.leaves += (int64_t)nc * nvalid;
+        c->stats.leaves += (int64_t)nch;
         nvtxRangePop();
         return VOTE_OK;
     }
@@ -749,18 +780,13 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     int64_t new_cells = (int64_t)c->h_sc->n_cells, new_slots = (int64_t)c->h_sc->n_recs;
     if (new_slots > 0) {
         TRY(ensure_level(c, N, l + 1, (size_t)(N.nrecs + new_slots), 0));
-        TRY(ensure(c, c->tdst, (size_t)nt * ns * 8));
-        ch.out = rec_view(c, c->ls[l + 1]);
-        ch.tdst = (unsigned long long *)c->tdst.p;
+        ch.out = rec_view(c, N);
         ev_mark(c, -1);
-        launch_next_tiles(ch, new_cells, c->stream);
-        launch_tile_dst(ch, c->stream);
-        ev_mark(c, VOTE_K_CHILDREN);
         if (!launch_emit(ch, c->stream)) {
             set_err("internal: no emit pass for record formats %d -> %d", lev.q16, lev.q16_next);
             return VOTE_EINTERNAL;
         }
-        c->stats.launches += 3;
+        c->stats.launches += 1;
         ev_mark(c, VOTE_K_TEST_EMIT);
         c->kbytes[VOTE_K_TEST_EMIT] += (double)nt * 32 * rb + (double)nt * ns * 4 +
                                        (double)new_slots * rec_bytes_at(c, l + 1);
@@ -1048,7 +1074,6 @@ vote_status vote_create(int family, int d, int k, const double *eps, const doubl
         delete c;
         return s;
     }
-    c->ns = 1 << d;
     // step size measured fastest on GB300 (1e6-surface workloads): planes keep almost
     // every cell above the bound, so larger steps only remove per-step overhead;
     // 3DoF prunes well and needs fine depth-first steps
@@ -1512,8 +1537,7 @@ void vote_destroy(vote_ctx *c) {
         release(c, s.key); release(c, s.rbeg); release(c, s.rcnt); release(c, s.ub); release(c, s.lb);
     }
     DevBuf *bufs[] = {&c->levs_dev, &c->path, &c->scal, &c->alive, &c->geo64, &c->geo32, &c->geo32lo, &c->cnt, &c->tinfo,
-                      &c->ballot, &c->tdst,
-                      &c->child_idx, &c->cursor, &c->keepflag, &c->recn, &c->bsums, &c->tr_level, &c->tr_key,
+                      &c->ballot, &c->lballot, &c->uns, &c->off, &c->cbase, &c->child_idx, &c->keepflag, &c->recn, &c->bsums, &c->tr_level, &c->tr_key,
                       &c->tr_ub, &c->tr_lb, &c->surf_tmp, &c->mask_tmp, &c->ss_partial,
                       &c->ss_io, &c->g_table, &c->g_owner, &c->g_newpos, &c->g_ccount, &c->g_ccur,
                       &c->g_rbeg, &c->g_rec, &c->g_mult, &c->g_tile, &c->beam_sel, &c->beam_src};

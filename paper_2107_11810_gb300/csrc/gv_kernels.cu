@@ -7,8 +7,10 @@
 //                 family's basis functions from the cell centre to each child
 //                 centre (own sin/cos, FP64)
 //   (k_count, k_emit: the proximity test itself, in gv_count.cu and gv_emit.cu)
-//   k_child_*     best lower bound, pruning, allocation of surviving children,
-//                 leaf argmax as a packed 64-bit atomicMax
+//   k_tile_scan   per child its counts, per tile and child its records' place, best
+//                 lower bound, all from the count pass's ballots
+//   k_child_*     pruning, allocation of surviving children, leaf argmax as a packed
+//                 64-bit atomicMax
 //   k_path_geo,   replay of every original surface along one root-to-cell path:
 //   k_replay      inlier mask of the best leaf and per-cell counts
 #include <cstdio>
@@ -126,8 +128,7 @@ __device__ __forceinline__ void parent_psi(const Problem &P, const Level &lev, u
     if (!F::LINEAR_BASIS) F::basis(P, cpar, psi);
 }
 
-// One thread per (cell, free-coordinate child slot fs); the 2^k threads of a cell
-// are consecutive lanes.  Writes the FP64 basis changes (for the exact recheck) and
+// One thread per (cell, free slot fs); the nfs threads of a cell are consecutive lanes.  Writes the FP64 basis changes (for the exact recheck) and
 // the screen's coefficients G[fs][j][m] = coef_jm(dpsi) * s_t,m / s_f,j rounded to
 // FP32, their remainders (G64 - G, rounded to FP32: the double-float tier's low
 // parts; G64 is exact, coef only copies or negates and s_t / s_f is a power of two),
@@ -138,12 +139,12 @@ __device__ __forceinline__ void parent_psi(const Problem &P, const Level &lev, u
 template <int FAM>
 __global__ void k_cell_geo(Chunk c) {
     using F = Fam<FAM>;
-    constexpr int NF = 1 << F::K;
-    constexpr int GF = geo32_floats(NF, F::ND, F::LE);
-    static_assert(32 % NF == 0, "a cell's threads must lie in one warp");
+    static_assert(32 % (1 << F::K) == 0, "a cell's threads must lie in one warp");
+    const int NF = c.nfs, GF = c.gf;
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int cell = gid / NF, fs = gid % NF;
+    const int cell = gid >> c.kf, fs = gid & (NF - 1);
     const bool in = cell < c.nc;
+    if (gid == 0) c.sc->n_uns = 0u;                  // this step's recheck queue
     const Problem &P = c.P;
     const Level &lev = c.lev;
     float ga[F::ND * F::LE];
@@ -156,13 +157,11 @@ __global__ void k_cell_geo(Chunk c) {
             c.alive[cell] = c.cells.ub[c.c0 + cell] >= thr ? 1 : 0;
         }
         double dpsi[F::NB];
-#pragma unroll
-        for (int m = 0; m < F::NB; ++m) dpsi[m] = 0.0;
-        if (!(fs & ~lev.split_mask & (NF - 1))) {
+        {
             uint64_t key = c.cells.key[c.c0 + cell];
             double psi_par[F::NB];
             parent_psi<FAM>(P, lev, key, psi_par);
-            child_dpsi<FAM>(P, lev, key, fs, psi_par, dpsi);
+            child_dpsi<FAM>(P, lev, key, expand_bits(fs, lev.split_mask & ((1 << F::K) - 1)), psi_par, dpsi);
         }
 #pragma unroll
         for (int m = 0; m < F::NB; ++m) c.geo64[((size_t)cell * NF + fs) * F::NB + m] = dpsi[m];
@@ -179,7 +178,6 @@ __global__ void k_cell_geo(Chunk c) {
             else if (gx != 0.0 && ge > kNoExp) ge = min(ge, lowbit_exp(gx));
         }
     }
-#pragma unroll
     for (int o = 1; o < NF; o <<= 1) {
 #pragma unroll
         for (int x = 0; x < F::ND * F::LE; ++x) ga[x] = fmaxf(ga[x], __shfl_xor_sync(kFull, ga[x], o));
@@ -223,32 +221,21 @@ __device__ __forceinline__ unsigned long long block_excl_scan(unsigned long long
 // ---------------------------------------------------------------------------
 // A5 best lower bound, pruning, allocation of surviving children, leaf argmax
 // ---------------------------------------------------------------------------
-template <int NS>
-__global__ void k_child_lbmax(Chunk c) {
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    int cl = idx / NS, s = idx % NS;
-    unsigned v = 0;
-    if (cl < c.nc && !(s & ~c.lev.split_mask) && c.alive[cl]) v = c.cnt[(size_t)idx * 3 + 1];
-    v = __reduce_max_sync(kFull, v);
-    if ((threadIdx.x & 31) == 0 && v) atomicMax(&c.sc->best_lb, v);
-}
-
 // Phase A: per child of the chunk -- trace, pruning decision, leaf argmax, and
 // per-block totals of surviving children and their records.
-template <int NS>
 __global__ void __launch_bounds__(256) k_child_mark(Chunk c, uint32_t *keepflag, uint32_t *recn,
                                                     unsigned long long *bs_cells, unsigned long long *bs_recs) {
     const Problem &P = c.P;
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    int cl = idx / NS, s = idx % NS;
-    bool exists = cl < c.nc && !(s & ~c.lev.split_mask) && c.alive[cl];
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int cl = idx >> c.lns, s = idx & (c.ns - 1);
+    const bool exists = cl < c.nc && c.alive[cl];
     unsigned ub = 0, lb = 0, nrec = 0;
     uint64_t key = 0;
     if (exists) {
-        ub = c.cnt[(size_t)idx * 3];
-        lb = c.cnt[(size_t)idx * 3 + 1];
-        nrec = c.cnt[(size_t)idx * 3 + 2];
-        key = child_key(P, c.cells.key[c.c0 + cl], c.lev.l, s);
+        ub = c.cub[idx];
+        if (c.lb) lb = c.clb[idx];
+        nrec = c.crec[idx];
+        key = child_key(P, c.cells.key[c.c0 + cl], c.lev.l, expand_bits(s, c.lev.split_mask));
         if (c.trace.cap) {
             unsigned long long t = atomicAdd(&c.sc->trace_n, 1ull);
             if (t < c.trace.cap) {
@@ -271,7 +258,7 @@ __global__ void __launch_bounds__(256) k_child_mark(Chunk c, uint32_t *keepflag,
     }
     // a child's records start at a multiple of 32 (whole tiles)
     const unsigned slots = keep ? (nrec + 31u) & ~31u : 0u;
-    if (idx < c.nc * NS) {
+    if (idx < c.nc << c.lns) {
         keepflag[idx] = keep ? 1u : 0u;
         recn[idx] = slots;
     }
@@ -308,30 +295,31 @@ __global__ void __launch_bounds__(256) k_scan_sums(unsigned long long *a, unsign
 
 // Phase C: surviving children get consecutive cell indices and record ranges in
 // (parent, slot) order; recn holds the slots (record count rounded up to 32).
-template <int NS>
 __global__ void __launch_bounds__(256) k_child_write(Chunk c, const uint32_t *keepflag, const uint32_t *recn,
                                                      const unsigned long long *bs_cells,
                                                      const unsigned long long *bs_recs) {
-    int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    bool in = idx < c.nc * NS;
+    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = idx < c.nc << c.lns;
     unsigned keep = in ? keepflag[idx] : 0u;
     unsigned nrec = in ? recn[idx] : 0u;
     unsigned long long tc, tr;
     unsigned long long ec = block_excl_scan(keep, &tc);
     unsigned long long er = block_excl_scan(nrec, &tr);
     if (!in) return;
-    if (keep) {
-        int cl = idx / NS, s = idx % NS;
-        unsigned long long ci = c.next_c0 + bs_cells[blockIdx.x] + ec;
-        c.next_cells.key[ci] = child_key(c.P, c.cells.key[c.c0 + cl], c.lev.l, s);
-        c.next_cells.rbeg[ci] = c.next_r0 + bs_recs[blockIdx.x] + er;
-        c.next_cells.rcnt[ci] = c.cnt[(size_t)idx * 3 + 2];
-        c.next_cells.ub[ci] = c.cnt[(size_t)idx * 3];
-        c.next_cells.lb[ci] = c.cnt[(size_t)idx * 3 + 1];
-        c.child_idx[idx] = (int32_t)ci;
-    } else {
-        c.child_idx[idx] = -1;
+    if (!keep) {
+        c.cbase[idx] = ~0ull;
+        return;
     }
+    const int cl = idx >> c.lns, s = idx & (c.ns - 1);
+    const unsigned long long ci = c.next_c0 + bs_cells[blockIdx.x] + ec;
+    const unsigned long long rb = c.next_r0 + bs_recs[blockIdx.x] + er;
+    c.next_cells.key[ci] = child_key(c.P, c.cells.key[c.c0 + cl], c.lev.l, expand_bits(s, c.lev.split_mask));
+    c.next_cells.rbeg[ci] = rb;
+    c.next_cells.rcnt[ci] = c.crec[idx];
+    c.next_cells.ub[ci] = c.cub[idx];
+    c.next_cells.lb[ci] = c.lb ? c.clb[idx] : 0u;
+    c.child_idx[idx] = (int32_t)ci;
+    c.cbase[idx] = rb;
 }
 
 // ---------------------------------------------------------------------------
@@ -512,68 +500,128 @@ __global__ void __launch_bounds__(256) k_beam_gather(RecView in, RecView out, Ce
 // stream their inputs with bulk copies and never chase a pointer per tile.
 // ---------------------------------------------------------------------------
 
-// per tile: the chunk-local cell (-1 if it was pruned) and how many of its 32 lanes
-// hold records
+// per tile: the chunk-local cell (-1 if it was pruned), how many of its 32 lanes hold
+// records, whether it is the cell's first or last tile
 __global__ void k_tile_info(Chunk c) {
     const int64_t t = c.t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= c.t1) return;
+    if (c.sc->err & kErrTimeout) {                   // an emit pass gave up: its tiles name no cells
+        c.tinfo[t - c.t0] = make_int2(-1, 0);
+        return;
+    }
     const int64_t cell = (int64_t)c.in.tile_cell[t];
     const int cl = (int)(cell - c.in_c0);
-    const int64_t left = (int64_t)c.in_rbeg[cell] + (int64_t)c.in_rcnt[cell] - 32 * t;
-    c.tinfo[t - c.t0] = make_int2(c.alive[cl] ? cl : -1, left < 32 ? (int)left : 32);
+    const int64_t r0 = (int64_t)c.in_rbeg[cell], left = r0 + (int64_t)c.in_rcnt[cell] - 32 * t;
+    c.tinfo[t - c.t0] = make_int2(c.alive[cl] ? cl : -1, (left < 32 ? (int)left : 32) | (32 * t == r0 ? kTileFirst : 0) |
+                                                             (left <= 32 ? kTileLast : 0));
 }
 
-// the next level's tile -> cell table: one warp per new cell writes its tiles
-__global__ void k_next_tiles(CellView next, RecView out, int64_t c0, int64_t ncells) {
-    const int64_t cell = c0 + ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
+// Counts and output positions from the ballots.  A warp takes 32 consecutive tiles,
+// one per lane, and per child slot a segmented scan over them (segments = runs of one
+// cell; UB-passing records in the low half of a word, LB-passing ones in the high
+// half): a tile's records get consecutive places in the child, after those of the
+// run's earlier tiles.  A run that is the whole cell owns the child's counters; any
+// other run reserves its places with one atomic on them.  Partial LB sums are valid
+// lower bounds, and each child's last addition returns its whole sum, so the best LB
+// is raised here.  W: child slots per load (2 or 4).
+template <int W>
+__global__ void __launch_bounds__(256) k_tile_scan(const __grid_constant__ Chunk c) {
     const int lane = threadIdx.x & 31;
-    if (cell >= c0 + ncells) return;
-    const int64_t t0 = (int64_t)(next.rbeg[cell] >> 5), nt = ((int64_t)next.rcnt[cell] + 31) >> 5;
-    for (int64_t i = lane; i < nt; i += 32) out.tile_cell[t0 + i] = (uint32_t)cell;
-}
-
-// Output positions of the emit pass.  A block takes 32 consecutive tiles;
-// warp w handles child slots w, w + 8, ... with one lane per tile: a segmented scan over the
-// tiles (segments = runs of one cell) gives every tile its offset inside the run,
-// the run's last lane reserves the run's records in the child with one atomic on
-// the child's cursor, and the run's base is broadcast back.  tdst[tile][s] = first
-// slot of the tile's records in child s, or ~0 when the tile writes none there.
-template <int NS>
-__global__ void __launch_bounds__(256) k_tile_dst(Chunk c) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    constexpr int NWARP = NS < 8 ? NS : 8;
-    if (w >= NWARP) return;
-    const int64_t t = c.t0 + (int64_t)blockIdx.x * 32 + lane;
-    const bool in = t < c.t1;
-    const int cl = in ? c.tinfo[t - c.t0].x : -1;
-    // segments: maximal runs of lanes with the same cell
+    const int64_t nt = c.t1 - c.t0;
+    const int64_t t = (blockIdx.x * 8ll + (threadIdx.x >> 5)) * 32 + lane;
+    if (t - lane >= nt) return;                                          // uniform
+    const int2 ti = t < nt ? c.tinfo[t] : make_int2(-1, 0);
+    const int cl = ti.x;
     const int prev = __shfl_up_sync(kFull, cl, 1);
     const unsigned heads = __ballot_sync(kFull, lane == 0 || prev != cl);
     const int next = __shfl_down_sync(kFull, cl, 1);
     const unsigned tails = __ballot_sync(kFull, lane == 31 || next != cl);
     const int head = 31 - __clz(heads & ((2u << lane) - 1u));          // this lane's segment head
     const int tail = __ffs(tails & ~((1u << lane) - 1u)) - 1;          // this lane's segment tail
+    const int yh = __shfl_sync(kFull, ti.y, head), yt = __shfl_sync(kFull, ti.y, tail);   // by every lane
+    const bool whole = (yh & kTileFirst) && (yt & kTileLast);
+    const bool last = lane == tail && cl >= 0;
+    const uint32_t *bp = c.ballot + (size_t)t * c.ns, *lp = c.lballot + (size_t)t * c.ns;
+    unsigned best = 0;
 #pragma unroll 1
-    for (int s = w; s < NS; s += NWARP) {
-        unsigned n = 0;
-        int ci = -1;
-        if (cl >= 0) {
-            ci = c.child_idx[(size_t)cl * NS + s];
-            if (ci >= 0) n = __popc(c.ballot[(size_t)(t - c.t0) * NS + s]);
-        }
-        // inclusive scan of n inside the segment
-        unsigned x = n;
+    for (int s0 = 0; s0 < c.ns; s0 += W) {
+        unsigned bw[W], lw[W], of[W];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            unsigned y = __shfl_up_sync(kFull, x, o);
-            if (lane - o >= head) x += y;
+        for (int q = 0; q < W; ++q) bw[q] = lw[q] = 0u;
+        if (cl >= 0) {
+            if constexpr (W == 4) {
+                const uint4 b = *reinterpret_cast<const uint4 *>(bp + s0);
+                bw[0] = b.x; bw[1] = b.y; bw[2] = b.z; bw[3] = b.w;
+                if (c.lb) {
+                    const uint4 l = *reinterpret_cast<const uint4 *>(lp + s0);
+                    lw[0] = l.x; lw[1] = l.y; lw[2] = l.z; lw[3] = l.w;
+                }
+            } else {
+                const uint2 b = *reinterpret_cast<const uint2 *>(bp + s0);
+                bw[0] = b.x; bw[1] = b.y;
+                if (c.lb) {
+                    const uint2 l = *reinterpret_cast<const uint2 *>(lp + s0);
+                    lw[0] = l.x; lw[1] = l.y;
+                }
+            }
         }
-        unsigned long long base = 0;
-        if (((tails >> lane) & 1) && cl >= 0 && ci >= 0 && x)
-            base = c.next_cells.rbeg[ci] + atomicAdd(&c.cursor[(size_t)cl * NS + s], x);
-        base = __shfl_sync(kFull, base, tail);
-        if (in) c.tdst[(size_t)(t - c.t0) * NS + s] = n ? base + (x - n) : ~0ull;
+#pragma unroll
+        for (int q = 0; q < W; ++q) {
+            const unsigned n = __popc(bw[q]);
+            unsigned x = n | ((unsigned)__popc(lw[q]) << 16);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned y = __shfl_up_sync(kFull, x, o);
+                if (lane - o >= head) x += y;
+            }
+            unsigned base = 0;
+            if (last) {
+                const size_t i = (size_t)cl * c.ns + s0 + q;
+                unsigned lb = x >> 16;
+                if (whole) {
+                    c.crec[i] = x & 0xffffu;
+                    if (c.lb) c.clb[i] = lb;
+                } else {
+                    if (x & 0xffffu) base = atomicAdd(c.crec + i, x & 0xffffu);
+                    if (lb) lb += atomicAdd(c.clb + i, lb);
+                }
+                best = lb > best ? lb : best;
+            }
+            base = __shfl_sync(kFull, base, tail);
+            of[q] = base + (x & 0xffffu) - n;
+        }
+        if (t < nt) {
+            if constexpr (W == 4) *reinterpret_cast<uint4 *>(c.off + (size_t)t * c.ns + s0) = make_uint4(of[0], of[1], of[2], of[3]);
+            else *reinterpret_cast<uint2 *>(c.off + (size_t)t * c.ns + s0) = make_uint2(of[0], of[1]);
+        }
     }
+    best = __reduce_max_sync(kFull, best);
+    if (lane == 0 && best > *(volatile unsigned *)&c.sc->best_lb) atomicMax(&c.sc->best_lb, best);
+}
+
+// The same with multiplicities (grouping): a warp per tile.
+__global__ void __launch_bounds__(256) k_tile_scan_weighted(const __grid_constant__ Chunk c) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nt = c.t1 - c.t0;
+    const int64_t t = blockIdx.x * 8ll + (threadIdx.x >> 5);
+    if (t >= nt) return;                                                 // uniform
+    const int2 ti = c.tinfo[t];
+    if (ti.x < 0) return;                                                // uniform
+    const uint32_t mult = lane < (ti.y & 63) ? c.in.mult[(c.t0 + t) * 32 + lane] : 0u;
+    unsigned best = 0;
+    for (int s = 0; s < c.ns; ++s) {
+        const size_t i = (size_t)ti.x * c.ns + s;
+        const unsigned b = c.ballot[(size_t)t * c.ns + s], l = c.lb ? c.lballot[(size_t)t * c.ns + s] : 0u;
+        const unsigned ub = __reduce_add_sync(kFull, (b >> lane) & 1u ? mult : 0u);
+        unsigned lb = __reduce_add_sync(kFull, (l >> lane) & 1u ? mult : 0u);
+        if (lane == 0) {
+            c.off[(size_t)t * c.ns + s] = b ? atomicAdd(c.crec + i, (unsigned)__popc(b)) : 0u;
+            if (ub) atomicAdd(c.cub + i, ub);
+            if (lb) lb += atomicAdd(c.clb + i, lb);
+            best = lb > best ? lb : best;
+        }
+    }
+    if (lane == 0 && best) atomicMax(&c.sc->best_lb, best);
 }
 
 // ---------------------------------------------------------------------------
@@ -652,6 +700,7 @@ __global__ void __launch_bounds__(256) k_replay(Problem P, const Level *__restri
 // A record slot of the chunk: its chunk-local cell, or -1 for the padding after a
 // cell's last record.
 __device__ __forceinline__ int slot_cell(const Chunk &c, int64_t r) {
+    if (c.sc->err & kErrTimeout) return -1;          // an emit pass gave up: its tiles name no cells
     int64_t cell = (int64_t)c.in.tile_cell[r >> 5];
     int cl = (int)(cell - c.in_c0);
     return r < (int64_t)c.in_rbeg[cell] + (int64_t)c.in_rcnt[cell] ? cl : -1;
@@ -792,7 +841,17 @@ void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t
 
 void launch_cell_geo(const Chunk &c, cudaStream_t st) {
     if (c.nc <= 0) return;
-    GV_DISPATCH(c.P.fam, (k_cell_geo<FAMV><<<blocks_for((int64_t)c.nc << Fam<FAMV>::K, 64), 64, 0, st>>>(c)));
+    GV_DISPATCH(c.P.fam, (k_cell_geo<FAMV><<<blocks_for((int64_t)c.nc << c.kf, 64), 64, 0, st>>>(c)));
+}
+
+int sm_count() {
+    static const int sms = [] {
+        int dev = 0, n = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        return n > 0 ? n : 1;
+    }();
+    return sms;
 }
 
 // Persistent grid: as many blocks as fit on the device at once (the kernel's
@@ -801,16 +860,9 @@ void launch_cell_geo(const Chunk &c, cudaStream_t st) {
 void launch_persistent(const void *kern, size_t smem, int64_t groups, const Chunk &c, cudaStream_t st) {
     static std::mutex mu;
     static std::map<std::pair<const void *, size_t>, int> occ;
-    static int sms = 0;
     int per_sm = 0;
     {
         std::lock_guard<std::mutex> lock(mu);
-        if (!sms) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (sms <= 0) sms = 1;
-        }
         auto it = occ.find({kern, smem});
         if (it == occ.end()) {
             if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -821,7 +873,7 @@ void launch_persistent(const void *kern, size_t smem, int64_t groups, const Chun
             per_sm = it->second;
         }
     }
-    int64_t g = (int64_t)sms * per_sm;
+    int64_t g = (int64_t)sm_count() * per_sm;
     if (g > groups) g = groups;
     void *args[] = {(void *)&c};
     cudaLaunchKernel(kern, dim3((unsigned)g), dim3(256), args, smem, st);
@@ -832,51 +884,24 @@ void launch_tile_info(const Chunk &c, cudaStream_t st) {
     if (nt > 0) k_tile_info<<<blocks_for(nt, 256), 256, 0, st>>>(c);
 }
 
-void launch_next_tiles(const Chunk &c, int64_t ncells, cudaStream_t st) {
-    if (ncells > 0) k_next_tiles<<<blocks_for(ncells * 32, 256), 256, 0, st>>>(c.next_cells, c.out, c.next_c0, ncells);
-}
-
-void launch_tile_dst(const Chunk &c, cudaStream_t st) {
+void launch_tile_scan(const Chunk &c, cudaStream_t st) {
     const int64_t nt = c.t1 - c.t0;
     if (nt <= 0) return;
-    const int ns = 1 << c.P.d;
-    if (ns == 4) k_tile_dst<4><<<blocks_for(nt, 32), 32 * 4, 0, st>>>(c);
-    else if (ns == 8) k_tile_dst<8><<<blocks_for(nt, 32), 32 * 8, 0, st>>>(c);
-    else if (ns == 16) k_tile_dst<16><<<blocks_for(nt, 32), 32 * 8, 0, st>>>(c);
-    else if (ns == 32) k_tile_dst<32><<<blocks_for(nt, 32), 32 * 8, 0, st>>>(c);
-    else k_tile_dst<64><<<blocks_for(nt, 32), 32 * 8, 0, st>>>(c);
-}
-
-void launch_child_lbmax(const Chunk &c, cudaStream_t st) {
-    int ns = 1 << c.P.d;
-    int64_t n = (int64_t)c.nc * ns;
-    if (n <= 0) return;
-    if (ns == 4) k_child_lbmax<4><<<blocks_for(n, 256), 256, 0, st>>>(c);
-    else if (ns == 8) k_child_lbmax<8><<<blocks_for(n, 256), 256, 0, st>>>(c);
-    else if (ns == 16) k_child_lbmax<16><<<blocks_for(n, 256), 256, 0, st>>>(c);
-    else if (ns == 32) k_child_lbmax<32><<<blocks_for(n, 256), 256, 0, st>>>(c);
-    else k_child_lbmax<64><<<blocks_for(n, 256), 256, 0, st>>>(c);
+    if (c.in.mult) k_tile_scan_weighted<<<blocks_for(nt, 8), 256, 0, st>>>(c);
+    else if (c.ns == 2) k_tile_scan<2><<<blocks_for(nt, 256), 256, 0, st>>>(c);
+    else k_tile_scan<4><<<blocks_for(nt, 256), 256, 0, st>>>(c);
 }
 
 void launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
                         cudaStream_t st) {
-    int ns = 1 << c.P.d;
-    int64_t n = (int64_t)c.nc * ns;
+    const int64_t n = (int64_t)c.nc << c.lns;
     if (n <= 0) return;
     unsigned nb = blocks_for(n, 256);
     unsigned long long *ba = bsums, *bb = bsums + nb;
-    if (ns == 4) k_child_mark<4><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
-    else if (ns == 8) k_child_mark<8><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
-    else if (ns == 16) k_child_mark<16><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
-    else if (ns == 32) k_child_mark<32><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
-    else k_child_mark<64><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
+    k_child_mark<<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
     if (c.lev.leaf_children) return;
     k_scan_sums<<<1, 256, 0, st>>>(ba, bb, (int)nb, c.sc);
-    if (ns == 4) k_child_write<4><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
-    else if (ns == 8) k_child_write<8><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
-    else if (ns == 16) k_child_write<16><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
-    else if (ns == 32) k_child_write<32><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
-    else k_child_write<64><<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
+    k_child_write<<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
 }
 
 void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, BeamSel *sel,

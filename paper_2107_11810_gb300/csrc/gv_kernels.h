@@ -32,7 +32,7 @@ struct CellView {
 // Device-resident scalars of one solve.
 struct Scalars {
     unsigned int best_lb;            // largest lower bound seen
-    unsigned int pad;
+    unsigned int n_uns;              // entries of the step's recheck queue
     unsigned long long best_key;     // (UB << coord_bits) | ~leaf key (max = best leaf)
     unsigned long long n_cells;      // cells written to the next level
     unsigned long long n_recs;       // record slots (32-aligned per cell) of the next level
@@ -56,27 +56,40 @@ struct Trace {
 };
 
 // Everything one expansion step (a chunk of cells of one level) needs.
+//
+// Children are numbered over the coordinates that still split at this level ("child
+// slots"): slot = free bits | dependent bits << kf, each the bits of the level's
+// split mask in coordinate order, so a cell has ns = 2^(splitting coordinates) slots
+// and nothing is computed, stored or read for children that do not exist.
 struct Chunk {
     Problem P;
     Level lev;
     CellView cells;          // cells of level l (key, ub: absolute index c0 + cl)
     int64_t c0;              // first cell of the chunk
     int nc;                  // number of cells in the chunk
+    int ns, lns;             // child slots per cell, log2
+    int nfs, kf;             // free slots (basis changes) per cell, log2
+    int dm;                  // bit j: dependent coordinate j splits
+    int gf;                  // floats of one cell's screen geometry
     RecView in;              // records of the chunk (tile_cell values: in_c0 + cl)
     const uint64_t *in_rbeg; // first record of chunk cell cl at in_rbeg[in_c0 + cl]
     const uint32_t *in_rcnt; // its record count
     int64_t in_c0;
     int64_t t0, t1;          // tile range of the chunk
     uint8_t *alive;          // [nc]   cell still above the pruning threshold
-    double *geo64;           // [nc][2^k][NB]          basis change per free child slot
-    float *geo32;            // [nc][2^k * ND * LE + ND * LE + 1] screen coefficients G, max |G|, exponent
-    float *geo32lo;          // [nc][2^k * ND * LE]   G64 - G rounded to FP32 (double-float tier)
-    uint32_t *cnt;           // [nc][2^d][3]      UB, LB, records per child
-    int2 *tinfo;             // [t1 - t0]         per tile: chunk-local cell (-1: pruned), valid lanes
-    uint32_t *ballot;        // [t1 - t0][2^d]    per tile and child: UB-pass lanes
-    unsigned long long *tdst;// [t1 - t0][2^d]    per tile and child: first output slot (~0: none)
-    int32_t *child_idx;      // [nc][2^d]         index of the child cell or -1
-    uint32_t *cursor;        // [nc][2^d]         next free record of the child
+    double *geo64;           // [nc][nfs][NB]          basis change per free slot
+    float *geo32;            // [nc][gf] screen coefficients G, max |G|, exponent
+    float *geo32lo;          // [nc][nfs * ND * LE]    G64 - G rounded to FP32 (double-float tier)
+    uint32_t *crec, *clb;    // [nc][ns]  records (UB-passing) and LB sum per child
+    uint32_t *cub;           // [nc][ns]  UB sum per child (= crec without multiplicities)
+    int2 *tinfo;             // [t1 - t0] per tile: chunk-local cell (-1: pruned), valid lanes | kTileFirst |
+                             //           kTileLast
+    uint32_t *ballot;        // [t1 - t0][ns] per tile and child: UB-passing lanes
+    uint32_t *lballot;       // [t1 - t0][ns] the same for the LB test
+    uint2 *uns;              // queue of (tile, lanes) the FP32 screen left undecided, sc->n_uns entries
+    uint32_t *off;           // [t1 - t0][ns] per tile and child: its records' first place in the child
+    unsigned long long *cbase; // [nc][ns] first record slot of the child (~0: pruned)
+    int32_t *child_idx;      // [nc][ns] index of the child cell (where cbase is not ~0)
     CellView next_cells;     // cells of level l+1
     int64_t next_c0, next_r0;// its cells and record slots before this step (the step appends)
     RecView out;             // records of level l+1
@@ -84,10 +97,12 @@ struct Chunk {
     Trace trace;
     int prune;
     int precision;           // 0 = FP64, 1 = FP32 screen + FP64 recheck
+    int lb;                  // lower bounds are wanted (lballot, clb)
     unsigned spin;           // polls of a bounded wait for a bulk copy before giving up
 };
+constexpr int kTileFirst = 64, kTileLast = 128;   // flags in tinfo.y: first / last tile of its cell
 
-// Size in floats of one cell's screen geometry: G[2^k][ND][LE], per (j, m) the
+// Size in floats of one cell's screen geometry: G[nfs][ND][LE], per (j, m) the
 // largest |G| over the free slots (rounded up), and the cell's exactness exponent e
 // (every G is FP32-exact and a multiple of 2^e; kNoExp when not).
 __host__ __device__ constexpr int geo32_floats(int nfs, int nd, int le) { return nfs * nd * le + nd * le + 1; }
@@ -114,21 +129,24 @@ void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t
 void launch_cell_geo(const Chunk &c, cudaStream_t st);
 // launch a persistent kernel taking one Chunk: one block per resident slot on the
 // device, at most `groups` blocks, 256 threads, smem bytes of dynamic shared memory
+// SMs of the device (read once)
+int sm_count();
 void launch_persistent(const void *kern, size_t smem, int64_t groups, const Chunk &c, cudaStream_t st);
 // per tile of the chunk: tinfo (after k_cell_geo has set alive)
 void launch_tile_info(const Chunk &c, cudaStream_t st);
+// the ballots of every tile and child, by the FP32 screen (undecided records queued)
+// or, in plain FP64 mode, by the definition
 void launch_count(const Chunk &c, cudaStream_t st);
-// the count and emit passes of families with 64 child slots (gv_wide.cu)
 void launch_count_wide(const Chunk &c, cudaStream_t st);
+// the definition: the queued records' bits are added to the ballots; every record
+void launch_recheck(const Chunk &c, cudaStream_t st);
+void launch_count_exact(const Chunk &c, cudaStream_t st);
+// per child its counts, per tile and child its records' place in the child, best LB
+void launch_tile_scan(const Chunk &c, cudaStream_t st);
 bool launch_emit_wide(const Chunk &c, cudaStream_t st);
-// after the children are laid out: the next level's tile -> cell table for cells
-// [next_c0, next_c0 + ncells) and every tile's output positions (tdst)
-void launch_next_tiles(const Chunk &c, int64_t ncells, cudaStream_t st);
-void launch_tile_dst(const Chunk &c, cudaStream_t st);
 // false if the level's record formats have no emit pass (never chosen by the engine)
 bool launch_emit(const Chunk &c, cudaStream_t st);
-void launch_child_lbmax(const Chunk &c, cudaStream_t st);
-// keepflag, recn: [nc * 2^d]; bsums: 2 * ceil(nc * 2^d / 256)
+// keepflag, recn: [nc * ns]; bsums: 2 * ceil(nc * ns / 256)
 void launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
                         cudaStream_t st);
 // the cells of a level (whose sum of record slots exceeds budget) with the largest UBs and LBs:

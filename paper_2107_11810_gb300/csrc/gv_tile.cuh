@@ -172,12 +172,16 @@ __device__ __forceinline__ void radius64(const Level &lev, const double *t, doub
     }
 }
 
+// shift of dependent coordinate j for the dependent bits ds of a child (dm: the
+// dependent coordinates that split; bit j of ds is 0 where j does not)
 template <int FAM>
-__device__ __forceinline__ double dep_shift64(const Level &lev, int j, int s) {
+__device__ __forceinline__ double dep_shift64(const Level &lev, int j, int ds, int dm) {
     constexpr int K = Fam<FAM>::K;
-    bool split = (lev.split_mask >> (K + j)) & 1;
-    return split ? (((s >> (K + j)) & 1) ? lev.h1[K + j] : -lev.h1[K + j]) : 0.0;
+    return ((dm >> j) & 1) ? (((ds >> j) & 1) ? lev.h1[K + j] : -lev.h1[K + j]) : 0.0;
 }
+
+// the child slot of free slot f and dependent bits ds (a subset of dm, at most two bits)
+__device__ __forceinline__ int child_slot(int f, int ds, int dm, int kf) { return f | ((dm == 2 ? ds >> 1 : ds) << kf); }
 
 template <int FAM>
 __device__ __forceinline__ void shifts64(const Level &lev, int s, double *sh) {
@@ -213,13 +217,13 @@ template <int FAM>
 using SlotMask = typename std::conditional<((1 << Fam<FAM>::D) > 32), unsigned long long, unsigned>::type;
 
 // UB/LB pass masks of one record (integer fields) against every child slot, exactly
-// as the definition evaluates them.  g64: the cell's basis changes [2^k][NB].
+// as the definition evaluates them.  g64: the cell's basis changes [nfs][NB].
 template <int FAM>
 __device__ __forceinline__ void eval64(const Problem &P, const Level &lev, const int *qf, const int *qt,
-                                       const double *g64, SlotMask<FAM> &ubm, SlotMask<FAM> &lbm) {
+                                       const double *g64, int kf, int dm, SlotMask<FAM> &ubm, SlotMask<FAM> &lbm) {
     using F = Fam<FAM>;
     using Mask = SlotMask<FAM>;
-    constexpr int NS = 1 << F::D, NFS = 1 << F::K;
+    static_assert(F::ND <= 2, "two dependent coordinates at most");
     double f[F::ND], t[F::LE], R[F::ND];
 #pragma unroll
     for (int j = 0; j < F::ND; ++j) f[j] = dmul((double)qf[j], P.s_f[j]);
@@ -228,21 +232,21 @@ __device__ __forceinline__ void eval64(const Problem &P, const Level &lev, const
     radius64<FAM>(lev, t, R);
     ubm = 0;
     lbm = 0;
-#pragma unroll
-    for (int fs = 0; fs < NFS; ++fs) {
-        if (fs & ~lev.split_mask) continue;
+#pragma unroll 1
+    for (int fs = 0; fs < (1 << kf); ++fs) {
         double pr[F::ND];
         F::partial64(f, t, g64 + fs * F::NB, pr);
 #pragma unroll
-        for (int s = fs; s < NS; s += NFS) {
-            if (s & ~lev.split_mask) continue;
+        for (int ds = 0; ds < (1 << F::ND); ++ds) {
+            if (ds & ~dm) continue;
             int ub = 1, lb = 1;
 #pragma unroll
             for (int j = 0; j < F::ND; ++j) {
-                double a = fabs(dsub(pr[j], dep_shift64<FAM>(lev, j, s)));
+                double a = fabs(dsub(pr[j], dep_shift64<FAM>(lev, j, ds, dm)));
                 ub &= a <= R[j];
                 lb &= a <= lev.rlb[j];
             }
+            const int s = child_slot(fs, ds, dm, kf);
             ubm |= (Mask)ub << s;
             lbm |= (Mask)lb << s;
         }
@@ -264,59 +268,25 @@ __device__ __forceinline__ RecWords rec_words_of(const uint32_t *w) {
     return r;
 }
 
-// Exact UB/LB masks of one record from its words, out of line (the FP32 screen
-// needs it rarely): x = UB mask, y = LB mask.
+// Exact FP64 snap of one record's free parameters at a child centre (g64: the basis
+// change of its free slot, ds: its dependent bits), out of line (the FP32 path needs
+// it rarely): the snapped values (x, y: dependent coordinates 0 and 1) and z != 0 if
+// a value leaves the representable range.
 template <int FAM, bool Q16>
-__device__ __noinline__ uint2 eval64_words(const Problem *P, const Level *lev, RecWords rw, const double *g64) {
-    using F = Fam<FAM>;
-    int qf[F::ND], qt[F::LE];
-#pragma unroll
-    for (int j = 0; j < F::ND; ++j) qf[j] = field_i<Q16>(rw.w, j);
-#pragma unroll
-    for (int m = 0; m < F::LE; ++m) qt[m] = field_i<Q16>(rw.w, F::ND + m);
-    SlotMask<FAM> ubm, lbm;
-    eval64<FAM>(*P, *lev, qf, qt, g64, ubm, lbm);
-    if constexpr (sizeof(SlotMask<FAM>) == 8) {
-        // families with more than 32 child slots use eval64_words_wide
-        return make_uint2(0u, 0u);
-    } else {
-        return make_uint2(ubm, lbm);
-    }
-}
-
-// The same for families with more than 32 child slots: x = UB mask, y = LB mask.
-template <int FAM, bool Q16>
-__device__ __noinline__ ulonglong2 eval64_words_wide(const Problem *P, const Level *lev, RecWords rw,
-                                                    const double *g64) {
-    using F = Fam<FAM>;
-    int qf[F::ND], qt[F::LE];
-#pragma unroll
-    for (int j = 0; j < F::ND; ++j) qf[j] = field_i<Q16>(rw.w, j);
-#pragma unroll
-    for (int m = 0; m < F::LE; ++m) qt[m] = field_i<Q16>(rw.w, F::ND + m);
-    SlotMask<FAM> ubm, lbm;
-    eval64<FAM>(*P, *lev, qf, qt, g64, ubm, lbm);
-    return make_ulonglong2((unsigned long long)ubm, (unsigned long long)lbm);
-}
-
-// Exact FP64 snap of one record's free parameters at the centre of child s, out of
-// line (the FP32 path needs it rarely): the snapped values (x, y: dependent
-// coordinates 0 and 1) and z != 0 if a value leaves the representable range.
-template <int FAM, bool Q16>
-__device__ __noinline__ int3 snap64_words(const Problem *P, const Level *lev, RecWords rw, const double *g64, int s) {
+__device__ __noinline__ int3 snap64_words(const Problem *P, const Level *lev, RecWords rw, const double *g64, int ds,
+                                          int dm) {
     using F = Fam<FAM>;
     static_assert(F::ND <= 2, "two dependent coordinates at most");
-    constexpr int NFS = 1 << F::K;
     double f[F::ND], t[F::LE], pr[F::ND];
 #pragma unroll
     for (int j = 0; j < F::ND; ++j) f[j] = dmul((double)field_i<Q16>(rw.w, j), P->s_f[j]);
 #pragma unroll
     for (int m = 0; m < F::LE; ++m) t[m] = dmul((double)field_i<Q16>(rw.w, F::ND + m), lev->s_t[m]);
-    F::partial64(f, t, g64 + (s & (NFS - 1)) * F::NB, pr);
+    F::partial64(f, t, g64, pr);
     int bad = 0, qn[2] = {0, 0};
 #pragma unroll
     for (int j = 0; j < F::ND; ++j) {
-        double q = rint(dmul(dsub(pr[j], dep_shift64<FAM>(*lev, j, s)), P->inv_s_f[j]));
+        double q = rint(dmul(dsub(pr[j], dep_shift64<FAM>(*lev, j, ds, dm)), P->inv_s_f[j]));
         bad |= !(fabs(q) < 1073741824.0);
         qn[j] = bad ? 0 : (int)q;
     }
@@ -339,19 +309,17 @@ __device__ __forceinline__ float two_sum(float a, float b, float &err) {
     return s;
 }
 
-// The snap of one record's dependent coordinates at the centre of child s, from
-// the residual q_f,j + sum_m q_t,m G64[fs][j][m] -+ h1_j / s_f,j evaluated as a
-// double-float (G64 = Gh + Gl, the cell's coefficients and their remainders):
+// The snap of one record's dependent coordinates at a child centre (dependent bits
+// ds), from the residual q_f,j + sum_m q_t,m G64[j][m] -+ h1_j / s_f,j evaluated as a
+// double-float (G64 = Gh + Gl, the free slot's coefficients and their remainders):
 // (x, y) the snapped values, z = 1 when both are decided (the value is more than
 // bd_j away from a rounding tie and below lim in magnitude), else 0 (the FP64
 // definition decides).  Out of line: the FP32 screen needs it rarely.
 template <int FAM, bool Q16>
-__device__ __noinline__ int3 snap_df_words(const Level *lev, RecWords rw, const float *Gh, const float *Gl, int s,
+__device__ __noinline__ int3 snap_df_words(const Level *lev, RecWords rw, const float *Gh, const float *Gl, int ds,
                                            float bd0, float bd1, float lim) {
     using F = Fam<FAM>;
     static_assert(F::ND <= 2, "two dependent coordinates at most");
-    constexpr int NFS = 1 << F::K;
-    const int fs = s & (NFS - 1);
     int qn[2] = {0, 0}, ok = 1;
 #pragma unroll
     for (int j = 0; j < F::ND; ++j) {
@@ -362,7 +330,7 @@ __device__ __noinline__ int3 snap_df_words(const Level *lev, RecWords rw, const 
             if (!F::uses(j, m)) continue;
             float th, tl;
             split_int(field_i<Q16>(rw.w, F::ND + m), th, tl);
-            const int x = (fs * F::ND + j) * F::LE + m;
+            const int x = j * F::LE + m;
             const float gh = __ldg(Gh + x), gl = __ldg(Gl + x);
             const float p = __fmul_rn(th, gh);
             const float e = __fmaf_rn(th, gh, -p);                  // th gh = p + e exactly
@@ -372,7 +340,7 @@ __device__ __noinline__ int3 snap_df_words(const Level *lev, RecWords rw, const 
         }
         if ((lev->split_mask >> (F::K + j)) & 1) {
             // the residual at the child centre: partial - h1 when the dependent bit is set
-            const bool up = (s >> (F::K + j)) & 1;
+            const bool up = (ds >> j) & 1;
             const float h = up ? -lev->Hs[j] : lev->Hs[j], hl = up ? -lev->Hs_lo[j] : lev->Hs_lo[j];
             float err;
             hi = two_sum(hi, h, err);
@@ -421,25 +389,136 @@ __device__ __forceinline__ void magnitudes(const float *qf, const float *qt, con
     }
 }
 
-// One (record, child slot) decision of the screen.  hs: dependent shifts in steps
-// (0 where the coordinate does not split); Rlo/Rhi = radius -+ band, Llo/Lhi the
-// same for the lower-bound radius.  ub/lb: the decision if it is certain; uns: a
-// comparison fell inside the band (the FP64 definition decides).
-template <int FAM>
-__device__ __forceinline__ void screen(int ds, const float *u, const float *hs, const float *Rlo, const float *Rhi,
-                                       const float *Llo, const float *Lhi, bool &ub, bool &lb, bool &uns) {
+// Two FP32 values in one 64-bit register: the packed FP32 operations of sm_100+ (each
+// half rounded as the scalar operation), two for one issue slot.
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 f2_make(float x, float y) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void f2_get(f2 v, float &x, float &y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// min(|a|, |b|, |c|)
+__device__ __forceinline__ float min3_abs(float a, float b, float c) {
+    float r;
+    asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
+// The screen's decisions on a pair of residuals y = (y0, y1) of one dependent coordinate
+// against the squared radius: y^2 - R^2 < 0, by its sign; the smallest |y^2 - R^2| of the
+// record goes into near, which leaves the record undecided when it falls below its band:
+// one packed multiply-add, two compares and one minimum for two tests.
+__device__ __forceinline__ void screen2(f2 y, float negr2, bool &p0, bool &p1, float &near) {
+    float d0, d1;
+    f2_get(f2_fma(y, y, f2_make(negr2, negr2)), d0, d1);
+    p0 = d0 < 0.0f;
+    p1 = d1 < 0.0f;
+    near = min3_abs(near, d0, d1);
+}
+
+// number of dependent shifts (children per free slot) for the dependent split mask
+__host__ __device__ constexpr int dep_slots(int dm) { return dm == 3 ? 4 : (dm ? 2 : 1); }
+
+// Ballots of FG free slots (1, 2 or 4) times their dependent shifts: bu/bl[ds * FG + f].
+// u[j][f]: residuals before the dependent shift.  A child passes when every dependent
+// coordinate passes, and the test of coordinate j depends only on its own shift, so with
+// two coordinates the four children of a free slot take four tests, not eight: their
+// ballots are combined.
+template <int ND, int FG, int DM, bool LB>
+__device__ __forceinline__ void test_children(const float (&u)[ND][FG], const float *hs, const float *negR2,
+                                              const float *negL2, float *near, float *nearL, unsigned *bu,
+                                              unsigned *bl) {
+    constexpr int NDS = dep_slots(DM);
+    unsigned au[ND][2][FG], al[ND][2][FG];
+#pragma unroll
+    for (int j = 0; j < ND; ++j) {
+        const bool split = (DM >> j) & 1;
+        if constexpr (FG >= 2) {
+#pragma unroll
+            for (int p = 0; p < FG; p += 2) {
+                const f2 u2 = f2_make(u[j][p], u[j][p + 1]);
+#pragma unroll
+                for (int v = 0; v < (split ? 2 : 1); ++v) {
+                    f2 y = u2;
+                    if (split) y = f2_add(u2, v ? f2_make(-hs[j], -hs[j]) : f2_make(hs[j], hs[j]));
+                    bool p0, p1;
+                    screen2(y, negR2[j], p0, p1, near[j]);
+                    au[j][v][p] = __ballot_sync(kFull, p0);
+                    au[j][v][p + 1] = __ballot_sync(kFull, p1);
+                    if constexpr (LB) {
+                        screen2(y, negL2[j], p0, p1, nearL[j]);
+                        al[j][v][p] = __ballot_sync(kFull, p0);
+                        al[j][v][p + 1] = __ballot_sync(kFull, p1);
+                    }
+                }
+            }
+        } else if (split) {
+            const f2 y = f2_add(f2_make(u[j][0], u[j][0]), f2_make(hs[j], -hs[j]));
+            bool p0, p1;
+            screen2(y, negR2[j], p0, p1, near[j]);
+            au[j][0][0] = __ballot_sync(kFull, p0);
+            au[j][1][0] = __ballot_sync(kFull, p1);
+            if constexpr (LB) {
+                screen2(y, negL2[j], p0, p1, nearL[j]);
+                al[j][0][0] = __ballot_sync(kFull, p0);
+                al[j][1][0] = __ballot_sync(kFull, p1);
+            }
+        } else {
+            const float d = __fmaf_rn(u[j][0], u[j][0], negR2[j]);
+            near[j] = fminf(near[j], fabsf(d));
+            au[j][0][0] = __ballot_sync(kFull, d < 0.0f);
+            if constexpr (LB) {
+                const float e = __fmaf_rn(u[j][0], u[j][0], negL2[j]);
+                nearL[j] = fminf(nearL[j], fabsf(e));
+                al[j][0][0] = __ballot_sync(kFull, e < 0.0f);
+            }
+        }
+    }
+#pragma unroll
+    for (int x = 0; x < NDS; ++x) {
+        const int ds = DM == 2 ? x << 1 : x;                        // dependent bits of shift x
+#pragma unroll
+        for (int f = 0; f < FG; ++f) {
+            unsigned b = kFull, l = kFull;
+#pragma unroll
+            for (int j = 0; j < ND; ++j) {
+                b &= au[j][(ds >> j) & 1][f];
+                if constexpr (LB) l &= al[j][(ds >> j) & 1][f];
+            }
+            bu[x * FG + f] = b;
+            if constexpr (LB) bl[x * FG + f] = l;
+        }
+    }
+}
+
+// Per record: squared radii (negated), and whether the screen's decisions stand.  The
+// band is proportional to the radius (Level::bandR, bandL: see finalize_levels): a
+// residual is within bandR R of the radius only if |y^2 - R^2| < bandR (2 + bandR) R^2.
+template <int FAM, bool LB>
+__device__ __forceinline__ bool undecided(const Level &lev, const float *R, const float *negR2, const float *near,
+                                          const float *nearL) {
     using F = Fam<FAM>;
-    ub = true;
-    lb = true;
+    bool u = false;
 #pragma unroll
     for (int j = 0; j < F::ND; ++j) {
-        float a = fabsf(((ds >> j) & 1) ? u[j] - hs[j] : u[j] + hs[j]);
-        bool um = a <= Rhi[j], us = a < Rlo[j];
-        bool lm = a <= Lhi[j], ls = a < Llo[j];
-        ub &= um;
-        lb &= lm;
-        uns |= (um != us) | (lm != ls);
+        u |= near[j] < -negR2[j] * lev.kappa[j];
+        if constexpr (LB) {
+            const float e = __fmaf_rn(lev.bandL[j], R[j], lev.bandL0[j]);
+            u |= nearL[j] < e * (e + 2.0f * lev.Lc[j]);
+        }
     }
+    return u;
 }
 
 }  // namespace gv

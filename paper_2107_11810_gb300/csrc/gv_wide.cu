@@ -1,11 +1,11 @@
 // gv_wide.cu -- the proximity test's count and emit passes for families whose
-// cells split into 16, 32 or 64 children (d = 4, 5, 6: Algorithm 2's 2^d
+// cells split into up to 16, 32 or 64 children (d = 4, 5, 6: Algorithm 2's 2^d
 // sub-boxes).  The same tests as gv_count.cu and gv_emit.cu (the surface-box test
 // of Sec. 3.2 with the FP32 screen and FP64 recheck, and the snap of the child
-// records for the next level), laid out for many child slots: lane s % 32 keeps the
-// counters and the ballot of child slot s, and the screen's coefficients of the
-// cell (the same for every lane of a warp) are staged in the warp's part of shared
-// memory once per run of tiles of one cell.
+// records for the next level), with a loop over groups of free slots: the screen's
+// coefficients of the cell (the same for every lane of a warp) are staged in the
+// warp's part of shared memory once per run of tiles of one cell, transposed so that
+// one load serves the coefficients of a whole group.
 //
 // Each warp takes a contiguous range of the chunk's tiles (so runs of tiles of one
 // cell stay together) and reads its records with plain loads; there are no
@@ -14,256 +14,190 @@
 
 namespace gv {
 
-template <int FAM, bool Q16, int PREC, bool WEIGHTED>
+// FG: free slots per group (4, or all of them when fewer split)
+template <int FAM, bool Q16, int FG, int DM, bool LB>
 __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chunk c) {
     using F = Fam<FAM>;
-    using Mask = SlotMask<FAM>;
-    constexpr int NS = 1 << F::D, NFS = 1 << F::K, NDS = 1 << F::ND, ND = F::ND, LE = F::LE;
-    static_assert(NS >= 16 && NS <= 64, "16 to 64 child slots");
-    constexpr int SPL = NS > 32 ? NS / 32 : 1;                     // child slots per lane
+    constexpr int ND = F::ND, LE = F::LE, NDS = dep_slots(DM), NX = ND * LE;
     constexpr int NW = rec_words(F::NFP, Q16);
-    constexpr int GF = geo32_floats(NFS, ND, LE);
+    constexpr int GMAX = (1 << F::K) * NX;
     const int lane = threadIdx.x & 31;
-    // the current cell's screen coefficients, staged once per run of tiles of the
-    // cell in the warp's part of shared memory (the per-free-slot loads then wait
-    // on shared memory, not on the cache hierarchy); blocks of 8 warps
-    __shared__ float s_g[8][GF];
-    float *sg = s_g[threadIdx.x >> 5];
-    int gcell = -1;
-    auto stage = [&](int cell) {
-        if (cell == gcell) return;                                  // uniform
-        __syncwarp();                                               // the old cell's reads are done
-        const float *src = c.geo32 + (size_t)cell * GF;
-        for (int i = lane; i < GF; i += 32) sg[i] = src[i];
-        __syncwarp();
-        gcell = cell;
-    };
+    __shared__ __align__(16) float s_g[8][GMAX];
+    float *sg = s_g[threadIdx.x >> 5];                              // [j * LE + m][nfs]
+    const int nfs = c.nfs;
+    int run = -1;
     const int64_t nt = c.t1 - c.t0;
-    const int64_t nwarp = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;        // chunk-relative tiles
+    const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
     const Level &lev = c.lev;
-    const int smask = lev.split_mask;
-    float hs[ND], Lc[ND];
+    float hs[ND], negL2[ND];
 #pragma unroll
     for (int j = 0; j < ND; ++j) {
-        hs[j] = ((smask >> (F::K + j)) & 1) ? lev.Hs[j] : 0.0f;
-        Lc[j] = lev.Lc[j];
+        hs[j] = lev.Hs[j];
+        negL2[j] = -lev.Lc[j] * lev.Lc[j];
     }
-    unsigned nvslot = 0;
-#pragma unroll
-    for (int s = 0; s < NS; ++s) nvslot += !(s & ~smask);
-
-    // counters of the current run of tiles of one cell, for slots lane + 32 h
-    unsigned cu[SPL], cl[SPL], cn[SPL];
-#pragma unroll
-    for (int h = 0; h < SPL; ++h) cu[h] = cl[h] = cn[h] = 0u;
-    int run = -1;
-    unsigned ntest = 0, nrechk = 0, nrec = 0;
-    auto flush = [&]() {
-        if (run < 0) return;
-#pragma unroll
-        for (int h = 0; h < SPL; ++h) {
-            if (lane + 32 * h >= NS) break;
-            uint32_t *bc = c.cnt + ((size_t)run * NS + lane + 32 * h) * 3;
-            if (cu[h]) atomicAdd(bc, cu[h]);
-            if (cl[h]) atomicAdd(bc + 1, cl[h]);
-            if (cn[h]) atomicAdd(bc + 2, cn[h]);
-            cu[h] = cl[h] = cn[h] = 0u;
-        }
-    };
+    unsigned nrec = 0;
 
 #pragma unroll 1
     for (int64_t tt = ta; tt < tb; ++tt) {
         const int2 ti = c.tinfo[tt];
         const int cell = ti.x;
         if (cell < 0) continue;                                     // uniform: the cell was pruned
+        uint32_t w[NW];
+        load_words<NW>(c.in.rec, (c.t0 + tt) * 32 + lane, w);       // whole tiles are allocated
         if (cell != run) {                                          // uniform: a new cell
-            flush();
+            __syncwarp();                                           // the old cell's reads are done
+            const float *src = c.geo32 + (size_t)cell * c.gf;
+            for (int i = lane; i < nfs * NX; i += 32) sg[(i % NX) * nfs + i / NX] = src[i];
+            __syncwarp();
             run = cell;
         }
-        const int64_t tile = c.t0 + tt;
-        const int nvalid = ti.y;
-        const bool act = lane < nvalid;
-        const int64_t r = tile * 32 + lane;
-        ntest += (unsigned)nvalid * nvslot;
+        const int nvalid = ti.y & 63;
         nrec += (unsigned)nvalid;
-        uint32_t w[NW];
-        load_words<NW>(c.in.rec, r, w);                             // whole tiles are allocated
-        const uint32_t mult = WEIGHTED ? (act ? c.in.mult[r] : 0u) : 1u;
-        if constexpr (PREC == 1) stage(cell);
-        const float *G = sg;
-        const double *g64 = c.geo64 + (size_t)cell * NFS * F::NB;
-        unsigned bw[SPL];                                           // ballots of slots lane + 32 h
+        float qf[ND], qt[LE], R[ND], negR2[ND], near[ND], nearL[ND];
 #pragma unroll
-        for (int h = 0; h < SPL; ++h) bw[h] = 0u;
-        // child slot s: the warp's ballots and sums go to lane s % 32
-        auto count = [&](int s, bool ub, bool lb) {
-            const unsigned bu = __ballot_sync(kFull, ub);
-            unsigned au, al;
-            if constexpr (WEIGHTED) {
-                au = __reduce_add_sync(kFull, ub ? mult : 0u);
-                al = __reduce_add_sync(kFull, lb ? mult : 0u);
-            } else {
-                au = __popc(bu);
-                al = __popc(__ballot_sync(kFull, lb));
-            }
-            if (lane == (s & 31)) {
-                bw[s >> 5] = bu;
-                cu[s >> 5] += au;
-                cl[s >> 5] += al;
-                cn[s >> 5] += (unsigned)__popc(bu);
-            }
-        };
-        if constexpr (PREC == 1) {
-            float qf[ND], qt[LE], R[ND], M[ND], Rlo[ND], Rhi[ND], Llo[ND], Lhi[ND];
+        for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
 #pragma unroll
-            for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
+        for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
+        F::radius32(lev, qt, R);
 #pragma unroll
-            for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
-            F::radius32(lev, qt, R);
-            magnitudes<FAM>(qf, qt, G + NFS * ND * LE, hs, M);
+        for (int j = 0; j < ND; ++j) {
+            negR2[j] = -R[j] * R[j];
+            near[j] = nearL[j] = 3.0e38f;
+        }
+        // a lane without a record fails every test (its residual is out of reach)
+        if (lane >= nvalid) qf[0] = 1.0e15f;
+        uint32_t *bp = c.ballot + (size_t)tt * c.ns, *lp = c.lballot + (size_t)tt * c.ns;
+#pragma unroll 1
+        for (int fs = 0; fs < nfs; fs += FG) {
+            float u[ND][FG];
 #pragma unroll
             for (int j = 0; j < ND; ++j) {
-                const float e = kBandTest * (M[j] + R[j]);
-                Rlo[j] = R[j] - e;
-                Rhi[j] = R[j] + e;
-                Llo[j] = Lc[j] - e;
-                Lhi[j] = Lc[j] + e;
-            }
-            // a lane without a record fails every test (its residual is out of reach)
-            if (!act) qf[0] = 1.0e30f;
-            bool uns = false;
-#pragma unroll 1
-            for (int fs = 0; fs < NFS; ++fs) {
-                float u[ND];
-                partial32<FAM>(qf, qt, G, fs, u);
+                f2 v[FG >= 2 ? FG / 2 : 1];
+                float v1 = qf[j];
 #pragma unroll
-                for (int ds = 0; ds < NDS; ++ds) {
-                    bool ub, lb;
-                    screen<FAM>(ds, u, hs, Rlo, Rhi, Llo, Lhi, ub, lb, uns);
-                    count(fs | (ds << F::K), ub, lb);
-                }
-            }
-            const unsigned unsb = __ballot_sync(kFull, act && uns);
-            if (unsb) {
-                // rare: the lanes whose screen was unsure take the FP64 definition; the
-                // difference to what was counted goes to the cell's counters directly
-                Mask m64u = 0;
-                if ((unsb >> lane) & 1) {
-                    Mask m32u = 0, m32l = 0;
-#pragma unroll 1
-                    for (int fs = 0; fs < NFS; ++fs) {
-                        float u[ND];
-                        partial32<FAM>(qf, qt, G, fs, u);
+                for (int p = 0; p < FG / 2; ++p) v[p] = f2_make(qf[j], qf[j]);
 #pragma unroll
-                        for (int ds = 0; ds < NDS; ++ds) {
-                            const int s = fs | (ds << F::K);
-                            bool ub, lb, un = false;
-                            screen<FAM>(ds, u, hs, Rlo, Rhi, Llo, Lhi, ub, lb, un);
-                            m32u |= (Mask)ub << s;
-                            m32l |= (Mask)lb << s;
-                        }
-                    }
-                    const ulonglong2 m64 = eval64_words_wide<FAM, Q16>(&c.P, &c.lev, rec_words_of<NW>(w), g64);
-                    m64u = (Mask)m64.x;
-                    nrechk += nvslot;
-                    for (Mask d = (m32u ^ (Mask)m64.x) | (m32l ^ (Mask)m64.y); d; d &= d - 1) {
-                        const int s = __ffsll((long long)d) - 1;
-                        const int du = (int)((m64.x >> s) & 1) - (int)((m32u >> s) & 1);
-                        const int dl = (int)((m64.y >> s) & 1) - (int)((m32l >> s) & 1);
-                        uint32_t *bc = c.cnt + ((size_t)cell * NS + s) * 3;
-                        if (du) {
-                            atomicAdd(bc, (unsigned)(du * (int)mult));
-                            atomicAdd(bc + 2, (unsigned)du);
-                        }
-                        if (dl) atomicAdd(bc + 1, (unsigned)(dl * (int)mult));
+                for (int m = 0; m < LE; ++m) {
+                    if (!F::uses(j, m)) continue;
+                    const float *g = sg + (j * LE + m) * nfs + fs;
+                    if constexpr (FG == 4) {
+                        const float4 g4 = *reinterpret_cast<const float4 *>(g);
+                        v[0] = f2_fma(f2_make(qt[m], qt[m]), f2_make(g4.x, g4.y), v[0]);
+                        v[1] = f2_fma(f2_make(qt[m], qt[m]), f2_make(g4.z, g4.w), v[1]);
+                    } else if constexpr (FG == 2) {
+                        const float2 g2 = *reinterpret_cast<const float2 *>(g);
+                        v[0] = f2_fma(f2_make(qt[m], qt[m]), f2_make(g2.x, g2.y), v[0]);
+                    } else {
+                        v1 = __fmaf_rn(qt[m], g[0], v1);
                     }
                 }
-#pragma unroll 1
-                for (int s = 0; s < NS; ++s) {
-                    const unsigned fix = __ballot_sync(kFull, ((unsb >> lane) & 1) && ((m64u >> s) & 1));
-                    if (lane == (s & 31)) bw[s >> 5] = (bw[s >> 5] & ~unsb) | fix;
+                if constexpr (FG == 1) {
+                    u[j][0] = v1;
+                } else {
+#pragma unroll
+                    for (int p = 0; p < FG / 2; ++p) f2_get(v[p], u[j][2 * p], u[j][2 * p + 1]);
                 }
             }
-        } else {
-            // plain FP64: every record by the definition
-            ulonglong2 m64 = make_ulonglong2(0ull, 0ull);
-            if (act) m64 = eval64_words_wide<FAM, Q16>(&c.P, &c.lev, rec_words_of<NW>(w), g64);
-#pragma unroll 1
-            for (int s = 0; s < NS; ++s) count(s, (m64.x >> s) & 1, (m64.y >> s) & 1);
+            unsigned bu[FG * NDS], bl[FG * NDS];
+            test_children<ND, FG, DM, LB>(u, hs, negR2, negL2, near, nearL, bu, bl);
+            if (lane == 0) {
+#pragma unroll
+                for (int x = 0; x < NDS; ++x) {
+                    uint32_t *b = bp + x * nfs + fs, *l = lp + x * nfs + fs;
+                    if constexpr (FG == 4) {
+                        *reinterpret_cast<uint4 *>(b) = make_uint4(bu[4 * x], bu[4 * x + 1], bu[4 * x + 2], bu[4 * x + 3]);
+                        if constexpr (LB)
+                            *reinterpret_cast<uint4 *>(l) = make_uint4(bl[4 * x], bl[4 * x + 1], bl[4 * x + 2], bl[4 * x + 3]);
+                    } else {
+#pragma unroll
+                        for (int f = 0; f < FG; ++f) {
+                            b[f] = bu[FG * x + f];
+                            if constexpr (LB) l[f] = bl[FG * x + f];
+                        }
+                    }
+                }
+            }
         }
-        // the tile's ballots, one word per child slot
-        uint32_t *bp = c.ballot + (size_t)tt * NS;
-#pragma unroll
-        for (int h = 0; h < SPL; ++h)
-            if (lane + 32 * h < NS) bp[lane + 32 * h] = bw[h];
+        const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
+        const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, negR2, near, nearL)) & act;
+        if (unsb) {                                                 // rare: left to the definition
+            __syncwarp();                                           // lane 0's stores
+            for (int s = lane; s < c.ns; s += 32) {
+                bp[s] &= ~unsb;
+                if constexpr (LB) lp[s] &= ~unsb;
+            }
+            if (lane == 0) c.uns[atomicAdd(&c.sc->n_uns, 1u)] = make_uint2((unsigned)tt, unsb);
+        }
     }
-    flush();
-    ntest = __reduce_add_sync(kFull, lane == 0 ? ntest : 0u);
-    nrec = __reduce_add_sync(kFull, lane == 0 ? nrec : 0u);
-    nrechk = __reduce_add_sync(kFull, nrechk);
-    if (lane == 0) {
-        if (ntest) atomicAdd(&c.sc->tests, (unsigned long long)ntest);
-        if (nrec) atomicAdd(&c.sc->records, (unsigned long long)nrec);
-        if (nrechk) atomicAdd(&c.sc->rechecks, (unsigned long long)nrechk);
+    if (lane == 0 && nrec) {
+        atomicAdd(&c.sc->records, (unsigned long long)nrec);
+        atomicAdd(&c.sc->tests, (unsigned long long)nrec * c.ns);
     }
 }
 
-template <int FAM, bool QI16, bool QO16, int PREC>
+// The emit pass (see gv_emit.cu): slot rows of a tile (output address, passing lanes)
+// staged by one lane per slot, then a loop over the free slots with the snaps of their
+// dependent shifts (taken once per coordinate and shift) and one predicated store per
+// child.
+template <int FAM, bool QI16, bool QO16>
 __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk c) {
     using F = Fam<FAM>;
-    constexpr int NS = 1 << F::D, NFS = 1 << F::K, NDS = 1 << F::ND, ND = F::ND, LE = F::LE, NFP = F::NFP;
-    static_assert(NS >= 16 && NS <= 64 && ND <= 2, "16 to 64 child slots, two dependent coordinates");
+    constexpr int NDS = 1 << F::ND, ND = F::ND, LE = F::LE, NFP = F::NFP;
+    static_assert(F::D <= 6 && ND <= 2, "at most 64 child slots, two dependent coordinates");
     constexpr int NWI = rec_words(NFP, QI16), NWO = rec_words(NFP, QO16);
-    constexpr int GF = geo32_floats(NFS, ND, LE);
-    const int lane = threadIdx.x & 31;
+    constexpr int GF = geo32_floats(1 << F::K, ND, LE);
+    const int NS = c.ns, nfs = c.nfs;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the current cell's screen coefficients, staged once per run of tiles of the
-    // cell in the warp's part of shared memory (the per-free-slot loads then wait
-    // on shared memory, not on the cache hierarchy); blocks of 8 warps
+    // cell in the warp's part of shared memory; the slot rows of the tile at hand
     __shared__ float s_g[8][GF];
-    float *sg = s_g[threadIdx.x >> 5];
+    __shared__ uint4 s_rows[8][1 << F::D];
+    float *G = s_g[warp];
+    uint4 *s_row = s_rows[warp];
     int gcell = -1;
-    auto stage = [&](int cell) {
-        if (cell == gcell) return;                                  // uniform
-        __syncwarp();                                               // the old cell's reads are done
-        const float *src = c.geo32 + (size_t)cell * GF;
-        for (int i = lane; i < GF; i += 32) sg[i] = src[i];
-        __syncwarp();
-        gcell = cell;
-    };
-    const unsigned below = (1u << lane) - 1u;
+    const unsigned below = (1u << lane) - 1u, lanebit = 1u << lane;
     const int64_t nt = c.t1 - c.t0;
-    const int64_t nwarp = (int64_t)gridDim.x * (blockDim.x >> 5);
-    const int64_t gw = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + warp;
     const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
     const Level &lev = c.lev;
-    const int smask = lev.split_mask;
     float hs[ND];
 #pragma unroll
-    for (int j = 0; j < ND; ++j) hs[j] = ((smask >> (F::K + j)) & 1) ? lev.Hs[j] : 0.0f;
+    for (int j = 0; j < ND; ++j) hs[j] = ((c.dm >> j) & 1) ? lev.Hs[j] : 0.0f;
     unsigned nrechk = 0, ndf = 0, bad = 0;
 
 #pragma unroll 1
     for (int64_t tt = ta; tt < tb; ++tt) {
         const int cell = c.tinfo[tt].x;
         if (cell < 0) continue;                                     // uniform
-        const uint32_t *bp = c.ballot + (size_t)tt * NS;
-        const unsigned long long *dp = c.tdst + (size_t)tt * NS;
-        // slots lane (A) and lane + 32 (B)
-        const bool hasA = lane < NS, hasB = lane + 32 < NS;
-        const unsigned balA = hasA ? bp[lane] : 0u, balB = hasB ? bp[32 + lane] : 0u;
-        const unsigned long long dA = hasA ? dp[lane] : ~0ull, dB = hasB ? dp[32 + lane] : ~0ull;
-        // child slots this tile writes (bit s of vA: slot s, of vB: slot 32 + s)
-        const unsigned vA = __ballot_sync(kFull, dA != ~0ull && balA != 0u);
-        const unsigned vB = __ballot_sync(kFull, dB != ~0ull && balB != 0u);
-        if (!(vA | vB)) continue;                                   // uniform
+        __syncwarp();                                               // the last tile's rows are read
+        unsigned v[2] = {0u, 0u};                                   // child slots this tile writes
+#pragma unroll
+        for (int h = 0; h < (F::D > 5 ? 2 : 1); ++h) {
+            const int s = lane + 32 * h;
+            unsigned bal = 0;
+            if (s < NS) {
+                const unsigned long long base = c.cbase[(size_t)cell * NS + s];
+                const unsigned long long p0 = base + c.off[(size_t)tt * NS + s];
+                bal = base == ~0ull ? 0u : c.ballot[(size_t)tt * NS + s];
+                const unsigned long long q = (p0 + 31) >> 5;
+                if (bal && (q << 5) < p0 + (unsigned)__popc(bal))
+                    c.out.tile_cell[q] = (uint32_t)c.child_idx[(size_t)cell * NS + s];
+                const unsigned long long p = (unsigned long long)(c.out.rec + p0 * NWO);
+                s_row[s] = make_uint4((unsigned)p, (unsigned)(p >> 32), bal, 0u);
+            }
+            v[h] = __ballot_sync(kFull, bal != 0u);
+        }
+        if (!(v[0] | v[1])) continue;                               // uniform: nothing to write
         const int64_t r = (c.t0 + tt) * 32 + lane;
         uint32_t w[NWI];
         load_words<NWI>(c.in.rec, r, w);
-        if (PREC == 1) stage(cell);
-        const float *G = sg;
-        const double *g64 = c.geo64 + (size_t)cell * NFS * F::NB;
+        if (cell != gcell) {                                        // uniform
+            const float *src = c.geo32 + (size_t)cell * c.gf;
+            for (int i = lane; i < c.gf; i += 32) G[i] = src[i];
+            gcell = cell;
+        }
+        __syncwarp();
         // the child's essential parameters (re-snapped when the step doubles)
         uint32_t fb[NFP];
 #pragma unroll
@@ -276,95 +210,114 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
             qt[m] = field_f<QI16>(w, ND + m);
             if constexpr (QO16) {
                 // adding kMagic16 rounds to an integer, ties to even, biased by 2^15
-                float v = lev.st_ratio_log2[m] ? __fmaf_rn(qt[m], 0.5f, kMagic16) : qt[m] + kMagic16;
-                fb[ND + m] = __float_as_uint(v);
+                float x = lev.st_ratio_log2[m] ? __fmaf_rn(qt[m], 0.5f, kMagic16) : qt[m] + kMagic16;
+                fb[ND + m] = __float_as_uint(x);
             } else {
                 const int q = field_i<QI16>(w, ND + m);
                 fb[ND + m] = (uint32_t)(lev.st_ratio_log2[m] ? resnap_half(q) : q);
             }
         }
-        const uint32_t mult = c.out.mult ? c.in.mult[r] : 1u;
-        float es[ND], bd[ND];                                       // the snaps' bands (steps)
-            bool xs[ND];                                                // FP32 residual exact
-        if (PREC == 1) {
-            float M[ND];
+        float es[ND], M[ND];                                        // a snap is certain within es of an integer
+        {
             // every term a multiple of 2^ex and M below 2^(24 + ex): the FP32 residual, and
             // the definition's FP64 one, are exact, so a tie rounds to even in both
-            const int ex = min(__float2int_rn(G[GF - 1]), lev.hs_exp);
+            const int ex = min(__float2int_rn(G[c.gf - 1]), lev.hs_exp);
             const float tq = ex > -100 ? __int_as_float((127 + 24 + ex) << 23) : 0.0f;
-            magnitudes<FAM>(qf, qt, G + NFS * ND * LE, hs, M);
+            magnitudes<FAM>(qf, qt, G + nfs * ND * LE, hs, M);
 #pragma unroll
             for (int j = 0; j < ND; ++j) {
-                es[j] = 0.5f - kBandSnap * M[j];
-                bd[j] = __fmaf_ru(kBandDF, M[j], kBandDFAbs);
-                xs[j] = M[j] < tq;
+                es[j] = M[j] < tq ? 1.0f : 0.5f - kBandSnap * M[j];
+                if (c.precision == 0) es[j] = -1.0f;                // plain FP64 mode: by the definition
             }
         }
+        const uint32_t mult = c.out.mult ? c.in.mult[r] : 1u;
+        unsigned long long um = 0ull;                               // slots whose snap FP32 leaves undecided
 #pragma unroll 1
-        for (int fs = 0; fs < NFS; ++fs) {
-            unsigned any = 0;
+        for (int f = 0; f < nfs; ++f) {
+            unsigned any = 0;                                       // this free slot's children, bit ds
 #pragma unroll
             for (int ds = 0; ds < NDS; ++ds) {
-                const int s = fs | (ds << F::K);
-                any |= (s < 32 ? (vA >> s) : (vB >> (s - 32))) & 1u;
+                if (ds & ~c.dm) continue;
+                const int s = child_slot(f, ds, c.dm, c.kf);
+                any |= ((s < 32 ? (v[0] >> s) : (v[1] >> (s - 32))) & 1u) << ds;
             }
             if (!any) continue;                                     // uniform
             float u[ND];
+            partial32<FAM>(qf, qt, G, f, u);
+            uint32_t sv[ND][2];
+            bool so[ND][2];
 #pragma unroll
-            for (int j = 0; j < ND; ++j) u[j] = 0.0f;
-            if (PREC == 1) partial32<FAM>(qf, qt, G, fs, u);
+            for (int j = 0; j < ND; ++j)
 #pragma unroll
-            for (int ds = 0; ds < NDS; ++ds) {
-                const int s = fs | (ds << F::K);
-                if (!((s < 32 ? (vA >> s) : (vB >> (s - 32))) & 1u)) continue;    // uniform
-                const unsigned bs = __shfl_sync(kFull, s < 32 ? balA : balB, s & 31);
-                const unsigned long long d0 = __shfl_sync(kFull, s < 32 ? dA : dB, s & 31);
-                if (!((bs >> lane) & 1)) continue;
-                const unsigned long long pos = d0 + (unsigned)__popc(bs & below);
-                bool done = PREC == 1;
-                if (PREC == 1) {
-#pragma unroll
-                    for (int j = 0; j < ND; ++j) {
-                        const float y = ((ds >> j) & 1) ? u[j] - hs[j] : u[j] + hs[j];
-                        if constexpr (QO16) {
-                            const float t = y + kMagic16;
-                            done &= (fabsf(y - (t - kMagic16)) < es[j] || xs[j]) && fabsf(y) < 32767.0f;
-                            fb[j] = __float_as_uint(t);
-                        } else {
-                            const float t = y + kMagic;
-                            done &= (fabsf(y - (t - kMagic)) < es[j] || xs[j]) && fabsf(y) < 4.0e6f;
-                            fb[j] = (uint32_t)(__float_as_int(t) - 0x4B400000);
-                        }
+                for (int k = 0; k < 2; ++k) {
+                    // a coordinate that does not split has ds bit 0 and shift 0
+                    const float y = k ? u[j] - hs[j] : u[j] + hs[j];
+                    if constexpr (QO16) {
+                        // |y| <= 32000: the record passed this level's UB test (finalize_levels)
+                        const float t = y + kMagic16;
+                        so[j][k] = fabsf(y - (t - kMagic16)) < es[j];
+                        sv[j][k] = __float_as_uint(t);
+                    } else {
+                        const float t = y + kMagic;
+                        so[j][k] = fabsf(y - (t - kMagic)) < es[j] && fabsf(y) < 4.0e6f;
+                        sv[j][k] = (uint32_t)(__float_as_int(t) - 0x4B400000);
                     }
                 }
-                if (!done) {
-                    int3 q = make_int3(0, 0, 0);
-                    if constexpr (PREC == 1) {                              // the double-float tier
-                        q = snap_df_words<FAM, QI16>(&c.lev, rec_words_of<NWI>(w), c.geo32 + (size_t)cell * GF,
-                                                     c.geo32lo + (size_t)cell * (NFS * ND * LE), s, bd[0],
-                                                     bd[ND - 1], QO16 ? 32767.0f : 1.0e9f);
-                        ++ndf;
-                    }
-                    if (!q.z) {                                             // the FP64 definition
-                        q = snap64_words<FAM, QI16>(&c.P, &c.lev, rec_words_of<NWI>(w), g64, s);
-                        bad |= (unsigned)(q.z != 0);
-                        nrechk += PREC == 1;
-                    }
-                    const int qn[2] = {q.x, q.y};
 #pragma unroll
-                    for (int j = 0; j < ND; ++j) {
-                        if constexpr (QO16) {
-                            bad |= (unsigned)(qn[j] < -32768 || qn[j] > 32767) << 1;
-                            fb[j] = (uint32_t)(qn[j] + 32768);
-                        } else {
-                            fb[j] = (uint32_t)qn[j];
-                        }
+            for (int ds = 0; ds < NDS; ++ds) {
+                if (!((any >> ds) & 1)) continue;                   // uniform
+                const int s = child_slot(f, ds, c.dm, c.kf);
+                const uint4 rw = s_row[s];
+                bool sure = true;
+#pragma unroll
+                for (int j = 0; j < ND; ++j) {
+                    fb[j] = sv[j][(ds >> j) & 1];
+                    sure &= so[j][(ds >> j) & 1];
+                }
+                uint32_t wo[NWO];
+                pack<NFP, QO16>(fb, wo);
+                const unsigned k = (unsigned)__popc(rw.z & below);
+                uint32_t *op = reinterpret_cast<uint32_t *>(((unsigned long long)rw.y << 32) | rw.x);
+                if (rw.z & lanebit) {
+                    store_words<NWO>(op, k, wo);
+                    if (!sure) um |= 1ull << s;
+                    if (c.out.mult) c.out.mult[(op - c.out.rec) / NWO + k] = mult;
+                }
+            }
+        }
+        if (um) {                                                   // rare
+            const RecWords rwords = rec_words_of<NWI>(w);
+            for (unsigned long long m = um; m; m &= m - 1) {
+                const int s = __ffsll((long long)m) - 1, f = s & (nfs - 1), x = s >> c.kf, ds = c.dm == 2 ? x << 1 : x;
+                const uint4 rw = s_row[s];
+                int3 q = make_int3(0, 0, 0);
+                if (c.precision == 1) {                             // the double-float tier
+                    q = snap_df_words<FAM, QI16>(&c.lev, rwords, c.geo32 + (size_t)cell * c.gf + f * ND * LE,
+                                                 c.geo32lo + ((size_t)cell * nfs + f) * ND * LE, ds,
+                                                 __fmaf_ru(kBandDF, M[0], kBandDFAbs),
+                                                 __fmaf_ru(kBandDF, M[ND - 1], kBandDFAbs), QO16 ? 32767.0f : 1.0e9f);
+                    ++ndf;
+                }
+                if (!q.z) {                                         // the FP64 definition
+                    q = snap64_words<FAM, QI16>(&c.P, &c.lev, rwords, c.geo64 + ((size_t)cell * nfs + f) * F::NB, ds,
+                                                c.dm);
+                    bad |= (unsigned)(q.z != 0);
+                    nrechk += c.precision == 1;
+                }
+                const int qn[2] = {q.x, q.y};
+#pragma unroll
+                for (int j = 0; j < ND; ++j) {
+                    if constexpr (QO16) {
+                        bad |= (unsigned)(qn[j] < -32768 || qn[j] > 32767) << 1;
+                        fb[j] = (uint32_t)(qn[j] + 32768);
+                    } else {
+                        fb[j] = (uint32_t)qn[j];
                     }
                 }
                 uint32_t wo[NWO];
                 pack<NFP, QO16>(fb, wo);
-                store_words<NWO>(c.out.rec, (int64_t)pos, wo);
-                if (c.out.mult) c.out.mult[pos] = mult;
+                store_words<NWO>(reinterpret_cast<uint32_t *>(((unsigned long long)rw.y << 32) | rw.x),
+                                 (unsigned)__popc(rw.z & below), wo);
             }
         }
     }
@@ -380,15 +333,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
 
 // a grid of 8-warp blocks: enough warps to fill the device, at most one per tile
 static unsigned wide_blocks(int64_t nt) {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 1;
-    }
-    int64_t want = (int64_t)sms * 8;                    // blocks of 8 warps, 8 blocks per SM
-    int64_t need = (nt + 7) / 8;
+    const int64_t want = (int64_t)sm_count() * 8, need = (nt + 7) / 8;
     return (unsigned)(want < need ? want : need);
 }
 
@@ -401,24 +346,37 @@ static unsigned wide_blocks(int64_t nt) {
     default: break;                                                            \
     }
 
+template <int FAM, bool Q16, int FG, int DM>
+static void launch_wide(const Chunk &c, cudaStream_t st) {
+    if constexpr (DM < (1 << Fam<FAM>::ND) && (FG > 1 || DM)) {
+        const unsigned g = wide_blocks(c.t1 - c.t0);
+        if (c.lb) k_count_wide<FAM, Q16, FG, DM, true><<<g, 256, 0, st>>>(c);
+        else k_count_wide<FAM, Q16, FG, DM, false><<<g, 256, 0, st>>>(c);
+    }
+}
+
+template <int FAM, bool Q16, int FG>
+static void launch_wide_dm(const Chunk &c, cudaStream_t st) {
+    if (c.dm == 0) launch_wide<FAM, Q16, FG, 0>(c, st);
+    else if (c.dm == 1) launch_wide<FAM, Q16, FG, 1>(c, st);
+    else if (c.dm == 2) launch_wide<FAM, Q16, FG, 2>(c, st);
+    else launch_wide<FAM, Q16, FG, 3>(c, st);
+}
+
+template <int FAM, bool Q16>
+static void launch_wide_fam(const Chunk &c, cudaStream_t st) {
+    if (c.kf >= 2) launch_wide_dm<FAM, Q16, 4>(c, st);
+    else if (c.kf == 1) launch_wide_dm<FAM, Q16, 2>(c, st);
+    else launch_wide_dm<FAM, Q16, 1>(c, st);
+}
+
 void launch_count_wide(const Chunk &c, cudaStream_t st) {
-    const int64_t nt = c.t1 - c.t0;
-    if (nt <= 0) return;
-    const unsigned g = wide_blocks(nt);
-    const bool w = c.in.mult != nullptr;
-#define GV_COUNT_WIDE(Q16, PREC)                                                         \
-    {                                                                                   \
-        if (w) k_count_wide<FAMV, Q16, PREC, true><<<g, 256, 0, st>>>(c);               \
-        else k_count_wide<FAMV, Q16, PREC, false><<<g, 256, 0, st>>>(c);                \
-    }
-    if (c.precision == 0) {
-        GV_DISPATCH_WIDE(c.P.fam, GV_COUNT_WIDE(false, 0));
-    } else if (c.lev.q16) {
-        GV_DISPATCH_WIDE(c.P.fam, GV_COUNT_WIDE(true, 1));
+    if (c.lev.q16) {
+        GV_DISPATCH_WIDE(c.P.fam, (launch_wide_fam<FAMV, true>(c, st)));
     } else {
-        GV_DISPATCH_WIDE(c.P.fam, GV_COUNT_WIDE(false, 1));
+        GV_DISPATCH_WIDE(c.P.fam, (launch_wide_fam<FAMV, false>(c, st)));
     }
-#undef GV_COUNT_WIDE
+    launch_recheck(c, st);
 }
 
 bool launch_emit_wide(const Chunk &c, cudaStream_t st) {
@@ -429,17 +387,15 @@ bool launch_emit_wide(const Chunk &c, cudaStream_t st) {
     bool known = false;
     GV_DISPATCH_WIDE(c.P.fam, (known = FAMV > 0));
     if (!known) return false;
-    if (c.precision == 0) {
-        if (q || qn) return false;                  // plain FP64 mode keeps 32-bit records
-        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, false, false, 0><<<g, 256, 0, st>>>(c)));
-    } else if (q && qn) {
-        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, true, true, 1><<<g, 256, 0, st>>>(c)));
+    if (c.precision == 0 && (q || qn)) return false;    // plain FP64 mode keeps 32-bit records
+    if (q && qn) {
+        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, true, true><<<g, 256, 0, st>>>(c)));
     } else if (!q && qn) {
-        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, false, true, 1><<<g, 256, 0, st>>>(c)));
+        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, false, true><<<g, 256, 0, st>>>(c)));
     } else if (!q && !qn) {
-        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, false, false, 1><<<g, 256, 0, st>>>(c)));
+        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, false, false><<<g, 256, 0, st>>>(c)));
     } else {
-        return false;                               // 16-bit to 32-bit: never chosen
+        return false;                                   // 16-bit to 32-bit: never chosen
     }
     return true;
 }
