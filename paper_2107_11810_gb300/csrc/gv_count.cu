@@ -31,11 +31,13 @@ __device__ __forceinline__ void store_row(uint32_t *p, const unsigned *v) {
 // KF: free coordinates that split, DM: dependent coordinates that split (bit mask).
 // Each warp takes a contiguous range of the chunk's tiles (runs of tiles of one cell
 // stay together: the cell's coefficients are spread from one register per lane only
-// when the cell changes).
+// when the cell changes).  Loads run one tile ahead of the tests and tile information
+// two: records and tile information are padded past their ends, so the loop has no
+// boundary case.
 template <int FAM, bool Q16, int KF, int DM, bool LB>
 __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk c) {
     using F = Fam<FAM>;
-    constexpr int ND = F::ND, LE = F::LE, NFS = 1 << KF, NS = NFS * dep_slots(DM);
+    constexpr int ND = F::ND, LE = F::LE, NFS = 1 << KF, NS = NFS * dep_slots(DM), NP = (NFS + 1) / 2;
     constexpr int NW = rec_words(F::NFP, Q16), NG = NFS * ND * LE;
     static_assert(NG <= 32 && NS >= 2 && NS <= 8, "coefficients of a cell fit one register per lane");
     const int lane = threadIdx.x & 31;
@@ -43,97 +45,99 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
     const int64_t nt = c.t1 - c.t0;
     const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
-    float hs[ND], negL2[ND];
+    if (ta >= tb) return;
+    float hs[ND];
+    f2 negL2[ND];
 #pragma unroll
     for (int j = 0; j < ND; ++j) {
         hs[j] = lev.Hs[j];
-        negL2[j] = -lev.Lc[j] * lev.Lc[j];
+        negL2[j] = f2_dup(-lev.Lc[j] * lev.Lc[j]);
     }
     const float *gp = c.geo32 + (lane < NG ? lane : 0);
-    auto load_g = [&](int cell) { return __ldg(gp + (size_t)(cell < 0 ? 0 : cell) * c.gf); };
+    auto load_g = [&](int cell) { return __ldg(gp + (unsigned)(cell < 0 ? 0 : cell) * (size_t)c.gf); };
     int run = -1;
-    float G[NG];
+    f2 G[ND][LE][NP];
 #pragma unroll
-    for (int i = 0; i < NG; ++i) G[i] = 0.0f;
+    for (int i = 0; i < ND * LE * NP; ++i) G[i / (LE * NP)][i / NP % LE][i % NP] = 0ull;
     unsigned nrec = 0;
-    if (ta < tb) {
-        // one tile ahead: records and the lane's coefficient; tile information two ahead
-        int2 ti1 = c.tinfo[ta], ti2 = c.tinfo[ta + 1 < tb ? ta + 1 : ta];
-        uint32_t w1[NW];
-        load_words<NW>(c.in.rec, (c.t0 + ta) * 32 + lane, w1);
-        float g1 = load_g(ti1.x);
+    const uint32_t *rp = c.in.rec + ((c.t0 + ta) * 32 + lane) * NW;
+    const int2 *tp = c.tinfo + ta;
+    uint32_t *bp = c.ballot + ta * NS, *lp = c.lballot + ta * NS;
+    int2 ti1 = tp[0], ti2 = tp[1];
+    uint32_t w1[NW];
+    load_words<NW>(rp, 0, w1);
+    float g1 = load_g(ti1.x);
+    unsigned tt = (unsigned)ta;
 #pragma unroll 1
-        for (int64_t tt = ta; tt < tb; ++tt) {
-            const int2 ti = ti1;
-            const float g = g1;
-            uint32_t w[NW];
+    for (int k = (int)(tb - ta); k > 0; --k, ++tt, bp += NS, lp += NS) {
+        const int2 ti = ti1;
+        const float g = g1;
+        uint32_t w[NW];
 #pragma unroll
-            for (int i = 0; i < NW; ++i) w[i] = w1[i];
-            if (tt + 1 < tb) {
-                ti1 = ti2;
-                load_words<NW>(c.in.rec, (c.t0 + tt + 1) * 32 + lane, w1);
-                g1 = load_g(ti1.x);
-                if (tt + 2 < tb) ti2 = c.tinfo[tt + 2];
-            }
-            if (ti.x < 0) continue;                                 // uniform: the cell was pruned
-            if (ti.x != run) {                                      // uniform: a new cell
-                run = ti.x;
+        for (int i = 0; i < NW; ++i) w[i] = w1[i];
+        rp += 32 * NW;
+        ++tp;
+        load_words<NW>(rp, 0, w1);
+        ti1 = ti2;
+        g1 = load_g(ti1.x);
+        ti2 = tp[1];
+        if (ti.x < 0) continue;                                     // uniform: the cell was pruned
+        if (ti.x != run) {                                          // uniform: a new cell
+            run = ti.x;
 #pragma unroll
-                for (int i = 0; i < NG; ++i) G[i] = __shfl_sync(kFull, g, i);
-            }
-            const int nvalid = ti.y & 63;
-            nrec += (unsigned)nvalid;
-            float qf[ND], qt[LE], R[ND], negR2[ND], near[ND], nearL[ND];
+            for (int j = 0; j < ND; ++j)
 #pragma unroll
-            for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
+                for (int m = 0; m < LE; ++m)
 #pragma unroll
-            for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
-            F::radius32(lev, qt, R);
-#pragma unroll
-            for (int j = 0; j < ND; ++j) {
-                negR2[j] = -R[j] * R[j];
-                near[j] = nearL[j] = 3.0e38f;
-            }
-            // a lane without a record fails every test (its residual is out of reach)
-            if (lane >= nvalid) qf[0] = 1.0e15f;
-            float u[ND][NFS];
-#pragma unroll
-            for (int j = 0; j < ND; ++j) {
-                if constexpr (NFS >= 2) {
-#pragma unroll
-                    for (int f = 0; f < NFS; f += 2) {
-                        f2 v = f2_make(qf[j], qf[j]);
-#pragma unroll
-                        for (int m = 0; m < LE; ++m)
-                            if (F::uses(j, m))
-                                v = f2_fma(f2_make(qt[m], qt[m]),
-                                           f2_make(G[(f * ND + j) * LE + m], G[((f + 1) * ND + j) * LE + m]), v);
-                        f2_get(v, u[j][f], u[j][f + 1]);
+                    for (int p = 0; p < NP; ++p) {
+                        if (!F::uses(j, m)) continue;
+                        const int f1 = NFS > 1 ? 2 * p + 1 : 0;     // one free slot: the pair holds it twice
+                        G[j][m][p] = f2_make(__shfl_sync(kFull, g, (2 * p * ND + j) * LE + m),
+                                             __shfl_sync(kFull, g, (f1 * ND + j) * LE + m));
                     }
-                } else {
-                    float v = qf[j];
+        }
+        const int nvalid = ti.y & 63;
+        nrec += (unsigned)nvalid;
+        float qf[ND], qt[LE], R[ND], near[ND], nearL[ND];
+        f2 negR2[ND], u[ND][NP];
 #pragma unroll
-                    for (int m = 0; m < LE; ++m)
-                        if (F::uses(j, m)) v = __fmaf_rn(qt[m], G[j * LE + m], v);
-                    u[j][0] = v;
-                }
-            }
-            unsigned bu[NS], bl[NS];
-            test_children<ND, NFS, DM, LB>(u, hs, negR2, negL2, near, nearL, bu, bl);
-            const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
-            const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, negR2, near, nearL)) & act;
-            if (unsb) {                                             // rare: left to the definition
+        for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
 #pragma unroll
-                for (int s = 0; s < NS; ++s) {
-                    bu[s] &= ~unsb;
-                    bl[s] &= ~unsb;
-                }
-                if (lane == 0) c.uns[atomicAdd(&c.sc->n_uns, 1u)] = make_uint2((unsigned)tt, unsb);
+        for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
+        F::radius32(lev, qt, R);
+        // a lane without a record fails every test (its residual is out of reach)
+        if (lane >= nvalid) qf[0] = 1.0e15f;
+#pragma unroll
+        for (int j = 0; j < ND; ++j) {
+            negR2[j] = f2_dup(-R[j] * R[j]);
+            near[j] = nearL[j] = 3.0e38f;
+#pragma unroll
+            for (int p = 0; p < NP; ++p) u[j][p] = f2_dup(qf[j]);
+        }
+#pragma unroll
+        for (int m = 0; m < LE; ++m) {
+            const f2 q2 = f2_dup(qt[m]);
+#pragma unroll
+            for (int j = 0; j < ND; ++j)
+#pragma unroll
+                for (int p = 0; p < NP; ++p)
+                    if (F::uses(j, m)) u[j][p] = f2_fma(q2, G[j][m][p], u[j][p]);
+        }
+        unsigned bu[NS], bl[NS];
+        test_children<ND, NFS, DM, LB>(u, hs, negR2, negL2, near, nearL, bu, bl);
+        if (lane == 0) {
+            store_row<NS>(bp, bu);
+            if constexpr (LB) store_row<NS>(lp, bl);
+        }
+        const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
+        const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, near, nearL)) & act;
+        if (unsb) {                                                 // rare: left to the definition
+            __syncwarp();                                           // lane 0's stores
+            if (lane < NS) {
+                bp[lane] &= ~unsb;
+                if constexpr (LB) lp[lane] &= ~unsb;
             }
-            if (lane == 0) {
-                store_row<NS>(c.ballot + (size_t)tt * NS, bu);
-                if constexpr (LB) store_row<NS>(c.lballot + (size_t)tt * NS, bl);
-            }
+            if (lane == 0) c.uns[atomicAdd(&c.sc->n_uns, 1u)] = make_uint2(tt, unsb);
         }
     }
     if (lane == 0 && nrec) {

@@ -41,6 +41,7 @@ struct Level {                 // tests of the children of a level-l cell
     int split_mask;            // bit j: coordinate j splits at this level
     int leaf_children;         // children are leaves (l + 1 == L)
     int st_ratio_log2[GV_MAXT];// log2(s_t(l+1) / s_t(l)), 0 or 1
+    float st_scale[GV_MAXT];   // s_t(l) / s_t(l+1), 1 or 0.5
     double h[GV_MAXD];         // half-widths at level l
     double h1[GV_MAXD];        // half-widths at level l+1
     double s_t[GV_MAXT];       // essential-parameter snap step at level l
@@ -73,6 +74,14 @@ __device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a,
 __device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double dsqrt(double a) { return __dsqrt_rn(a); }
 __device__ __forceinline__ double ddiv(double a, double b) { return __ddiv_rn(a, b); }
+
+// FP32 square root of the screen's radii: the hardware approximation, without the
+// scaling of subnormal inputs (they are squares of steps)
+__device__ __forceinline__ float sqrt32(float a) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
 
 // ---------------------------------------------------------------------------
 // sin / cos of cell-centre angles: Cody-Waite reduction by pi/2 with a three-part
@@ -255,7 +264,7 @@ template <> struct Fam<FAM_PLANE3D_SPH> {
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
         float xy = __fmaf_rn(qt[1], qt[1], qt[0] * qt[0]);
         float all = __fmaf_rn(qt[2] * lev.rho2, qt[2], xy);
-        R[0] = __fmaf_rn(lev.lam_c[0], sqrtf(all), __fmaf_rn(lev.lam_c[1], sqrtf(xy), lev.rc0[0]));
+        R[0] = __fmaf_rn(lev.lam_c[0], sqrt32(all), __fmaf_rn(lev.lam_c[1], sqrt32(xy), lev.rc0[0]));
     }
 };
 
@@ -299,7 +308,7 @@ template <> struct Fam<FAM_POSE3DOF> {
     }
     // s_t,a = s_t,b: sqrt(a^2 + b^2) = s_t sqrt(qa^2 + qb^2)
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
-        float r = sqrtf(__fmaf_rn(qt[1], qt[1], qt[0] * qt[0]));
+        float r = sqrt32(__fmaf_rn(qt[1], qt[1], qt[0] * qt[0]));
         R[0] = __fmaf_rn(lev.lam_c[0], r, lev.rc0[0]);
         R[1] = __fmaf_rn(lev.lam_c[1], r, lev.rc0[1]);
     }
@@ -541,9 +550,9 @@ template <> struct Fam<FAM_POSE6DOF> {
     // s_t equal for the nine rotation coefficients and for xi, eta:
     // |w| + |xi w| = s_t (|q_w| + |q_xiw|); lam_c: [x rotation, x z, y rotation, y z]
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
-        const float nw = sqrtf(__fmaf_rn(qt[2], qt[2], __fmaf_rn(qt[1], qt[1], qt[0] * qt[0])));
-        const float nxw = sqrtf(__fmaf_rn(qt[5], qt[5], __fmaf_rn(qt[4], qt[4], qt[3] * qt[3])));
-        const float nyw = sqrtf(__fmaf_rn(qt[8], qt[8], __fmaf_rn(qt[7], qt[7], qt[6] * qt[6])));
+        const float nw = sqrt32(__fmaf_rn(qt[2], qt[2], __fmaf_rn(qt[1], qt[1], qt[0] * qt[0])));
+        const float nxw = sqrt32(__fmaf_rn(qt[5], qt[5], __fmaf_rn(qt[4], qt[4], qt[3] * qt[3])));
+        const float nyw = sqrt32(__fmaf_rn(qt[8], qt[8], __fmaf_rn(qt[7], qt[7], qt[6] * qt[6])));
         R[0] = __fmaf_rn(lev.lam_c[0], nxw + nw, __fmaf_rn(lev.lam_c[1], fabsf(qt[9]), lev.rc0[0]));
         R[1] = __fmaf_rn(lev.lam_c[2], nyw + nw, __fmaf_rn(lev.lam_c[3], fabsf(qt[10]), lev.rc0[1]));
     }
@@ -607,8 +616,8 @@ template <> struct Fam<FAM_RADIAL5DOF> {
     // s_t equal for the six rotation coefficients: |rho w| + |w| = s_t (|q_rw| + |q_w|);
     // lam_c: [rotation, y]
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
-        const float nrw = sqrtf(__fmaf_rn(qt[2], qt[2], __fmaf_rn(qt[1], qt[1], qt[0] * qt[0])));
-        const float nw = sqrtf(__fmaf_rn(qt[5], qt[5], __fmaf_rn(qt[4], qt[4], qt[3] * qt[3])));
+        const float nrw = sqrt32(__fmaf_rn(qt[2], qt[2], __fmaf_rn(qt[1], qt[1], qt[0] * qt[0])));
+        const float nw = sqrt32(__fmaf_rn(qt[5], qt[5], __fmaf_rn(qt[4], qt[4], qt[3] * qt[3])));
         R[0] = __fmaf_rn(lev.lam_c[0], nrw + nw, __fmaf_rn(lev.lam_c[1], fabsf(qt[6]), lev.rc0[0]));
     }
 };

@@ -24,6 +24,8 @@
 namespace gv {
 
 constexpr int kEmitTiles = 4;                        // tiles per warp and buffer
+constexpr int kEmitUnit = 16;                        // consecutive tiles a warp takes at a time (kEmitTiles
+                                                     // while that leaves under four units per warp)
 
 // Shared memory of one block (8 warps): per warp two buffers of kEmitTiles tiles of
 // records, ballots and positions, and the slot rows of the tile at hand (two, by turns).
@@ -33,15 +35,18 @@ __host__ __device__ constexpr size_t emit_warp_bytes(int ns) {
 }
 
 // KF: free coordinates that split, DM: dependent coordinates that split (bit mask).
-// Each warp takes a contiguous range of groups of kEmitTiles tiles and streams them
-// through its own two buffers (bulk copies completing on the warp's mbarriers), so
-// warps never wait for each other.
+// Warps take units of kEmitUnit tiles by turns; the groups of kEmitTiles tiles of a unit
+// with a cell that has surviving children stream through the warp's own two buffers
+// (bulk copies completing on the warp's mbarriers), so warps never wait for each other,
+// and neither reading nor the work falls to tiles that have nothing to write.
 template <int FAM, bool QI16, bool QO16, int KF, int DM>
-__global__ void __launch_bounds__(256, 4) k_emit(const __grid_constant__ Chunk c) {
+__global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c) {
     using F = Fam<FAM>;
     constexpr int ND = F::ND, LE = F::LE, NFP = F::NFP, NFS = 1 << KF, NDS = dep_slots(DM), NS = NFS * NDS;
     constexpr int NWI = rec_words(NFP, QI16), NWO = rec_words(NFP, QO16), RW = 32 * NWI, NG = NFS * ND * LE;
-    constexpr int GT = kEmitTiles;
+    constexpr int GT = kEmitTiles, NP = (NFS + 1) / 2;
+    // child slots of free slot 0 (those of free slot f: shifted left by f)
+    constexpr unsigned kFsSlots = NDS == 4 ? 1u | 1u << NFS | 1u << 2 * NFS | 1u << 3 * NFS : (NDS == 2 ? 1u | 1u << NFS : 1u);
     static_assert(geo32_floats(NFS, ND, LE) <= 32, "a cell's coefficients fit one register per lane");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Level &lev = c.lev;
@@ -53,41 +58,69 @@ __global__ void __launch_bounds__(256, 4) k_emit(const __grid_constant__ Chunk c
     __shared__ __align__(8) uint64_t s_bars[8][2];
     uint64_t *s_bar = s_bars[warp];
 
-    const int64_t nt = c.t1 - c.t0, ng = (nt + GT - 1) / GT;
-    const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + warp;
-    const int64_t g0 = gw * ng / nwarp, g1 = (gw + 1) * ng / nwarp;
+    const int nt = (int)(c.t1 - c.t0);
+    const int nwarp = gridDim.x * 8, gw = blockIdx.x * 8 + warp;
+    const int ut = nt > 4 * kEmitUnit * nwarp ? kEmitUnit : GT, nunits = (nt + ut - 1) / ut;
     if (lane == 0) {
         mbar_init(&s_bar[0], 1);
         mbar_init(&s_bar[1], 1);
         mbar_init_fence();
     }
     __syncwarp();
-    auto issue = [&](int64_t g) {                                   // lane 0
-        const int b = (int)((g - g0) & 1);
-        const int64_t ta = g * GT;
-        const int ntl = (int)((ta + GT < nt ? ta + GT : nt) - ta);
+
+    // units of this warp: lane k < ut holds the cell of the unit's tile k (-1: nothing to
+    // write); the next unit's are loaded, and the tile information of the one after it, so
+    // no load waits for another
+    int unit = gw, ucells, pcells, tcells;
+    auto load_cells = [&](int u) {
+        const int t = u * ut + lane;
+        if (lane >= ut || u >= nunits || t >= nt) return -1;
+        return c.tinfo[t].x;
+    };
+    auto live = [&](int cell) { return cell >= 0 && (c.alive[cell] & 2) ? cell : -1; };
+    ucells = live(load_cells(unit));
+    unsigned umask = __ballot_sync(kFull, ucells >= 0);             // the unit's tiles still to be taken
+    pcells = live(load_cells(unit + nwarp));
+    tcells = load_cells(unit + 2 * nwarp);
+    // the next group with something to write: its first tile (-1: none is left), its cells
+    auto next_group = [&](int &t0, int &cells) {
+        while (!umask) {
+            unit += nwarp;
+            if (unit >= nunits) {
+                t0 = -1;
+                cells = -1;
+                return;
+            }
+            ucells = pcells;
+            umask = __ballot_sync(kFull, ucells >= 0);
+            pcells = live(tcells);
+            tcells = load_cells(unit + 2 * nwarp);
+        }
+        const int g = (__ffs(umask) - 1) / GT;
+        umask &= ~(((1u << GT) - 1u) << (g * GT));
+        t0 = unit * ut + g * GT;
+        cells = __shfl_sync(kFull, ucells, g * GT + (lane & (GT - 1)));
+    };
+    // lane 0: copy number n (buffer n & 1)
+    auto issue = [&](int n, int t0) {
+        const int b = n & 1, ntl = t0 + GT < nt ? GT : nt - t0;
         // bulk copies take multiples of 16 bytes (the arrays are padded past the last tile)
         const unsigned rbytes = (unsigned)ntl * RW * 4, bbytes = ((unsigned)ntl * NS * 4 + 15u) & ~15u;
         mbar_expect_tx(&s_bar[b], rbytes + 2 * bbytes);
-        bulk_load(s_rec + b * GT * RW, c.in.rec + (c.t0 + ta) * RW, rbytes, &s_bar[b]);
-        bulk_load(s_bal + b * GT * NS, c.ballot + ta * NS, bbytes, &s_bar[b]);
-        bulk_load(s_off + b * GT * NS, c.off + ta * NS, bbytes, &s_bar[b]);
-    };
-    // lane k: the cell of tile k of group g (-1: pruned, or past the end)
-    auto load_cells = [&](int64_t g) {
-        const int64_t t = g * GT + lane;
-        return g < g1 && lane < GT && t < nt ? c.tinfo[t].x : -1;
+        bulk_load(s_rec + b * GT * RW, c.in.rec + (c.t0 + t0) * RW, rbytes, &s_bar[b]);
+        bulk_load(s_bal + b * GT * NS, c.ballot + (size_t)t0 * NS, bbytes, &s_bar[b]);
+        bulk_load(s_off + b * GT * NS, c.off + (size_t)t0 * NS, bbytes, &s_bar[b]);
     };
     // a cell's data, one word per lane: coefficient, child's first slot and index
     float pg = 0.0f;
     unsigned long long pbase = ~0ull;
     int pidx = 0;
     auto prefetch = [&](int cell) {
-        const int x = cell < 0 ? 0 : cell;
-        if (lane < c.gf) pg = __ldg(c.geo32 + (size_t)x * c.gf + lane);
+        if (cell < 0) return;                                       // uniform
+        if (lane < c.gf) pg = __ldg(c.geo32 + (size_t)cell * c.gf + lane);
         if (lane < NS) {
-            pbase = c.cbase[(size_t)x * NS + lane];
-            pidx = c.child_idx[(size_t)x * NS + lane];
+            pbase = c.cbase[(size_t)cell * NS + lane];
+            pidx = c.child_idx[(size_t)cell * NS + lane];
         }
     };
 
@@ -95,72 +128,91 @@ __global__ void __launch_bounds__(256, 4) k_emit(const __grid_constant__ Chunk c
 #pragma unroll
     for (int j = 0; j < ND; ++j) hs[j] = ((DM >> j) & 1) ? lev.Hs[j] : 0.0f;
     const unsigned below = (1u << lane) - 1u, lanebit = 1u << lane;
-    int cur = -1, row = 0;
-    float G[NG], Gmax[ND * LE], gexp = 0.0f;
-    unsigned long long base = ~0ull;
+    int cur = -1, pcell = -1, row = 0;                              // the cell at hand, the prefetched one
+    f2 G[ND][LE][NP];
+    float Gmax[ND * LE], tq = 0.0f;
+    const float es0 = c.precision == 1 ? 0.5f : -1.0f;              // plain FP64 mode: no snap is certain
+    unsigned long long crec = 0;                                    // lane s: child s's first record, 0 when pruned
+    uint32_t *ctile = nullptr;                                      // and its first tile -> cell entry
     int cidx = 0;
 #pragma unroll
-    for (int i = 0; i < NG; ++i) G[i] = 0.0f;
+    for (int i = 0; i < ND * LE * NP; ++i) G[i / (LE * NP)][i / NP % LE][i % NP] = 0ull;
 #pragma unroll
     for (int i = 0; i < ND * LE; ++i) Gmax[i] = 0.0f;
     unsigned nrechk = 0, ndf = 0, bad = 0;
-    int64_t gfail = -1;                                             // group whose copy did not arrive
-    int cells1 = load_cells(g0);
-    if (g0 < g1) {
-        if (lane == 0) issue(g0);
-        prefetch(__shfl_sync(kFull, cells1, 0));
-    }
+    int t1, cells1, nfail = -1;                                     // copy that did not arrive
+    next_group(t1, cells1);
+    if (t1 >= 0 && lane == 0) issue(0, t1);
 #pragma unroll 1
-    for (int64_t g = g0; g < g1; ++g) {
-        const int b = (int)((g - g0) & 1);
-        if (lane == 0 && g + 1 < g1) issue(g + 1);
-        const int cells = cells1;
-        cells1 = load_cells(g + 1);
-        const bool ok = mbar_wait(&s_bar[b], (unsigned)(((g - g0) >> 1) & 1), c.spin, &c.sc->err);
+    for (int n = 0; t1 >= 0; ++n) {
+        const int b = n & 1, t0 = t1, cells = cells1;
+        next_group(t1, cells1);
+        if (t1 >= 0 && lane == 0) issue(n + 1, t1);
+        const unsigned gm = __ballot_sync(kFull, cells >= 0) & ((1u << GT) - 1u);
+        if (pcell < 0) {                                            // the first group
+            pcell = __shfl_sync(kFull, cells, __ffs(gm) - 1);
+            prefetch(pcell);
+        }
+        const bool ok = mbar_wait(&s_bar[b], (unsigned)(n >> 1) & 1u, c.spin, &c.sc->err);
         if (!__all_sync(kFull, ok)) {
-            gfail = g;
+            nfail = n;
             break;
         }
 #pragma unroll 1
-        for (int lt = 0; lt < GT; ++lt) {
-            const int cl = __shfl_sync(kFull, cells, lt);
-            const float g_ = pg;
-            const unsigned long long base_ = pbase;
-            const int idx_ = pidx;
-            {
-                const int a = __shfl_sync(kFull, cells, (lt + 1) & (GT - 1)), n1 = __shfl_sync(kFull, cells1, 0);
-                prefetch(lt + 1 < GT ? a : n1);
-            }
-            if (cl < 0) continue;                                   // uniform
-            if (cl != cur) {                                        // uniform: a new cell
+        for (unsigned m = gm; m; m &= m - 1) {
+            const int lt = __ffs(m) - 1, cl = __shfl_sync(kFull, cells, lt);
+            if (cl != cur) {                                        // uniform: a new cell, prefetched
                 cur = cl;
-                base = base_;
-                cidx = idx_;
+                crec = pbase == ~0ull ? 0ull : (unsigned long long)(c.out.rec + pbase * NWO);
+                ctile = c.out.tile_cell + (pbase >> 5);
+                cidx = pidx;
 #pragma unroll
-                for (int i = 0; i < NG; ++i) G[i] = __shfl_sync(kFull, g_, i);
+                for (int j = 0; j < ND; ++j)
 #pragma unroll
-                for (int i = 0; i < ND * LE; ++i) Gmax[i] = __shfl_sync(kFull, g_, NG + i);
-                gexp = __shfl_sync(kFull, g_, NG + ND * LE);
+                    for (int x = 0; x < LE; ++x)
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) {
+                            if (!F::uses(j, x)) continue;
+                            const int f1 = NFS > 1 ? 2 * p + 1 : 0;
+                            G[j][x][p] = f2_make(__shfl_sync(kFull, pg, (2 * p * ND + j) * LE + x),
+                                                 __shfl_sync(kFull, pg, (f1 * ND + j) * LE + x));
+                        }
+#pragma unroll
+                for (int i = 0; i < ND * LE; ++i) Gmax[i] = __shfl_sync(kFull, pg, NG + i);
+                // every term a multiple of 2^ex and M below 2^(24 + ex): the FP32 residual, and
+                // the definition's FP64 one, are exact, so a tie rounds to even in both
+                const int ex = min(__float2int_rn(__shfl_sync(kFull, pg, NG + ND * LE)), lev.hs_exp);
+                tq = ex > -100 && c.precision == 1 ? __int_as_float((127 + 24 + ex) << 23) : 0.0f;
             }
-            const int64_t tt = g * GT + lt;
+            {
+                // the cell of the next tile to be taken
+                const unsigned rest = m & (m - 1);
+                const unsigned gn = __ballot_sync(kFull, cells1 >= 0) & ((1u << GT) - 1u);
+                const int a = __shfl_sync(kFull, cells, rest ? __ffs(rest) - 1 : 0);
+                const int z = __shfl_sync(kFull, cells1, gn ? __ffs(gn) - 1 : 0);
+                const int nx = rest ? a : z;
+                if (nx >= 0 && nx != pcell) {                       // uniform
+                    pcell = nx;
+                    prefetch(nx);
+                }
+            }
             // slot rows: output address and passing lanes; the next level's tile -> cell
             // table for the one tile whose first slot this tile may fill
             row ^= NS;
             unsigned bal = 0;
             if (lane < NS) {
-                const unsigned long long p0 = base + s_off[b * GT * NS + lt * NS + lane];
-                bal = base == ~0ull ? 0u : s_bal[b * GT * NS + lt * NS + lane];
-                const unsigned long long q = (p0 + 31) >> 5;
-                if (bal && (q << 5) < p0 + (unsigned)__popc(bal)) c.out.tile_cell[q] = (uint32_t)cidx;
-                const unsigned long long p = (unsigned long long)(c.out.rec + p0 * NWO);
+                const unsigned off = s_off[b * GT * NS + lt * NS + lane];
+                bal = crec ? s_bal[b * GT * NS + lt * NS + lane] : 0u;
+                const unsigned first = (off + 31u) & ~31u;
+                if (first < off + (unsigned)__popc(bal)) ctile[first >> 5] = (uint32_t)cidx;
+                const unsigned long long p = crec + off * (unsigned long long)(NWO * 4);
                 s_row[row + lane] = make_uint4((unsigned)p, (unsigned)(p >> 32), bal, 0u);
             }
             const unsigned vmask = __ballot_sync(kFull, bal != 0u);  // child slots this tile writes
             __syncwarp();
             if (!vmask) continue;                                   // uniform: nothing to write
             uint32_t w[NWI];
-#pragma unroll
-            for (int i = 0; i < NWI; ++i) w[i] = s_rec[b * GT * RW + lt * RW + lane * NWI + i];
+            load_words<NWI>(s_rec + b * GT * RW + lt * RW, lane, w);
             // the child's essential parameters (re-snapped when the step doubles)
             uint32_t fb[NFP];
 #pragma unroll
@@ -169,80 +221,95 @@ __global__ void __launch_bounds__(256, 4) k_emit(const __grid_constant__ Chunk c
 #pragma unroll
             for (int j = 0; j < ND; ++j) qf[j] = field_f<QI16>(w, j);
 #pragma unroll
-            for (int m = 0; m < LE; ++m) {
-                qt[m] = field_f<QI16>(w, ND + m);
+            for (int x = 0; x < LE; ++x) {
+                qt[x] = field_f<QI16>(w, ND + x);
                 if constexpr (QO16) {
                     // adding kMagic16 rounds to an integer, ties to even, biased by 2^15
-                    float v = lev.st_ratio_log2[m] ? __fmaf_rn(qt[m], 0.5f, kMagic16) : qt[m] + kMagic16;
-                    fb[ND + m] = __float_as_uint(v);
+                    fb[ND + x] = __float_as_uint(__fmaf_rn(qt[x], lev.st_scale[x], kMagic16));
                 } else {
-                    const int q = field_i<QI16>(w, ND + m);
-                    fb[ND + m] = (uint32_t)(lev.st_ratio_log2[m] ? resnap_half(q) : q);
+                    const int q = field_i<QI16>(w, ND + x);
+                    fb[ND + x] = (uint32_t)(lev.st_ratio_log2[x] ? resnap_half(q) : q);
                 }
             }
             float es[ND], M[ND];                                    // a snap is certain within es of an integer
-            {
-                // every term a multiple of 2^ex and M below 2^(24 + ex): the FP32 residual, and
-                // the definition's FP64 one, are exact, so a tie rounds to even in both
-                const int ex = min(__float2int_rn(gexp), lev.hs_exp);
-                const float tq = ex > -100 ? __int_as_float((127 + 24 + ex) << 23) : 0.0f;
-                magnitudes<FAM>(qf, qt, Gmax, hs, M);
+            magnitudes<FAM>(qf, qt, Gmax, hs, M);
 #pragma unroll
-                for (int j = 0; j < ND; ++j) {
-                    es[j] = M[j] < tq ? 1.0f : 0.5f - kBandSnap * M[j];
-                    if (c.precision == 0) es[j] = -1.0f;            // plain FP64 mode: by the definition
-                }
-            }
-            const uint32_t mult = c.out.mult ? c.in.mult[(c.t0 + tt) * 32 + lane] : 1u;
+            for (int j = 0; j < ND; ++j) es[j] = M[j] < tq ? 1.0f : __fmaf_rn(-kBandSnap, M[j], es0);
             unsigned um = 0;                                        // slots whose snap FP32 leaves undecided
 #pragma unroll
-            for (int f = 0; f < NFS; ++f) {
-                float u[ND];
-                partial32<FAM>(qf, qt, G, f, u);
-                uint32_t sv[ND][2];
-                bool so[ND][2];
+            for (int p = 0; p < NP; ++p) {
+                constexpr unsigned kPair = NFS > 1 ? kFsSlots | kFsSlots << 1 : kFsSlots;
+                if (!(vmask & (kPair << (2 * p)))) continue;        // uniform: no child of these free slots
+                // snapped residuals of (free slots 2 p and 2 p + 1) x shift, or, with one free
+                // slot, of the two shifts: y + kMagic(16) rounds to an integer, ties to even
+                float sv[ND][2][2], er[ND][2][2];
 #pragma unroll
-                for (int j = 0; j < ND; ++j)
+                for (int j = 0; j < ND; ++j) {
+                    f2 u = f2_dup(qf[j]);
 #pragma unroll
-                    for (int v = 0; v < (((DM >> j) & 1) ? 2 : 1); ++v) {
-                        const float y = ((DM >> j) & 1) ? (v ? u[j] - hs[j] : u[j] + hs[j]) : u[j];
-                        if constexpr (QO16) {
-                            // |y| <= 32000: the record passed this level's UB test (finalize_levels)
-                            const float t = y + kMagic16;
-                            so[j][v] = fabsf(y - (t - kMagic16)) < es[j];
-                            sv[j][v] = __float_as_uint(t);
+                    for (int x = 0; x < LE; ++x)
+                        if (F::uses(j, x)) u = f2_fma(f2_dup(qt[x]), G[j][x][p], u);
+                    constexpr float kM = QO16 ? kMagic16 : kMagic;
+                    const bool split = (DM >> j) & 1;
+#pragma unroll
+                    for (int v = 0; v < (NFS > 1 && split ? 2 : 1); ++v) {
+                        f2 y = u;
+                        if (split) y = f2_add(u, NFS > 1 ? f2_dup(v ? -hs[j] : hs[j]) : f2_make(hs[j], -hs[j]));
+                        const f2 t = f2_add(y, f2_dup(kM));
+                        // y - (t - kM), exact
+                        const f2 e = f2_fma(f2_add(t, f2_dup(-kM)), f2_dup(-1.0f), y);
+                        float a0, a1, b0, b1;
+                        f2_get(t, a0, a1);
+                        f2_get(e, b0, b1);
+                        if constexpr (!QO16) {                      // 16-bit children: |y| <= 32000 (finalize_levels)
+                            float y0, y1;
+                            f2_get(y, y0, y1);
+                            b0 = fabsf(y0) < 4.0e6f ? b0 : 1.0f;
+                            b1 = fabsf(y1) < 4.0e6f ? b1 : 1.0f;
+                        }
+                        if (NFS > 1) {
+                            sv[j][v][0] = a0; er[j][v][0] = b0;
+                            sv[j][v][1] = a1; er[j][v][1] = b1;
                         } else {
-                            const float t = y + kMagic;
-                            so[j][v] = fabsf(y - (t - kMagic)) < es[j] && fabsf(y) < 4.0e6f;
-                            sv[j][v] = (uint32_t)(__float_as_int(t) - 0x4B400000);
+                            sv[j][0][0] = a0; er[j][0][0] = b0;
+                            sv[j][1][0] = a1; er[j][1][0] = b1;
                         }
                     }
+                }
 #pragma unroll
-                for (int x = 0; x < NDS; ++x) {
-                    const int s = x * NFS + f, ds = DM == 2 ? x << 1 : x;
-                    if (!((vmask >> s) & 1)) continue;              // uniform
+                for (int h = 0; h < (NFS > 1 ? 2 : 1); ++h) {
+                    const int f = 2 * p + h;
+                    if (NFS > 1 && !(vmask & (kFsSlots << f))) continue;   // uniform
+#pragma unroll
+                    for (int x = 0; x < NDS; ++x) {
+                        const int s = x * NFS + f, ds = DM == 2 ? x << 1 : x;
+                        const uint4 rw = s_row[row + s];            // no passing lane: nothing is stored
+#pragma unroll
+                        for (int j = 0; j < ND; ++j) {
+                            const float t = sv[j][(ds >> j) & 1][h];
+                            fb[j] = QO16 ? __float_as_uint(t) : (uint32_t)(__float_as_int(t) - 0x4B400000);
+                        }
+                        uint32_t wo[NWO];
+                        pack<NFP, QO16>(fb, wo);
+                        store_child<NWO, ND>(rw.z, lanebit, row_address(rw) + (unsigned)__popc(rw.z & below) * (NWO * 4u),
+                                             wo, er[0][ds & 1][h], es[0], er[ND - 1][ND == 2 ? ds >> 1 : 0][h],
+                                             es[ND - 1], um, 1u << s);
+                    }
+                }
+            }
+            if (c.out.mult) {                                       // grouping: the records' multiplicities
+                const uint32_t mult = c.in.mult[(c.t0 + t0 + lt) * 32 + lane];
+                for (int s = 0; s < NS; ++s) {
                     const uint4 rw = s_row[row + s];
-                    bool sure = true;
-#pragma unroll
-                    for (int j = 0; j < ND; ++j) {
-                        fb[j] = sv[j][(ds >> j) & 1];
-                        sure &= so[j][(ds >> j) & 1];
-                    }
-                    uint32_t wo[NWO];
-                    pack<NFP, QO16>(fb, wo);
-                    const unsigned k = (unsigned)__popc(rw.z & below);
-                    uint32_t *op = reinterpret_cast<uint32_t *>(((unsigned long long)rw.y << 32) | rw.x);
-                    if (rw.z & lanebit) {
-                        store_words<NWO>(op, k, wo);
-                        if (!sure) um |= 1u << s;
-                        if (c.out.mult) c.out.mult[(op - c.out.rec) / NWO + k] = mult;
-                    }
+                    const unsigned long long i =
+                        (row_address(rw) - (unsigned long long)c.out.rec) / (NWO * 4u) + (unsigned)__popc(rw.z & below);
+                    if (rw.z & lanebit) c.out.mult[i] = mult;
                 }
             }
             if (um) {                                               // rare
                 const RecWords rwords = rec_words_of<NWI>(w);
-                for (unsigned m = um; m; m &= m - 1) {
-                    const int s = __ffs(m) - 1, f = s & (NFS - 1), x = s >> KF, ds = DM == 2 ? x << 1 : x;
+                for (unsigned r = um; r; r &= r - 1) {
+                    const int s = __ffs(r) - 1, f = s & (NFS - 1), x = s >> KF, ds = DM == 2 ? x << 1 : x;
                     const uint4 rw = s_row[row + s];
                     int3 q = make_int3(0, 0, 0);
                     if (c.precision == 1) {                         // the double-float tier
@@ -270,22 +337,17 @@ __global__ void __launch_bounds__(256, 4) k_emit(const __grid_constant__ Chunk c
                     }
                     uint32_t wo[NWO];
                     pack<NFP, QO16>(fb, wo);
-                    store_words<NWO>(reinterpret_cast<uint32_t *>(((unsigned long long)rw.y << 32) | rw.x),
-                                     (unsigned)__popc(rw.z & below), wo);
+                    store_words_if<NWO>(1u, row_address(rw) + (unsigned)__popc(rw.z & below) * (NWO * 4u), wo);
                 }
             }
         }
         __syncwarp();                                               // buffer b is free again
     }
-    if (gfail >= 0 && lane == 0) {
-        // the copies of groups gfail and gfail + 1 (no later one was issued) may still
-        // be in flight: wait for them, bounded, before the block's shared memory is
-        // released
-        const int64_t ge = gfail + 2 < g1 ? gfail + 2 : g1;
-        for (int64_t g = gfail; g < ge; ++g) {
-            const int b = (int)((g - g0) & 1);
-            if (!mbar_wait(&s_bar[b], (unsigned)(((g - g0) >> 1) & 1), GV_SPIN_LIMIT, &c.sc->err)) break;
-        }
+    if (nfail >= 0 && lane == 0) {
+        // the copies nfail and nfail + 1 (no later one was issued) may still be in flight:
+        // wait for them, bounded, before the block's shared memory is released
+        for (int n = nfail; n < nfail + (t1 >= 0 ? 2 : 1); ++n)
+            if (!mbar_wait(&s_bar[n & 1], (unsigned)(n >> 1) & 1u, GV_SPIN_LIMIT, &c.sc->err)) break;
     }
     nrechk = __reduce_add_sync(kFull, nrechk);
     ndf = __reduce_add_sync(kFull, ndf);

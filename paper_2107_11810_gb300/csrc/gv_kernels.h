@@ -76,13 +76,14 @@ struct Chunk {
     const uint32_t *in_rcnt; // its record count
     int64_t in_c0;
     int64_t t0, t1;          // tile range of the chunk
-    uint8_t *alive;          // [nc]   cell still above the pruning threshold
+    uint8_t *alive;          // [nc]   bit 0: cell still above the pruning threshold; bit 1: it has a
+                             //        surviving child
     double *geo64;           // [nc][nfs][NB]          basis change per free slot
     float *geo32;            // [nc][gf] screen coefficients G, max |G|, exponent
     float *geo32lo;          // [nc][nfs * ND * LE]    G64 - G rounded to FP32 (double-float tier)
     uint32_t *crec, *clb;    // [nc][ns]  records (UB-passing) and LB sum per child
     uint32_t *cub;           // [nc][ns]  UB sum per child (= crec without multiplicities)
-    int2 *tinfo;             // [t1 - t0] per tile: chunk-local cell (-1: pruned), valid lanes | kTileFirst |
+    int2 *tinfo;             // [t1 - t0 + 2] per tile: chunk-local cell (-1: pruned), valid lanes | kTileFirst |
                              //           kTileLast
     uint32_t *ballot;        // [t1 - t0][ns] per tile and child: UB-passing lanes
     uint32_t *lballot;       // [t1 - t0][ns] the same for the LB test
@@ -149,10 +150,10 @@ bool launch_emit(const Chunk &c, cudaStream_t st);
 // keepflag, recn: [nc * ns]; bsums: 2 * ceil(nc * ns / 256)
 void launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
                         cudaStream_t st);
-// the cells of a level (whose sum of record slots exceeds budget) with the largest UBs and LBs:
+// the cells of a level (whose sum of record slots exceeds budget) with the largest UBs (nk = 2: and LBs):
 // out and src_rbeg receive them ([ncells] at most), sc->n_cells / n_recs their number
 // and slots; bsums: 2 * ceil(ncells / 256); then their records
-void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, BeamSel *sel,
+void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, int nk, BeamSel *sel,
                         unsigned long long *bsums, const CellView &out, uint64_t *src_rbeg, Scalars *sc,
                         cudaStream_t st);
 void launch_beam_gather(const RecView &in, const RecView &out, const CellView &sel, const uint64_t *src_rbeg,

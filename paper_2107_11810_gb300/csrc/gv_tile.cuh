@@ -117,6 +117,64 @@ __device__ __forceinline__ void store_words(uint32_t *base, int64_t r, const uin
     }
 }
 
+// The emit pass's slot rows: (output address, passing lanes) of one child slot of a tile.
+__device__ __forceinline__ unsigned long long row_address(const uint4 &rw) {
+    return ((unsigned long long)rw.y << 32) | rw.x;
+}
+
+// A record's words to a global address, if this lane passes (bal & lanebit), and the slot's
+// bit into um if it passes and its snap is not certain (|e0| >= es0 or |e1| >= es1; e1 is
+// unused with one dependent coordinate): one predicate, one predicated store, no branch.
+template <int NW, int ND>
+__device__ __forceinline__ void store_child(unsigned bal, unsigned lanebit, unsigned long long p, const uint32_t *w,
+                                            float e0, float es0, float e1, float es1, unsigned &um, unsigned bit) {
+    static_assert(NW == 1 || NW == 2 || NW == 4, "records of at most four words");
+    const float x0 = fabsf(e0), x1 = fabsf(e1);
+#define GV_STORE_CHILD(ST, ...)                                                                                \
+    if constexpr (ND == 1)                                                                                     \
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\tand.b32 t, %1, %2;\n\tsetp.ne.u32 p, t, 0;\n\t" ST    \
+                     "setp.ge.and.f32 q, %4, %5, p;\n\t@q or.b32 %0, %0, %6;\n\t}"                              \
+                     : "+r"(um)                                                                                \
+                     : "r"(bal), "r"(lanebit), "l"(p), "f"(x0), "f"(es0), "r"(bit), "f"(x1), "f"(es1), __VA_ARGS__ \
+                     : "memory");                                                                              \
+    else                                                                                                       \
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 t;\n\tand.b32 t, %1, %2;\n\tsetp.ne.u32 p, t, 0;\n\t" ST    \
+                     "setp.ge.f32 q, %4, %5;\n\tsetp.ge.or.f32 q, %7, %8, q;\n\tand.pred q, q, p;\n\t"          \
+                     "@q or.b32 %0, %0, %6;\n\t}"                                                              \
+                     : "+r"(um)                                                                                \
+                     : "r"(bal), "r"(lanebit), "l"(p), "f"(x0), "f"(es0), "r"(bit), "f"(x1), "f"(es1), __VA_ARGS__ \
+                     : "memory")
+    if constexpr (NW == 1) {
+        GV_STORE_CHILD("@p st.global.u32 [%3], %9;\n\t", "r"(w[0]));
+    } else if constexpr (NW == 2) {
+        GV_STORE_CHILD("@p st.global.v2.u32 [%3], {%9, %10};\n\t", "r"(w[0]), "r"(w[1]));
+    } else {
+        GV_STORE_CHILD("@p st.global.v4.u32 [%3], {%9, %10, %11, %12};\n\t", "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]));
+    }
+#undef GV_STORE_CHILD
+}
+
+// one record's words to a global address where on != 0 (predicated stores, no branch)
+template <int NW>
+__device__ __forceinline__ void store_words_if(unsigned on, unsigned long long p, const uint32_t *w) {
+    if constexpr (NW == 1) {
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.global.u32 [%1], %2;\n\t}" ::"r"(on), "l"(p),
+                     "r"(w[0])
+                     : "memory");
+    } else if constexpr (NW == 2) {
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.global.v2.u32 [%1], {%2, %3};\n\t}" ::"r"(on),
+                     "l"(p), "r"(w[0]), "r"(w[1])
+                     : "memory");
+    } else {
+#pragma unroll
+        for (int i = 0; i < NW; i += 4)
+            asm volatile(
+                "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.global.v4.u32 [%1], {%2, %3, %4, %5};\n\t}" ::"r"(on),
+                "l"(p + 4u * i), "r"(w[i]), "r"(w[i + 1]), "r"(w[i + 2]), "r"(w[i + 3])
+                : "memory");
+    }
+}
+
 // Field i of a record as a float (exact: 16-bit fields always, 32-bit fields below 2^24).
 template <bool Q16>
 __device__ __forceinline__ float field_f(const uint32_t *w, int i) {
@@ -415,13 +473,15 @@ __device__ __forceinline__ float min3_abs(float a, float b, float c) {
     return r;
 }
 
+__device__ __forceinline__ f2 f2_dup(float x) { return f2_make(x, x); }
+
 // The screen's decisions on a pair of residuals y = (y0, y1) of one dependent coordinate
 // against the squared radius: y^2 - R^2 < 0, by its sign; the smallest |y^2 - R^2| of the
 // record goes into near, which leaves the record undecided when it falls below its band:
 // one packed multiply-add, two compares and one minimum for two tests.
-__device__ __forceinline__ void screen2(f2 y, float negr2, bool &p0, bool &p1, float &near) {
+__device__ __forceinline__ void screen2(f2 y, f2 negr2, bool &p0, bool &p1, float &near) {
     float d0, d1;
-    f2_get(f2_fma(y, y, f2_make(negr2, negr2)), d0, d1);
+    f2_get(f2_fma(y, y, negr2), d0, d1);
     p0 = d0 < 0.0f;
     p1 = d1 < 0.0f;
     near = min3_abs(near, d0, d1);
@@ -431,13 +491,13 @@ __device__ __forceinline__ void screen2(f2 y, float negr2, bool &p0, bool &p1, f
 __host__ __device__ constexpr int dep_slots(int dm) { return dm == 3 ? 4 : (dm ? 2 : 1); }
 
 // Ballots of FG free slots (1, 2 or 4) times their dependent shifts: bu/bl[ds * FG + f].
-// u[j][f]: residuals before the dependent shift.  A child passes when every dependent
-// coordinate passes, and the test of coordinate j depends only on its own shift, so with
-// two coordinates the four children of a free slot take four tests, not eight: their
-// ballots are combined.
+// u[j][p]: residuals before the dependent shift, of free slots 2 p and 2 p + 1 (FG = 1:
+// of the one slot, twice).  A child passes when every dependent coordinate passes, and
+// the test of coordinate j depends only on its own shift, so with two coordinates the
+// four children of a free slot take four tests, not eight: their ballots are combined.
 template <int ND, int FG, int DM, bool LB>
-__device__ __forceinline__ void test_children(const float (&u)[ND][FG], const float *hs, const float *negR2,
-                                              const float *negL2, float *near, float *nearL, unsigned *bu,
+__device__ __forceinline__ void test_children(const f2 (&u)[ND][(FG + 1) / 2], const float *hs, const f2 *negR2,
+                                              const f2 *negL2, float *near, float *nearL, unsigned *bu,
                                               unsigned *bl) {
     constexpr int NDS = dep_slots(DM);
     unsigned au[ND][2][FG], al[ND][2][FG];
@@ -447,11 +507,10 @@ __device__ __forceinline__ void test_children(const float (&u)[ND][FG], const fl
         if constexpr (FG >= 2) {
 #pragma unroll
             for (int p = 0; p < FG; p += 2) {
-                const f2 u2 = f2_make(u[j][p], u[j][p + 1]);
 #pragma unroll
                 for (int v = 0; v < (split ? 2 : 1); ++v) {
-                    f2 y = u2;
-                    if (split) y = f2_add(u2, v ? f2_make(-hs[j], -hs[j]) : f2_make(hs[j], hs[j]));
+                    f2 y = u[j][p / 2];
+                    if (split) y = f2_add(y, f2_dup(v ? -hs[j] : hs[j]));
                     bool p0, p1;
                     screen2(y, negR2[j], p0, p1, near[j]);
                     au[j][v][p] = __ballot_sync(kFull, p0);
@@ -463,25 +522,17 @@ __device__ __forceinline__ void test_children(const float (&u)[ND][FG], const fl
                     }
                 }
             }
-        } else if (split) {
-            const f2 y = f2_add(f2_make(u[j][0], u[j][0]), f2_make(hs[j], -hs[j]));
+        } else {
+            // the pair is the coordinate's two shifts (the same value twice without one)
+            const f2 y = split ? f2_add(u[j][0], f2_make(hs[j], -hs[j])) : u[j][0];
             bool p0, p1;
             screen2(y, negR2[j], p0, p1, near[j]);
             au[j][0][0] = __ballot_sync(kFull, p0);
-            au[j][1][0] = __ballot_sync(kFull, p1);
+            if (split) au[j][1][0] = __ballot_sync(kFull, p1);
             if constexpr (LB) {
                 screen2(y, negL2[j], p0, p1, nearL[j]);
                 al[j][0][0] = __ballot_sync(kFull, p0);
-                al[j][1][0] = __ballot_sync(kFull, p1);
-            }
-        } else {
-            const float d = __fmaf_rn(u[j][0], u[j][0], negR2[j]);
-            near[j] = fminf(near[j], fabsf(d));
-            au[j][0][0] = __ballot_sync(kFull, d < 0.0f);
-            if constexpr (LB) {
-                const float e = __fmaf_rn(u[j][0], u[j][0], negL2[j]);
-                nearL[j] = fminf(nearL[j], fabsf(e));
-                al[j][0][0] = __ballot_sync(kFull, e < 0.0f);
+                if (split) al[j][1][0] = __ballot_sync(kFull, p1);
             }
         }
     }
@@ -490,11 +541,10 @@ __device__ __forceinline__ void test_children(const float (&u)[ND][FG], const fl
         const int ds = DM == 2 ? x << 1 : x;                        // dependent bits of shift x
 #pragma unroll
         for (int f = 0; f < FG; ++f) {
-            unsigned b = kFull, l = kFull;
-#pragma unroll
-            for (int j = 0; j < ND; ++j) {
-                b &= au[j][(ds >> j) & 1][f];
-                if constexpr (LB) l &= al[j][(ds >> j) & 1][f];
+            unsigned b = au[0][ds & 1][f], l = LB ? al[0][ds & 1][f] : 0u;
+            if constexpr (ND == 2) {
+                b &= au[ND - 1][ds >> 1][f];
+                if constexpr (LB) l &= al[ND - 1][ds >> 1][f];
             }
             bu[x * FG + f] = b;
             if constexpr (LB) bl[x * FG + f] = l;
@@ -502,17 +552,15 @@ __device__ __forceinline__ void test_children(const float (&u)[ND][FG], const fl
     }
 }
 
-// Per record: squared radii (negated), and whether the screen's decisions stand.  The
-// band is proportional to the radius (Level::bandR, bandL: see finalize_levels): a
+// Whether the screen leaves a record undecided.  The band is proportional to the radius (Level::bandR, bandL: see finalize_levels): a
 // residual is within bandR R of the radius only if |y^2 - R^2| < bandR (2 + bandR) R^2.
 template <int FAM, bool LB>
-__device__ __forceinline__ bool undecided(const Level &lev, const float *R, const float *negR2, const float *near,
-                                          const float *nearL) {
+__device__ __forceinline__ bool undecided(const Level &lev, const float *R, const float *near, const float *nearL) {
     using F = Fam<FAM>;
     bool u = false;
 #pragma unroll
     for (int j = 0; j < F::ND; ++j) {
-        u |= near[j] < -negR2[j] * lev.kappa[j];
+        u |= near[j] < R[j] * R[j] * lev.kappa[j];
         if constexpr (LB) {
             const float e = __fmaf_rn(lev.bandL[j], R[j], lev.bandL0[j]);
             u |= nearL[j] < e * (e + 2.0f * lev.Lc[j]);

@@ -30,11 +30,12 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
     const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
     const Level &lev = c.lev;
-    float hs[ND], negL2[ND];
+    float hs[ND];
+    f2 negL2[ND];
 #pragma unroll
     for (int j = 0; j < ND; ++j) {
         hs[j] = lev.Hs[j];
-        negL2[j] = -lev.Lc[j] * lev.Lc[j];
+        negL2[j] = f2_dup(-lev.Lc[j] * lev.Lc[j]);
     }
     unsigned nrec = 0;
 
@@ -54,7 +55,8 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
         }
         const int nvalid = ti.y & 63;
         nrec += (unsigned)nvalid;
-        float qf[ND], qt[LE], R[ND], negR2[ND], near[ND], nearL[ND];
+        float qf[ND], qt[LE], R[ND], near[ND], nearL[ND];
+        f2 negR2[ND];
 #pragma unroll
         for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
 #pragma unroll
@@ -62,7 +64,7 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
         F::radius32(lev, qt, R);
 #pragma unroll
         for (int j = 0; j < ND; ++j) {
-            negR2[j] = -R[j] * R[j];
+            negR2[j] = f2_dup(-R[j] * R[j]);
             near[j] = nearL[j] = 3.0e38f;
         }
         // a lane without a record fails every test (its residual is out of reach)
@@ -70,33 +72,25 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
         uint32_t *bp = c.ballot + (size_t)tt * c.ns, *lp = c.lballot + (size_t)tt * c.ns;
 #pragma unroll 1
         for (int fs = 0; fs < nfs; fs += FG) {
-            float u[ND][FG];
+            f2 u[ND][(FG + 1) / 2];
 #pragma unroll
             for (int j = 0; j < ND; ++j) {
-                f2 v[FG >= 2 ? FG / 2 : 1];
-                float v1 = qf[j];
 #pragma unroll
-                for (int p = 0; p < FG / 2; ++p) v[p] = f2_make(qf[j], qf[j]);
+                for (int p = 0; p < (FG + 1) / 2; ++p) u[j][p] = f2_dup(qf[j]);
 #pragma unroll
                 for (int m = 0; m < LE; ++m) {
                     if (!F::uses(j, m)) continue;
                     const float *g = sg + (j * LE + m) * nfs + fs;
+                    const f2 q2 = f2_dup(qt[m]);
                     if constexpr (FG == 4) {
-                        const float4 g4 = *reinterpret_cast<const float4 *>(g);
-                        v[0] = f2_fma(f2_make(qt[m], qt[m]), f2_make(g4.x, g4.y), v[0]);
-                        v[1] = f2_fma(f2_make(qt[m], qt[m]), f2_make(g4.z, g4.w), v[1]);
+                        const ulonglong2 g4 = *reinterpret_cast<const ulonglong2 *>(g);
+                        u[j][0] = f2_fma(q2, g4.x, u[j][0]);
+                        u[j][1] = f2_fma(q2, g4.y, u[j][1]);
                     } else if constexpr (FG == 2) {
-                        const float2 g2 = *reinterpret_cast<const float2 *>(g);
-                        v[0] = f2_fma(f2_make(qt[m], qt[m]), f2_make(g2.x, g2.y), v[0]);
+                        u[j][0] = f2_fma(q2, *reinterpret_cast<const f2 *>(g), u[j][0]);
                     } else {
-                        v1 = __fmaf_rn(qt[m], g[0], v1);
+                        u[j][0] = f2_fma(q2, f2_dup(g[0]), u[j][0]);
                     }
-                }
-                if constexpr (FG == 1) {
-                    u[j][0] = v1;
-                } else {
-#pragma unroll
-                    for (int p = 0; p < FG / 2; ++p) f2_get(v[p], u[j][2 * p], u[j][2 * p + 1]);
                 }
             }
             unsigned bu[FG * NDS], bl[FG * NDS];
@@ -120,7 +114,7 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
             }
         }
         const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
-        const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, negR2, near, nearL)) & act;
+        const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, near, nearL)) & act;
         if (unsb) {                                                 // rare: left to the definition
             __syncwarp();                                           // lane 0's stores
             for (int s = lane; s < c.ns; s += 32) {
@@ -210,8 +204,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
             qt[m] = field_f<QI16>(w, ND + m);
             if constexpr (QO16) {
                 // adding kMagic16 rounds to an integer, ties to even, biased by 2^15
-                float x = lev.st_ratio_log2[m] ? __fmaf_rn(qt[m], 0.5f, kMagic16) : qt[m] + kMagic16;
-                fb[ND + m] = __float_as_uint(x);
+                fb[ND + m] = __float_as_uint(__fmaf_rn(qt[m], lev.st_scale[m], kMagic16));
             } else {
                 const int q = field_i<QI16>(w, ND + m);
                 fb[ND + m] = (uint32_t)(lev.st_ratio_log2[m] ? resnap_half(q) : q);
@@ -222,15 +215,14 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
             // every term a multiple of 2^ex and M below 2^(24 + ex): the FP32 residual, and
             // the definition's FP64 one, are exact, so a tie rounds to even in both
             const int ex = min(__float2int_rn(G[c.gf - 1]), lev.hs_exp);
-            const float tq = ex > -100 ? __int_as_float((127 + 24 + ex) << 23) : 0.0f;
+            const float tq = ex > -100 && c.precision == 1 ? __int_as_float((127 + 24 + ex) << 23) : 0.0f;
             magnitudes<FAM>(qf, qt, G + nfs * ND * LE, hs, M);
 #pragma unroll
             for (int j = 0; j < ND; ++j) {
-                es[j] = M[j] < tq ? 1.0f : 0.5f - kBandSnap * M[j];
-                if (c.precision == 0) es[j] = -1.0f;                // plain FP64 mode: by the definition
+                // plain FP64 mode: no snap is certain
+                es[j] = M[j] < tq ? 1.0f : __fmaf_rn(-kBandSnap, M[j], c.precision == 1 ? 0.5f : -1.0f);
             }
         }
-        const uint32_t mult = c.out.mult ? c.in.mult[r] : 1u;
         unsigned long long um = 0ull;                               // slots whose snap FP32 leaves undecided
 #pragma unroll 1
         for (int f = 0; f < nfs; ++f) {
@@ -276,13 +268,17 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
                 }
                 uint32_t wo[NWO];
                 pack<NFP, QO16>(fb, wo);
-                const unsigned k = (unsigned)__popc(rw.z & below);
-                uint32_t *op = reinterpret_cast<uint32_t *>(((unsigned long long)rw.y << 32) | rw.x);
-                if (rw.z & lanebit) {
-                    store_words<NWO>(op, k, wo);
-                    if (!sure) um |= 1ull << s;
-                    if (c.out.mult) c.out.mult[(op - c.out.rec) / NWO + k] = mult;
-                }
+                store_words_if<NWO>(rw.z & lanebit, row_address(rw) + (unsigned)__popc(rw.z & below) * (NWO * 4u), wo);
+                if ((rw.z & lanebit) && !sure) um |= 1ull << s;
+            }
+        }
+        if (c.out.mult) {                                           // grouping: the records' multiplicities
+            const uint32_t mult = c.in.mult[r];
+            for (int s = 0; s < NS; ++s) {
+                const uint4 rw = s_row[s];
+                const unsigned long long i =
+                    (row_address(rw) - (unsigned long long)c.out.rec) / (NWO * 4u) + (unsigned)__popc(rw.z & below);
+                if (rw.z & lanebit) c.out.mult[i] = mult;
             }
         }
         if (um) {                                                   // rare
@@ -316,8 +312,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
                 }
                 uint32_t wo[NWO];
                 pack<NFP, QO16>(fb, wo);
-                store_words<NWO>(reinterpret_cast<uint32_t *>(((unsigned long long)rw.y << 32) | rw.x),
-                                 (unsigned)__popc(rw.z & below), wo);
+                store_words_if<NWO>(1u, row_address(rw) + (unsigned)__popc(rw.z & below) * (NWO * 4u), wo);
             }
         }
     }
