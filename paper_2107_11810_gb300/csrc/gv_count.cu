@@ -38,8 +38,8 @@ template <int FAM, bool Q16, int KF, int DM, bool LB>
 __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk c) {
     using F = Fam<FAM>;
     constexpr int ND = F::ND, LE = F::LE, NFS = 1 << KF, NS = NFS * dep_slots(DM), NP = (NFS + 1) / 2;
-    constexpr int NW = rec_words(F::NFP, Q16), NG = NFS * ND * LE;
-    static_assert(NG <= 32 && NS >= 2 && NS <= 8, "coefficients of a cell fit one register per lane");
+    constexpr int NW = rec_words(F::NFP, Q16), NG = F::NBG * NFS;
+    static_assert(NG <= 32 && NS >= 2 && NS <= 8, "a cell's basis changes fit one register per lane");
     const int lane = threadIdx.x & 31;
     const Level &lev = c.lev;
     const int64_t nt = c.t1 - c.t0;
@@ -54,11 +54,24 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
         negL2[j] = f2_dup(-lev.Lc[j] * lev.Lc[j]);
     }
     const float *gp = c.geo32 + (lane < NG ? lane : 0);
-    auto load_g = [&](int cell) { return __ldg(gp + (unsigned)(cell < 0 ? 0 : cell) * (size_t)c.gf); };
+    auto load_g = [&](int cell) {
+        if constexpr (NG == 0) return 0.0f;
+        else return __ldg(gp + (unsigned)(cell < 0 ? 0 : cell) * (size_t)c.gf);
+    };
     int run = -1;
     f2 G[ND][LE][NP];
 #pragma unroll
-    for (int i = 0; i < ND * LE * NP; ++i) G[i / (LE * NP)][i / NP % LE][i % NP] = 0ull;
+    for (int j = 0; j < ND; ++j)
+#pragma unroll
+        for (int m = 0; m < LE; ++m)
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                G[j][m][p] = 0ull;
+                if constexpr (NG == 0)                              // a linear basis: the same for every cell
+                    if (F::uses(j, m))
+                        G[j][m][p] = f2_make(coef32<FAM>(lev, j, m, lin_change<FAM>(c, F::cb(j, m), 2 * p, false)),
+                                             coef32<FAM>(lev, j, m, lin_change<FAM>(c, F::cb(j, m), NFS > 1 ? 2 * p + 1 : 0, false)));
+            }
     unsigned nrec = 0;
     const uint32_t *rp = c.in.rec + ((c.t0 + ta) * 32 + lane) * NW;
     const int2 *tp = c.tinfo + ta;
@@ -82,19 +95,24 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
         g1 = load_g(ti1.x);
         ti2 = tp[1];
         if (ti.x < 0) continue;                                     // uniform: the cell was pruned
-        if (ti.x != run) {                                          // uniform: a new cell
-            run = ti.x;
+        if constexpr (NG > 0) {
+            if (ti.x != run) {                                      // uniform: a new cell
+                run = ti.x;
+                float d[F::NBG ? F::NBG : 1][NFS];
 #pragma unroll
-            for (int j = 0; j < ND; ++j)
+                for (int x = 0; x < F::NBG; ++x)
 #pragma unroll
-                for (int m = 0; m < LE; ++m)
+                    for (int f = 0; f < NFS; ++f) d[x][f] = __shfl_sync(kFull, g, x * NFS + f);
 #pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        if (!F::uses(j, m)) continue;
-                        const int f1 = NFS > 1 ? 2 * p + 1 : 0;     // one free slot: the pair holds it twice
-                        G[j][m][p] = f2_make(__shfl_sync(kFull, g, (2 * p * ND + j) * LE + m),
-                                             __shfl_sync(kFull, g, (f1 * ND + j) * LE + m));
-                    }
+                for (int j = 0; j < ND; ++j)
+#pragma unroll
+                    for (int m = 0; m < LE; ++m)
+#pragma unroll
+                        for (int p = 0; p < NP; ++p)                // one free slot: the pair holds it twice
+                            if (F::uses(j, m))
+                                G[j][m][p] = f2_make(coef32<FAM>(lev, j, m, d[F::cb(j, m)][2 * p]),
+                                                     coef32<FAM>(lev, j, m, d[F::cb(j, m)][NFS > 1 ? 2 * p + 1 : 0]));
+            }
         }
         const int nvalid = ti.y & 63;
         nrec += (unsigned)nvalid;

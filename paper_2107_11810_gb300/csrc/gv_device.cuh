@@ -50,6 +50,10 @@ struct Level {                 // tests of the children of a level-l cell
     double A1[GV_MAXD];        // accumulated canonization error at level l+1
     double rlb[GV_MAXD];       // eps_j - A1_j             (lower-bound radius)
     double gscale[GV_MAXD][GV_MAXT];  // s_t,m / s_f,j (a power of two)
+    float gs[GV_MAXD][GV_MAXT];       // the same
+    float h1f[GV_MAXD], h1f_lo[GV_MAXD];  // h1 rounded to FP32 and what that leaves
+    int g_exp;                 // linear bases: every coefficient is FP32-exact and a multiple of 2^g_exp
+                               // (<= 0); -1000 otherwise
     // FP32 screen constants, in units of s_f,j (dependent coordinate j)
     float Hs[GV_MAXD];         // h1 of dependent coordinate j
     float Hs_lo[GV_MAXD];      // h1 / s_f,j - Hs rounded to FP32 (the double-float tier's low part)
@@ -185,9 +189,10 @@ __device__ __forceinline__ uint64_t child_key(const Problem &P, uint64_t key, in
 // Families.  For each: D, K (free coords), ND (dependent), LE (essential params),
 // NP (input rows), NB (basis values), NFP (record fields, padded so that a record
 // is 1, 2 or a multiple of 4 words); basis(), lift(), residual64(), partial64(),
-// lipschitz64() (the exact FP64 definition), and for the FP32 screen coef()
-// (coefficient of t_m in dependent residual j for a basis change), uses(j, m)
-// (whether t_m enters residual j at all) and radius32() (the UB radius in steps).
+// lipschitz64() (the exact FP64 definition), and for the FP32 screen uses(j, m)
+// (whether t_m enters residual j at all), cb(j, m) and cneg(j, m) (the basis value whose
+// change is its coefficient there, and whether negated), NBG (the basis values, the
+// first ones, whose changes depend on the cell) and radius32() (the UB radius in steps).
 // LINEAR_BASIS: the basis is the free coordinate itself; LINEAR_TAIL: the last
 // basis value is the last free coordinate (its change is the exact child shift).
 // ---------------------------------------------------------------------------
@@ -199,7 +204,7 @@ template <int FAM> struct Fam;
 // LINE2D: coords (m, b); b = y - x m.  t = x, psi = m (linear: its change across a
 // child shift is the shift itself).
 template <> struct Fam<FAM_LINE2D> {
-    static constexpr int D = 2, K = 1, ND = 1, LE = 1, NP = 2, NB = 1, NFP = 2;
+    static constexpr int D = 2, K = 1, ND = 1, LE = 1, NP = 2, NB = 1, NFP = 2, NBG = 0;
     static constexpr bool LINEAR_BASIS = true, LINEAR_TAIL = false;
     __host__ __device__ static constexpr bool uses(int, int) { return true; }
     __device__ static void basis(const Problem &, const double *c, double *psi) { psi[0] = c[0]; }
@@ -219,7 +224,8 @@ template <> struct Fam<FAM_LINE2D> {
     __device__ static void partial64(const double *f, const double *t, const double *dpsi, double *p) {
         p[0] = dsub(f[0], dmul(t[0], dpsi[0]));
     }
-    __device__ static void coef(const double *dpsi, double *g) { g[0] = -dpsi[0]; }
+    __host__ __device__ static constexpr int cb(int j, int m) { return 0; }
+    __host__ __device__ static constexpr bool cneg(int j, int m) { return true; }
     // |t| = s_t |q_t|: radius = rc0 + lam_c[0] |q_t|
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
         R[0] = __fmaf_rn(lev.lam_c[0], fabsf(qt[0]), lev.rc0[0]);
@@ -228,7 +234,7 @@ template <> struct Fam<FAM_LINE2D> {
 
 // PLANE3D_SPH: coords (theta, phi, d); d = q . n(theta, phi).  t = q; psi = n.
 template <> struct Fam<FAM_PLANE3D_SPH> {
-    static constexpr int D = 3, K = 2, ND = 1, LE = 3, NP = 3, NB = 3, NFP = 4;
+    static constexpr int D = 3, K = 2, ND = 1, LE = 3, NP = 3, NB = 3, NFP = 4, NBG = 3;
     static constexpr bool LINEAR_BASIS = false, LINEAR_TAIL = false;
     __host__ __device__ static constexpr bool uses(int, int) { return true; }
     __device__ static void basis(const Problem &, const double *c, double *psi) {
@@ -258,7 +264,8 @@ template <> struct Fam<FAM_PLANE3D_SPH> {
         lam[0] = dsqrt(dadd(xy, dmul(t[2], t[2])));
         lam[1] = dsqrt(xy);
     }
-    __device__ static void coef(const double *dpsi, double *g) { g[0] = dpsi[0]; g[1] = dpsi[1]; g[2] = dpsi[2]; }
+    __host__ __device__ static constexpr int cb(int j, int m) { return m; }
+    __host__ __device__ static constexpr bool cneg(int j, int m) { return false; }
     // s_t,x = s_t,y (their sigma bounds are equal) and s_t,z = s_t,x sqrt(rho2):
     // |q| = s_t,x sqrt(qx^2 + qy^2 + rho2 qz^2), |q_xy| = s_t,x sqrt(qx^2 + qy^2)
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
@@ -271,7 +278,7 @@ template <> struct Fam<FAM_PLANE3D_SPH> {
 // POSE3DOF: coords (yaw, x, y); x = w1 - (a cos yaw - b sin yaw),
 // y = w2 - (a sin yaw + b cos yaw).  t = (a, b); psi = (cos yaw, sin yaw).
 template <> struct Fam<FAM_POSE3DOF> {
-    static constexpr int D = 3, K = 1, ND = 2, LE = 2, NP = 4, NB = 2, NFP = 4;
+    static constexpr int D = 3, K = 1, ND = 2, LE = 2, NP = 4, NB = 2, NFP = 4, NBG = 2;
     static constexpr bool LINEAR_BASIS = false, LINEAR_TAIL = false;
     __host__ __device__ static constexpr bool uses(int, int) { return true; }
     __device__ static void basis(const Problem &, const double *c, double *psi) {
@@ -302,10 +309,8 @@ template <> struct Fam<FAM_POSE3DOF> {
         lam[1] = r;
     }
     // x residual: -a dcos + b dsin; y residual: -a dsin - b dcos
-    __device__ static void coef(const double *dpsi, double *g) {
-        g[0] = -dpsi[0]; g[1] = dpsi[1];
-        g[2] = -dpsi[1]; g[3] = -dpsi[0];
-    }
+    __host__ __device__ static constexpr int cb(int j, int m) { return j == m ? 0 : 1; }
+    __host__ __device__ static constexpr bool cneg(int j, int m) { return !(j == 0 && m == 1); }
     // s_t,a = s_t,b: sqrt(a^2 + b^2) = s_t sqrt(qa^2 + qb^2)
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
         float r = sqrt32(__fmaf_rn(qt[1], qt[1], qt[0] * qt[0]));
@@ -317,7 +322,7 @@ template <> struct Fam<FAM_POSE3DOF> {
 // RAYS3D: rays in 3-space (Sec. 4.3); coords (x, y, z); y = a x + b, z = c x + d.
 // t = (a, c); psi = x (linear: its change across a child shift is the shift itself).
 template <> struct Fam<FAM_RAYS3D> {
-    static constexpr int D = 3, K = 1, ND = 2, LE = 2, NP = 4, NB = 1, NFP = 4;
+    static constexpr int D = 3, K = 1, ND = 2, LE = 2, NP = 4, NB = 1, NFP = 4, NBG = 0;
     static constexpr bool LINEAR_BASIS = true, LINEAR_TAIL = false;
     __host__ __device__ static constexpr bool uses(int j, int m) { return j == m; }
     __device__ static void basis(const Problem &, const double *c, double *psi) { psi[0] = c[0]; }
@@ -342,10 +347,8 @@ template <> struct Fam<FAM_RAYS3D> {
         lam[0] = fabs(t[0]);
         lam[1] = fabs(t[1]);
     }
-    __device__ static void coef(const double *dpsi, double *g) {
-        g[0] = dpsi[0]; g[1] = 0.0;
-        g[2] = 0.0; g[3] = dpsi[0];
-    }
+    __host__ __device__ static constexpr int cb(int j, int m) { return 0; }
+    __host__ __device__ static constexpr bool cneg(int j, int m) { return false; }
     // |a| h1_x = lam_c[0] |q_a|, |c| h1_x = lam_c[1] |q_c|
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
         R[0] = __fmaf_rn(lev.lam_c[0], fabsf(qt[0]), lev.rc0[0]);
@@ -357,7 +360,7 @@ template <> struct Fam<FAM_RAYS3D> {
 // d = 4); coords (a1, a2, a3, b), dual surface b = x4 - a . x.  t = (x1, x2, x3);
 // psi = (a1, a2, a3) (linear: their changes across a child shift are the shifts).
 template <> struct Fam<FAM_AFFINE4D> {
-    static constexpr int D = 4, K = 3, ND = 1, LE = 3, NP = 4, NB = 3, NFP = 4;
+    static constexpr int D = 4, K = 3, ND = 1, LE = 3, NP = 4, NB = 3, NFP = 4, NBG = 0;
     static constexpr bool LINEAR_BASIS = true, LINEAR_TAIL = false;
     __host__ __device__ static constexpr bool uses(int, int) { return true; }
     __device__ static void basis(const Problem &, const double *c, double *psi) {
@@ -388,11 +391,8 @@ template <> struct Fam<FAM_AFFINE4D> {
         lam[1] = fabs(t[1]);
         lam[2] = fabs(t[2]);
     }
-    __device__ static void coef(const double *dpsi, double *g) {
-        g[0] = -dpsi[0];
-        g[1] = -dpsi[1];
-        g[2] = -dpsi[2];
-    }
+    __host__ __device__ static constexpr int cb(int j, int m) { return m; }
+    __host__ __device__ static constexpr bool cneg(int j, int m) { return true; }
     // sum_i |x_i| h1_i = sum_i lam_c[i] |q_i|
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
         R[0] = __fmaf_rn(lev.lam_c[0], fabsf(qt[0]),
@@ -405,7 +405,7 @@ template <> struct Fam<FAM_AFFINE4D> {
 // a = g_a - u c - v d and b = g_b - v c + u d, u = p_x/|p|^2, v = p_y/|p|^2; t = (u, v),
 // psi = (c, d) (linear: their changes across a child shift are the shifts).
 template <> struct Fam<FAM_POINTSET2D> {
-    static constexpr int D = 4, K = 2, ND = 2, LE = 2, NP = 4, NB = 2, NFP = 4;
+    static constexpr int D = 4, K = 2, ND = 2, LE = 2, NP = 4, NB = 2, NFP = 4, NBG = 0;
     static constexpr bool LINEAR_BASIS = true, LINEAR_TAIL = false;
     __host__ __device__ static constexpr bool uses(int, int) { return true; }
     __device__ static void basis(const Problem &, const double *c, double *psi) {
@@ -440,10 +440,8 @@ template <> struct Fam<FAM_POINTSET2D> {
         lam[2] = fabs(t[1]);
         lam[3] = fabs(t[0]);
     }
-    __device__ static void coef(const double *dpsi, double *g) {
-        g[0] = -dpsi[0]; g[1] = -dpsi[1];      // a: -(u dc + v dd)
-        g[2] = dpsi[1]; g[3] = -dpsi[0];       // b: -(v dc - u dd)
-    }
+    __host__ __device__ static constexpr int cb(int j, int m) { return j == m ? 0 : 1; }
+    __host__ __device__ static constexpr bool cneg(int j, int m) { return !(j == 1 && m == 0); }
     // lam_c: [a with |u|, a with |v|, b with |v|, b with |u|]
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
         const float au = fabsf(qt[0]), av = fabsf(qt[1]);
@@ -459,7 +457,7 @@ template <> struct Fam<FAM_POINTSET2D> {
 // t = (w, xi w, eta w, xi, eta).  R by Rodrigues' formula with its three scalar
 // functions as power series in theta^2 (no division by theta, no sin/cos).
 template <> struct Fam<FAM_POSE6DOF> {
-    static constexpr int D = 6, K = 4, ND = 2, LE = 11, NP = 5, NB = 10, NFP = 16;
+    static constexpr int D = 6, K = 4, ND = 2, LE = 11, NP = 5, NB = 10, NFP = 16, NBG = 9;
     static constexpr bool LINEAR_BASIS = false, LINEAR_TAIL = true;
     // x uses w (with r1), xi w (r3), xi (z); y uses w (r2), eta w (r3), eta (z)
     __host__ __device__ static constexpr bool uses(int j, int m) {
@@ -533,20 +531,9 @@ template <> struct Fam<FAM_POSE6DOF> {
         lam[0] = lx; lam[1] = lx; lam[2] = lx; lam[3] = fabs(t[9]);
         lam[4] = ly; lam[5] = ly; lam[6] = ly; lam[7] = fabs(t[10]);
     }
-    // g[j * LE + m]: coefficient of t_m in residual j for basis changes dpsi
-    __device__ static void coef(const double *dpsi, double *g) {
-#pragma unroll
-        for (int x = 0; x < ND * LE; ++x) g[x] = 0.0;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            g[i] = -dpsi[i];                 // x: -r1 . w
-            g[3 + i] = dpsi[6 + i];          // x: xi w . r3
-            g[LE + i] = -dpsi[3 + i];        // y: -r2 . w
-            g[LE + 6 + i] = dpsi[6 + i];     // y: eta w . r3
-        }
-        g[9] = dpsi[9];                      // x: xi z
-        g[LE + 10] = dpsi[9];                // y: eta z
-    }
+    // x: -r1 . w + xi w . r3 + xi z; y: -r2 . w + eta w . r3 + eta z
+    __host__ __device__ static constexpr int cb(int j, int m) { return m >= 9 ? 9 : (m >= 6 ? m : (m >= 3 ? m + 3 : 3 * j + m)); }
+    __host__ __device__ static constexpr bool cneg(int j, int m) { return m < 3; }
     // s_t equal for the nine rotation coefficients and for xi, eta:
     // |w| + |xi w| = s_t (|q_w| + |q_xiw|); lam_c: [x rotation, x z, y rotation, y z]
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {
@@ -564,7 +551,7 @@ template <> struct Fam<FAM_POSE6DOF> {
 // rho y, affine in the basis psi = (rows of R(phi), y) (r3 unused) with coefficients
 // t = (rho w, w, rho).
 template <> struct Fam<FAM_RADIAL5DOF> {
-    static constexpr int D = 5, K = 4, ND = 1, LE = 7, NP = 5, NB = 10, NFP = 8;
+    static constexpr int D = 5, K = 4, ND = 1, LE = 7, NP = 5, NB = 10, NFP = 8, NBG = 6;
     static constexpr bool LINEAR_BASIS = false, LINEAR_TAIL = true;
     __host__ __device__ static constexpr bool uses(int, int) { return true; }
     __device__ static void basis(const Problem &P, const double *c, double *psi) {
@@ -604,15 +591,9 @@ template <> struct Fam<FAM_RADIAL5DOF> {
         const double lx = dadd(nrw, nw);
         lam[0] = lx; lam[1] = lx; lam[2] = lx; lam[3] = fabs(t[6]);
     }
-    // g[m]: coefficient of t_m in x for basis changes dpsi
-    __device__ static void coef(const double *dpsi, double *g) {
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            g[i] = dpsi[i];                  // rho w . r1
-            g[3 + i] = -dpsi[3 + i];         // -w . r2
-        }
-        g[6] = -dpsi[9];                     // -rho y
-    }
+    // rho w . r1 - w . r2 - rho y
+    __host__ __device__ static constexpr int cb(int j, int m) { return m == 6 ? 9 : m; }
+    __host__ __device__ static constexpr bool cneg(int j, int m) { return m >= 3; }
     // s_t equal for the six rotation coefficients: |rho w| + |w| = s_t (|q_rw| + |q_w|);
     // lam_c: [rotation, y]
     __device__ static void radius32(const Level &lev, const float *qt, float *R) {

@@ -43,11 +43,11 @@ template <int FAM, bool QI16, bool QO16, int KF, int DM>
 __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c) {
     using F = Fam<FAM>;
     constexpr int ND = F::ND, LE = F::LE, NFP = F::NFP, NFS = 1 << KF, NDS = dep_slots(DM), NS = NFS * NDS;
-    constexpr int NWI = rec_words(NFP, QI16), NWO = rec_words(NFP, QO16), RW = 32 * NWI, NG = NFS * ND * LE;
+    constexpr int NWI = rec_words(NFP, QI16), NWO = rec_words(NFP, QO16), RW = 32 * NWI, NG = F::NBG * NFS;
     constexpr int GT = kEmitTiles, NP = (NFS + 1) / 2;
     // child slots of free slot 0 (those of free slot f: shifted left by f)
     constexpr unsigned kFsSlots = NDS == 4 ? 1u | 1u << NFS | 1u << 2 * NFS | 1u << 3 * NFS : (NDS == 2 ? 1u | 1u << NFS : 1u);
-    static_assert(geo32_floats(NFS, ND, LE) <= 32, "a cell's coefficients fit one register per lane");
+    static_assert(NG + F::NBG <= 32, "a cell's basis changes fit one register per lane");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Level &lev = c.lev;
     extern __shared__ __align__(128) uint8_t s_dyn[];
@@ -111,13 +111,13 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
         bulk_load(s_bal + b * GT * NS, c.ballot + (size_t)t0 * NS, bbytes, &s_bar[b]);
         bulk_load(s_off + b * GT * NS, c.off + (size_t)t0 * NS, bbytes, &s_bar[b]);
     };
-    // a cell's data, one word per lane: coefficient, child's first slot and index
+    // a cell's data, one word per lane: basis change, child's first slot and index
     float pg = 0.0f;
     unsigned long long pbase = ~0ull;
     int pidx = 0;
     auto prefetch = [&](int cell) {
         if (cell < 0) return;                                       // uniform
-        if (lane < c.gf) pg = __ldg(c.geo32 + (size_t)cell * c.gf + lane);
+        if (lane < NG + F::NBG) pg = __ldg(c.geo32 + (size_t)cell * c.gf + lane);
         if (lane < NS) {
             pbase = c.cbase[(size_t)cell * NS + lane];
             pidx = c.child_idx[(size_t)cell * NS + lane];
@@ -130,15 +130,31 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
     const unsigned below = (1u << lane) - 1u, lanebit = 1u << lane;
     int cur = -1, pcell = -1, row = 0;                              // the cell at hand, the prefetched one
     f2 G[ND][LE][NP];
-    float Gmax[ND * LE], tq = 0.0f;
+    float Gmax[ND * LE];
+    // every term a multiple of 2^ex and M below 2^(24 + ex): the FP32 residual, and the
+    // definition's FP64 one, are exact, so a tie rounds to even in both
+    const int ex = min(lev.g_exp, lev.hs_exp);
+    const float tq = ex > -100 && c.precision == 1 ? __int_as_float((127 + 24 + ex) << 23) : 0.0f;
     const float es0 = c.precision == 1 ? 0.5f : -1.0f;              // plain FP64 mode: no snap is certain
     unsigned long long crec = 0;                                    // lane s: child s's first record, 0 when pruned
     uint32_t *ctile = nullptr;                                      // and its first tile -> cell entry
     int cidx = 0;
 #pragma unroll
-    for (int i = 0; i < ND * LE * NP; ++i) G[i / (LE * NP)][i / NP % LE][i % NP] = 0ull;
+    for (int j = 0; j < ND; ++j)
 #pragma unroll
-    for (int i = 0; i < ND * LE; ++i) Gmax[i] = 0.0f;
+        for (int x = 0; x < LE; ++x) {
+            Gmax[j * LE + x] = 0.0f;
+#pragma unroll
+            for (int p = 0; p < NP; ++p) G[j][x][p] = 0ull;
+            if constexpr (NG == 0) {                                // a linear basis: the same for every cell
+                if (!F::uses(j, x)) continue;
+#pragma unroll
+                for (int p = 0; p < NP; ++p)
+                    G[j][x][p] = f2_make(coef32<FAM>(lev, j, x, lin_change<FAM>(c, F::cb(j, x), 2 * p, false)),
+                                         coef32<FAM>(lev, j, x, lin_change<FAM>(c, F::cb(j, x), NFS > 1 ? 2 * p + 1 : 0, false)));
+                Gmax[j * LE + x] = fabsf(coef32<FAM>(lev, j, x, lin_change<FAM>(c, F::cb(j, x), 0, false)));
+            }
+        }
     unsigned nrechk = 0, ndf = 0, bad = 0;
     int t1, cells1, nfail = -1;                                     // copy that did not arrive
     next_group(t1, cells1);
@@ -166,23 +182,26 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
                 crec = pbase == ~0ull ? 0ull : (unsigned long long)(c.out.rec + pbase * NWO);
                 ctile = c.out.tile_cell + (pbase >> 5);
                 cidx = pidx;
+                if constexpr (NG > 0) {
+                    float d[F::NBG ? F::NBG : 1][NFS + 1];          // the last: the largest magnitude
 #pragma unroll
-                for (int j = 0; j < ND; ++j)
+                    for (int x = 0; x < F::NBG; ++x) {
 #pragma unroll
-                    for (int x = 0; x < LE; ++x)
+                        for (int f = 0; f < NFS; ++f) d[x][f] = __shfl_sync(kFull, pg, x * NFS + f);
+                        d[x][NFS] = __shfl_sync(kFull, pg, NG + x);
+                    }
 #pragma unroll
-                        for (int p = 0; p < NP; ++p) {
+                    for (int j = 0; j < ND; ++j)
+#pragma unroll
+                        for (int x = 0; x < LE; ++x) {
                             if (!F::uses(j, x)) continue;
-                            const int f1 = NFS > 1 ? 2 * p + 1 : 0;
-                            G[j][x][p] = f2_make(__shfl_sync(kFull, pg, (2 * p * ND + j) * LE + x),
-                                                 __shfl_sync(kFull, pg, (f1 * ND + j) * LE + x));
-                        }
 #pragma unroll
-                for (int i = 0; i < ND * LE; ++i) Gmax[i] = __shfl_sync(kFull, pg, NG + i);
-                // every term a multiple of 2^ex and M below 2^(24 + ex): the FP32 residual, and
-                // the definition's FP64 one, are exact, so a tie rounds to even in both
-                const int ex = min(__float2int_rn(__shfl_sync(kFull, pg, NG + ND * LE)), lev.hs_exp);
-                tq = ex > -100 && c.precision == 1 ? __int_as_float((127 + 24 + ex) << 23) : 0.0f;
+                            for (int p = 0; p < NP; ++p)
+                                G[j][x][p] = f2_make(coef32<FAM>(lev, j, x, d[F::cb(j, x)][2 * p]),
+                                                     coef32<FAM>(lev, j, x, d[F::cb(j, x)][NFS > 1 ? 2 * p + 1 : 0]));
+                            Gmax[j * LE + x] = d[F::cb(j, x)][NFS] * lev.gs[j][x];
+                        }
+                }
             }
             {
                 // the cell of the next tile to be taken
@@ -307,21 +326,18 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
                 }
             }
             if (um) {                                               // rare
-                const RecWords rwords = rec_words_of<NWI>(w);
+                const RecWords<NWI> rwords = rec_words_of<NWI>(w);
                 for (unsigned r = um; r; r &= r - 1) {
                     const int s = __ffs(r) - 1, f = s & (NFS - 1), x = s >> KF, ds = DM == 2 ? x << 1 : x;
                     const uint4 rw = s_row[row + s];
                     int3 q = make_int3(0, 0, 0);
                     if (c.precision == 1) {                         // the double-float tier
-                        q = snap_df_words<FAM, QI16>(&c.lev, rwords, c.geo32 + (size_t)cl * c.gf + f * ND * LE,
-                                                     c.geo32lo + ((size_t)cl * NFS + f) * ND * LE, ds,
-                                                     __fmaf_ru(kBandDF, M[0], kBandDFAbs),
+                        q = snap_df_words<FAM, QI16>(&c, rwords, cl, f, ds, __fmaf_ru(kBandDF, M[0], kBandDFAbs),
                                                      __fmaf_ru(kBandDF, M[ND - 1], kBandDFAbs), QO16 ? 32767.0f : 1.0e9f);
                         ++ndf;
                     }
                     if (!q.z) {                                     // the FP64 definition
-                        q = snap64_words<FAM, QI16>(&c.P, &c.lev, rwords,
-                                                    c.geo64 + ((size_t)cl * NFS + f) * F::NB, ds, c.dm);
+                        q = snap64_words<FAM, QI16>(&c, rwords, cl, f, ds);
                         bad |= (unsigned)(q.z != 0);
                         nrechk += c.precision == 1;
                     }

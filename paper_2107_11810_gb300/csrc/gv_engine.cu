@@ -99,6 +99,8 @@ struct vote_ctx {
     LevelStore ls[GV_MAXL + 1];
     LevelStore beam;           // the selected cells of one level, during the dive
     DevBuf beam_sel, beam_src;
+    DevBuf sctab[2];           // (sin, cos) tables of the angular coordinates (launch_sincos_table)
+    DevBuf rot[GV_MAXL + 1], rotflag[GV_MAXL + 1];   // rotation tables per level (k_rot_fill)
     DevBuf levs_dev, path, scal, alive, geo64, geo32, geo32lo, cnt, tinfo, ballot, lballot, uns, off, cbase, child_idx;
     DevBuf keepflag, recn, bsums;
     DevBuf tr_level, tr_key, tr_ub, tr_lb, surf_tmp, mask_tmp;
@@ -183,6 +185,33 @@ static double pow2_floor(double x, int *e_out) {
     std::frexp(x, &e);
     if (e_out) *e_out = e - 1;
     return std::ldexp(1.0, e - 1);
+}
+
+// Linear bases: the largest e <= 0 with every coefficient h1_b s_t,m / s_f,j of the
+// screen an FP32-exact multiple of 2^e; kNoExp when one is not, and for other bases.
+template <int FAM>
+static int linear_exp_fam(const Problem &, const Level &v) {
+    using F = Fam<FAM>;
+    if (!F::LINEAR_BASIS) return kNoExp;
+    int e = 0;
+    for (int j = 0; j < F::ND; ++j)
+        for (int m = 0; m < F::LE; ++m) {
+            const int b = F::cb(j, m);
+            if (!F::uses(j, m) || !((v.split_mask >> b) & 1)) continue;
+            const double g = v.h1[b] * v.gscale[j][m];
+            if ((double)(float)g != g) return kNoExp;
+            if (g != 0.0) e = std::min(e, lowbit_exp(g));
+        }
+    return e;
+}
+static int linear_exp(const Problem &P, const Level &v) {
+    switch (P.fam) {
+    case VOTE_LINE2D: return linear_exp_fam<FAM_LINE2D>(P, v);
+    case VOTE_RAYS3D: return linear_exp_fam<FAM_RAYS3D>(P, v);
+    case VOTE_POINTSET2D: return linear_exp_fam<FAM_POINTSET2D>(P, v);
+    case VOTE_AFFINE4D: return linear_exp_fam<FAM_AFFINE4D>(P, v);
+    default: return kNoExp;
+    }
 }
 
 static vote_status problem_init(vote_ctx *c, int fam, int d, int k, const double *eps, const double *bounds) {
@@ -287,7 +316,10 @@ static vote_status problem_init(vote_ctx *c, int fam, int d, int k, const double
             v.A1[j] = A[l + 1][j];
             v.rlb[j] = P.eps[k + j] - A[l + 1][j];
             // FP32 screen constants in steps of s_f,j (rounding is covered by its band)
-            for (int m = 0; m < le; ++m) v.gscale[j][m] = s_t[l][m] / P.s_f[j];
+            for (int m = 0; m < le; ++m) {
+                v.gscale[j][m] = s_t[l][m] / P.s_f[j];
+                v.gs[j][m] = (float)v.gscale[j][m];
+            }
             v.Hs[j] = (float)(h[l + 1][k + j] / P.s_f[j]);
             v.Hs_lo[j] = (float)(h[l + 1][k + j] / P.s_f[j] - (double)v.Hs[j]);
             if (l < P.Lj[k + j]) {              // the dependent coordinate splits: its shift enters
@@ -298,6 +330,11 @@ static vote_status problem_init(vote_ctx *c, int fam, int d, int k, const double
             v.rc0[j] = (float)((v.Rbase[j] + v.A1[j]) / P.s_f[j]);
             v.Lc[j] = (float)(v.rlb[j] / P.s_f[j]);
         }
+        for (int j = 0; j < d; ++j) {
+            v.h1f[j] = (float)v.h1[j];
+            v.h1f_lo[j] = (float)(v.h1[j] - (double)v.h1f[j]);
+        }
+        v.g_exp = linear_exp(P, v);
         // Lipschitz term of the radius from the essential parameters in steps
         switch (fam) {
         case VOTE_LINE2D:        // |t| h1_m
@@ -500,6 +537,17 @@ static int family_nb(int fam) {
     default: return Fam<FAM_POSE6DOF>::NB;
     }
 }
+// basis values whose changes depend on the cell
+static int family_nbg(int fam) {
+    switch (fam) {
+    case VOTE_PLANE3D_SPH: return Fam<FAM_PLANE3D_SPH>::NBG;
+    case VOTE_POSE3DOF: return Fam<FAM_POSE3DOF>::NBG;
+    case VOTE_POSE6DOF: return Fam<FAM_POSE6DOF>::NBG;
+    case VOTE_RADIAL5DOF: return Fam<FAM_RADIAL5DOF>::NBG;
+    default: return 0;
+    }
+}
+static bool family_rotation(int fam) { return fam == VOTE_POSE6DOF || fam == VOTE_RADIAL5DOF; }
 static_assert((int)VOTE_LINE2D == FAM_LINE2D && (int)VOTE_PLANE3D_SPH == FAM_PLANE3D_SPH &&
                   (int)VOTE_POSE3DOF == FAM_POSE3DOF && (int)VOTE_POSE6DOF == FAM_POSE6DOF &&
                   (int)VOTE_RAYS3D == FAM_RAYS3D && (int)VOTE_POINTSET2D == FAM_POINTSET2D &&
@@ -590,6 +638,12 @@ static void ev_collect(vote_ctx *c) {
 // search
 // ---------------------------------------------------------------------------
 
+// rotation tables hold at most 2^kRotBits cells of the rotation coordinates per level
+// (151 MB: seven levels of the 6DoF workload); deeper levels evaluate rotations directly
+static const int kRotBits = 21;
+// angular coordinates of at most this many splits have a (sin, cos) table (2 MB)
+static const int kSincosBits = 16;
+
 // records expanded with lower bounds outside dives
 static int64_t lb_records(int d) { return d <= 3 ? (int64_t)1 << 28 : (int64_t)1 << 22; }
 
@@ -629,14 +683,33 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     }
     nvtxRangePushA("expand_chunk");
     const int nc = (int)(c1 - c0);
-    const int NB = family_nb(P.fam);
-    const int gf = geo32_floats(nfs, P.nd, P.le);
+    const int NB = family_nb(P.fam), NBG = family_nbg(P.fam);
+    const bool rotation = family_rotation(P.fam);
+    // geometry slots: the free slots, without the linear tail coordinate's bit
+    const int kg = rotation ? kf - ((lev.split_mask >> (P.k - 1)) & 1) : kf, ng = 1 << kg;
+    const int gf = NBG * ng + NBG;
     const size_t nch = (size_t)nc * ns;
     const size_t cnt_arrays = c->group ? 3 : 2;
     TRY(ensure(c, c->alive, nc));
-    TRY(ensure(c, c->geo64, (size_t)nc * nfs * NB * 8));
-    TRY(ensure(c, c->geo32, (size_t)nc * gf * 4));
-    TRY(ensure(c, c->geo32lo, (size_t)nc * nfs * P.nd * P.le * 4));
+    bool need64 = c->precision == 0;
+    if (NBG) {
+        TRY(ensure(c, c->geo32, (size_t)nc * gf * 4));
+        TRY(ensure(c, c->geo32lo, (size_t)nc * NBG * ng * 4));
+    }
+    if (rotation) {
+        for (int x = l; x <= l + 1; ++x) {       // tables of this level's and the next level's rotations
+            int bits = 0;
+            for (int j = 0; j < 3; ++j) bits += std::min(x, P.Lj[j]);
+            if (bits > kRotBits || c->rot[x].p) continue;
+            TRY(ensure(c, c->rot[x], ((size_t)72 << bits)));
+            TRY(ensure(c, c->rotflag[x], (((size_t)1 << bits) / 32 + 1) * 4));
+            CK(cudaMemsetAsync(c->rotflag[x].p, 0, (((size_t)1 << bits) / 32 + 1) * 4, c->stream));
+        }
+        need64 |= !c->rot[l].p || !c->rot[l + 1].p;
+    } else if (NBG) {
+        for (int j = 0; j < P.k; ++j) need64 |= !c->sctab[j].p;
+    }
+    if (need64) TRY(ensure(c, c->geo64, (size_t)nc * nfs * NB * 8));
     TRY(ensure(c, c->cnt, nch * 4 * cnt_arrays));
     TRY(ensure(c, c->child_idx, nch * 4));
     TRY(ensure(c, c->cbase, nch * 8));
@@ -666,7 +739,15 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     ch.t0 = r0 / 32;
     ch.t1 = r1 / 32;
     ch.alive = (uint8_t *)c->alive.p;
-    ch.geo64 = (double *)c->geo64.p;
+    ch.ng = ng;
+    ch.kg = kg;
+    ch.geo64 = need64 ? (double *)c->geo64.p : nullptr;
+    for (int j = 0; j < 2; ++j) ch.sincos[j] = (const double2 *)c->sctab[j].p;
+    if (rotation) {
+        ch.rot_par = (double *)c->rot[l].p;
+        ch.rot_ch = (double *)c->rot[l + 1].p;
+        ch.rot_flag = (unsigned *)c->rotflag[l + 1].p;
+    }
     ch.geo32 = (float *)c->geo32.p;
     ch.geo32lo = (float *)c->geo32lo.p;
     ch.crec = (uint32_t *)c->cnt.p;
@@ -756,8 +837,7 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
         ch.out = rec_view(c, c->ls[l + 1]);
     }
     ev_mark(c, -1);
-    launch_cell_geo(ch, c->stream);
-    launch_tile_info(ch, c->stream);
+    const int nprep = launch_prep(ch, c->stream);
     ev_mark(c, VOTE_K_CELL_GEO);
     launch_count(ch, c->stream);
     ev_mark(c, VOTE_K_TEST_COUNT);
@@ -770,7 +850,7 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     c->kbytes[VOTE_K_CELL_GEO] += (double)nc * (8 + 4);
     CK(cudaGetLastError());
     c->stats.chunks++;
-    c->stats.launches += (lev.leaf_children ? 5 : 7) + (c->precision == 1);
+    c->stats.launches += (lev.leaf_children ? 3 : 5) + nprep + (c->precision == 1);
     c->stats.cells += nc;
     c->lv_cells[l] += nc;
     c->lv_recs[l] += nt * 32;
@@ -1112,6 +1192,12 @@ vote_status vote_create(int family, int d, int k, const double *eps, const doubl
     if (s == VOTE_OK) s = ensure(c, c->levs_dev, sizeof(Level) * (c->P.L > 0 ? c->P.L : 1));
     if (s == VOTE_OK) s = ensure(c, c->path, sizeof(PathStep) * (c->P.L > 0 ? c->P.L : 1));
     if (s == VOTE_OK && c->P.L > 0) {
+        const int nang = family == VOTE_PLANE3D_SPH ? 2 : (family == VOTE_POSE3DOF ? 1 : 0);
+        for (int j = 0; j < nang && s == VOTE_OK; ++j)
+            if (c->P.Lj[j] <= kSincosBits) {
+                s = ensure(c, c->sctab[j], sizeof(double2) * (((size_t)2 << c->P.Lj[j]) - 1));
+                if (s == VOTE_OK) launch_sincos_table(c->P, j, (double2 *)c->sctab[j].p, c->stream);
+            }
         e = cudaMemcpyAsync(c->levs_dev.p, c->lev, sizeof(Level) * c->P.L, cudaMemcpyHostToDevice, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) {
@@ -1554,6 +1640,8 @@ void vote_destroy(vote_ctx *c) {
                       &c->ss_io, &c->g_table, &c->g_owner, &c->g_newpos, &c->g_ccount, &c->g_ccur,
                       &c->g_rbeg, &c->g_rec, &c->g_mult, &c->g_tile, &c->beam_sel, &c->beam_src};
     for (DevBuf *b : bufs) release(c, *b);
+    for (DevBuf &b : c->sctab) release(c, b);
+    for (int l = 0; l <= GV_MAXL; ++l) release(c, c->rot[l]), release(c, c->rotflag[l]);
     cudaStreamSynchronize(c->stream);
     for (int i = 0; i < vote_ctx::kEv; ++i)
         if (c->ev[i]) cudaEventDestroy(c->ev[i]);

@@ -21,7 +21,7 @@ __device__ __forceinline__ void eval_record(const Chunk &c, int64_t r, int cell,
     for (int j = 0; j < F::ND; ++j) qf[j] = field_i<Q16>(w, j);
 #pragma unroll
     for (int m = 0; m < F::LE; ++m) qt[m] = field_i<Q16>(w, F::ND + m);
-    eval64<FAM>(c.P, c.lev, qf, qt, c.geo64 + (size_t)cell * c.nfs * F::NB, c.kf, c.dm, ubm, lbm);
+    eval64<FAM>(c, cell, qf, qt, ubm, lbm);
 }
 
 // One queue entry (a tile and its undecided lanes, almost always one) per thread; the

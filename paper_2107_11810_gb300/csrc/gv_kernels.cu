@@ -3,9 +3,9 @@
 //
 //   k_lift        root records of the original surfaces (Eq. 1 in the frame of the
 //                 domain centre), snapped for level 0
-//   k_cell_geo    per cell of a chunk: pruning re-check and the change of the
+//   k_prep        per cell of a chunk: pruning re-check and the change of the
 //                 family's basis functions from the cell centre to each child
-//                 centre (own sin/cos, FP64)
+//                 centre (own sin/cos, FP64, from tables); per tile its cell
 //   (k_count, k_emit: the proximity test itself, in gv_count.cu and gv_emit.cu)
 //   k_tile_scan   per child its counts, per tile and child its records' place, best
 //                 lower bound, all from the count pass's ballots
@@ -23,8 +23,9 @@ namespace gv {
 
 __device__ __forceinline__ unsigned prune_threshold(const Problem &P, const Scalars *sc, int prune) {
     if (!prune) return 1u;
-    unsigned lb = *(volatile const unsigned *)&sc->best_lb;
-    unsigned long long bk = *(volatile const unsigned long long *)&sc->best_key;
+    // plain (cached) loads: every thread of a kernel reads them, and an older value is valid
+    unsigned lb = sc->best_lb;
+    unsigned long long bk = sc->best_key;
     unsigned leaf = (unsigned)(bk >> P.coord_bits);
     unsigned t = lb > leaf ? lb : leaf;
     return t > 1u ? t : 1u;
@@ -128,65 +129,115 @@ __device__ __forceinline__ void parent_psi(const Problem &P, const Level &lev, u
     if (!F::LINEAR_BASIS) F::basis(P, cpar, psi);
 }
 
-// One thread per (cell, free slot fs); the nfs threads of a cell are consecutive lanes.  Writes the FP64 basis changes (for the exact recheck) and
-// the screen's coefficients G[fs][j][m] = coef_jm(dpsi) * s_t,m / s_f,j rounded to
-// FP32, their remainders (G64 - G, rounded to FP32: the double-float tier's low
-// parts; G64 is exact, coef only copies or negates and s_t / s_f is a power of two),
-// per (j, m) the largest |G| over the child slots (rounded up), which bounds the
-// magnitudes the screen's band scales with, and the cell's exactness exponent: the
-// least e with every G a multiple of 2^e (at most 0), or kNoExp when some G is not
-// exactly an FP32 value.
+// (sin, cos) of every cell centre of an angular coordinate, by the same operations as
+// Fam::basis: a cell's geometry then takes table reads and a few FP64 operations instead
+// of two evaluations per child slot (the FP64 pipe issues one lane per clock and SM and
+// bounded this pass: 84 % busy).
+__global__ void k_sincos_table(Problem P, int j, double2 *tab, int64_t n) {
+    const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (x >= n) return;
+    const int e = 63 - __clzll(x + 1);
+    const int64_t i = x + 1 - (1ll << e);
+    double h[GV_MAXD], sn, cs;
+    h[j] = ldexp(P.W[j], -(e + 1));                  // the half-width after e splits
+    vsincos(cell_center(P, h, j, i), &sn, &cs);
+    tab[x] = make_double2(sn, cs);
+}
+
+// Rotation families: the rotations of the child centres that no earlier step has filled
+// in.  A thread per (cell, geometry slot) claims its entry; claimed entries are complete
+// at the end of the kernel.  Cells that share their rotation coordinates share them.
 template <int FAM>
-__global__ void k_cell_geo(Chunk c) {
-    using F = Fam<FAM>;
-    static_assert(32 % (1 << F::K) == 0, "a cell's threads must lie in one warp");
-    const int NF = c.nfs, GF = c.gf;
-    const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int cell = gid >> c.kf, fs = gid & (NF - 1);
-    const bool in = cell < c.nc;
-    if (gid == 0) c.sc->n_uns = 0u;                  // this step's recheck queue
+__global__ void __launch_bounds__(256) k_rot_fill(const __grid_constant__ Chunk c) {
+    const int64_t gid = blockIdx.x * 256ll + threadIdx.x;
     const Problem &P = c.P;
     const Level &lev = c.lev;
-    float ga[F::ND * F::LE];
+    if (gid == 0 && lev.l == 0) {                    // the root's own
+        double ph[3];
+        for (int j = 0; j < 3; ++j) ph[j] = cell_center(P, lev.h, j, 0);
+        Fam<FAM_POSE6DOF>::rotation(P, ph, c.rot_par);
+    }
+    const int64_t cell = gid >> c.kg;
+    if (cell >= c.nc || c.cells.ub[c.c0 + cell] < prune_threshold(P, c.sc, c.prune)) return;
+    int64_t ix[3];
+    geo_coords<FAM>(c, c.cells.key[c.c0 + cell], (int)(gid & (c.ng - 1)), true, ix);
+    const int64_t e = rot_entry(P, lev.l + 1, ix);
+    const unsigned bit = 1u << (e & 31);
+    if (c.rot_flag[e >> 5] & bit) return;
+    if (atomicOr(c.rot_flag + (e >> 5), bit) & bit) return;
+    double ph[3];
+    for (int j = 0; j < 3; ++j) ph[j] = cell_center(P, lev.h1, j, ix[j]);
+    Fam<FAM_POSE6DOF>::rotation(P, ph, c.rot_ch + 9 * e);
+}
+
+// Cells and tiles of a chunk.  Per cell whether it is still above the threshold; per
+// (cell, geometry slot) the FP32 basis changes and remainders (G64 = change times a power
+// of two; the screen's coefficient is the rounded change times that power), and per basis
+// value the largest magnitude (rounded up), which bounds the snap's band; in plain FP64
+// mode, and where there are no tables, the FP64 changes too.  Per tile its cell (-1: pruned), how many of its 32 lanes
+// hold records, and whether it is its cell's first or last tile.
+__device__ __forceinline__ void tile_info(const Chunk &c, int64_t i, unsigned thr) {
+    const int64_t nt = c.t1 - c.t0;
+    if (i >= nt + 2) return;
+    // two entries of padding: the count pass loads ahead; after an emit pass gave up its
+    // tiles name no cells
+    int2 ti = make_int2(-1, 0);
+    if (i < nt && !(c.sc->err & kErrTimeout)) {
+        const int64_t t = c.t0 + i, cell = (int64_t)c.in.tile_cell[t];
+        const int cl = (int)(cell - c.in_c0);
+        const int64_t r0 = (int64_t)c.in_rbeg[cell], left = r0 + (int64_t)c.in_rcnt[cell] - 32 * t;
+        ti = make_int2(c.cells.ub[c.c0 + cl] >= thr ? cl : -1, (left < 32 ? (int)left : 32) |
+                                                                   (32 * t == r0 ? kTileFirst : 0) |
+                                                                   (left <= 32 ? kTileLast : 0));
+    }
+    c.tinfo[i] = ti;
+}
+
+template <int FAM>
+__global__ void __launch_bounds__(256) k_prep(const __grid_constant__ Chunk c) {
+    using F = Fam<FAM>;
+    static_assert(32 % (1 << F::K) == 0, "a cell's threads must lie in one warp");
+    const int64_t gid = blockIdx.x * 256ll + threadIdx.x;
+    const unsigned thr = prune_threshold(c.P, c.sc, c.prune);
+    if (gid == 0) c.sc->n_uns = 0u;                  // this step's recheck queue
+    if (gid < c.nc) c.alive[gid] = c.cells.ub[c.c0 + gid] >= thr ? 1 : 0;
+    tile_info(c, gid, thr);
+    if (c.geo64) {
+        const int64_t cell = gid >> c.kf;
+        if (cell < c.nc) {
+            const int fs = (int)(gid & (c.nfs - 1));
+            double d[F::NB];
+            cell_change<FAM, false>(c, c.cells.key[c.c0 + cell], fs, d);
 #pragma unroll
-    for (int x = 0; x < F::ND * F::LE; ++x) ga[x] = 0.0f;
-    int ge = 0;                                      // exactness exponent (<= 0) of this thread's G
-    if (in) {
-        if (fs == 0) {
-            unsigned thr = prune_threshold(P, c.sc, c.prune);
-            c.alive[cell] = c.cells.ub[c.c0 + cell] >= thr ? 1 : 0;
-        }
-        double dpsi[F::NB];
-        {
-            uint64_t key = c.cells.key[c.c0 + cell];
-            double psi_par[F::NB];
-            parent_psi<FAM>(P, lev, key, psi_par);
-            child_dpsi<FAM>(P, lev, key, expand_bits(fs, lev.split_mask & ((1 << F::K) - 1)), psi_par, dpsi);
-        }
-#pragma unroll
-        for (int m = 0; m < F::NB; ++m) c.geo64[((size_t)cell * NF + fs) * F::NB + m] = dpsi[m];
-        double g[F::ND * F::LE];
-        F::coef(dpsi, g);
-#pragma unroll
-        for (int x = 0; x < F::ND * F::LE; ++x) {
-            const double gx = g[x] * lev.gscale[x / F::LE][x % F::LE];
-            const float gh = (float)gx;
-            c.geo32[(size_t)cell * GF + fs * F::ND * F::LE + x] = gh;
-            c.geo32lo[((size_t)cell * NF + fs) * F::ND * F::LE + x] = (float)(gx - (double)gh);
-            ga[x] = __double2float_ru(fabs(gx));
-            if ((double)gh != gx) ge = kNoExp;
-            else if (gx != 0.0 && ge > kNoExp) ge = min(ge, lowbit_exp(gx));
+            for (int m = 0; m < F::NB; ++m) c.geo64[((size_t)cell * c.nfs + fs) * F::NB + m] = d[m];
         }
     }
-    for (int o = 1; o < NF; o <<= 1) {
+    if constexpr (F::NBG > 0) {
+        const int64_t cell = gid >> c.kg;
+        const int r = (int)(gid & (c.ng - 1));
+        if ((gid & ~31ll) >> c.kg >= c.nc) return;   // uniform: this warp only has tiles
+        const bool in = cell < c.nc && c.cells.ub[c.c0 + cell] >= thr;
+        float ga[F::NBG];
 #pragma unroll
-        for (int x = 0; x < F::ND * F::LE; ++x) ga[x] = fmaxf(ga[x], __shfl_xor_sync(kFull, ga[x], o));
-        ge = min(ge, __shfl_xor_sync(kFull, ge, o));
-    }
-    if (in && fs == 0) {
+        for (int x = 0; x < F::NBG; ++x) ga[x] = 0.0f;
+        if (in) {
+            double d[F::NBG];
+            geo_change<FAM, false>(c, c.cells.key[c.c0 + cell], r, d);
+            float *gh = c.geo32 + (size_t)cell * c.gf + r, *gl = c.geo32lo + (size_t)cell * F::NBG * c.ng + r;
 #pragma unroll
-        for (int x = 0; x < F::ND * F::LE; ++x) c.geo32[(size_t)cell * GF + NF * F::ND * F::LE + x] = ga[x];
-        c.geo32[(size_t)cell * GF + GF - 1] = (float)ge;
+            for (int x = 0; x < F::NBG; ++x) {
+                const float h = (float)d[x];
+                gh[x * c.ng] = h;
+                gl[x * c.ng] = (float)dsub(d[x], (double)h);
+                ga[x] = __uint_as_float(__float_as_uint(fabsf(h)) + 1u);   // at least |d|
+            }
+        }
+        for (int o = 1; o < c.ng; o <<= 1)
+#pragma unroll
+            for (int x = 0; x < F::NBG; ++x) ga[x] = fmaxf(ga[x], __shfl_xor_sync(kFull, ga[x], o));
+        if (in && r == 0)
+#pragma unroll
+            for (int x = 0; x < F::NBG; ++x) c.geo32[(size_t)cell * c.gf + F::NBG * c.ng + x] = ga[x];
     }
 }
 
@@ -502,25 +553,6 @@ __global__ void __launch_bounds__(256) k_beam_gather(RecView in, RecView out, Ce
 // Per-tile bookkeeping of the proximity test, so that the count and emit passes
 // stream their inputs with bulk copies and never chase a pointer per tile.
 // ---------------------------------------------------------------------------
-
-// per tile: the chunk-local cell (-1 if it was pruned), how many of its 32 lanes hold
-// records, whether it is the cell's first or last tile
-__global__ void k_tile_info(Chunk c) {
-    const int64_t t = c.t0 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= c.t1) {                                 // two entries of padding: the count pass loads ahead
-        if (t < c.t1 + 2) c.tinfo[t - c.t0] = make_int2(-1, 0);
-        return;
-    }
-    if (c.sc->err & kErrTimeout) {                   // an emit pass gave up: its tiles name no cells
-        c.tinfo[t - c.t0] = make_int2(-1, 0);
-        return;
-    }
-    const int64_t cell = (int64_t)c.in.tile_cell[t];
-    const int cl = (int)(cell - c.in_c0);
-    const int64_t r0 = (int64_t)c.in_rbeg[cell], left = r0 + (int64_t)c.in_rcnt[cell] - 32 * t;
-    c.tinfo[t - c.t0] = make_int2(c.alive[cl] ? cl : -1, (left < 32 ? (int)left : 32) | (32 * t == r0 ? kTileFirst : 0) |
-                                                             (left <= 32 ? kTileLast : 0));
-}
 
 // Counts and output positions from the ballots.  A warp takes 32 consecutive tiles,
 // one per lane, and per child slot a segmented scan over them (segments = runs of one
@@ -845,9 +877,23 @@ void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t
     GV_DISPATCH(P.fam, (k_lift<FAMV><<<blocks_for(n, 256), 256, 0, st>>>(P, lev0, prm, n, out, sc)));
 }
 
-void launch_cell_geo(const Chunk &c, cudaStream_t st) {
-    if (c.nc <= 0) return;
-    GV_DISPATCH(c.P.fam, (k_cell_geo<FAMV><<<blocks_for((int64_t)c.nc << c.kf, 64), 64, 0, st>>>(c)));
+void launch_sincos_table(const Problem &P, int j, double2 *tab, cudaStream_t st) {
+    const int64_t n = ((int64_t)2 << P.Lj[j]) - 1;
+    k_sincos_table<<<blocks_for(n, 128), 128, 0, st>>>(P, j, tab, n);
+}
+
+int launch_prep(const Chunk &c, cudaStream_t st) {
+    int n = 1;
+    const int64_t geo = (int64_t)c.nc << (c.geo64 ? c.kf : c.kg);
+    if (c.rot_ch) {                                  // rotation families only
+        const unsigned g = blocks_for((int64_t)c.nc << c.kg, 256);
+        if (c.P.fam == FAM_POSE6DOF) k_rot_fill<FAM_POSE6DOF><<<g, 256, 0, st>>>(c);
+        else k_rot_fill<FAM_RADIAL5DOF><<<g, 256, 0, st>>>(c);
+        n = 2;
+    }
+    const int64_t nt = c.t1 - c.t0 + 2, g = nt > geo ? nt : geo;
+    GV_DISPATCH(c.P.fam, (k_prep<FAMV><<<blocks_for(g, 256), 256, 0, st>>>(c)));
+    return n;
 }
 
 int sm_count() {
@@ -883,11 +929,6 @@ void launch_persistent(const void *kern, size_t smem, int64_t groups, const Chun
     if (g > groups) g = groups;
     void *args[] = {(void *)&c};
     cudaLaunchKernel(kern, dim3((unsigned)g), dim3(256), args, smem, st);
-}
-
-void launch_tile_info(const Chunk &c, cudaStream_t st) {
-    const int64_t nt = c.t1 - c.t0;
-    if (nt > 0) k_tile_info<<<blocks_for(nt + 2, 256), 256, 0, st>>>(c);
 }
 
 void launch_tile_scan(const Chunk &c, cudaStream_t st) {

@@ -78,9 +78,18 @@ struct Chunk {
     int64_t t0, t1;          // tile range of the chunk
     uint8_t *alive;          // [nc]   bit 0: cell still above the pruning threshold; bit 1: it has a
                              //        surviving child
-    double *geo64;           // [nc][nfs][NB]          basis change per free slot
-    float *geo32;            // [nc][gf] screen coefficients G, max |G|, exponent
-    float *geo32lo;          // [nc][nfs * ND * LE]    G64 - G rounded to FP32 (double-float tier)
+    // cell geometry: the changes of the cell-dependent basis values (Fam::NBG) from the
+    // cell centre to the child centres, one per geometry slot (the free slots without a
+    // linear tail coordinate's bit)
+    int ng, kg;              // geometry slots, log2
+    float *geo32;            // [nc][gf]: [NBG][ng] rounded to FP32, then [NBG] the largest magnitudes
+    float *geo32lo;          // [nc][NBG][ng] what that rounding leaves, rounded to FP32
+    double *geo64;           // [nc][nfs][NB] in plain FP64 mode and where a table is missing, else NULL
+    const double2 *sincos[2];// (sin, cos) of every centre of angular coordinate 0, 1 (entry 2^e - 1 + i for
+                             // cell i after e splits), or NULL
+    double *rot_par, *rot_ch;// rotations (9 values) of every cell of the rotation coordinates at this level and
+                             // the next, filled on demand, or NULL
+    unsigned *rot_flag;      // bit per entry of rot_ch: filled
     uint32_t *crec, *clb;    // [nc][ns]  records (UB-passing) and LB sum per child
     uint32_t *cub;           // [nc][ns]  UB sum per child (= crec without multiplicities)
     int2 *tinfo;             // [t1 - t0 + 2] per tile: chunk-local cell (-1: pruned), valid lanes | kTileFirst |
@@ -103,10 +112,6 @@ struct Chunk {
 };
 constexpr int kTileFirst = 64, kTileLast = 128;   // flags in tinfo.y: first / last tile of its cell
 
-// Size in floats of one cell's screen geometry: G[nfs][ND][LE], per (j, m) the
-// largest |G| over the free slots (rounded up), and the cell's exactness exponent e
-// (every G is FP32-exact and a multiple of 2^e; kNoExp when not).
-__host__ __device__ constexpr int geo32_floats(int nfs, int nd, int le) { return nfs * nd * le + nd * le + 1; }
 constexpr int kNoExp = -1000;
 
 // Selection of a level's cells with the largest UBs (index 0) and LBs (index 1)
@@ -127,14 +132,15 @@ struct PathStep {
 
 void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t n, RecView out, Scalars *sc,
                  cudaStream_t st);
-void launch_cell_geo(const Chunk &c, cudaStream_t st);
+// the (sin, cos) table of an angular coordinate (2^(splits + 1) - 1 entries)
+void launch_sincos_table(const Problem &P, int j, double2 *tab, cudaStream_t st);
+// cells (alive, geometry) and tiles (tinfo) of the chunk; returns the kernels launched
+int launch_prep(const Chunk &c, cudaStream_t st);
 // launch a persistent kernel taking one Chunk: one block per resident slot on the
 // device, at most `groups` blocks, 256 threads, smem bytes of dynamic shared memory
 // SMs of the device (read once)
 int sm_count();
 void launch_persistent(const void *kern, size_t smem, int64_t groups, const Chunk &c, cudaStream_t st);
-// per tile of the chunk: tinfo (after k_cell_geo has set alive)
-void launch_tile_info(const Chunk &c, cudaStream_t st);
 // the ballots of every tile and child, by the FP32 screen (undecided records queued)
 // or, in plain FP64 mode, by the definition
 void launch_count(const Chunk &c, cudaStream_t st);

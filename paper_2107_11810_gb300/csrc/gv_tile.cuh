@@ -212,6 +212,147 @@ __device__ __forceinline__ int32_t resnap_half(int32_t q) {
 }
 
 // ---------------------------------------------------------------------------
+// Cell geometry: the changes of the basis values from a cell's centre to its children's.
+// ---------------------------------------------------------------------------
+
+// entry of a rotation table: the packed coordinates of a cell of the rotation
+// coordinates 0..2 at level l
+__device__ __forceinline__ int64_t rot_entry(const Problem &P, int l, const int64_t *ix) {
+    return (((ix[0] << splits_at(P, l, 1)) | ix[1]) << splits_at(P, l, 2)) | ix[2];
+}
+
+// coordinates (of those the stored basis values depend on) of the cell itself or of the
+// child of geometry slot r
+template <int FAM>
+__device__ __forceinline__ void geo_coords(const Chunk &c, uint64_t key, int r, bool child, int64_t *ix) {
+    using F = Fam<FAM>;
+    constexpr int NC = F::LINEAR_TAIL ? F::K - 1 : F::K;
+    int bits = r;
+#pragma unroll
+    for (int j = 0; j < NC; ++j) {
+        ix[j] = cell_coord(c.P, key, c.lev.l, j);
+        if (child && ((c.lev.split_mask >> j) & 1)) {
+            ix[j] = 2 * ix[j] + (bits & 1);
+            bits >>= 1;
+        }
+    }
+}
+
+// the stored basis values at a cell (level l: half-widths h) of these coordinates.  TAB: the
+// tables hold them (else they are evaluated where there is no table).
+template <int FAM, bool TAB>
+__device__ __forceinline__ void geo_basis(const Chunk &c, int l, const double *h, const double *rot, const int64_t *ix,
+                                          double *psi) {
+    using F = Fam<FAM>;
+    if constexpr (F::LINEAR_TAIL) {
+        double R[9];
+        if (TAB || rot) {
+            const double *p = rot + 9 * rot_entry(c.P, l, ix);
+#pragma unroll
+            for (int m = 0; m < F::NBG; ++m) psi[m] = p[m];
+            return;
+        }
+        double ph[3];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) ph[j] = cell_center(c.P, h, j, ix[j]);
+        Fam<FAM_POSE6DOF>::rotation(c.P, ph, R);
+#pragma unroll
+        for (int m = 0; m < F::NBG; ++m) psi[m] = R[m];
+    } else {
+        constexpr int NC = F::K;
+        double sn[2], cs[2];
+        static_assert(FAM == FAM_PLANE3D_SPH || FAM == FAM_POSE3DOF, "angular coordinates");
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            if (TAB || c.sincos[j]) {
+                const double2 v = c.sincos[j][(1ll << splits_at(c.P, l, j)) - 1 + ix[j]];
+                sn[j] = v.x;
+                cs[j] = v.y;
+            } else {
+                vsincos(cell_center(c.P, h, j, ix[j]), &sn[j], &cs[j]);
+            }
+        }
+        if constexpr (FAM == FAM_PLANE3D_SPH) {     // as Fam::basis
+            psi[0] = dmul(sn[0], cs[1]);
+            psi[1] = dmul(sn[0], sn[1]);
+            psi[2] = cs[0];
+        } else {
+            psi[0] = cs[0];
+            psi[1] = sn[0];
+        }
+    }
+}
+
+// changes of the stored basis values for geometry slot r
+template <int FAM, bool TAB>
+__device__ __forceinline__ void geo_change(const Chunk &c, uint64_t key, int r, double *d) {
+    using F = Fam<FAM>;
+    int64_t ix[3];
+    double par[F::NBG], ch[F::NBG];
+    geo_coords<FAM>(c, key, r, false, ix);
+    geo_basis<FAM, TAB>(c, c.lev.l, c.lev.h, c.rot_par, ix, par);
+    geo_coords<FAM>(c, key, r, true, ix);
+    geo_basis<FAM, TAB>(c, c.lev.l + 1, c.lev.h1, c.rot_ch, ix, ch);
+#pragma unroll
+    for (int m = 0; m < F::NBG; ++m) d[m] = dsub(ch[m], par[m]);
+}
+
+// changes of all basis values for free slot fs (the definition's)
+template <int FAM, bool TAB>
+__device__ __forceinline__ void cell_change(const Chunk &c, uint64_t key, int fs, double *d) {
+    using F = Fam<FAM>;
+    if constexpr (F::LINEAR_BASIS) {
+        // psi is the free coordinates themselves: their changes are the exact child shifts
+        int bits = fs;
+#pragma unroll
+        for (int m = 0; m < F::NB; ++m) {
+            const bool split = (c.lev.split_mask >> m) & 1;
+            d[m] = split ? ((bits & 1) ? c.lev.h1[m] : -c.lev.h1[m]) : 0.0;
+            if (split) bits >>= 1;
+        }
+    } else {
+        geo_change<FAM, TAB>(c, key, fs & (c.ng - 1), d);
+        if constexpr (F::LINEAR_TAIL) {
+            // the last basis value is the last free coordinate: its change is the exact shift
+            constexpr int j = F::K - 1;
+#pragma unroll
+            for (int m = F::NBG; m < F::NB - 1; ++m) d[m] = 0.0;    // not used by the family
+            d[F::NB - 1] = ((c.lev.split_mask >> j) & 1) ? ((fs >> c.kg) ? c.lev.h1[j] : -c.lev.h1[j]) : 0.0;
+        }
+    }
+}
+
+// the same of a chunk's cell, from its FP64 geometry where that is kept (plain FP64 mode,
+// and where there are no tables: so the rare paths hold no evaluation)
+template <int FAM>
+__device__ __forceinline__ void chunk_change(const Chunk &c, int cell, int fs, double *d) {
+    using F = Fam<FAM>;
+    if (c.geo64) {
+#pragma unroll
+        for (int m = 0; m < F::NB; ++m) d[m] = c.geo64[((size_t)cell * c.nfs + fs) * F::NB + m];
+    } else {
+        cell_change<FAM, true>(c, c.cells.key[c.c0 + cell], fs, d);
+    }
+}
+
+// FP32 change of basis value b for free slot f where it does not depend on the cell (a
+// linear basis or tail coordinate), and what the rounding leaves
+template <int FAM>
+__device__ __forceinline__ float lin_change(const Chunk &c, int b, int f, bool low) {
+    using F = Fam<FAM>;
+    const int j = F::LINEAR_TAIL ? F::K - 1 : b;
+    if (!((c.lev.split_mask >> j) & 1)) return 0.0f;
+    const float h = low ? c.lev.h1f_lo[j] : c.lev.h1f[j];
+    return (f >> __popc(c.lev.split_mask & ((1 << j) - 1))) & 1 ? h : -h;
+}
+
+// the screen's coefficient of t_m in residual j from the change of its basis value
+template <int FAM>
+__device__ __forceinline__ float coef32(const Level &lev, int j, int m, float d) {
+    return (Fam<FAM>::cneg(j, m) ? -d : d) * lev.gs[j][m];
+}
+
+// ---------------------------------------------------------------------------
 // Exact FP64 definition (the recheck of the screen, and the plain FP64 mode).
 // ---------------------------------------------------------------------------
 
@@ -275,11 +416,14 @@ template <int FAM>
 using SlotMask = typename std::conditional<((1 << Fam<FAM>::D) > 32), unsigned long long, unsigned>::type;
 
 // UB/LB pass masks of one record (integer fields) against every child slot, exactly
-// as the definition evaluates them.  g64: the cell's basis changes [nfs][NB].
+// as the definition evaluates them.
 template <int FAM>
-__device__ __forceinline__ void eval64(const Problem &P, const Level &lev, const int *qf, const int *qt,
-                                       const double *g64, int kf, int dm, SlotMask<FAM> &ubm, SlotMask<FAM> &lbm) {
+__device__ __forceinline__ void eval64(const Chunk &c, int cell, const int *qf, const int *qt, SlotMask<FAM> &ubm,
+                                       SlotMask<FAM> &lbm) {
     using F = Fam<FAM>;
+    const Problem &P = c.P;
+    const Level &lev = c.lev;
+    const int kf = c.kf, dm = c.dm;
     using Mask = SlotMask<FAM>;
     static_assert(F::ND <= 2, "two dependent coordinates at most");
     double f[F::ND], t[F::LE], R[F::ND];
@@ -292,8 +436,9 @@ __device__ __forceinline__ void eval64(const Problem &P, const Level &lev, const
     lbm = 0;
 #pragma unroll 1
     for (int fs = 0; fs < (1 << kf); ++fs) {
-        double pr[F::ND];
-        F::partial64(f, t, g64 + fs * F::NB, pr);
+        double pr[F::ND], d[F::NB];
+        chunk_change<FAM>(c, cell, fs, d);
+        F::partial64(f, t, d, pr);
 #pragma unroll
         for (int ds = 0; ds < (1 << F::ND); ++ds) {
             if (ds & ~dm) continue;
@@ -313,29 +458,32 @@ __device__ __forceinline__ void eval64(const Problem &P, const Level &lev, const
 
 // Record words passed by value to the out-of-line FP64 helpers below (so that the
 // caller's arrays stay in registers).
+template <int NW>
 struct RecWords {
-    uint32_t w[16];
+    uint32_t w[NW];
 };
 
 template <int NW>
-__device__ __forceinline__ RecWords rec_words_of(const uint32_t *w) {
-    static_assert(NW <= 16, "record words");
-    RecWords r;
+__device__ __forceinline__ RecWords<NW> rec_words_of(const uint32_t *w) {
+    RecWords<NW> r;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) r.w[i] = i < NW ? w[i] : 0u;
+    for (int i = 0; i < NW; ++i) r.w[i] = w[i];
     return r;
 }
 
-// Exact FP64 snap of one record's free parameters at a child centre (g64: the basis
-// change of its free slot, ds: its dependent bits), out of line (the FP32 path needs
-// it rarely): the snapped values (x, y: dependent coordinates 0 and 1) and z != 0 if
-// a value leaves the representable range.
+// Exact FP64 snap of one record's free parameters at a child centre (free slot fs,
+// dependent bits ds), out of line (the FP32 path needs it rarely): the snapped values
+// (x, y: dependent coordinates 0 and 1) and z != 0 if a value leaves the representable
+// range.
 template <int FAM, bool Q16>
-__device__ __noinline__ int3 snap64_words(const Problem *P, const Level *lev, RecWords rw, const double *g64, int ds,
-                                          int dm) {
+__device__ __noinline__ int3 snap64_words(const Chunk *c, RecWords<rec_words(Fam<FAM>::NFP, Q16)> rw, int cell, int fs, int ds) {
     using F = Fam<FAM>;
     static_assert(F::ND <= 2, "two dependent coordinates at most");
-    double f[F::ND], t[F::LE], pr[F::ND];
+    const Problem *P = &c->P;
+    const Level *lev = &c->lev;
+    const int dm = c->dm;
+    double f[F::ND], t[F::LE], pr[F::ND], g64[F::NB];
+    chunk_change<FAM>(*c, cell, fs, g64);
 #pragma unroll
     for (int j = 0; j < F::ND; ++j) f[j] = dmul((double)field_i<Q16>(rw.w, j), P->s_f[j]);
 #pragma unroll
@@ -367,17 +515,19 @@ __device__ __forceinline__ float two_sum(float a, float b, float &err) {
     return s;
 }
 
-// The snap of one record's dependent coordinates at a child centre (dependent bits
-// ds), from the residual q_f,j + sum_m q_t,m G64[j][m] -+ h1_j / s_f,j evaluated as a
-// double-float (G64 = Gh + Gl, the free slot's coefficients and their remainders):
+// The snap of one record's dependent coordinates at a child centre (free slot fs,
+// dependent bits ds), from the residual q_f,j + sum_m q_t,m G64[j][m] -+ h1_j / s_f,j
+// evaluated as a double-float (G64 = Gh + Gl, the slot's coefficients and their remainders):
 // (x, y) the snapped values, z = 1 when both are decided (the value is more than
 // bd_j away from a rounding tie and below lim in magnitude), else 0 (the FP64
 // definition decides).  Out of line: the FP32 screen needs it rarely.
 template <int FAM, bool Q16>
-__device__ __noinline__ int3 snap_df_words(const Level *lev, RecWords rw, const float *Gh, const float *Gl, int ds,
-                                           float bd0, float bd1, float lim) {
+__device__ __noinline__ int3 snap_df_words(const Chunk *c, RecWords<rec_words(Fam<FAM>::NFP, Q16)> rw, int cell,
+                                           int fs, int ds, float bd0, float bd1, float lim) {
     using F = Fam<FAM>;
     static_assert(F::ND <= 2, "two dependent coordinates at most");
+    const Level *lev = &c->lev;
+    const int r = fs & (c->ng - 1);
     int qn[2] = {0, 0}, ok = 1;
 #pragma unroll
     for (int j = 0; j < F::ND; ++j) {
@@ -388,8 +538,16 @@ __device__ __noinline__ int3 snap_df_words(const Level *lev, RecWords rw, const 
             if (!F::uses(j, m)) continue;
             float th, tl;
             split_int(field_i<Q16>(rw.w, F::ND + m), th, tl);
-            const int x = j * F::LE + m;
-            const float gh = __ldg(Gh + x), gl = __ldg(Gl + x);
+            const int b = F::cb(j, m);
+            float dh, dl;
+            if (b < F::NBG) {
+                dh = __ldg(c->geo32 + (size_t)cell * c->gf + b * c->ng + r);
+                dl = __ldg(c->geo32lo + ((size_t)cell * F::NBG + b) * c->ng + r);
+            } else {
+                dh = lin_change<FAM>(*c, b, fs, false);
+                dl = lin_change<FAM>(*c, b, fs, true);
+            }
+            const float gh = coef32<FAM>(*lev, j, m, dh), gl = coef32<FAM>(*lev, j, m, dl);
             const float p = __fmul_rn(th, gh);
             const float e = __fmaf_rn(th, gh, -p);                  // th gh = p + e exactly
             float err;
@@ -415,23 +573,10 @@ __device__ __noinline__ int3 snap_df_words(const Level *lev, RecWords rw, const 
 }
 
 // ---------------------------------------------------------------------------
-// FP32 screen (in steps of s_f): residual before the dependent shift for free
-// slot fs, from the record's fields and the cell's coefficients G[fs][j][m].
+// FP32 screen (in steps of s_f).
 // ---------------------------------------------------------------------------
-template <int FAM>
-__device__ __forceinline__ void partial32(const float *qf, const float *qt, const float *G, int fs, float *u) {
-    using F = Fam<FAM>;
-#pragma unroll
-    for (int j = 0; j < F::ND; ++j) {
-        float v = qf[j];
-#pragma unroll
-        for (int m = 0; m < F::LE; ++m)
-            if (F::uses(j, m)) v = __fmaf_rn(qt[m], G[(fs * F::ND + j) * F::LE + m], v);
-        u[j] = v;
-    }
-}
 
-// The magnitudes the screen's band scales with (steps): M_j = |q_f,j| + |H_j| +
+// The magnitudes the snap's band scales with (steps): M_j = |q_f,j| + |H_j| +
 // sum_m |q_t,m| Gmax_jm, Gmax = the cell's largest |G| per (j, m).
 template <int FAM>
 __device__ __forceinline__ void magnitudes(const float *qf, const float *qt, const float *Gmax, const float *hs,

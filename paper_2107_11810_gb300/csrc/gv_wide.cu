@@ -14,6 +14,28 @@
 
 namespace gv {
 
+// The screen's coefficients of a cell, transposed: sg[(j * LE + m) * nfs + f], by all lanes
+// of a warp; per (j, m) the largest magnitude at sg[ND * LE * nfs + j * LE + m].
+template <int FAM, bool MAX>
+__device__ __forceinline__ void stage_coefs(const Chunk &c, int cell, float *sg, int lane) {
+    using F = Fam<FAM>;
+    const float *geo = c.geo32 + (size_t)cell * c.gf;
+    const int f = lane & (c.nfs - 1);
+#pragma unroll
+    for (int j = 0; j < F::ND; ++j)
+#pragma unroll
+        for (int m = 0; m < F::LE; ++m) {
+            if (!F::uses(j, m)) continue;
+            const int b = F::cb(j, m), x = j * F::LE + m;
+            const float d = b < F::NBG ? __ldg(geo + b * c.ng + (f & (c.ng - 1))) : lin_change<FAM>(c, b, f, false);
+            if (lane < c.nfs) sg[x * c.nfs + f] = coef32<FAM>(c.lev, j, m, d);
+            if constexpr (MAX) {
+                const float g = b < F::NBG ? __ldg(geo + F::NBG * c.ng + b) : fabsf(d);
+                if (lane == 0) sg[F::ND * F::LE * c.nfs + x] = g * c.lev.gs[j][m];
+            }
+        }
+}
+
 // FG: free slots per group (4, or all of them when fewer split)
 template <int FAM, bool Q16, int FG, int DM, bool LB>
 __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chunk c) {
@@ -46,10 +68,9 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
         if (cell < 0) continue;                                     // uniform: the cell was pruned
         uint32_t w[NW];
         load_words<NW>(c.in.rec, (c.t0 + tt) * 32 + lane, w);       // whole tiles are allocated
-        if (cell != run) {                                          // uniform: a new cell
+        if (F::NBG > 0 ? cell != run : run < 0) {                   // uniform: a new cell (linear bases: once)
             __syncwarp();                                           // the old cell's reads are done
-            const float *src = c.geo32 + (size_t)cell * c.gf;
-            for (int i = lane; i < nfs * NX; i += 32) sg[(i % NX) * nfs + i / NX] = src[i];
+            stage_coefs<FAM, false>(c, cell, sg, lane);
             __syncwarp();
             run = cell;
         }
@@ -140,7 +161,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
     constexpr int NDS = 1 << F::ND, ND = F::ND, LE = F::LE, NFP = F::NFP;
     static_assert(F::D <= 6 && ND <= 2, "at most 64 child slots, two dependent coordinates");
     constexpr int NWI = rec_words(NFP, QI16), NWO = rec_words(NFP, QO16);
-    constexpr int GF = geo32_floats(1 << F::K, ND, LE);
+    constexpr int GF = ((1 << F::K) + 1) * ND * LE;
     const int NS = c.ns, nfs = c.nfs;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the current cell's screen coefficients, staged once per run of tiles of the
@@ -186,9 +207,8 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
         const int64_t r = (c.t0 + tt) * 32 + lane;
         uint32_t w[NWI];
         load_words<NWI>(c.in.rec, r, w);
-        if (cell != gcell) {                                        // uniform
-            const float *src = c.geo32 + (size_t)cell * c.gf;
-            for (int i = lane; i < c.gf; i += 32) G[i] = src[i];
+        if (F::NBG > 0 ? cell != gcell : gcell < 0) {               // uniform (linear bases: once)
+            stage_coefs<FAM, true>(c, cell, G, lane);
             gcell = cell;
         }
         __syncwarp();
@@ -214,7 +234,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
         {
             // every term a multiple of 2^ex and M below 2^(24 + ex): the FP32 residual, and
             // the definition's FP64 one, are exact, so a tie rounds to even in both
-            const int ex = min(__float2int_rn(G[c.gf - 1]), lev.hs_exp);
+            const int ex = min(lev.g_exp, lev.hs_exp);
             const float tq = ex > -100 && c.precision == 1 ? __int_as_float((127 + 24 + ex) << 23) : 0.0f;
             magnitudes<FAM>(qf, qt, G + nfs * ND * LE, hs, M);
 #pragma unroll
@@ -235,7 +255,13 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
             }
             if (!any) continue;                                     // uniform
             float u[ND];
-            partial32<FAM>(qf, qt, G, f, u);
+#pragma unroll
+            for (int j = 0; j < ND; ++j) {
+                u[j] = qf[j];
+#pragma unroll
+                for (int m = 0; m < LE; ++m)
+                    if (F::uses(j, m)) u[j] = __fmaf_rn(qt[m], G[(j * LE + m) * nfs + f], u[j]);
+            }
             uint32_t sv[ND][2];
             bool so[ND][2];
 #pragma unroll
@@ -282,21 +308,18 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
             }
         }
         if (um) {                                                   // rare
-            const RecWords rwords = rec_words_of<NWI>(w);
+            const RecWords<NWI> rwords = rec_words_of<NWI>(w);
             for (unsigned long long m = um; m; m &= m - 1) {
                 const int s = __ffsll((long long)m) - 1, f = s & (nfs - 1), x = s >> c.kf, ds = c.dm == 2 ? x << 1 : x;
                 const uint4 rw = s_row[s];
                 int3 q = make_int3(0, 0, 0);
                 if (c.precision == 1) {                             // the double-float tier
-                    q = snap_df_words<FAM, QI16>(&c.lev, rwords, c.geo32 + (size_t)cell * c.gf + f * ND * LE,
-                                                 c.geo32lo + ((size_t)cell * nfs + f) * ND * LE, ds,
-                                                 __fmaf_ru(kBandDF, M[0], kBandDFAbs),
+                    q = snap_df_words<FAM, QI16>(&c, rwords, cell, f, ds, __fmaf_ru(kBandDF, M[0], kBandDFAbs),
                                                  __fmaf_ru(kBandDF, M[ND - 1], kBandDFAbs), QO16 ? 32767.0f : 1.0e9f);
                     ++ndf;
                 }
                 if (!q.z) {                                         // the FP64 definition
-                    q = snap64_words<FAM, QI16>(&c.P, &c.lev, rwords, c.geo64 + ((size_t)cell * nfs + f) * F::NB, ds,
-                                                c.dm);
+                    q = snap64_words<FAM, QI16>(&c, rwords, cell, f, ds);
                     bad |= (unsigned)(q.z != 0);
                     nrechk += c.precision == 1;
                 }
