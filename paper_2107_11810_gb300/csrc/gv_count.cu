@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
     static_assert(NG <= 32 && NS >= 2 && NS <= 8, "a cell's basis changes fit one register per lane");
     const int lane = threadIdx.x & 31;
     const Level &lev = c.lev;
-    const int64_t nt = c.t1 - c.t0;
+    const int64_t nt = chunk_tiles(c);
     const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
     if (ta >= tb) return;

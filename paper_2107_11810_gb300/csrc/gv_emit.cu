@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
     // child slots of free slot 0 (those of free slot f: shifted left by f)
     constexpr unsigned kFsSlots = NDS == 4 ? 1u | 1u << NFS | 1u << 2 * NFS | 1u << 3 * NFS : (NDS == 2 ? 1u | 1u << NFS : 1u);
     static_assert(NG + F::NBG <= 32, "a cell's basis changes fit one register per lane");
+    if (c.dyn && c.dyn->overflow) return;                           // the children were not laid out
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const Level &lev = c.lev;
     extern __shared__ __align__(128) uint8_t s_dyn[];
@@ -58,7 +59,7 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
     __shared__ __align__(8) uint64_t s_bars[8][2];
     uint64_t *s_bar = s_bars[warp];
 
-    const int nt = (int)(c.t1 - c.t0);
+    const int nt = (int)chunk_tiles(c);
     const int nwarp = gridDim.x * 8, gw = blockIdx.x * 8 + warp;
     const int ut = nt > 4 * kEmitUnit * nwarp ? kEmitUnit : GT, nunits = (nt + ut - 1) / ut;
     if (lane == 0) {

@@ -98,7 +98,9 @@ struct vote_ctx {
     int64_t fault_alloc_at = 0, alloc_count = 0;
     LevelStore ls[GV_MAXL + 1];
     LevelStore beam;           // the selected cells of one level, during the dive
-    DevBuf beam_sel, beam_src;
+    DevBuf beam_sel, beam_src, linfo;
+    LevInfo *h_info = nullptr; // pinned: the steps' reports, per level; the last for single steps
+    long long steps = 0;       // numbers them
     DevBuf sctab[2];           // (sin, cos) tables of the angular coordinates (launch_sincos_table)
     DevBuf rot[GV_MAXL + 1], rotflag[GV_MAXL + 1];   // rotation tables per level (k_rot_fill)
     DevBuf levs_dev, path, scal, alive, geo64, geo32, geo32lo, cnt, tinfo, ballot, lballot, uns, off, cbase, child_idx;
@@ -647,19 +649,185 @@ static const int kSincosBits = 16;
 // records expanded with lower bounds outside dives
 static int64_t lb_records(int d) { return d <= 3 ? (int64_t)1 << 28 : (int64_t)1 << 22; }
 
+// Shape of a level's expansion steps.
+struct StepDims {
+    int kf, dm, lns, ns, nfs;  // child slots (see Chunk)
+    int kg, ng, gf, NB, NBG;   // geometry slots, floats per cell, basis values
+    bool rotation;
+};
+
+static StepDims step_dims(const vote_ctx *c, int l) {
+    const Problem &P = c->P;
+    const Level &lev = c->lev[l];
+    StepDims s;
+    s.kf = s.lns = 0;
+    s.dm = lev.split_mask >> P.k;
+    for (int j = 0; j < P.d; ++j) {
+        const int split = (lev.split_mask >> j) & 1;
+        s.lns += split;
+        if (j < P.k) s.kf += split;
+    }
+    s.ns = 1 << s.lns;
+    s.nfs = 1 << s.kf;
+    s.NB = family_nb(P.fam);
+    s.NBG = family_nbg(P.fam);
+    s.rotation = family_rotation(P.fam);
+    // geometry slots: the free slots, without the linear tail coordinate's bit
+    s.kg = s.rotation ? s.kf - ((lev.split_mask >> (P.k - 1)) & 1) : s.kf;
+    s.ng = 1 << s.kg;
+    s.gf = s.NBG * s.ng + s.NBG;
+    return s;
+}
+
+// Tables of a level's geometry; need64: the FP64 changes are stored per cell (plain FP64
+// mode, or a table is missing).
+static vote_status ensure_tables(vote_ctx *c, int l, const StepDims &s, bool *need64) {
+    const Problem &P = c->P;
+    *need64 = c->precision == 0;
+    if (s.rotation) {
+        for (int x = l; x <= l + 1; ++x) {       // this level's and the next level's rotations
+            int bits = 0;
+            for (int j = 0; j < 3; ++j) bits += std::min(x, P.Lj[j]);
+            if (bits > kRotBits || c->rot[x].p) continue;
+            const size_t flags = (((size_t)1 << bits) / 32 + 1) * 4;
+            TRY(ensure(c, c->rotflag[x], flags));
+            CK(cudaMemsetAsync(c->rotflag[x].p, 0, flags, c->stream));
+            TRY(ensure(c, c->rot[x], (size_t)72 << bits));
+        }
+        *need64 |= !c->rot[l].p || !c->rot[l + 1].p;
+    } else if (s.NBG) {
+        for (int j = 0; j < P.k; ++j) *need64 |= !c->sctab[j].p;
+    }
+    return VOTE_OK;
+}
+
+// Scratch of a step of nc cells and nt tiles; fits: only whether all of it is there.
+static vote_status ensure_scratch(vote_ctx *c, const StepDims &s, size_t nc, size_t nt, bool lb, bool need64,
+                                  bool *fits = nullptr) {
+    const size_t nch = nc * s.ns, ntp = nt > 0 ? nt : 1;
+    auto need = [&](DevBuf &b, size_t bytes) {
+        if (!fits) return ensure(c, b, bytes);
+        if (!b.p || b.bytes < bytes) *fits = false;
+        return VOTE_OK;
+    };
+    if (fits) *fits = true;
+    TRY(need(c->alive, nc));
+    if (s.NBG) {
+        TRY(need(c->geo32, nc * s.gf * 4));
+        TRY(need(c->geo32lo, nc * s.NBG * s.ng * 4));
+    }
+    if (need64) TRY(need(c->geo64, nc * s.nfs * s.NB * 8));
+    TRY(need(c->cnt, nch * 4 * (c->group ? 3 : 2)));
+    TRY(need(c->child_idx, nch * 4));
+    TRY(need(c->cbase, nch * 8));
+    TRY(need(c->keepflag, nch * 4));
+    TRY(need(c->recn, nch * 4));
+    TRY(need(c->bsums, ((nch + 255) / 256) * 16 + 16));
+    TRY(need(c->tinfo, (ntp + 2) * 8));
+    TRY(need(c->ballot, ntp * s.ns * 4 + 16));       // bulk copies round up to 16 bytes
+    TRY(need(c->off, ntp * s.ns * 4 + 16));
+    if (lb) TRY(need(c->lballot, ntp * s.ns * 4));
+    if (c->precision == 1) TRY(need(c->uns, ntp * 8));
+    return VOTE_OK;
+}
+
+// A step's chunk over nc cells and nt tiles from (c0, t0) of S, with the scratch's arrays.
+static void fill_chunk(vote_ctx *c, int l, const LevelStore &S, const StepDims &s, int64_t c0, int64_t nc, int64_t t0,
+                       int64_t nt, bool lb, bool need64, Chunk &ch) {
+    const size_t nch = (size_t)nc * s.ns;
+    std::memset(&ch, 0, sizeof(ch));
+    ch.P = c->P;
+    ch.lev = c->lev[l];
+    ch.cells = cell_view(S);
+    ch.c0 = c0;
+    ch.nc = (int)nc;
+    ch.ns = s.ns;
+    ch.lns = s.lns;
+    ch.nfs = s.nfs;
+    ch.kf = s.kf;
+    ch.dm = s.dm;
+    ch.ng = s.ng;
+    ch.kg = s.kg;
+    ch.gf = s.gf;
+    ch.in = rec_view(c, S);
+    ch.in_rbeg = (const uint64_t *)S.rbeg.p;
+    ch.in_rcnt = (const uint32_t *)S.rcnt.p;
+    ch.in_c0 = c0;
+    ch.t0 = t0;
+    ch.t1 = t0 + nt;
+    ch.alive = (uint8_t *)c->alive.p;
+    ch.geo64 = need64 ? (double *)c->geo64.p : nullptr;
+    for (int j = 0; j < 2; ++j) ch.sincos[j] = (const double2 *)c->sctab[j].p;
+    if (s.rotation) {
+        ch.rot_par = (double *)c->rot[l].p;
+        ch.rot_ch = (double *)c->rot[l + 1].p;
+        ch.rot_flag = (unsigned *)c->rotflag[l + 1].p;
+    }
+    ch.geo32 = (float *)c->geo32.p;
+    ch.geo32lo = (float *)c->geo32lo.p;
+    ch.crec = (uint32_t *)c->cnt.p;
+    ch.clb = ch.crec + nch;
+    ch.cub = c->group ? ch.crec + 2 * nch : ch.crec;
+    ch.weighted = c->group;
+    ch.child_idx = (int32_t *)c->child_idx.p;
+    ch.cbase = (unsigned long long *)c->cbase.p;
+    ch.sc = dsc(c);
+    if (c->trace_cap > 0) {
+        ch.trace.cap = (unsigned long long)c->trace_cap;
+        ch.trace.level = (int32_t *)c->tr_level.p;
+        ch.trace.key = (uint64_t *)c->tr_key.p;
+        ch.trace.ub = (uint32_t *)c->tr_ub.p;
+        ch.trace.lb = (uint32_t *)c->tr_lb.p;
+    }
+    ch.prune = c->prune;
+    ch.precision = c->precision;
+    ch.lb = lb;
+    ch.spin = c->spin_limit;
+    ch.tinfo = (int2 *)c->tinfo.p;
+    ch.ballot = (uint32_t *)c->ballot.p;
+    ch.lballot = (uint32_t *)c->lballot.p;
+    ch.uns = (uint2 *)c->uns.p;
+    ch.off = (uint32_t *)c->off.p;
+    if (!ch.lev.leaf_children) {
+        ch.next_cells = cell_view(c->ls[l + 1]);
+        ch.next_c0 = c->ls[l + 1].ncells;
+        ch.next_r0 = c->ls[l + 1].nrecs;
+        ch.out = rec_view(c, c->ls[l + 1]);
+    }
+}
+
+// Waits until step number seq has reported into v (every step's report is its last but one
+// or last kernel; the stream's state is looked at now and then, so a failed launch ends it).
+static vote_status wait_report(vote_ctx *c, const LevInfo *v, long long seq) {
+    for (unsigned i = 1;; ++i) {
+        if (__atomic_load_n(&v->seq, __ATOMIC_ACQUIRE) == seq) return VOTE_OK;
+        if (i & 1023u) continue;
+        const cudaError_t e = cudaStreamQuery(c->stream);
+        if (e == cudaErrorNotReady) {
+            cudaGetLastError();
+            continue;
+        }
+        CK(e);
+        if (__atomic_load_n(&v->seq, __ATOMIC_ACQUIRE) == seq) return VOTE_OK;
+        set_err("internal: an expansion step ended without its report");
+        return VOTE_EINTERNAL;
+    }
+}
+
+// Lower bounds cost a third of the count pass.  Leaves need none (their own counts are
+// one).  Above them they prune before the first leaf is reached, and with d <= 3 they
+// rank the cells of a dive; once lb_records() records are expanded, only dives take them.
+// All steps / none / this rule, ms: planes of 1e4 points 38 / 98 / 34, of 1e6 points
+// 810 / 741 / 744, 10,000 lines 0.67 / 0.96 / 0.67, affine 4-space 46 / 40 / 41.
+static bool wants_lb(const vote_ctx *c, int l, bool beam) {
+    return c->trace_cap > 0 || (!c->lev[l].leaf_children && (beam || c->expanded < lb_records(c->P.d)));
+}
+
 // Expand a chunk of level-l cells taken from the top of the level's stack, or, in the
 // dive, all cells of the beam store (a selection of level l).
 static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
-    const Problem &P = c->P;
     LevelStore &S = beam ? c->beam : c->ls[l];
     const Level &lev = c->lev[l];
-    int kf = 0, dm = lev.split_mask >> P.k, lns = 0;
-    for (int j = 0; j < P.d; ++j) {
-        const int split = (lev.split_mask >> j) & 1;
-        lns += split;
-        if (j < P.k) kf += split;
-    }
-    const int ns = 1 << lns, nfs = 1 << kf;
     // chunk: cells [c0, c1) from the top of the stack, about chunk_records records
     const int64_t c1 = S.ncells, r1 = S.nrecs;
     int64_t avg = S.nrecs / (S.ncells > 0 ? S.ncells : 1);
@@ -683,99 +851,22 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     }
     nvtxRangePushA("expand_chunk");
     const int nc = (int)(c1 - c0);
-    const int NB = family_nb(P.fam), NBG = family_nbg(P.fam);
-    const bool rotation = family_rotation(P.fam);
-    // geometry slots: the free slots, without the linear tail coordinate's bit
-    const int kg = rotation ? kf - ((lev.split_mask >> (P.k - 1)) & 1) : kf, ng = 1 << kg;
-    const int gf = NBG * ng + NBG;
+    const StepDims dims = step_dims(c, l);
+    const int ns = dims.ns;
     const size_t nch = (size_t)nc * ns;
-    const size_t cnt_arrays = c->group ? 3 : 2;
-    TRY(ensure(c, c->alive, nc));
-    bool need64 = c->precision == 0;
-    if (NBG) {
-        TRY(ensure(c, c->geo32, (size_t)nc * gf * 4));
-        TRY(ensure(c, c->geo32lo, (size_t)nc * NBG * ng * 4));
-    }
-    if (rotation) {
-        for (int x = l; x <= l + 1; ++x) {       // tables of this level's and the next level's rotations
-            int bits = 0;
-            for (int j = 0; j < 3; ++j) bits += std::min(x, P.Lj[j]);
-            if (bits > kRotBits || c->rot[x].p) continue;
-            TRY(ensure(c, c->rot[x], ((size_t)72 << bits)));
-            TRY(ensure(c, c->rotflag[x], (((size_t)1 << bits) / 32 + 1) * 4));
-            CK(cudaMemsetAsync(c->rotflag[x].p, 0, (((size_t)1 << bits) / 32 + 1) * 4, c->stream));
-        }
-        need64 |= !c->rot[l].p || !c->rot[l + 1].p;
-    } else if (NBG) {
-        for (int j = 0; j < P.k; ++j) need64 |= !c->sctab[j].p;
-    }
-    if (need64) TRY(ensure(c, c->geo64, (size_t)nc * nfs * NB * 8));
-    TRY(ensure(c, c->cnt, nch * 4 * cnt_arrays));
-    TRY(ensure(c, c->child_idx, nch * 4));
-    TRY(ensure(c, c->cbase, nch * 8));
-    TRY(ensure(c, c->keepflag, nch * 4));
-    TRY(ensure(c, c->recn, nch * 4));
-    TRY(ensure(c, c->bsums, ((nch + 255) / 256) * 16 + 16));
-    if (!lev.leaf_children) TRY(ensure_level(c, c->ls[l + 1], l + 1, 0, (size_t)c->ls[l + 1].ncells + nch));
-    CK(cudaMemsetAsync(c->cnt.p, 0, nch * 4 * cnt_arrays, c->stream));
-
-    Chunk ch;
-    std::memset(&ch, 0, sizeof(ch));
-    ch.P = P;
-    ch.lev = lev;
-    ch.cells = cell_view(S);
-    ch.c0 = c0;
-    ch.nc = nc;
-    ch.ns = ns;
-    ch.lns = lns;
-    ch.nfs = nfs;
-    ch.kf = kf;
-    ch.dm = dm;
-    ch.gf = gf;
-    ch.in = rec_view(c, S);
-    ch.in_rbeg = (const uint64_t *)S.rbeg.p;
-    ch.in_rcnt = (const uint32_t *)S.rcnt.p;
-    ch.in_c0 = c0;
-    ch.t0 = r0 / 32;
-    ch.t1 = r1 / 32;
-    ch.alive = (uint8_t *)c->alive.p;
-    ch.ng = ng;
-    ch.kg = kg;
-    ch.geo64 = need64 ? (double *)c->geo64.p : nullptr;
-    for (int j = 0; j < 2; ++j) ch.sincos[j] = (const double2 *)c->sctab[j].p;
-    if (rotation) {
-        ch.rot_par = (double *)c->rot[l].p;
-        ch.rot_ch = (double *)c->rot[l + 1].p;
-        ch.rot_flag = (unsigned *)c->rotflag[l + 1].p;
-    }
-    ch.geo32 = (float *)c->geo32.p;
-    ch.geo32lo = (float *)c->geo32lo.p;
-    ch.crec = (uint32_t *)c->cnt.p;
-    ch.clb = ch.crec + nch;
-    ch.cub = c->group ? ch.crec + 2 * nch : ch.crec;
-    ch.child_idx = (int32_t *)c->child_idx.p;
-    ch.cbase = (unsigned long long *)c->cbase.p;
-    ch.sc = dsc(c);
-    if (c->trace_cap > 0) {
-        ch.trace.cap = (unsigned long long)c->trace_cap;
-        ch.trace.level = (int32_t *)c->tr_level.p;
-        ch.trace.key = (uint64_t *)c->tr_key.p;
-        ch.trace.ub = (uint32_t *)c->tr_ub.p;
-        ch.trace.lb = (uint32_t *)c->tr_lb.p;
-    }
-    ch.prune = c->prune;
-    ch.precision = c->precision;
-    // Lower bounds cost a third of the count pass.  Leaves need none (their own counts are
-    // one).  Above them they prune before the first leaf is reached, and with d <= 3 they
-    // rank the cells of a dive; once lb_records() records are expanded, only dives take them.
-    // All steps / none / this rule, ms: planes of 1e4 points 38 / 98 / 34, of 1e6 points
-    // 810 / 741 / 744, 10,000 lines 0.67 / 0.96 / 0.67, affine 4-space 46 / 40 / 41.
-    ch.lb = c->trace_cap > 0 || (!lev.leaf_children && (beam || c->expanded < lb_records(P.d)));
-    c->expanded += r1 - r0;
-    ch.spin = c->spin_limit;
-
     const int rb = rec_bytes_at(c, l);
-    if (c->group && r1 - r0 > 32) {
+    bool need64;
+    TRY(ensure_tables(c, l, dims, &need64));
+    if (!lev.leaf_children) TRY(ensure_level(c, c->ls[l + 1], l + 1, 0, (size_t)c->ls[l + 1].ncells + nch));
+    const bool lb = wants_lb(c, l, beam), grouping = c->group && r1 - r0 > 32;
+    c->expanded += r1 - r0;
+    // canonical records need at most the slots of the originals plus one tile per cell
+    const size_t gslots = (size_t)(r1 - r0) + 32 * (size_t)nc;
+    TRY(ensure_scratch(c, dims, (size_t)nc, grouping ? gslots / 32 : (size_t)(r1 - r0) / 32, lb, need64));
+    Chunk ch;
+    fill_chunk(c, l, S, dims, c0, nc, r0 / 32, (r1 - r0) / 32, lb, need64, ch);
+
+    if (grouping) {
         // canonization's grouping: merge records with equal (cell, q_f, q_t)
         const size_t nr = (size_t)(r1 - r0);
         size_t cap = 1;
@@ -786,8 +877,6 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
         TRY(ensure(c, c->g_ccount, (size_t)nc * 4));
         TRY(ensure(c, c->g_ccur, (size_t)nc * 4));
         TRY(ensure(c, c->g_rbeg, (size_t)nc * 8));
-        // canonical records need at most the slots of the originals plus one tile per cell
-        const size_t gslots = nr + 32 * (size_t)nc;
         TRY(ensure(c, c->g_rec, (gslots + 32) * rb));       // one tile of padding, as for a level
         TRY(ensure(c, c->g_mult, gslots * 4));
         TRY(ensure(c, c->g_tile, (gslots / 32) * 4));
@@ -819,38 +908,23 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
         ch.t1 = gs / 32;
     }
     const int64_t nt = ch.t1 - ch.t0;
-    const size_t ntp = (size_t)(nt > 0 ? nt : 1);
-    TRY(ensure(c, c->tinfo, (ntp + 2) * 8));
-    TRY(ensure(c, c->ballot, ntp * ns * 4 + 16));      // bulk copies round up to 16 bytes
-    TRY(ensure(c, c->off, ntp * ns * 4 + 16));
-    if (ch.lb) TRY(ensure(c, c->lballot, ntp * ns * 4));
-    if (c->precision == 1) TRY(ensure(c, c->uns, ntp * 8));
-    ch.tinfo = (int2 *)c->tinfo.p;
-    ch.ballot = (uint32_t *)c->ballot.p;
-    ch.lballot = (uint32_t *)c->lballot.p;
-    ch.uns = (uint2 *)c->uns.p;
-    ch.off = (uint32_t *)c->off.p;
-    if (!lev.leaf_children) {
-        ch.next_cells = cell_view(c->ls[l + 1]);
-        ch.next_c0 = c->ls[l + 1].ncells;
-        ch.next_r0 = c->ls[l + 1].nrecs;
-        ch.out = rec_view(c, c->ls[l + 1]);
-    }
+    ch.host = c->h_info + GV_MAXL + 1;
+    ch.seq = ++c->steps;
     ev_mark(c, -1);
     const int nprep = launch_prep(ch, c->stream);
     ev_mark(c, VOTE_K_CELL_GEO);
     launch_count(ch, c->stream);
     ev_mark(c, VOTE_K_TEST_COUNT);
     launch_tile_scan(ch, c->stream);
-    launch_child_alloc(ch, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p, (unsigned long long *)c->bsums.p,
-                       c->stream);
+    const int nchild = launch_child_alloc(ch, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
+                                          (unsigned long long *)c->bsums.p, c->stream);
     ev_mark(c, VOTE_K_CHILDREN);
     // algorithmic bytes: the records of whole tiles read, the ballots written
     c->kbytes[VOTE_K_TEST_COUNT] += (double)nt * 32 * rb + (double)nt * ns * 4;
     c->kbytes[VOTE_K_CELL_GEO] += (double)nc * (8 + 4);
     CK(cudaGetLastError());
     c->stats.chunks++;
-    c->stats.launches += (lev.leaf_children ? 3 : 5) + nprep + (c->precision == 1);
+    c->stats.launches += 2 + nprep + nchild + (c->precision == 1);
     c->stats.cells += nc;
     c->lv_cells[l] += nc;
     c->lv_recs[l] += nt * 32;
@@ -865,10 +939,9 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
         nvtxRangePop();
         return VOTE_OK;
     }
-    CK(cudaMemcpyAsync(&c->h_sc->n_cells, &dsc(c)->n_cells, 16, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    TRY(wait_report(c, ch.host, ch.seq));
     LevelStore &N = c->ls[l + 1];
-    int64_t new_cells = (int64_t)c->h_sc->n_cells, new_slots = (int64_t)c->h_sc->n_recs;
+    int64_t new_cells = ch.host->stored_cells, new_slots = ch.host->stored_recs;
     if (new_slots > 0) {
         TRY(ensure_level(c, N, l + 1, (size_t)(N.nrecs + new_slots), 0));
         ch.out = rec_view(c, N);
@@ -907,7 +980,8 @@ static vote_status replay(vote_ctx *c, const double *surfaces, int64_t n, int la
                           int64_t *ub, int64_t *lb) {
     CK(cudaMemsetAsync(&dsc(c)->replay_ub, 0, 16, c->stream));
     ev_mark(c, -1);
-    if (lam > 0) launch_path_geo(c->P, (const Level *)c->levs_dev.p, lam, key, (PathStep *)c->path.p, c->stream);
+    if (lam > 0)
+        launch_path_geo(c->P, (const Level *)c->levs_dev.p, lam, key, nullptr, (PathStep *)c->path.p, c->stream);
     launch_replay(c->P, (const Level *)c->levs_dev.p, (const PathStep *)c->path.p, lam, surfaces, n, reach,
                   dsc(c), c->stream);
     c->stats.launches += lam > 0 ? 2 : 1;
@@ -978,7 +1052,136 @@ static vote_status dive(vote_ctx *c, int l0) {
     return VOTE_OK;
 }
 
-// The search.  A dive from the root; then level by level, shallowest first, so that a
+// The chain: from the root, levels that hold at most kBeamRecords records are expanded
+// whole, one after the other.  A level's sizes pass on to the next on the device, and the
+// host queues each level's step while the one before runs, with grids and scratch sized
+// by bounds from the level before that: without it every step of a few hundred surfaces
+// waited 40 us for the host beside 20 us of kernels.  The chain ends at the leaves, at a
+// level too large to expand whole (stored for the dives; the step queued for it finds no
+// cells), or where nothing is left.  *replayed: the best leaf's mask was replayed into mask.
+static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_t *mask, bool *replayed) {
+    const Problem &P = c->P;
+    const int L = P.L;
+    *replayed = false;
+    const int64_t slots0 = c->ls[0].nrecs, fit = std::min(kBeamRecords, c->chunk_records) & ~(int64_t)31;
+    if (slots0 > fit || c->group || c->kernel_timing || c->log >= 2) return VOTE_OK;
+    TRY(ensure(c, c->linfo, sizeof(LevInfo) * (GV_MAXL + 1)));
+    LevInfo *di = (LevInfo *)c->linfo.p;
+    Chunk ch, last;                          // of the level at hand, of the one before
+    int64_t cells = 1, recs = slots0;        // sizes of the level at hand, once known
+    int64_t pcells = 0;                      // and of the one before
+    StepDims dims, pdims;
+    bool known = true;
+    int launches = 0;
+    for (int l = 0;;) {
+        dims = step_dims(c, l);
+        const bool lb = wants_lb(c, l, c->dive && c->prune);
+        bool need64, fits;
+        TRY(ensure_tables(c, l, dims, &need64));
+        // every cell holds at least a tile, and at most as many as the root
+        int64_t cb = cells, tb = recs / 32;
+        if (!known) {
+            cb = std::min(pcells * pdims.ns, fit / 32);
+            tb = std::min(cb * (slots0 / 32), fit / 32);
+            // the step before may still need the scratch that would grow
+            TRY(ensure_scratch(c, dims, (size_t)cb, (size_t)tb, lb, need64, &fits));
+        }
+        if (known || fits) {
+            if (l + 1 < L) {
+                // room for the next level: most levels need less; else see below
+                const int64_t rc = std::min(cb * dims.ns, (int64_t)1 << 14);
+                TRY(ensure_level(c, c->ls[l + 1], l + 1, (size_t)std::min(rc * slots0, (int64_t)1 << 17), (size_t)rc));
+            }
+            if (known) {
+                TRY(ensure_scratch(c, dims, (size_t)cb, (size_t)tb, lb, need64));
+                launch_chain_start(di + l, cells, recs, c->stream);
+            }
+            fill_chunk(c, l, c->ls[l], dims, 0, cb, 0, tb, lb, need64, ch);
+            ch.dyn = di + l;
+            ch.host = c->h_info + l + 1;
+            ch.seq = ++c->steps;
+            ch.fit_recs = fit;
+            if (l + 1 < L) {
+                const LevelStore &N = c->ls[l + 1];
+                ch.cap_cells = (int64_t)std::min(std::min(N.key.bytes, N.rbeg.bytes) / 8,
+                                                 std::min(std::min(N.rcnt.bytes, N.ub.bytes), N.lb.bytes) / 4);
+                ch.cap_recs = std::min((int64_t)(N.rec.bytes / rec_bytes_at(c, l + 1)) - 32,
+                                       (int64_t)(N.tile_cell.bytes / 4) * 32);
+            }
+            const int nprep = launch_prep(ch, c->stream);
+            launch_count(ch, c->stream);
+            launch_tile_scan(ch, c->stream);
+            const int nchild = launch_child_alloc(ch, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
+                                                  (unsigned long long *)c->bsums.p, c->stream);
+            if (l + 1 < L && !launch_emit(ch, c->stream)) {
+                set_err("internal: no emit pass for record formats %d -> %d", ch.lev.q16, ch.lev.q16_next);
+                return VOTE_EINTERNAL;
+            }
+            CK(cudaGetLastError());
+            launches = 2 + nprep + nchild + (c->precision == 1) + (l + 1 < L);
+        }
+        if (!known) {                        // what the step before stored
+            const LevInfo *v = last.host;
+            TRY(wait_report(c, v, last.seq));
+            cells = v->stored_cells;
+            recs = v->stored_recs;
+            c->ls[l].ncells = cells;
+            c->ls[l].nrecs = recs;
+            if (recs > c->stats.peak_records) c->stats.peak_records = recs;
+            if (v->overflow) {
+                // its counts and ballots stand: make room, lay the children out, emit
+                const unsigned stride = (unsigned)(((int64_t)last.nc * last.ns + 255) / 256);   // of the block totals
+                LevelStore &N = c->ls[l];
+                N.ncells = N.nrecs = 0;
+                TRY(ensure_level(c, N, l, (size_t)recs, (size_t)cells));
+                last.nc = (int)pcells;
+                last.t1 = c->ls[l - 1].nrecs / 32;
+                last.dyn = nullptr;
+                last.host = nullptr;
+                last.next_cells = cell_view(N);
+                last.out = rec_view(c, N);
+                launch_child_write(last, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
+                                   (unsigned long long *)c->bsums.p, stride, c->stream);
+                launch_emit(last, c->stream);
+                CK(cudaGetLastError());
+                N.ncells = cells;
+                N.nrecs = recs;
+            }
+            c->ls[l - 1].ncells = c->ls[l - 1].nrecs = 0;
+            if (cells == 0 || recs > fit) return VOTE_OK;
+            known = true;
+            if (v->overflow || !fits) continue;      // no step is queued for this level yet
+        }
+        // the level's step is queued and its sizes are known
+        c->stats.chunks++;
+        c->stats.launches += launches;       // of the steps that ran: the same whatever was allocated before
+        c->stats.cells += cells;
+        c->lv_cells[l] += cells;
+        c->lv_recs[l] += recs;
+        c->expanded += recs;
+        c->kbytes[VOTE_K_TEST_COUNT] += (double)recs * rec_bytes_at(c, l) + (double)recs / 32 * dims.ns * 4;
+        if (++l == L) {
+            c->ls[l - 1].ncells = c->ls[l - 1].nrecs = 0;
+            c->stats.leaves += cells * dims.ns;
+            break;
+        }
+        last = ch;
+        pcells = cells;
+        pdims = dims;
+        known = false;
+    }
+    if (mask) {
+        launch_path_geo(P, (const Level *)c->levs_dev.p, L, 0, dsc(c), (PathStep *)c->path.p, c->stream);
+        launch_replay(P, (const Level *)c->levs_dev.p, (const PathStep *)c->path.p, L, surfaces, n, mask, dsc(c),
+                      c->stream);
+        CK(cudaGetLastError());
+        c->stats.launches += 2;
+        *replayed = true;
+    }
+    return VOTE_OK;
+}
+
+// The search.  The chain from the root; a dive from where it ends; then level by level, shallowest first, so that a
 // level's bounds are raised by all of its cells before its children are opened, while
 // the next level holds less than one step's records; when every level below is full,
 // the deepest first, which bounds the memory (room for 4 steps: a first solve of planes
@@ -989,13 +1192,19 @@ static vote_status dive(vote_ctx *c, int l0) {
 // radial 70 -> 22, affine 4-space 204 -> 55, planes of 1e4 points 110 -> 54, 3DoF with
 // 1e6 matches 12.5 -> 7.9; with the final depth known from the start (VOTE_OPT_INITIAL_LB)
 // they took 13.5, -, 19, 52, 47 and 4.4 ms.
-static vote_status search(vote_ctx *c) {
+static vote_status search(vote_ctx *c, const double *surfaces, int64_t n, uint32_t *mask, bool *replayed) {
     const int L = c->P.L;
     const bool dives = c->dive && c->prune;
     const int64_t full = std::min(c->chunk_records, (int64_t)1 << 34);
     int64_t since[GV_MAXL + 1];          // records expanded into the level since its last dive
     for (int l = 0; l <= L; ++l) since[l] = -1;
-    if (dives) TRY(dive(c, 0));
+    TRY(chain(c, surfaces, n, mask, replayed));
+    if (dives)
+        for (int l = 0; l < L; ++l)
+            if (c->ls[l].ncells > 0) {               // from where the chain ended
+                TRY(dive(c, l));
+                break;
+            }
     for (;;) {
         int l = -1;
         for (int x = 0; x < L; ++x)
@@ -1040,6 +1249,7 @@ static vote_status solve_device(vote_ctx *c, const double *surfaces, int64_t n, 
                                 int64_t *best_leaf, int64_t *depth, uint32_t *mask) {
     nvtxRangePushA("vote_solve");
     vote_status st = solve_inner(c, surfaces, n, best_point, best_leaf, depth, mask);
+    if (st != VOTE_OK) cudaStreamSynchronize(c->stream);   // steps in flight report into this context
     nvtxRangePop();
     if (c->log) log_solve(c, st);
     return st;
@@ -1070,24 +1280,17 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
     for (int l = 0; l <= P.L; ++l) c->ls[l].ncells = c->ls[l].nrecs = 0;
     uint64_t leafkey = 0;
     int64_t dep = 0;
+    bool mask_done = false;
     if (n > 0 && P.L == 0) {
         dep = n;                                   // the domain is a leaf: every surface counts
     } else if (n > 0) {
         const int64_t slots0 = (n + 31) & ~(int64_t)31;
         TRY(ensure_level(c, c->ls[0], 0, (size_t)slots0, 1));
         ev_mark(c, -1);
-        launch_lift(P, c->lev[0], surfaces, n, rec_view(c, c->ls[0]), dsc(c), c->stream);
+        launch_lift(P, c->lev[0], surfaces, n, rec_view(c, c->ls[0]), cell_view(c->ls[0]), dsc(c), c->stream);
         c->stats.launches += 1;
         ev_mark(c, VOTE_K_LIFT);
         CK(cudaGetLastError());
-        uint64_t key0 = 0, rb0 = 0;
-        uint32_t cnt0 = (uint32_t)n;
-        CK(cudaMemcpyAsync(c->ls[0].key.p, &key0, 8, cudaMemcpyHostToDevice, c->stream));
-        CK(cudaMemcpyAsync(c->ls[0].rbeg.p, &rb0, 8, cudaMemcpyHostToDevice, c->stream));
-        CK(cudaMemcpyAsync(c->ls[0].rcnt.p, &cnt0, 4, cudaMemcpyHostToDevice, c->stream));
-        CK(cudaMemcpyAsync(c->ls[0].ub.p, &cnt0, 4, cudaMemcpyHostToDevice, c->stream));
-        CK(cudaMemsetAsync(c->ls[0].lb.p, 0, 4, c->stream));
-        CK(cudaStreamSynchronize(c->stream));    // host sources above live on this frame
         c->ls[0].ncells = 1;
         c->ls[0].nrecs = slots0;
         TRY(read_scalars(c));
@@ -1098,7 +1301,8 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
             return VOTE_EINVAL;
         }
         finalize_levels(c, c->h_sc->qmax);
-        TRY(search(c));
+        bool replayed = false;
+        TRY(search(c, surfaces, n, mask, &replayed));
         TRY(read_scalars(c));
         ev_collect(c);
         if (c->h_sc->err & kErrTimeout) {
@@ -1109,6 +1313,7 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
             set_err("internal: residual out of range (err %u)", c->h_sc->err);
             return VOTE_EINTERNAL;
         }
+        mask_done = replayed;
         unsigned long long bk = c->h_sc->best_key;
         if (bk) {
             dep = (int64_t)(bk >> P.coord_bits);
@@ -1127,7 +1332,12 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
         best_point[j] = P.lo[j] + (double)(2 * i + 1) * c->h_leaf[j];
     }
     if (mask && n > 0) {
-        if (dep > 0) {
+        if (dep > 0 && mask_done) {
+            if ((int64_t)c->h_sc->replay_ub != dep) {
+                set_err("internal: replayed inlier count %lld != depth %lld", (long long)c->h_sc->replay_ub, (long long)dep);
+                return VOTE_EINTERNAL;
+            }
+        } else if (dep > 0) {
             int64_t ub = 0, lb = 0;
             TRY(replay(c, surfaces, n, P.L, leafkey, mask, &ub, &lb));
             if (ub != dep) {
@@ -1183,6 +1393,8 @@ vote_status vote_create(int family, int d, int k, const double *eps, const doubl
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_sc, sizeof(Scalars));
     if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_tmp, 64);
+    if (e == cudaSuccess) e = cudaMallocHost((void **)&c->h_info, sizeof(LevInfo) * (GV_MAXL + 2));
+    if (e == cudaSuccess) std::memset(c->h_info, 0, sizeof(LevInfo) * (GV_MAXL + 2));
     if (e != cudaSuccess) {
         set_err("CUDA unavailable: %s", cudaGetErrorString(e));
         delete c;
@@ -1638,7 +1850,7 @@ void vote_destroy(vote_ctx *c) {
                       &c->ballot, &c->lballot, &c->uns, &c->off, &c->cbase, &c->child_idx, &c->keepflag, &c->recn, &c->bsums, &c->tr_level, &c->tr_key,
                       &c->tr_ub, &c->tr_lb, &c->surf_tmp, &c->mask_tmp, &c->ss_partial,
                       &c->ss_io, &c->g_table, &c->g_owner, &c->g_newpos, &c->g_ccount, &c->g_ccur,
-                      &c->g_rbeg, &c->g_rec, &c->g_mult, &c->g_tile, &c->beam_sel, &c->beam_src};
+                      &c->g_rbeg, &c->g_rec, &c->g_mult, &c->g_tile, &c->beam_sel, &c->beam_src, &c->linfo};
     for (DevBuf *b : bufs) release(c, *b);
     for (DevBuf &b : c->sctab) release(c, b);
     for (int l = 0; l <= GV_MAXL; ++l) release(c, c->rot[l]), release(c, c->rotflag[l]);
@@ -1647,6 +1859,7 @@ void vote_destroy(vote_ctx *c) {
         if (c->ev[i]) cudaEventDestroy(c->ev[i]);
     if (c->h_sc) cudaFreeHost(c->h_sc);
     if (c->h_tmp) cudaFreeHost(c->h_tmp);
+    if (c->h_info) cudaFreeHost(c->h_info);
     delete c;
 }
 
@@ -1720,7 +1933,7 @@ extern "C" vote_status vote_cell_counts_noalloc(int family, int d, int k, const 
     Scalars *sc = (Scalars *)(base + kNaScalars);
     if (P.L > 0) CK(cudaMemcpyAsync(levs, tmp.lev, sizeof(Level) * P.L, cudaMemcpyHostToDevice, st));
     CK(cudaMemsetAsync(sc, 0, sizeof(Scalars), st));        // the counters must start at zero
-    if (level > 0) launch_path_geo(P, levs, level, key, path, st);
+    if (level > 0) launch_path_geo(P, levs, level, key, nullptr, path, st);
     launch_replay(P, levs, path, level, surfaces, n, reach, sc, st);
     CK(cudaGetLastError());
     unsigned long long cnt[2] = {0, 0};

@@ -28,6 +28,7 @@ __device__ __forceinline__ void eval_record(const Chunk &c, int64_t r, int cell,
 // screen left those lanes' bits clear, so the passing ones are set here.
 template <int FAM, bool Q16>
 __global__ void __launch_bounds__(128) k_recheck(const __grid_constant__ Chunk c) {
+    if (chunk_tiles(c) == 0) return;                                // the chain has stopped: not its queue
     const unsigned nq = c.sc->n_uns;
     unsigned long long done = 0;
     for (unsigned i = blockIdx.x * 128u + threadIdx.x; i < nq; i += gridDim.x * 128u) {
@@ -51,7 +52,7 @@ __global__ void __launch_bounds__(128) k_recheck(const __grid_constant__ Chunk c
 template <int FAM, bool Q16>
 __global__ void __launch_bounds__(256) k_count_exact(const __grid_constant__ Chunk c) {
     const int lane = threadIdx.x & 31;
-    const int64_t nwarp = (int64_t)gridDim.x * 8, nt = c.t1 - c.t0;
+    const int64_t nwarp = (int64_t)gridDim.x * 8, nt = chunk_tiles(c);
     unsigned nrec = 0;
     for (int64_t tt = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); tt < nt; tt += nwarp) {
         const int2 ti = c.tinfo[tt];

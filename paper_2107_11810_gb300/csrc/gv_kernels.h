@@ -55,6 +55,16 @@ struct Trace {
     uint32_t *ub, *lb;
 };
 
+// Sizes of one level in a chain (levels expanded whole, one after the other, without the
+// host): what its kernels expand, 0 once the chain has stopped; what the step before
+// stored; whether its own step found no room in the next level.
+struct LevInfo {
+    long long ncells, nrecs;
+    long long stored_cells, stored_recs;
+    long long overflow;
+    long long seq;           // the host's copy: written last, the number of the step
+};
+
 // Everything one expansion step (a chunk of cells of one level) needs.
 //
 // Children are numbered over the coordinates that still split at this level ("child
@@ -105,11 +115,19 @@ struct Chunk {
     RecView out;             // records of level l+1
     Scalars *sc;
     Trace trace;
+    LevInfo *dyn;            // in a chain of levels: this level's sizes (the next level's follow), else NULL
+    LevInfo *host;           // pinned: where the step reports what it stored, as step number seq
+    long long seq;
+    int64_t cap_cells, cap_recs, fit_recs;   // chain: room in the next level; what still is expanded whole
+    int weighted;            // multiplicities: cub is an array of its own
     int prune;
     int precision;           // 0 = FP64, 1 = FP32 screen + FP64 recheck
     int lb;                  // lower bounds are wanted (lballot, clb)
     unsigned spin;           // polls of a bounded wait for a bulk copy before giving up
 };
+// Sizes of a chunk: from the device in a chain of levels (the host's are then bounds).
+__device__ __forceinline__ int64_t chunk_tiles(const Chunk &c) { return c.dyn ? c.dyn->nrecs >> 5 : c.t1 - c.t0; }
+__device__ __forceinline__ int chunk_cells(const Chunk &c) { return c.dyn ? (int)c.dyn->ncells : c.nc; }
 constexpr int kTileFirst = 64, kTileLast = 128;   // flags in tinfo.y: first / last tile of its cell
 
 constexpr int kNoExp = -1000;
@@ -130,8 +148,9 @@ struct PathStep {
     double dpsi[GV_MAXT];
 };
 
-void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t n, RecView out, Scalars *sc,
-                 cudaStream_t st);
+// root records of the surfaces and the root cell
+void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t n, RecView out, CellView root,
+                 Scalars *sc, cudaStream_t st);
 // the (sin, cos) table of an angular coordinate (2^(splits + 1) - 1 entries)
 void launch_sincos_table(const Problem &P, int j, double2 *tab, cudaStream_t st);
 // cells (alive, geometry) and tiles (tinfo) of the chunk; returns the kernels launched
@@ -154,8 +173,14 @@ bool launch_emit_wide(const Chunk &c, cudaStream_t st);
 // false if the level's record formats have no emit pass (never chosen by the engine)
 bool launch_emit(const Chunk &c, cudaStream_t st);
 // keepflag, recn: [nc * ns]; bsums: 2 * ceil(nc * ns / 256)
-void launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
-                        cudaStream_t st);
+// sizes of the level that a chain starts from, or goes on from
+void launch_chain_start(LevInfo *info, int64_t cells, int64_t recs, cudaStream_t st);
+// returns the kernels launched
+int launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
+                       cudaStream_t st);
+// the last of them again (after a chain found no room in the next level)
+void launch_child_write(const Chunk &c, const uint32_t *keepflag, const uint32_t *recn, unsigned long long *bsums,
+                        unsigned stride, cudaStream_t st);
 // the cells of a level (whose sum of record slots exceeds budget) with the largest UBs (nk = 2: and LBs):
 // out and src_rbeg receive them ([ncells] at most), sc->n_cells / n_recs their number
 // and slots; bsums: 2 * ceil(ncells / 256); then their records
@@ -164,7 +189,8 @@ void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells,
                         cudaStream_t st);
 void launch_beam_gather(const RecView &in, const RecView &out, const CellView &sel, const uint64_t *src_rbeg,
                         int64_t ncells, int64_t ntiles, int rec_bytes, cudaStream_t st);
-void launch_path_geo(const Problem &P, const Level *levs_dev, int lam, uint64_t key, PathStep *path,
+// the path to cell `key` at level lam, or to the best leaf of sc when sc is not NULL
+void launch_path_geo(const Problem &P, const Level *levs_dev, int lam, uint64_t key, const Scalars *sc, PathStep *path,
                      cudaStream_t st);
 void launch_replay(const Problem &P, const Level *levs_dev, const PathStep *path, int lam, const double *prm,
                    int64_t n, uint32_t *reach, Scalars *sc, cudaStream_t st);

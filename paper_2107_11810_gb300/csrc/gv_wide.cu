@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
     float *sg = s_g[threadIdx.x >> 5];                              // [j * LE + m][nfs]
     const int nfs = c.nfs;
     int run = -1;
-    const int64_t nt = c.t1 - c.t0;
+    const int64_t nt = chunk_tiles(c);
     const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
     const Level &lev = c.lev;
@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
     static_assert(F::D <= 6 && ND <= 2, "at most 64 child slots, two dependent coordinates");
     constexpr int NWI = rec_words(NFP, QI16), NWO = rec_words(NFP, QO16);
     constexpr int GF = ((1 << F::K) + 1) * ND * LE;
+    if (c.dyn && c.dyn->overflow) return;                           // the children were not laid out
     const int NS = c.ns, nfs = c.nfs;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the current cell's screen coefficients, staged once per run of tiles of the
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
     uint4 *s_row = s_rows[warp];
     int gcell = -1;
     const unsigned below = (1u << lane) - 1u, lanebit = 1u << lane;
-    const int64_t nt = c.t1 - c.t0;
+    const int64_t nt = chunk_tiles(c);
     const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + warp;
     const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
     const Level &lev = c.lev;
