@@ -36,6 +36,7 @@ __device__ __forceinline__ void store_row(uint32_t *p, const unsigned *v) {
 // boundary case.
 template <int FAM, bool Q16, int KF, int DM, bool LB>
 __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk c) {
+    grid_start();
     using F = Fam<FAM>;
     constexpr int ND = F::ND, LE = F::LE, NFS = 1 << KF, NS = NFS * dep_slots(DM), NP = (NFS + 1) / 2;
     constexpr int NW = rec_words(F::NFP, Q16), NG = F::NBG * NFS;
@@ -56,7 +57,7 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
     const float *gp = c.geo32 + (lane < NG ? lane : 0);
     auto load_g = [&](int cell) {
         if constexpr (NG == 0) return 0.0f;
-        else return __ldg(gp + (unsigned)(cell < 0 ? 0 : cell) * (size_t)c.gf);
+        else return gp[(unsigned)(cell < 0 ? 0 : cell) * (size_t)c.gf];
     };
     int run = -1;
     f2 G[ND][LE][NP];
@@ -172,8 +173,8 @@ static void launch_kd(const Chunk &c, cudaStream_t st) {
         const int64_t nt = c.t1 - c.t0;
         const int64_t want = (int64_t)sm_count() * 4, need = (nt + 15) / 16;
         const unsigned g = (unsigned)(want < need ? want : need);
-        if (c.lb) k_count<FAM, Q16, KF, DM, true><<<g, 256, 0, st>>>(c);
-        else k_count<FAM, Q16, KF, DM, false><<<g, 256, 0, st>>>(c);
+        if (c.lb) launch(k_count<FAM, Q16, KF, DM, true>, g, 256, 0, st, c);
+        else launch(k_count<FAM, Q16, KF, DM, false>, g, 256, 0, st, c);
     }
 }
 

@@ -41,6 +41,7 @@ __host__ __device__ constexpr size_t emit_warp_bytes(int ns) {
 // and neither reading nor the work falls to tiles that have nothing to write.
 template <int FAM, bool QI16, bool QO16, int KF, int DM>
 __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c) {
+    grid_start();
     using F = Fam<FAM>;
     constexpr int ND = F::ND, LE = F::LE, NFP = F::NFP, NFS = 1 << KF, NDS = dep_slots(DM), NS = NFS * NDS;
     constexpr int NWI = rec_words(NFP, QI16), NWO = rec_words(NFP, QO16), RW = 32 * NWI, NG = F::NBG * NFS;
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
     int pidx = 0;
     auto prefetch = [&](int cell) {
         if (cell < 0) return;                                       // uniform
-        if (lane < NG + F::NBG) pg = __ldg(c.geo32 + (size_t)cell * c.gf + lane);
+        if (lane < NG + F::NBG) pg = c.geo32[(size_t)cell * c.gf + lane];
         if (lane < NS) {
             pbase = c.cbase[(size_t)cell * NS + lane];
             pidx = c.child_idx[(size_t)cell * NS + lane];

@@ -28,6 +28,7 @@ __device__ __forceinline__ void eval_record(const Chunk &c, int64_t r, int cell,
 // screen left those lanes' bits clear, so the passing ones are set here.
 template <int FAM, bool Q16>
 __global__ void __launch_bounds__(128) k_recheck(const __grid_constant__ Chunk c) {
+    grid_start();
     if (chunk_tiles(c) == 0) return;                                // the chain has stopped: not its queue
     const unsigned nq = c.sc->n_uns;
     unsigned long long done = 0;
@@ -51,6 +52,7 @@ __global__ void __launch_bounds__(128) k_recheck(const __grid_constant__ Chunk c
 // Plain FP64 mode: a warp per tile, every record by the definition.
 template <int FAM, bool Q16>
 __global__ void __launch_bounds__(256) k_count_exact(const __grid_constant__ Chunk c) {
+    grid_start();
     const int lane = threadIdx.x & 31;
     const int64_t nwarp = (int64_t)gridDim.x * 8, nt = chunk_tiles(c);
     unsigned nrec = 0;
@@ -96,9 +98,9 @@ void launch_recheck(const Chunk &c, cudaStream_t st) {
     // 8e7 tiles on, smaller chunks need fewer
     const unsigned g = (unsigned)(nt < 608 * 128 ? (nt + 127) / 128 : 608);
     if (c.lev.q16) {
-        GV_DISPATCH(c.P.fam, (k_recheck<FAMV, true><<<g, 128, 0, st>>>(c)));
+        GV_DISPATCH(c.P.fam, (launch(k_recheck<FAMV, true>, g, 128, 0, st, c)));
     } else {
-        GV_DISPATCH(c.P.fam, (k_recheck<FAMV, false><<<g, 128, 0, st>>>(c)));
+        GV_DISPATCH(c.P.fam, (launch(k_recheck<FAMV, false>, g, 128, 0, st, c)));
     }
 }
 
@@ -106,7 +108,7 @@ void launch_count_exact(const Chunk &c, cudaStream_t st) {
     const int64_t nt = c.t1 - c.t0;
     if (nt <= 0) return;
     const unsigned g = (unsigned)(nt < 8 * 152 * 8 ? (nt + 7) / 8 : 152 * 8);
-    GV_DISPATCH(c.P.fam, (k_count_exact<FAMV, false><<<g, 256, 0, st>>>(c)));   // 32-bit records in this mode
+    GV_DISPATCH(c.P.fam, (launch(k_count_exact<FAMV, false>, g, 256, 0, st, c)));   // 32-bit records in this mode
 }
 
 }  // namespace gv

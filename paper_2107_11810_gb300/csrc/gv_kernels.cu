@@ -37,6 +37,7 @@ __device__ __forceinline__ unsigned prune_threshold(const Problem &P, const Scal
 template <int FAM>
 __global__ void k_lift(Problem P, Level lev0, const double *prm, int64_t n, RecView out, CellView root,
                        Scalars *sc) {
+    grid_start();
     using F = Fam<FAM>;
     constexpr int NW = rec_words(F::NFP, false);
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -155,6 +156,7 @@ __global__ void k_sincos_table(Problem P, int j, double2 *tab, int64_t n) {
 // at the end of the kernel.  Cells that share their rotation coordinates share them.
 template <int FAM>
 __global__ void __launch_bounds__(256) k_rot_fill(const __grid_constant__ Chunk c) {
+    grid_start();
     const int64_t gid = blockIdx.x * 256ll + threadIdx.x;
     const Problem &P = c.P;
     const Level &lev = c.lev;
@@ -201,6 +203,7 @@ __device__ __forceinline__ void tile_info(const Chunk &c, int64_t i, unsigned th
 
 template <int FAM>
 __global__ void __launch_bounds__(256) k_prep(const __grid_constant__ Chunk c) {
+    grid_start();
     using F = Fam<FAM>;
     static_assert(32 % (1 << F::K) == 0, "a cell's threads must lie in one warp");
     const int64_t gid = blockIdx.x * 256ll + threadIdx.x;
@@ -289,6 +292,7 @@ __device__ __forceinline__ unsigned long long block_excl_scan(unsigned long long
 // per-block totals of surviving children and their records.
 __global__ void __launch_bounds__(256) k_child_mark(Chunk c, uint32_t *keepflag, uint32_t *recn,
                                                     unsigned long long *bs_cells, unsigned long long *bs_recs) {
+    grid_start();
     const Problem &P = c.P;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int cl = idx >> c.lns, s = idx & (c.ns - 1);
@@ -339,6 +343,7 @@ __global__ void __launch_bounds__(256) k_child_mark(Chunk c, uint32_t *keepflag,
 
 // Phase B: exclusive scan of the per-block totals (one block of 256 threads).
 __global__ void __launch_bounds__(256) k_scan_sums(unsigned long long *a, unsigned long long *b, int nb, Scalars *sc) {
+    grid_start();
     unsigned long long ca = 0, cb = 0;
     for (int base = 0; base < nb; base += 256) {
         int i = base + threadIdx.x;
@@ -379,6 +384,7 @@ __device__ __forceinline__ void report(const Chunk &c, unsigned long long cells,
 __global__ void __launch_bounds__(256) k_child_write(Chunk c, const uint32_t *keepflag, const uint32_t *recn,
                                                      const unsigned long long *bs_cells,
                                                      const unsigned long long *bs_recs, int scanned) {
+    grid_start();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     const int nch = chunk_cells(c) << c.lns, nb = (nch + 255) / 256;
     if ((int)blockIdx.x >= nb) return;                   // uniform
@@ -491,6 +497,7 @@ __device__ __forceinline__ unsigned long long warp_max64(unsigned long long v) {
 
 __global__ void __launch_bounds__(256) k_beam_hist(CellView cells, int64_t ncells, BeamSel *sel, int nk, Problem P,
                                                    const Scalars *sc) {
+    grid_start();
     __shared__ unsigned long long hist[2][kBeamBins];
     for (int i = threadIdx.x; i < 2 * kBeamBins; i += 256) hist[0][i] = 0ull;
     const unsigned thr = prune_threshold(P, sc, 1);
@@ -520,6 +527,7 @@ __global__ void __launch_bounds__(256) k_beam_hist(CellView cells, int64_t ncell
 }
 
 __global__ void __launch_bounds__(256) k_beam_pick(BeamSel *sel, unsigned long long budget) {
+    grid_start();
     // thread t owns bins [8 t', 8 t' + 8), t' counted from the top, so a prefix over the
     // threads is the slots of all higher bins
     constexpr int PER = kBeamBins / 256;
@@ -571,6 +579,7 @@ __device__ __forceinline__ bool beam_selected(const CellView &cells, int64_t i, 
 __global__ void __launch_bounds__(256) k_beam_mark(CellView cells, int64_t ncells, const BeamSel *sel, int nk, Problem P,
                                                    const Scalars *sc, unsigned long long *bs_cells,
                                                    unsigned long long *bs_recs) {
+    grid_start();
     const int64_t i = blockIdx.x * 256ll + threadIdx.x;
     const bool keep = beam_selected(cells, i, ncells, sel, nk, prune_threshold(P, sc, 1));
     unsigned long long tc, tr;
@@ -586,6 +595,7 @@ __global__ void __launch_bounds__(256) k_beam_write(CellView cells, int64_t ncel
                                                     const Scalars *sc, const unsigned long long *bs_cells,
                                                     const unsigned long long *bs_recs, CellView out,
                                                     uint64_t *src_rbeg) {
+    grid_start();
     const int64_t i = blockIdx.x * 256ll + threadIdx.x;
     const bool keep = beam_selected(cells, i, ncells, sel, nk, prune_threshold(P, sc, 1));
     unsigned long long tc, tr;
@@ -605,6 +615,7 @@ __global__ void __launch_bounds__(256) k_beam_write(CellView cells, int64_t ncel
 // nq: 16-byte words of one tile's records
 __global__ void __launch_bounds__(256) k_beam_gather(RecView in, RecView out, CellView sel, const uint64_t *src_rbeg,
                                                      int64_t ncells, int64_t ntiles, int nq) {
+    grid_start();
     const int64_t t = (blockIdx.x * 256ll + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (t >= ntiles) return;
@@ -637,6 +648,7 @@ __global__ void __launch_bounds__(256) k_beam_gather(RecView in, RecView out, Ce
 // is raised here.  W: child slots per load (2 or 4).
 template <int W>
 __global__ void __launch_bounds__(256) k_tile_scan(const __grid_constant__ Chunk c) {
+    grid_start();
     const int lane = threadIdx.x & 31;
     const int64_t nt = chunk_tiles(c);
     const int64_t t = (blockIdx.x * 8ll + (threadIdx.x >> 5)) * 32 + lane;
@@ -712,6 +724,7 @@ __global__ void __launch_bounds__(256) k_tile_scan(const __grid_constant__ Chunk
 
 // The same with multiplicities (grouping): a warp per tile.
 __global__ void __launch_bounds__(256) k_tile_scan_weighted(const __grid_constant__ Chunk c) {
+    grid_start();
     const int lane = threadIdx.x & 31;
     const int64_t nt = chunk_tiles(c);
     const int64_t t = blockIdx.x * 8ll + (threadIdx.x >> 5);
@@ -741,6 +754,7 @@ __global__ void __launch_bounds__(256) k_tile_scan_weighted(const __grid_constan
 template <int FAM>
 __global__ void k_path_geo(Problem P, const Level *levs, int lam, uint64_t key, const Scalars *sc,
                            PathStep *path) {
+    grid_start();
     using F = Fam<FAM>;
     int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= lam) return;
@@ -762,6 +776,7 @@ __global__ void __launch_bounds__(256) k_replay(Problem P, const Level *levs,
                                                const PathStep *path, int lam,
                                                const double *prm, int64_t n, uint32_t *reach,
                                                Scalars *sc) {
+    grid_start();
     using F = Fam<FAM>;
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int lane = threadIdx.x & 31;
@@ -949,7 +964,7 @@ static inline unsigned blocks_for(int64_t n, int bs) { return (unsigned)((n + bs
 void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t n, RecView out, CellView root,
                  Scalars *sc, cudaStream_t st) {
     if (n <= 0) return;
-    GV_DISPATCH(P.fam, (k_lift<FAMV><<<blocks_for(n, 256), 256, 0, st>>>(P, lev0, prm, n, out, root, sc)));
+    GV_DISPATCH(P.fam, (launch(k_lift<FAMV>, blocks_for(n, 256), 256, 0, st, P, lev0, prm, n, out, root, sc)));
 }
 
 void launch_sincos_table(const Problem &P, int j, double2 *tab, cudaStream_t st) {
@@ -962,12 +977,12 @@ int launch_prep(const Chunk &c, cudaStream_t st) {
     const int64_t geo = (int64_t)c.nc << (c.geo64 ? c.kf : c.kg);
     if (c.rot_ch) {                                  // rotation families only
         const unsigned g = blocks_for((int64_t)c.nc << c.kg, 256);
-        if (c.P.fam == FAM_POSE6DOF) k_rot_fill<FAM_POSE6DOF><<<g, 256, 0, st>>>(c);
-        else k_rot_fill<FAM_RADIAL5DOF><<<g, 256, 0, st>>>(c);
+        if (c.P.fam == FAM_POSE6DOF) launch(k_rot_fill<FAM_POSE6DOF>, g, 256, 0, st, c);
+        else launch(k_rot_fill<FAM_RADIAL5DOF>, g, 256, 0, st, c);
         n = 2;
     }
     const int64_t nt = c.t1 - c.t0 + 2, g = nt > geo ? nt : geo;
-    GV_DISPATCH(c.P.fam, (k_prep<FAMV><<<blocks_for(g, 256), 256, 0, st>>>(c)));
+    GV_DISPATCH(c.P.fam, (launch(k_prep<FAMV>, blocks_for(g, 256), 256, 0, st, c)));
     return n;
 }
 
@@ -1003,25 +1018,28 @@ void launch_persistent(const void *kern, size_t smem, int64_t groups, const Chun
     int64_t g = (int64_t)sm_count() * per_sm;
     if (g > groups) g = groups;
     void *args[] = {(void *)&c};
-    cudaLaunchKernel(kern, dim3((unsigned)g), dim3(256), args, smem, st);
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = launch_config((unsigned)g, 256, smem, st, &attr);
+    cudaLaunchKernelExC(&cfg, kern, args);
 }
 
 void launch_tile_scan(const Chunk &c, cudaStream_t st) {
     const int64_t nt = c.t1 - c.t0;
     if (nt <= 0) return;
-    if (c.in.mult) k_tile_scan_weighted<<<blocks_for(nt, 8), 256, 0, st>>>(c);
-    else if (c.ns == 2) k_tile_scan<2><<<blocks_for(nt, 256), 256, 0, st>>>(c);
-    else k_tile_scan<4><<<blocks_for(nt, 256), 256, 0, st>>>(c);
+    if (c.in.mult) launch(k_tile_scan_weighted, blocks_for(nt, 8), 256, 0, st, c);
+    else if (c.ns == 2) launch(k_tile_scan<2>, blocks_for(nt, 256), 256, 0, st, c);
+    else launch(k_tile_scan<4>, blocks_for(nt, 256), 256, 0, st, c);
 }
 
 __global__ void k_chain_start(LevInfo *info, long long cells, long long recs) {
+    grid_start();
     info->ncells = cells;
     info->nrecs = recs;
     info->overflow = 0;
 }
 
 void launch_chain_start(LevInfo *info, int64_t cells, int64_t recs, cudaStream_t st) {
-    k_chain_start<<<1, 1, 0, st>>>(info, cells, recs);
+    launch(k_chain_start, 1, 1, 0, st, info, cells, recs);
 }
 
 // blocks up to which k_child_write adds up the block totals itself (each block reads all
@@ -1034,21 +1052,21 @@ int launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsig
     if (n <= 0) return 0;
     unsigned nb = blocks_for(n, 256);
     unsigned long long *ba = bsums, *bb = bsums + nb;
-    k_child_mark<<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb);
+    launch(k_child_mark, nb, 256, 0, st, c, keepflag, recn, ba, bb);
     if (c.lev.leaf_children) return 1;
     if (!c.dyn && nb > kSelfScan) {
-        k_scan_sums<<<1, 256, 0, st>>>(ba, bb, (int)nb, c.sc);
-        k_child_write<<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb, 1);
+        launch(k_scan_sums, 1, 256, 0, st, ba, bb, (int)nb, c.sc);
+        launch(k_child_write, nb, 256, 0, st, c, keepflag, recn, ba, bb, 1);
         return 3;
     }
-    k_child_write<<<nb, 256, 0, st>>>(c, keepflag, recn, ba, bb, 0);
+    launch(k_child_write, nb, 256, 0, st, c, keepflag, recn, ba, bb, 0);
     return 2;
 }
 
 void launch_child_write(const Chunk &c, const uint32_t *keepflag, const uint32_t *recn, unsigned long long *bsums,
                         unsigned stride, cudaStream_t st) {
     const unsigned nb = blocks_for((int64_t)c.nc << c.lns, 256);
-    k_child_write<<<nb, 256, 0, st>>>(c, keepflag, recn, bsums, bsums + stride, 0);
+    launch(k_child_write, nb, 256, 0, st, c, keepflag, recn, bsums, bsums + stride, 0);
 }
 
 void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, int nk, BeamSel *sel,
@@ -1056,17 +1074,17 @@ void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells,
                         cudaStream_t st) {
     const unsigned nb = blocks_for(ncells, 256);
     unsigned long long *ba = bsums, *bb = bsums + nb;
-    k_beam_hist<<<nb < 1024u ? nb : 1024u, 256, 0, st>>>(cells, ncells, sel, nk, P, sc);
-    k_beam_pick<<<1, 256, 0, st>>>(sel, (unsigned long long)budget / nk);
-    k_beam_mark<<<nb, 256, 0, st>>>(cells, ncells, sel, nk, P, sc, ba, bb);
-    k_scan_sums<<<1, 256, 0, st>>>(ba, bb, (int)nb, sc);
-    k_beam_write<<<nb, 256, 0, st>>>(cells, ncells, sel, nk, P, sc, ba, bb, out, src_rbeg);
+    launch(k_beam_hist, nb < 1024u ? nb : 1024u, 256, 0, st, cells, ncells, sel, nk, P, sc);
+    launch(k_beam_pick, 1, 256, 0, st, sel, (unsigned long long)budget / nk);
+    launch(k_beam_mark, nb, 256, 0, st, cells, ncells, sel, nk, P, sc, ba, bb);
+    launch(k_scan_sums, 1, 256, 0, st, ba, bb, (int)nb, sc);
+    launch(k_beam_write, nb, 256, 0, st, cells, ncells, sel, nk, P, sc, ba, bb, out, src_rbeg);
 }
 
 void launch_beam_gather(const RecView &in, const RecView &out, const CellView &sel, const uint64_t *src_rbeg,
                         int64_t ncells, int64_t ntiles, int rec_bytes, cudaStream_t st) {
     if (ntiles > 0)
-        k_beam_gather<<<blocks_for(ntiles * 32, 256), 256, 0, st>>>(in, out, sel, src_rbeg, ncells, ntiles,
+        launch(k_beam_gather, blocks_for(ntiles * 32, 256), 256, 0, st, in, out, sel, src_rbeg, ncells, ntiles,
                                                                     32 * rec_bytes / 16);
 }
 
@@ -1093,13 +1111,13 @@ void launch_group(const Chunk &c, uint32_t *table, uint32_t tmask, uint32_t *own
 void launch_path_geo(const Problem &P, const Level *levs_dev, int lam, uint64_t key, const Scalars *sc, PathStep *path,
                      cudaStream_t st) {
     if (lam <= 0) return;
-    GV_DISPATCH(P.fam, (k_path_geo<FAMV><<<blocks_for(lam, 64), 64, 0, st>>>(P, levs_dev, lam, key, sc, path)));
+    GV_DISPATCH(P.fam, (launch(k_path_geo<FAMV>, blocks_for(lam, 64), 64, 0, st, P, levs_dev, lam, key, sc, path)));
 }
 
 void launch_replay(const Problem &P, const Level *levs_dev, const PathStep *path, int lam, const double *prm,
                    int64_t n, uint32_t *reach, Scalars *sc, cudaStream_t st) {
     if (n <= 0) return;
-    GV_DISPATCH(P.fam, (k_replay<FAMV><<<blocks_for(n, 256), 256, 0, st>>>(P, levs_dev, path, lam, prm, n,
+    GV_DISPATCH(P.fam, (launch(k_replay<FAMV>, blocks_for(n, 256), 256, 0, st, P, levs_dev, path, lam, prm, n,
                                                                             reach, sc)));
 }
 

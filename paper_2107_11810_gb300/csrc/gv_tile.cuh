@@ -541,8 +541,8 @@ __device__ __noinline__ int3 snap_df_words(const Chunk *c, RecWords<rec_words(Fa
             const int b = F::cb(j, m);
             float dh, dl;
             if (b < F::NBG) {
-                dh = __ldg(c->geo32 + (size_t)cell * c->gf + b * c->ng + r);
-                dl = __ldg(c->geo32lo + ((size_t)cell * F::NBG + b) * c->ng + r);
+                dh = c->geo32[(size_t)cell * c->gf + b * c->ng + r];
+                dl = c->geo32lo[((size_t)cell * F::NBG + b) * c->ng + r];
             } else {
                 dh = lin_change<FAM>(*c, b, fs, false);
                 dl = lin_change<FAM>(*c, b, fs, true);

@@ -27,10 +27,10 @@ __device__ __forceinline__ void stage_coefs(const Chunk &c, int cell, float *sg,
         for (int m = 0; m < F::LE; ++m) {
             if (!F::uses(j, m)) continue;
             const int b = F::cb(j, m), x = j * F::LE + m;
-            const float d = b < F::NBG ? __ldg(geo + b * c.ng + (f & (c.ng - 1))) : lin_change<FAM>(c, b, f, false);
+            const float d = b < F::NBG ? geo[b * c.ng + (f & (c.ng - 1))] : lin_change<FAM>(c, b, f, false);
             if (lane < c.nfs) sg[x * c.nfs + f] = coef32<FAM>(c.lev, j, m, d);
             if constexpr (MAX) {
-                const float g = b < F::NBG ? __ldg(geo + F::NBG * c.ng + b) : fabsf(d);
+                const float g = b < F::NBG ? geo[F::NBG * c.ng + b] : fabsf(d);
                 if (lane == 0) sg[F::ND * F::LE * c.nfs + x] = g * c.lev.gs[j][m];
             }
         }
@@ -39,6 +39,7 @@ __device__ __forceinline__ void stage_coefs(const Chunk &c, int cell, float *sg,
 // FG: free slots per group (4, or all of them when fewer split)
 template <int FAM, bool Q16, int FG, int DM, bool LB>
 __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chunk c) {
+    grid_start();
     using F = Fam<FAM>;
     constexpr int ND = F::ND, LE = F::LE, NDS = dep_slots(DM), NX = ND * LE;
     constexpr int NW = rec_words(F::NFP, Q16);
@@ -157,6 +158,7 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
 // child.
 template <int FAM, bool QI16, bool QO16>
 __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk c) {
+    grid_start();
     using F = Fam<FAM>;
     constexpr int NDS = 1 << F::ND, ND = F::ND, LE = F::LE, NFP = F::NFP;
     static_assert(F::D <= 6 && ND <= 2, "at most 64 child slots, two dependent coordinates");
@@ -369,8 +371,8 @@ template <int FAM, bool Q16, int FG, int DM>
 static void launch_wide(const Chunk &c, cudaStream_t st) {
     if constexpr (DM < (1 << Fam<FAM>::ND) && (FG > 1 || DM)) {
         const unsigned g = wide_blocks(c.t1 - c.t0);
-        if (c.lb) k_count_wide<FAM, Q16, FG, DM, true><<<g, 256, 0, st>>>(c);
-        else k_count_wide<FAM, Q16, FG, DM, false><<<g, 256, 0, st>>>(c);
+        if (c.lb) launch(k_count_wide<FAM, Q16, FG, DM, true>, g, 256, 0, st, c);
+        else launch(k_count_wide<FAM, Q16, FG, DM, false>, g, 256, 0, st, c);
     }
 }
 
@@ -408,11 +410,11 @@ bool launch_emit_wide(const Chunk &c, cudaStream_t st) {
     if (!known) return false;
     if (c.precision == 0 && (q || qn)) return false;    // plain FP64 mode keeps 32-bit records
     if (q && qn) {
-        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, true, true><<<g, 256, 0, st>>>(c)));
+        GV_DISPATCH_WIDE(c.P.fam, (launch(k_emit_wide<FAMV, true, true>, g, 256, 0, st, c)));
     } else if (!q && qn) {
-        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, false, true><<<g, 256, 0, st>>>(c)));
+        GV_DISPATCH_WIDE(c.P.fam, (launch(k_emit_wide<FAMV, false, true>, g, 256, 0, st, c)));
     } else if (!q && !qn) {
-        GV_DISPATCH_WIDE(c.P.fam, (k_emit_wide<FAMV, false, false><<<g, 256, 0, st>>>(c)));
+        GV_DISPATCH_WIDE(c.P.fam, (launch(k_emit_wide<FAMV, false, false>, g, 256, 0, st, c)));
     } else {
         return false;                                   // 16-bit to 32-bit: never chosen
     }
