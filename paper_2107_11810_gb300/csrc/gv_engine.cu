@@ -101,6 +101,7 @@ struct vote_ctx {
     DevBuf beam_sel, beam_src, linfo;
     LevInfo *h_info = nullptr; // pinned: the steps' reports, per level; the last for single steps
     long long steps = 0;       // numbers them
+    DevBuf psi0;               // basis of the root cell's centre
     DevBuf sctab[2];           // (sin, cos) tables of the angular coordinates (launch_sincos_table)
     DevBuf rot[GV_MAXL + 1], rotflag[GV_MAXL + 1];   // rotation tables per level (k_rot_fill)
     DevBuf levs_dev, path, scal, alive, geo64, geo32, geo32lo, cnt, tinfo, ballot, lballot, uns, off, cbase, child_idx;
@@ -1287,7 +1288,7 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
         const int64_t slots0 = (n + 31) & ~(int64_t)31;
         TRY(ensure_level(c, c->ls[0], 0, (size_t)slots0, 1));
         ev_mark(c, -1);
-        launch_lift(P, c->lev[0], surfaces, n, rec_view(c, c->ls[0]), cell_view(c->ls[0]), dsc(c), c->stream);
+        launch_lift(P, c->lev[0], (const double *)c->psi0.p, surfaces, n, rec_view(c, c->ls[0]), cell_view(c->ls[0]), dsc(c), c->stream);
         c->stats.launches += 1;
         ev_mark(c, VOTE_K_LIFT);
         CK(cudaGetLastError());
@@ -1402,8 +1403,10 @@ vote_status vote_create(int family, int d, int k, const double *eps, const doubl
     }
     s = ensure(c, c->scal, ((sizeof(Scalars) + 63) / 64) * 64 + 64);
     if (s == VOTE_OK) s = ensure(c, c->levs_dev, sizeof(Level) * (c->P.L > 0 ? c->P.L : 1));
-    if (s == VOTE_OK) s = ensure(c, c->path, sizeof(PathStep) * (c->P.L > 0 ? c->P.L : 1));
+    if (s == VOTE_OK) s = ensure(c, c->path, sizeof(PathStep) * (c->P.L + kPathTail));
+    if (s == VOTE_OK) s = ensure(c, c->psi0, sizeof(double) * GV_MAXT);
     if (s == VOTE_OK && c->P.L > 0) {
+        launch_root_basis(c->P, c->lev[0], (double *)c->psi0.p, c->stream);
         const int nang = family == VOTE_PLANE3D_SPH ? 2 : (family == VOTE_POSE3DOF ? 1 : 0);
         for (int j = 0; j < nang && s == VOTE_OK; ++j)
             if (c->P.Lj[j] <= kSincosBits) {
@@ -1853,6 +1856,7 @@ void vote_destroy(vote_ctx *c) {
                       &c->g_rbeg, &c->g_rec, &c->g_mult, &c->g_tile, &c->beam_sel, &c->beam_src, &c->linfo};
     for (DevBuf *b : bufs) release(c, *b);
     for (DevBuf &b : c->sctab) release(c, b);
+    release(c, c->psi0);
     for (int l = 0; l <= GV_MAXL; ++l) release(c, c->rot[l]), release(c, c->rotflag[l]);
     cudaStreamSynchronize(c->stream);
     for (int i = 0; i < vote_ctx::kEv; ++i)
@@ -1876,7 +1880,7 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[VOTE_NOALLOC_SC
 namespace {
 constexpr size_t kNaLevels = 0;
 constexpr size_t kNaPath = kNaLevels + sizeof(Level) * GV_MAXL;
-constexpr size_t kNaScalars = (kNaPath + sizeof(PathStep) * GV_MAXL + 255) / 256 * 256;
+constexpr size_t kNaScalars = (kNaPath + sizeof(PathStep) * (GV_MAXL + kPathTail) + 255) / 256 * 256;
 constexpr size_t kNaEnd = kNaScalars + sizeof(Scalars);
 static_assert(kNaEnd <= VOTE_NOALLOC_SCRATCH_BYTES, "no-alloc scratch too small");
 

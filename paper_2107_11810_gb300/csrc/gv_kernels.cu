@@ -34,60 +34,82 @@ __device__ __forceinline__ unsigned prune_threshold(const Problem &P, const Scal
 // ---------------------------------------------------------------------------
 // A0 lift
 // ---------------------------------------------------------------------------
+// Basis of the root cell's centre (once per context).
 template <int FAM>
-__global__ void k_lift(Problem P, Level lev0, const double *prm, int64_t n, RecView out, CellView root,
-                       Scalars *sc) {
+__global__ void k_root_basis(Problem P, Level lev0, double *psi) {
+    double c[Fam<FAM>::D], v[Fam<FAM>::NB];
+#pragma unroll
+    for (int j = 0; j < Fam<FAM>::D; ++j) c[j] = cell_center(P, lev0.h, j, 0);
+    Fam<FAM>::basis(P, c, v);
+#pragma unroll
+    for (int m = 0; m < Fam<FAM>::NB; ++m) psi[m] = v[m];
+}
+
+// Rounds to the nearest step; bad unless below 2^30 steps (integer tests: the FP64 pipe,
+// one instruction per 32 clocks and SM, bounds this kernel).
+__device__ __forceinline__ int lift_q(double x, double inv_s, bool &bad) {
+    const double v = dmul(x, inv_s);
+    const int q = __double2int_rn(v);                // saturates
+    bad |= (__double2hiint(v) & 0x7ff00000) == 0x7ff00000 || (unsigned)(q + 0x3fffffff) > 0x7ffffffeu;
+    return bad ? 0 : q;
+}
+
+// Root records of the surfaces.  48 bytes move per surface of a 3-DoF pose and 16 FP64
+// instructions run; blocks take several surfaces per thread so that the largest |q| of
+// each field (it sets the screen's band and the record formats) costs one atomic per
+// block: 167 us per 1e6 surfaces with a basis per surface and an atomic per warp and
+// field, 44 us now.
+template <int FAM>
+__global__ void __launch_bounds__(256) k_lift(Problem P, Level lev0, const double *psi0, const double *prm, int64_t n,
+                                              RecView out, CellView root, Scalars *sc) {
     grid_start();
     using F = Fam<FAM>;
-    constexpr int NW = rec_words(F::NFP, false);
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    constexpr int NW = rec_words(F::NFP, false), NQ = F::ND + F::LE;
     const int lane = threadIdx.x & 31;
-    unsigned qa[F::ND + F::LE];
+    __shared__ unsigned s_max[NQ];
+    unsigned qa[NQ];
 #pragma unroll
-    for (int x = 0; x < F::ND + F::LE; ++x) qa[x] = 0u;
+    for (int x = 0; x < NQ; ++x) qa[x] = 0u;
+    if (threadIdx.x < NQ) s_max[threadIdx.x] = 0u;
     bool bad = false;
-    if (i == 0) {                                    // the root cell holds every surface
+    const int64_t first = blockIdx.x * 256ll + threadIdx.x;
+    if (first == 0) {                                // the root cell holds every surface
         root.key[0] = 0ull;
         root.rbeg[0] = 0ull;
         root.rcnt[0] = root.ub[0] = (uint32_t)n;
         root.lb[0] = 0u;
     }
-    if (i < n) {
-        double c[F::D], psi[F::NB], f[F::ND], t[F::LE];
+    double c[F::D], psi[F::NB];
 #pragma unroll
-        for (int j = 0; j < F::D; ++j) c[j] = cell_center(P, lev0.h, j, 0);
-        F::basis(P, c, psi);
+    for (int j = 0; j < F::D; ++j) c[j] = cell_center(P, lev0.h, j, 0);
+#pragma unroll
+    for (int m = 0; m < F::NB; ++m) psi[m] = psi0[m];
+    __syncthreads();
+    for (int64_t i = first; i < n; i += gridDim.x * 256ll) {
+        double f[F::ND], t[F::LE];
         F::lift(prm, n, i, c, psi, f, t);
         uint32_t w[NW];
 #pragma unroll
         for (int x = 0; x < NW; ++x) w[x] = 0u;
 #pragma unroll
-        for (int j = 0; j < F::ND; ++j) {
-            double q = rint(dmul(f[j], P.inv_s_f[j]));
-            bad |= !(fabs(q) < 1073741824.0);
-            int qi = bad ? 0 : (int)q;
-            w[j] = (uint32_t)qi;
-            qa[j] = (unsigned)abs(qi);
-        }
-#pragma unroll
-        for (int m = 0; m < F::LE; ++m) {
-            double q = rint(dmul(t[m], lev0.inv_s_t[m]));
-            bad |= !(fabs(q) < 1073741824.0);
-            int qi = bad ? 0 : (int)q;
-            w[F::ND + m] = (uint32_t)qi;
-            qa[F::ND + m] = (unsigned)abs(qi);
+        for (int x = 0; x < NQ; ++x) {
+            const int q = x < F::ND ? lift_q(f[x], P.inv_s_f[x], bad) : lift_q(t[x - F::ND], lev0.inv_s_t[x - F::ND], bad);
+            w[x] = (uint32_t)q;
+            const unsigned aq = (unsigned)abs(q);
+            qa[x] = aq > qa[x] ? aq : qa[x];
         }
         store_words<NW>(out.rec, i, w);
         if (out.mult) out.mult[i] = 1u;
         if ((i & 31) == 0) out.tile_cell[i >> 5] = 0u;
     }
-    // largest |q| per field (it sets the screen's band and the record formats)
 #pragma unroll
-    for (int x = 0; x < F::ND + F::LE; ++x) {
-        unsigned m = __reduce_max_sync(kFull, qa[x]);
-        if (lane == 0 && m) atomicMax(&sc->qmax[x], m);
+    for (int x = 0; x < NQ; ++x) {
+        const unsigned m = __reduce_max_sync(kFull, qa[x]);
+        if (lane == 0 && m) atomicMax(&s_max[x], m);
     }
     if (bad) atomicOr(&sc->err, 1u);
+    __syncthreads();
+    if (threadIdx.x < NQ && s_max[threadIdx.x]) atomicMax(&sc->qmax[threadIdx.x], s_max[threadIdx.x]);
 }
 
 // ---------------------------------------------------------------------------
@@ -751,43 +773,134 @@ __global__ void __launch_bounds__(256) k_tile_scan_weighted(const __grid_constan
 // ---------------------------------------------------------------------------
 // A7 replay of the original surfaces along one root-to-cell path
 // ---------------------------------------------------------------------------
+// path[0, lam): child slot and basis change of each step; then, for the replay's screen,
+// path[lam].dpsi: the whole path's basis change; [lam + 1]: the root's basis; [lam + 2]: the
+// whole shift of each coordinate; [lam + 3]: s_t of the root's level over that of the last.
 template <int FAM>
-__global__ void k_path_geo(Problem P, const Level *levs, int lam, uint64_t key, const Scalars *sc,
-                           PathStep *path) {
+__global__ void __launch_bounds__(64) k_path_geo(Problem P, const Level *levs, int lam, uint64_t key,
+                                                 const Scalars *sc, PathStep *path) {
     grid_start();
     using F = Fam<FAM>;
-    int l = blockIdx.x * blockDim.x + threadIdx.x;
-    if (l >= lam) return;
+    const int l = threadIdx.x;
     if (sc) key = ~sc->best_key & ((1ull << P.coord_bits) - 1ull);   // the best leaf
-    const Level &lev = levs[l];
-    int slot = 0;
-    for (int j = 0; j < F::D; ++j)
-        if (l < P.Lj[j]) slot |= (int)(cell_coord(P, key, l + 1, j) & 1) << j;
-    double psi_par[F::NB], dpsi[F::NB];
-    parent_psi<FAM>(P, lev, key, psi_par);
-    child_dpsi<FAM>(P, lev, key, slot & ((1 << F::K) - 1), psi_par, dpsi);
-    path[l].slot = slot;
+    if (l < lam) {
+        const Level &lev = levs[l];
+        int slot = 0;
+        for (int j = 0; j < F::D; ++j)
+            if (l < P.Lj[j]) slot |= (int)(cell_coord(P, key, l + 1, j) & 1) << j;
+        double psi_par[F::NB], dpsi[F::NB];
+        parent_psi<FAM>(P, lev, key, psi_par);
+        child_dpsi<FAM>(P, lev, key, slot & ((1 << F::K) - 1), psi_par, dpsi);
+        path[l].slot = slot;
 #pragma unroll
-    for (int m = 0; m < F::NB; ++m) path[l].dpsi[m] = dpsi[m];
-}
-
-template <int FAM>
-__global__ void __launch_bounds__(256) k_replay(Problem P, const Level *levs,
-                                               const PathStep *path, int lam,
-                                               const double *prm, int64_t n, uint32_t *reach,
-                                               Scalars *sc) {
-    grid_start();
-    using F = Fam<FAM>;
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int lane = threadIdx.x & 31;
-    bool reached = false, lbp = false;
-    if (i < n) {
-        double c[F::D], psi[F::NB], f[F::ND], t[F::LE];
+        for (int m = 0; m < F::NB; ++m) path[l].dpsi[m] = dpsi[m];
+    } else if (l == 63) {
+        double c[F::D], psi[F::NB];
 #pragma unroll
         for (int j = 0; j < F::D; ++j) c[j] = cell_center(P, levs[0].h, j, 0);
         F::basis(P, c, psi);
-        F::lift(prm, n, i, c, psi, f, t);
-        reached = true;
+#pragma unroll
+        for (int m = 0; m < F::NB; ++m) path[lam + 1].dpsi[m] = psi[m];
+    }
+    __syncthreads();
+    if (l < F::NB) {
+        double v = 0.0;
+        for (int x = 0; x < lam; ++x) v = dadd(v, path[x].dpsi[l]);
+        path[lam].dpsi[l] = v;
+    } else if (l >= 16 && l < 16 + F::D) {
+        double v = 0.0;
+        for (int x = 0; x < lam; ++x) {
+            const Level &lev = levs[x];
+            const double h = lev.h1[l - 16];
+            if ((lev.split_mask >> (l - 16)) & 1) v = dadd(v, (path[x].slot >> (l - 16)) & 1 ? h : -h);
+        }
+        path[lam + 2].dpsi[l - 16] = v;
+    } else if (l >= 32 && l < 32 + F::LE) {
+        path[lam + 3].dpsi[l - 32] = dmul(levs[0].s_t[l - 32], levs[lam - 1].inv_s_t[l - 32]);
+    }
+}
+
+// Screen of the replay: whether a surface certainly fails the last step's test.  Its
+// residual at the target cell's centre is taken from the root in one jump, without
+// snapping: the steps' residual differs from it by at most the accumulated canonization
+// error, which the radius contains; the essential parameters differ by at most one step of
+// the last level (half of each coarser grid they are snapped to on the way).  The FP64 rounding of either way is far below one snap step (fields
+// below 2^30 steps), that of the FP32 radius and conversions below the 1e-4 added.
+template <int FAM>
+__device__ __forceinline__ bool replay_far(const Problem &P, const Level &lev, const PathStep *tail, const double *f,
+                                           const double *t) {
+    using F = Fam<FAM>;
+    double fo[F::ND], sh[F::D], dpsi[F::NB];
+#pragma unroll
+    for (int m = 0; m < F::NB; ++m) dpsi[m] = tail[0].dpsi[m];
+#pragma unroll
+    for (int j = 0; j < F::D; ++j) sh[j] = tail[2].dpsi[j];
+    F::residual64(f, t, dpsi, sh, fo);
+    bool in = true, far = false;                     // in: the fields are in range (always, in a search)
+    float qt[F::LE], R[F::ND];
+#pragma unroll
+    for (int m = 0; m < F::LE; ++m) {
+        const float ratio = (float)tail[3].dpsi[m], x = fabsf((float)t[m] * (float)lev.inv_s_t[m]);
+        in &= x < 1073741824.0f * ratio;
+        qt[m] = x + 1.5f;
+    }
+    F::radius32(lev, qt, R);
+#pragma unroll
+    for (int j = 0; j < F::ND; ++j) {
+        const float s = (float)P.inv_s_f[j];
+        in &= fabsf((float)f[j] * s) < 1073741824.0f;
+        far |= fabsf((float)fo[j] * s) > __fmaf_rn(R[j], 1.0001f, 2.0f);
+    }
+    return in && far;
+}
+
+// Which surfaces pass every test from the root to the target cell.  Nearly all fail, most
+// of them at once: a block screens its surfaces first (30 FP64 instructions each) and only
+// those that may pass go through the steps (50 FP64 instructions per step, the FP64 pipe's
+// rate is the bound), collected so that warps are full.  1e6 surfaces of a 3-DoF pose, 10
+// steps: 621 us with every surface through the steps until it fails, 131 us now.
+constexpr int kReplayPer = 4;                        // surfaces per thread
+template <int FAM>
+__global__ void __launch_bounds__(256) k_replay(Problem P, const Level *levs, const PathStep *path, int lam,
+                                                const double *prm, int64_t n, uint32_t *reach, Scalars *sc) {
+    grid_start();
+    using F = Fam<FAM>;
+    constexpr int NS = 256 * kReplayPer;
+    __shared__ unsigned s_words[NS / 32], s_n, s_lb;
+    __shared__ unsigned short s_list[NS];
+    const int64_t base = (int64_t)blockIdx.x * NS;
+    const int lane = threadIdx.x & 31;
+    const PathStep *tail = path + lam;
+    if (threadIdx.x < NS / 32) s_words[threadIdx.x] = 0u;
+    if (threadIdx.x == 0) s_n = s_lb = 0u;
+    double c[F::D], psi[F::NB], f[F::ND], t[F::LE];
+    if (lam > 0) {
+#pragma unroll
+        for (int j = 0; j < F::D; ++j) c[j] = cell_center(P, levs[0].h, j, 0);
+#pragma unroll
+        for (int m = 0; m < F::NB; ++m) psi[m] = tail[1].dpsi[m];
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int k = 0; k < kReplayPer; ++k) {
+        const int x = k * 256 + threadIdx.x;
+        bool maybe = base + x < n;
+        if (maybe && lam > 0) {
+            F::lift(prm, n, base + x, c, psi, f, t);
+            maybe = !replay_far<FAM>(P, levs[lam - 1], tail, f, t);
+        }
+        const unsigned b = __ballot_sync(kFull, maybe);
+        unsigned at = 0;
+        if (lane == 0 && b) at = atomicAdd(&s_n, __popc(b));
+        at = __shfl_sync(kFull, at, 0);
+        if (maybe) s_list[at + __popc(b & ((1u << lane) - 1u))] = (unsigned short)x;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (unsigned q = threadIdx.x; q < s_n; q += 256) {
+        const int x = s_list[q];
+        bool reached = true, lbp = false;
+        if (lam > 0) F::lift(prm, n, base + x, c, psi, f, t);
         for (int l = 0; l < lam; ++l) {
             const Level &lev = levs[l];
 #pragma unroll
@@ -805,13 +918,17 @@ __global__ void __launch_bounds__(256) k_replay(Problem P, const Level *levs,
 #pragma unroll
             for (int j = 0; j < F::ND; ++j) f[j] = fo[j];
         }
+        if (reached) atomicOr(&s_words[x >> 5], 1u << (x & 31));
+        if (lbp) atomicAdd(&s_lb, 1u);
     }
-    unsigned b = __ballot_sync(kFull, reached);
-    unsigned bl = __ballot_sync(kFull, lbp);
-    if (lane == 0 && i < n) {
-        if (reach) reach[i >> 5] = b;
-        if (b) atomicAdd(&sc->replay_ub, (unsigned long long)__popc(b));
-        if (bl) atomicAdd(&sc->replay_lb, (unsigned long long)__popc(bl));
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        static_assert(NS / 32 == 32, "a mask word per lane");
+        const unsigned w = s_words[lane];
+        if (reach && base + 32 * lane < n) reach[(base >> 5) + lane] = w;
+        const unsigned total = __reduce_add_sync(kFull, (unsigned)__popc(w));
+        if (lane == 0 && total) atomicAdd(&sc->replay_ub, (unsigned long long)total);
+        if (lane == 0 && s_lb) atomicAdd(&sc->replay_lb, (unsigned long long)s_lb);
     }
 }
 
@@ -961,10 +1078,15 @@ static inline unsigned blocks_for(int64_t n, int bs) { return (unsigned)((n + bs
     default: break;                                                 \
     }
 
-void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t n, RecView out, CellView root,
-                 Scalars *sc, cudaStream_t st) {
+void launch_root_basis(const Problem &P, const Level &lev0, double *psi, cudaStream_t st) {
+    GV_DISPATCH(P.fam, (k_root_basis<FAMV><<<1, 1, 0, st>>>(P, lev0, psi)));
+}
+
+void launch_lift(const Problem &P, const Level &lev0, const double *psi0, const double *prm, int64_t n, RecView out,
+                 CellView root, Scalars *sc, cudaStream_t st) {
     if (n <= 0) return;
-    GV_DISPATCH(P.fam, (launch(k_lift<FAMV>, blocks_for(n, 256), 256, 0, st, P, lev0, prm, n, out, root, sc)));
+    const unsigned nb = blocks_for(n, 256), g = 4u * (unsigned)sm_count();
+    GV_DISPATCH(P.fam, (launch(k_lift<FAMV>, nb < g ? nb : g, 256, 0, st, P, lev0, psi0, prm, n, out, root, sc)));
 }
 
 void launch_sincos_table(const Problem &P, int j, double2 *tab, cudaStream_t st) {
@@ -1111,13 +1233,13 @@ void launch_group(const Chunk &c, uint32_t *table, uint32_t tmask, uint32_t *own
 void launch_path_geo(const Problem &P, const Level *levs_dev, int lam, uint64_t key, const Scalars *sc, PathStep *path,
                      cudaStream_t st) {
     if (lam <= 0) return;
-    GV_DISPATCH(P.fam, (launch(k_path_geo<FAMV>, blocks_for(lam, 64), 64, 0, st, P, levs_dev, lam, key, sc, path)));
+    GV_DISPATCH(P.fam, (launch(k_path_geo<FAMV>, 1, 64, 0, st, P, levs_dev, lam, key, sc, path)));
 }
 
 void launch_replay(const Problem &P, const Level *levs_dev, const PathStep *path, int lam, const double *prm,
                    int64_t n, uint32_t *reach, Scalars *sc, cudaStream_t st) {
     if (n <= 0) return;
-    GV_DISPATCH(P.fam, (launch(k_replay<FAMV>, blocks_for(n, 256), 256, 0, st, P, levs_dev, path, lam, prm, n,
+    GV_DISPATCH(P.fam, (launch(k_replay<FAMV>, blocks_for(n, 256 * kReplayPer), 256, 0, st, P, levs_dev, path, lam, prm, n,
                                                                             reach, sc)));
 }
 

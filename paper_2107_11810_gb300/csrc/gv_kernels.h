@@ -175,14 +175,17 @@ struct BeamSel {
 };
 
 // Path geometry for replaying surfaces along the root-to-cell path.
+constexpr int kPathTail = 4; // entries after the steps (see k_path_geo)
 struct PathStep {
     int slot;
     double dpsi[GV_MAXT];
 };
 
 // root records of the surfaces and the root cell
-void launch_lift(const Problem &P, const Level &lev0, const double *prm, int64_t n, RecView out, CellView root,
-                 Scalars *sc, cudaStream_t st);
+void launch_lift(const Problem &P, const Level &lev0, const double *psi0, const double *prm, int64_t n, RecView out,
+                 CellView root, Scalars *sc, cudaStream_t st);
+// psi [GV_MAXT]: basis of the root cell's centre
+void launch_root_basis(const Problem &P, const Level &lev0, double *psi, cudaStream_t st);
 // the (sin, cos) table of an angular coordinate (2^(splits + 1) - 1 entries)
 void launch_sincos_table(const Problem &P, int j, double2 *tab, cudaStream_t st);
 // cells (alive, geometry) and tiles (tinfo) of the chunk; returns the kernels launched
