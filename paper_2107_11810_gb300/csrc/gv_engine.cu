@@ -824,6 +824,10 @@ static bool wants_lb(const vote_ctx *c, int l, bool beam) {
     return c->trace_cap > 0 || (!c->lev[l].leaf_children && (beam || c->expanded < lb_records(c->P.d)));
 }
 
+// Up to these children a kernel of one block lays them out; above, two kernels do.  The
+// chain only knows a bound, mostly several times the real number.
+static const int64_t kSmallStep = 2048, kSmallChain = 8192;
+
 // Expand a chunk of level-l cells taken from the top of the level's stack, or, in the
 // dive, all cells of the beam store (a selection of level l).
 static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
@@ -916,9 +920,10 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     ev_mark(c, VOTE_K_CELL_GEO);
     launch_count(ch, c->stream);
     ev_mark(c, VOTE_K_TEST_COUNT);
+    const bool small = !grouping && (int64_t)nch <= kSmallStep;
     launch_tile_scan(ch, c->stream);
-    const int nchild = launch_child_alloc(ch, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
-                                          (unsigned long long *)c->bsums.p, c->stream);
+    const int nchild = launch_child_alloc(ch, small, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
+                                                      (unsigned long long *)c->bsums.p, c->stream);
     ev_mark(c, VOTE_K_CHILDREN);
     // algorithmic bytes: the records of whole tiles read, the ballots written
     c->kbytes[VOTE_K_TEST_COUNT] += (double)nt * 32 * rb + (double)nt * ns * 4;
@@ -1025,18 +1030,21 @@ static vote_status dive(vote_ctx *c, int l0) {
         const int64_t m = S.ncells;
         c->beam.ncells = c->beam.nrecs = 0;
         TRY(ensure_level(c, c->beam, l, 0, (size_t)m));
-        TRY(ensure(c, c->beam_sel, sizeof(BeamSel)));
+        if (!c->beam_sel.p) {
+            TRY(ensure(c, c->beam_sel, sizeof(BeamSel)));
+            CK(cudaMemsetAsync(c->beam_sel.p, 0, sizeof(BeamSel), c->stream));   // every selection leaves it cleared
+        }
         TRY(ensure(c, c->beam_src, (size_t)m * 8));
         TRY(ensure(c, c->bsums, (size_t)((m + 255) / 256) * 16 + 16));
-        CK(cudaMemsetAsync(c->beam_sel.p, 0, sizeof(BeamSel), c->stream));
-        launch_beam_select(c->P, cell_view(S), m, budget, c->P.d <= 3 ? 2 : 1, (BeamSel *)c->beam_sel.p, (unsigned long long *)c->bsums.p,
-                           cell_view(c->beam), (uint64_t *)c->beam_src.p, dsc(c), c->stream);
+        const LevInfo *v = c->h_info + GV_MAXL + 1;
+        const long long seq = ++c->steps;
+        c->stats.launches +=
+            launch_beam_select(c->P, cell_view(S), m, budget, c->P.d <= 3 ? 2 : 1, (BeamSel *)c->beam_sel.p,
+                               (unsigned long long *)c->bsums.p, cell_view(c->beam), (uint64_t *)c->beam_src.p, dsc(c),
+                               c->h_info + GV_MAXL + 1, seq, c->stream);
         CK(cudaGetLastError());
-        CK(cudaMemcpyAsync(&c->h_sc->n_cells, &dsc(c)->n_cells, 16, cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
-        ev_collect(c);
-        const int64_t nsel = (int64_t)c->h_sc->n_cells, rsel = (int64_t)c->h_sc->n_recs;
-        c->stats.launches += 5;
+        TRY(wait_report(c, v, seq));
+        const int64_t nsel = v->stored_cells, rsel = v->stored_recs;
         if (nsel <= 0) {                 // no cell reaches the bound any more (it never falls)
             S.ncells = S.nrecs = 0;
             return VOTE_OK;
@@ -1081,8 +1089,10 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
         TRY(ensure_tables(c, l, dims, &need64));
         // every cell holds at least a tile, and at most as many as the root
         int64_t cb = cells, tb = recs / 32;
+        const int64_t cmax = l ? std::min(pcells * pdims.ns, fit / 32) : 1;
+        const bool small = cmax * dims.ns <= kSmallChain;
         if (!known) {
-            cb = std::min(pcells * pdims.ns, fit / 32);
+            cb = cmax;
             tb = std::min(cb * (slots0 / 32), fit / 32);
             // the step before may still need the scratch that would grow
             TRY(ensure_scratch(c, dims, (size_t)cb, (size_t)tb, lb, need64, &fits));
@@ -1112,8 +1122,8 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
             const int nprep = launch_prep(ch, c->stream);
             launch_count(ch, c->stream);
             launch_tile_scan(ch, c->stream);
-            const int nchild = launch_child_alloc(ch, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
-                                                  (unsigned long long *)c->bsums.p, c->stream);
+            const int nchild = launch_child_alloc(ch, small, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
+                                                              (unsigned long long *)c->bsums.p, c->stream);
             if (l + 1 < L && !launch_emit(ch, c->stream)) {
                 set_err("internal: no emit pass for record formats %d -> %d", ch.lev.q16, ch.lev.q16_next);
                 return VOTE_EINTERNAL;
@@ -1131,7 +1141,6 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
             if (recs > c->stats.peak_records) c->stats.peak_records = recs;
             if (v->overflow) {
                 // its counts and ballots stand: make room, lay the children out, emit
-                const unsigned stride = (unsigned)(((int64_t)last.nc * last.ns + 255) / 256);   // of the block totals
                 LevelStore &N = c->ls[l];
                 N.ncells = N.nrecs = 0;
                 TRY(ensure_level(c, N, l, (size_t)recs, (size_t)cells));
@@ -1139,10 +1148,11 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
                 last.t1 = c->ls[l - 1].nrecs / 32;
                 last.dyn = nullptr;
                 last.host = nullptr;
+                last.trace.cap = 0;          // its children are in the trace
                 last.next_cells = cell_view(N);
                 last.out = rec_view(c, N);
-                launch_child_write(last, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
-                                   (unsigned long long *)c->bsums.p, stride, c->stream);
+                launch_child_alloc(last, false, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
+                                   (unsigned long long *)c->bsums.p, c->stream);
                 launch_emit(last, c->stream);
                 CK(cudaGetLastError());
                 N.ncells = cells;

@@ -10,8 +10,8 @@
 namespace gv {
 
 template <int FAM, bool Q16>
-__device__ __forceinline__ void eval_record(const Chunk &c, int64_t r, int cell, SlotMask<FAM> &ubm,
-                                            SlotMask<FAM> &lbm) {
+__device__ __forceinline__ void eval_record(const Chunk &c, int64_t r, int cell, int fs0, int fs1,
+                                            SlotMask<FAM> &ubm, SlotMask<FAM> &lbm) {
     using F = Fam<FAM>;
     constexpr int NW = rec_words(F::NFP, Q16);
     uint32_t w[NW];
@@ -21,29 +21,36 @@ __device__ __forceinline__ void eval_record(const Chunk &c, int64_t r, int cell,
     for (int j = 0; j < F::ND; ++j) qf[j] = field_i<Q16>(w, j);
 #pragma unroll
     for (int m = 0; m < F::LE; ++m) qt[m] = field_i<Q16>(w, F::ND + m);
-    eval64<FAM>(c, cell, qf, qt, ubm, lbm);
+    eval64<FAM>(c, cell, qf, qt, fs0, fs1, ubm, lbm);
 }
 
-// One queue entry (a tile and its undecided lanes, almost always one) per thread; the
-// screen left those lanes' bits clear, so the passing ones are set here.
+// One queue entry (a tile and its undecided lanes, almost always one) per thread, or, of a
+// short queue, one entry's children of one free slot: then the kernel's time is a single
+// evaluation's (a chain of FP64 instructions, 40 clocks each: 8 children of a 3-DoF pose
+// 5 us, 64 of a 6-DoF pose 70 us), and the work that the split repeats costs nothing: 6-DoF
+// pose, 5000 matches: count and recheck 2.7 -> 1.1 ms.  The
+// screen left the lanes' bits clear, so the passing ones are set here.
 template <int FAM, bool Q16>
 __global__ void __launch_bounds__(128) k_recheck(const __grid_constant__ Chunk c) {
     grid_start();
     if (chunk_tiles(c) == 0) return;                                // the chain has stopped: not its queue
     const unsigned nq = c.sc->n_uns;
     unsigned long long done = 0;
-    for (unsigned i = blockIdx.x * 128u + threadIdx.x; i < nq; i += gridDim.x * 128u) {
+    const unsigned threads = gridDim.x * 128u, parts = nq * (unsigned)c.nfs <= threads ? (unsigned)c.nfs : 1u;
+    for (unsigned x = blockIdx.x * 128u + threadIdx.x; x < nq * parts; x += threads) {
+        const unsigned i = x / parts;
+        const int fs0 = (int)(x - i * parts), fs1 = parts > 1u ? fs0 + 1 : c.nfs;
         const uint2 e = c.uns[i];
         const int cell = c.tinfo[e.x].x;
         for (unsigned m = e.y; m; m &= m - 1) {
             const int bit = __ffs(m) - 1;
             SlotMask<FAM> ubm, lbm;
-            eval_record<FAM, Q16>(c, (c.t0 + e.x) * 32 + bit, cell, ubm, lbm);
+            eval_record<FAM, Q16>(c, (c.t0 + e.x) * 32 + bit, cell, fs0, fs1, ubm, lbm);
             uint32_t *bp = c.ballot + (size_t)e.x * c.ns, *lp = c.lballot + (size_t)e.x * c.ns;
             for (SlotMask<FAM> x = ubm; x; x &= x - 1) atomicOr(bp + __ffsll((long long)x) - 1, 1u << bit);
             if (c.lb)
                 for (SlotMask<FAM> x = lbm; x; x &= x - 1) atomicOr(lp + __ffsll((long long)x) - 1, 1u << bit);
-            done += (unsigned)c.ns;
+            if (fs0 == 0) done += (unsigned)c.ns;
         }
     }
     if (done) atomicAdd(&c.sc->rechecks, done);
@@ -62,7 +69,7 @@ __global__ void __launch_bounds__(256) k_count_exact(const __grid_constant__ Chu
         const int nvalid = ti.y & 63;
         nrec += (unsigned)nvalid;
         SlotMask<FAM> ubm = 0, lbm = 0;
-        if (lane < nvalid) eval_record<FAM, Q16>(c, (c.t0 + tt) * 32 + lane, ti.x, ubm, lbm);
+        if (lane < nvalid) eval_record<FAM, Q16>(c, (c.t0 + tt) * 32 + lane, ti.x, 0, c.nfs, ubm, lbm);
         uint32_t *bp = c.ballot + (size_t)tt * c.ns, *lp = c.lballot + (size_t)tt * c.ns;
         for (int s = 0; s < c.ns; ++s) {
             const unsigned bu = __ballot_sync(kFull, (ubm >> s) & 1), bl = __ballot_sync(kFull, (lbm >> s) & 1);
@@ -94,9 +101,9 @@ __global__ void __launch_bounds__(256) k_count_exact(const __grid_constant__ Chu
 void launch_recheck(const Chunk &c, cudaStream_t st) {
     const int64_t nt = c.t1 - c.t0;
     if (nt <= 0) return;
-    // at most one entry per tile; a queue of 10^-3 entries per tile fills 608 blocks from
-    // 8e7 tiles on, smaller chunks need fewer
-    const unsigned g = (unsigned)(nt < 608 * 128 ? (nt + 127) / 128 : 608);
+    // at most one entry per tile, nfs threads for each while the queue is short
+    const int64_t need = (nt * c.nfs + 127) / 128;
+    const unsigned g = (unsigned)(need < 608 ? need : 608);
     if (c.lev.q16) {
         GV_DISPATCH(c.P.fam, (launch(k_recheck<FAMV, true>, g, 128, 0, st, c)));
     } else {

@@ -279,6 +279,15 @@ __global__ void __launch_bounds__(256) k_prep(const __grid_constant__ Chunk c) {
     }
 }
 
+__device__ __forceinline__ unsigned long long warp_max64(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long y = __shfl_xor_sync(kFull, v, o);
+        v = y > v ? y : v;
+    }
+    return v;
+}
+
 // Block-wide exclusive scan of one 64-bit value per thread (blockDim = 256).
 __device__ __forceinline__ unsigned long long block_excl_scan(unsigned long long v, unsigned long long *total) {
     __shared__ unsigned long long warp_tot[8];
@@ -307,9 +316,44 @@ __device__ __forceinline__ unsigned long long block_excl_scan(unsigned long long
     return before + x - v;
 }
 
+// Cells and records of the blocks before this one (v[0], v[1]) and of all nb (v[2], v[3]).
+__device__ __forceinline__ void block_totals(const unsigned long long *cells, const unsigned long long *recs, int nb,
+                                             unsigned long long *v) {
+    __shared__ unsigned long long sum[8][4];
+    v[0] = v[1] = v[2] = v[3] = 0ull;
+    for (int i = threadIdx.x; i < nb; i += 256) {
+        const unsigned long long x = cells[i], y = recs[i];
+        if (i < (int)blockIdx.x) v[0] += x, v[1] += y;
+        v[2] += x;
+        v[3] += y;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(kFull, v[k], o);
+        if ((threadIdx.x & 31) == 0) sum[threadIdx.x >> 5][k] = v[k];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[k] = 0ull;
+        for (int w = 0; w < 8; ++w) v[k] += sum[w][k];
+    }
+    __syncthreads();
+}
+
 // ---------------------------------------------------------------------------
 // A5 best lower bound, pruning, allocation of surviving children, leaf argmax
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void trace_child(const Chunk &c, uint64_t key, unsigned ub, unsigned lb) {
+    const unsigned long long t = atomicAdd(&c.sc->trace_n, 1ull);
+    if (t >= c.trace.cap) return;
+    c.trace.level[t] = c.lev.l + 1;
+    c.trace.key[t] = key;
+    c.trace.ub[t] = ub;
+    c.trace.lb[t] = lb;
+}
+
 // Phase A: per child of the chunk -- trace, pruning decision, leaf argmax, and
 // per-block totals of surviving children and their records.
 __global__ void __launch_bounds__(256) k_child_mark(Chunk c, uint32_t *keepflag, uint32_t *recn,
@@ -329,13 +373,7 @@ __global__ void __launch_bounds__(256) k_child_mark(Chunk c, uint32_t *keepflag,
         nrec = c.crec[idx];
         key = child_key(P, c.cells.key[c.c0 + cl], c.lev.l, expand_bits(s, c.lev.split_mask));
         if (c.trace.cap) {
-            unsigned long long t = atomicAdd(&c.sc->trace_n, 1ull);
-            if (t < c.trace.cap) {
-                c.trace.level[t] = c.lev.l + 1;
-                c.trace.key[t] = key;
-                c.trace.ub[t] = ub;
-                c.trace.lb[t] = lb;
-            }
+            trace_child(c, key, ub, lb);
         }
     }
     unsigned thr = prune_threshold(P, c.sc, c.prune);
@@ -388,14 +426,107 @@ __global__ void __launch_bounds__(256) k_scan_sums(unsigned long long *a, unsign
 
 // What the step stores, to the host: it polls this instead of copying and synchronising
 // (4 us instead of 15 us per step).
-__device__ __forceinline__ void report(const Chunk &c, unsigned long long cells, unsigned long long recs, bool overflow) {
-    if (!c.host) return;
-    volatile LevInfo *h = c.host;
+__device__ __forceinline__ void report(LevInfo *host, long long seq, unsigned long long cells, unsigned long long recs,
+                                       bool overflow) {
+    if (!host) return;
+    volatile LevInfo *h = host;
     h->stored_cells = (long long)cells;
     h->stored_recs = (long long)recs;
     h->overflow = overflow;
     __threadfence_system();
-    h->seq = c.seq;
+    h->seq = seq;
+}
+
+// What a step stores: to the next level of a chain (it runs if there was room for it and
+// it is not too large) and to the host.  Returns whether there was room.
+__device__ __forceinline__ bool step_room(const Chunk &c, unsigned long long cells, unsigned long long recs) {
+    return !c.dyn || ((int64_t)cells <= c.cap_cells && (int64_t)recs <= c.cap_recs);
+}
+
+__device__ __forceinline__ void step_result(const Chunk &c, unsigned long long cells, unsigned long long recs) {
+    const bool room = step_room(c, cells, recs), runs = room && (int64_t)recs <= c.fit_recs;
+    c.sc->n_cells = cells;
+    c.sc->n_recs = recs;
+    if (c.dyn) {
+        c.dyn->overflow = !room;
+        c.dyn[1].ncells = runs ? (long long)cells : 0ll;
+        c.dyn[1].nrecs = runs ? (long long)recs : 0ll;
+    }
+    report(c.host, c.seq, cells, recs, !room);
+}
+
+// Lays out a kept child: cell index ci, records from rb.
+__device__ __forceinline__ void place_child(const Chunk &c, int idx, unsigned long long ci, unsigned long long rb) {
+    const int cl = idx >> c.lns, s = idx & (c.ns - 1);
+    c.next_cells.key[ci] = child_key(c.P, c.cells.key[c.c0 + cl], c.lev.l, expand_bits(s, c.lev.split_mask));
+    c.next_cells.rbeg[ci] = rb;
+    c.next_cells.rcnt[ci] = c.crec[idx];
+    c.next_cells.ub[ci] = c.cub[idx];
+    c.next_cells.lb[ci] = c.lb ? c.clb[idx] : 0u;
+    c.child_idx[idx] = (int32_t)ci;
+    c.cbase[idx] = rb;
+    c.alive[cl] = 3;                                 // the cell has something to write (every writer stores 3)
+}
+
+// Phases A to C of a small step in one block of 256 threads: 1024 children at a time,
+// four consecutive ones per thread (all their loads in flight at once).  8 us instead of 3
+// + 6.5 us; as the end of the tile scan it took longer than by itself.
+__global__ void __launch_bounds__(256) k_children(const __grid_constant__ Chunk c) {
+    grid_start();
+    const Problem &P = c.P;
+    const int nch = chunk_cells(c) << c.lns;
+    if (nch == 0) return;                            // the chain has stopped
+    const unsigned thr = prune_threshold(P, c.sc, c.prune);
+    unsigned long long cand = 0ull, cells = 0ull, recs = 0ull;
+    for (int base = 0; base < nch; base += 1024) {
+        const int first = base + 4 * (int)threadIdx.x;
+        unsigned ub[4], nrec[4];
+        bool exists[4], keep[4];
+        uint64_t key[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int idx = first + k < nch ? first + k : nch - 1, cl = idx >> c.lns;
+            exists[k] = c.alive[cl] && first + k < nch;
+            nrec[k] = c.crec[idx];
+            ub[k] = c.weighted ? c.cub[idx] : nrec[k];
+            key[k] = c.cells.key[c.c0 + cl];
+        }
+        unsigned long long v = 0ull;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            keep[k] = exists[k] && ub[k] >= thr;
+            key[k] = child_key(P, key[k], c.lev.l, expand_bits((first + k) & (c.ns - 1), c.lev.split_mask));
+            if (c.trace.cap && exists[k]) trace_child(c, key[k], ub[k], c.lb ? c.clb[first + k] : 0u);
+            const unsigned long long leafv =
+                ((unsigned long long)ub[k] << P.coord_bits) | (~key[k] & ((1ull << P.coord_bits) - 1ull));
+            if (keep[k] && leafv > cand) cand = leafv;
+            // a child's records start at a whole tile
+            if (keep[k]) v += (1ull << 40) + ((nrec[k] + 31u) & ~31u);
+        }
+        if (c.lev.leaf_children) continue;
+        unsigned long long total;
+        v = block_excl_scan(v, &total);
+        unsigned long long ci = c.next_c0 + cells + (v >> 40), rb = c.next_r0 + recs + (v & ((1ull << 40) - 1ull));
+        cells += total >> 40;
+        recs += total & ((1ull << 40) - 1ull);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (first + k >= nch) break;
+            // without room the host lays the children out again; nothing is written past the end
+            if (keep[k] && (!c.dyn || (int64_t)ci < c.cap_cells)) place_child(c, first + k, ci, rb);
+            else c.cbase[first + k] = ~0ull;
+            if (keep[k]) {
+                ++ci;
+                rb += (nrec[k] + 31u) & ~31u;
+            }
+        }
+    }
+    if (c.lev.leaf_children) {
+        cand = warp_max64(cand);
+        if ((threadIdx.x & 31) == 0 && cand) atomicMax(&c.sc->best_key, cand);
+    } else if (threadIdx.x == 0) {
+        step_result(c, cells, recs);
+    }
 }
 
 // Phase C: surviving children get consecutive cell indices and record ranges in
@@ -414,42 +545,14 @@ __global__ void __launch_bounds__(256) k_child_write(Chunk c, const uint32_t *ke
     if (scanned) {
         c_before = bs_cells[blockIdx.x];
         r_before = bs_recs[blockIdx.x];
-        if (blockIdx.x == 0 && threadIdx.x == 0) report(c, c.sc->n_cells, c.sc->n_recs, false);
+        if (blockIdx.x == 0 && threadIdx.x == 0) report(c.host, c.seq, c.sc->n_cells, c.sc->n_recs, false);
     } else {
-        __shared__ unsigned long long sum[8][4];
-        unsigned long long v[4] = {0ull, 0ull, 0ull, 0ull};      // cells, records: before this block, in all
-        for (int i = threadIdx.x; i < nb; i += 256) {
-            const unsigned long long x = bs_cells[i], y = bs_recs[i];
-            if (i < (int)blockIdx.x) v[0] += x, v[1] += y;
-            v[2] += x;
-            v[3] += y;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(kFull, v[k], o);
-            if ((threadIdx.x & 31) == 0) sum[threadIdx.x >> 5][k] = v[k];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            v[k] = 0ull;
-            for (int w = 0; w < 8; ++w) v[k] += sum[w][k];
-        }
-        __syncthreads();
+        unsigned long long v[4];
+        block_totals(bs_cells, bs_recs, nb, v);
         c_before = v[0];
         r_before = v[1];
-        const bool room = !c.dyn || ((int64_t)v[2] <= c.cap_cells && (int64_t)v[3] <= c.cap_recs);
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            const bool runs = room && (int64_t)v[3] <= c.fit_recs;
-            if (c.dyn) {
-                c.dyn->overflow = !room;
-                c.dyn[1].ncells = runs ? (long long)v[2] : 0ll;
-                c.dyn[1].nrecs = runs ? (long long)v[3] : 0ll;
-            }
-            report(c, v[2], v[3], !room);
-        }
-        if (!room) return;                               // uniform
+        if (blockIdx.x == 0 && threadIdx.x == 0) step_result(c, v[2], v[3]);
+        if (!step_room(c, v[2], v[3])) return;           // uniform
     }
     const bool in = idx < nch;
     unsigned keep = in ? keepflag[idx] : 0u;
@@ -462,17 +565,7 @@ __global__ void __launch_bounds__(256) k_child_write(Chunk c, const uint32_t *ke
         c.cbase[idx] = ~0ull;
         return;
     }
-    const int cl = idx >> c.lns, s = idx & (c.ns - 1);
-    const unsigned long long ci = c.next_c0 + c_before + ec;
-    const unsigned long long rb = c.next_r0 + r_before + er;
-    c.next_cells.key[ci] = child_key(c.P, c.cells.key[c.c0 + cl], c.lev.l, expand_bits(s, c.lev.split_mask));
-    c.next_cells.rbeg[ci] = rb;
-    c.next_cells.rcnt[ci] = c.crec[idx];
-    c.next_cells.ub[ci] = c.cub[idx];
-    c.next_cells.lb[ci] = c.lb ? c.clb[idx] : 0u;
-    c.child_idx[idx] = (int32_t)ci;
-    c.cbase[idx] = rb;
-    c.alive[cl] = 3;                                 // the cell has something to write (every writer stores 3)
+    place_child(c, idx, c.next_c0 + c_before + ec, c.next_r0 + r_before + er);
 }
 
 // ---------------------------------------------------------------------------
@@ -486,14 +579,17 @@ __global__ void __launch_bounds__(256) k_child_write(Chunk c, const uint32_t *ke
 // 9.2 ms).
 //
 // k_beam_hist: record slots per UB and LB bin (64 bins per octave) and the cells with
-// the largest UB and LB; k_beam_pick: the bin at which the slots of the bins above
-// reach the budget, and the share of that bin's cells that still fits; k_beam_mark:
+// the largest UB and LB; its last block finds the bin at which the slots of the bins above
+// reach the budget, and the share of that bin's cells that still fits.  k_beam_mark:
 // selected cells (the border bin's by a hash of their keys, so the choice depends on
-// nothing but the cells) and block totals; k_scan_sums; k_beam_write: the selected
-// cells in index order, their UB in the level set to 0 (no threshold is below 1, so
-// they are found pruned later and no cell is tested twice); k_beam_gather: their
+// nothing but the cells) and block totals; k_scan_sums (with many blocks); k_beam_write:
+// the selected cells in index order, their UB in the level set to 0 (no threshold is below
+// 1, so they are found pruned later and no cell is tested twice).  Of few cells, the last
+// block of k_beam_hist also takes those steps.  k_beam_gather: the selected cells'
 // records, copied so that one contiguous chunk holds them (a warp per tile, the owning
-// cell by binary search; the copy moves at most a few tens of MB).
+// cell by binary search; the copy moves at most a few tens of MB).  A 3-DoF search of 1e6
+// surfaces makes 28 selections: five kernels, a clear, a copy and a synchronisation for
+// each took 1.2 ms in all, 0.9 ms now.
 // ---------------------------------------------------------------------------
 
 // 64 bins per octave: the exponent and six mantissa bits of a count as a float
@@ -508,17 +604,92 @@ __device__ __forceinline__ unsigned beam_hash(uint64_t key) {
     return (unsigned)(key >> 32);
 }
 
-__device__ __forceinline__ unsigned long long warp_max64(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long y = __shfl_xor_sync(kFull, v, o);
-        v = y > v ? y : v;
+// Adds a value to a kernel's ticket; whether this is its last block (all 256 threads).
+__device__ __forceinline__ bool last_block(unsigned *ticket, unsigned blocks) {
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(ticket, 1u) == blocks - 1u;
+        if (s_last) *ticket = 0u;                    // for the next kernel
     }
-    return v;
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
 }
 
+__device__ __forceinline__ void beam_pick(BeamSel *sel, unsigned long long budget) {
+    // thread t owns bins [8 t', 8 t' + 8), t' counted from the top, so a prefix over the
+    // threads is the slots of all higher bins
+    constexpr int PER = kBeamBins / 256;
+    const int top = kBeamBins - 1 - (int)threadIdx.x * PER;
+    if (threadIdx.x < 2) {
+        sel->top[threadIdx.x] = __ldcg(&sel->best[threadIdx.x]);
+        sel->best[threadIdx.x] = 0ull;
+    }
+    for (int k = 0; k < 2; ++k) {
+        unsigned long long v[PER], sum = 0ull, total;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            v[i] = __ldcg(&sel->hist[k][top - i]);
+            sel->hist[k][top - i] = 0ull;            // for the next selection
+            sum += v[i];
+        }
+        unsigned long long above = block_excl_scan(sum, &total);
+        if (total <= budget) {
+            if (threadIdx.x == 0) {
+                sel->border[k] = -1;
+                sel->share[k] = 0u;
+            }
+            continue;
+        }
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            if (above <= budget && above + v[i] > budget) {
+                sel->border[k] = top - i;
+                sel->share[k] = (unsigned)((double)(budget - above) / (double)v[i] * 4294967295.0);
+            }
+            above += v[i];
+        }
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ bool beam_selected(const CellView &cells, int64_t i, int64_t ncells, const BeamSel *sel,
+                                              int nk, unsigned thr) {
+    if (i >= ncells) i = ncells - 1, thr = 0xffffffffu;
+    const unsigned ub = cells.ub[i];
+    const unsigned v[2] = {ub, cells.lb[i]};
+    const unsigned h = beam_hash(cells.key[i]);
+    bool keep = false;
+    if (ub < thr) return false;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (k >= nk || !v[k]) continue;
+        const int b = beam_bin(v[k]);
+        keep |= b > sel->border[k] || (b == sel->border[k] && h < sel->share[k]) ||
+                (unsigned)~(unsigned)sel->top[k] == (unsigned)i;
+    }
+    return keep;
+}
+
+// the selected cell i as cell o of the selection, its records from r
+__device__ __forceinline__ void beam_place(const CellView &cells, int64_t i, const CellView &out, uint64_t *src_rbeg,
+                                           unsigned long long o, unsigned long long r) {
+    out.key[o] = cells.key[i];
+    out.rbeg[o] = r;
+    out.rcnt[o] = cells.rcnt[i];
+    out.ub[o] = cells.ub[i];
+    src_rbeg[o] = cells.rbeg[i];
+    cells.ub[i] = 0u;
+}
+
+// up to kBeamSmall cells are selected by the last block
+constexpr int kBeamSmall = 2048;
+
 __global__ void __launch_bounds__(256) k_beam_hist(CellView cells, int64_t ncells, BeamSel *sel, int nk, Problem P,
-                                                   const Scalars *sc) {
+                                                   const Scalars *sc, unsigned long long budget, CellView out,
+                                                   uint64_t *src_rbeg, LevInfo *host, long long seq) {
     grid_start();
     __shared__ unsigned long long hist[2][kBeamBins];
     for (int i = threadIdx.x; i < 2 * kBeamBins; i += 256) hist[0][i] = 0ull;
@@ -546,56 +717,35 @@ __global__ void __launch_bounds__(256) k_beam_hist(CellView cells, int64_t ncell
     __syncthreads();
     for (int i = threadIdx.x; i < 2 * kBeamBins; i += 256)
         if (hist[0][i]) atomicAdd(&sel->hist[0][i], hist[0][i]);
-}
-
-__global__ void __launch_bounds__(256) k_beam_pick(BeamSel *sel, unsigned long long budget) {
-    grid_start();
-    // thread t owns bins [8 t', 8 t' + 8), t' counted from the top, so a prefix over the
-    // threads is the slots of all higher bins
-    constexpr int PER = kBeamBins / 256;
-    const int top = kBeamBins - 1 - (int)threadIdx.x * PER;
-    for (int k = 0; k < 2; ++k) {
-        unsigned long long v[PER], sum = 0ull, total;
+    if (!last_block(&sel->ticket, gridDim.x)) return;
+    beam_pick(sel, budget);
+    if (ncells > kBeamSmall) return;
+    unsigned long long tc = 0ull, tr = 0ull;
+    for (int base = 0; base < (int)ncells; base += 1024) {
+        const int first = base + 4 * (int)threadIdx.x;
+        bool keep[4];
+        unsigned slots[4];
+        unsigned long long x = 0ull, total;
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            v[i] = sel->hist[k][top - i];
-            sum += v[i];
+        for (int k = 0; k < 4; ++k) {
+            keep[k] = beam_selected(cells, first + k, ncells, sel, nk, thr);
+            slots[k] = keep[k] ? (cells.rcnt[first + k] + 31u) & ~31u : 0u;
         }
-        unsigned long long above = block_excl_scan(sum, &total);
-        if (total <= budget) {
-            if (threadIdx.x == 0) {
-                sel->border[k] = -1;
-                sel->share[k] = 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (keep[k]) x += (1ull << 40) + slots[k];
+        x = block_excl_scan(x, &total);
+        unsigned long long o = tc + (x >> 40), r = tr + (x & ((1ull << 40) - 1ull));
+        tc += total >> 40;
+        tr += total & ((1ull << 40) - 1ull);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (keep[k]) {
+                beam_place(cells, first + k, out, src_rbeg, o++, r);
+                r += slots[k];
             }
-            continue;
-        }
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            if (above <= budget && above + v[i] > budget) {
-                sel->border[k] = top - i;
-                sel->share[k] = (unsigned)((double)(budget - above) / (double)v[i] * 4294967295.0);
-            }
-            above += v[i];
-        }
     }
-}
-
-__device__ __forceinline__ bool beam_selected(const CellView &cells, int64_t i, int64_t ncells, const BeamSel *sel,
-                                              int nk, unsigned thr) {
-    if (i >= ncells) return false;
-    const unsigned ub = cells.ub[i];
-    if (ub < thr) return false;
-    const unsigned v[2] = {ub, cells.lb[i]};
-    const unsigned h = beam_hash(cells.key[i]);
-    bool keep = false;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        if (k >= nk || !v[k]) continue;
-        const int b = beam_bin(v[k]);
-        keep |= b > sel->border[k] || (b == sel->border[k] && h < sel->share[k]) ||
-                (unsigned)~(unsigned)sel->best[k] == (unsigned)i;
-    }
-    return keep;
+    if (threadIdx.x == 0) report(host, seq, tc, tr, false);
 }
 
 __global__ void __launch_bounds__(256) k_beam_mark(CellView cells, int64_t ncells, const BeamSel *sel, int nk, Problem P,
@@ -615,23 +765,28 @@ __global__ void __launch_bounds__(256) k_beam_mark(CellView cells, int64_t ncell
 
 __global__ void __launch_bounds__(256) k_beam_write(CellView cells, int64_t ncells, const BeamSel *sel, int nk, Problem P,
                                                     const Scalars *sc, const unsigned long long *bs_cells,
-                                                    const unsigned long long *bs_recs, CellView out,
-                                                    uint64_t *src_rbeg) {
+                                                    const unsigned long long *bs_recs, int scanned, CellView out,
+                                                    uint64_t *src_rbeg, LevInfo *host, long long seq) {
     grid_start();
+    unsigned long long c_before, r_before;
+    if (scanned) {
+        c_before = bs_cells[blockIdx.x];
+        r_before = bs_recs[blockIdx.x];
+        if (blockIdx.x == 0 && threadIdx.x == 0) report(host, seq, sc->n_cells, sc->n_recs, false);
+    } else {
+        unsigned long long v[4];
+        block_totals(bs_cells, bs_recs, (int)gridDim.x, v);
+        c_before = v[0];
+        r_before = v[1];
+        if (blockIdx.x == 0 && threadIdx.x == 0) report(host, seq, v[2], v[3], false);
+    }
     const int64_t i = blockIdx.x * 256ll + threadIdx.x;
     const bool keep = beam_selected(cells, i, ncells, sel, nk, prune_threshold(P, sc, 1));
     unsigned long long tc, tr;
     const unsigned long long ec = block_excl_scan(keep ? 1ull : 0ull, &tc);
     const unsigned long long er =
         block_excl_scan(keep ? (unsigned long long)((cells.rcnt[i] + 31u) & ~31u) : 0ull, &tr);
-    if (!keep) return;
-    const unsigned long long o = bs_cells[blockIdx.x] + ec;
-    out.key[o] = cells.key[i];
-    out.rbeg[o] = bs_recs[blockIdx.x] + er;
-    out.rcnt[o] = cells.rcnt[i];
-    out.ub[o] = cells.ub[i];
-    src_rbeg[o] = cells.rbeg[i];
-    cells.ub[i] = 0u;
+    if (keep) beam_place(cells, i, out, src_rbeg, c_before + ec, r_before + er);
 }
 
 // nq: 16-byte words of one tile's records
@@ -858,17 +1013,19 @@ __device__ __forceinline__ bool replay_far(const Problem &P, const Level &lev, c
 // of them at once: a block screens its surfaces first (30 FP64 instructions each) and only
 // those that may pass go through the steps (50 FP64 instructions per step, the FP64 pipe's
 // rate is the bound), collected so that warps are full.  1e6 surfaces of a 3-DoF pose, 10
-// steps: 621 us with every surface through the steps until it fails, 131 us now.
-constexpr int kReplayPer = 4;                        // surfaces per thread
+// steps: 621 us with every surface through the steps until it fails, 120 us now.
+// per: surfaces per block, a multiple of 32; at most 1024, fewer when the chip would be
+// idle otherwise (the steps of 1024 surfaces on one SM take 40 us).
 template <int FAM>
 __global__ void __launch_bounds__(256) k_replay(Problem P, const Level *levs, const PathStep *path, int lam,
-                                                const double *prm, int64_t n, uint32_t *reach, Scalars *sc) {
+                                                const double *prm, int64_t n, int per, uint32_t *reach, Scalars *sc) {
     grid_start();
     using F = Fam<FAM>;
-    constexpr int NS = 256 * kReplayPer;
+    constexpr int NS = 1024;
     __shared__ unsigned s_words[NS / 32], s_n, s_lb;
     __shared__ unsigned short s_list[NS];
-    const int64_t base = (int64_t)blockIdx.x * NS;
+    const int64_t base = (int64_t)blockIdx.x * per, left = n - base;
+    const int share = left < per ? (int)left : per;
     const int lane = threadIdx.x & 31;
     const PathStep *tail = path + lam;
     if (threadIdx.x < NS / 32) s_words[threadIdx.x] = 0u;
@@ -882,9 +1039,9 @@ __global__ void __launch_bounds__(256) k_replay(Problem P, const Level *levs, co
     }
     __syncthreads();
 #pragma unroll 1
-    for (int k = 0; k < kReplayPer; ++k) {
-        const int x = k * 256 + threadIdx.x;
-        bool maybe = base + x < n;
+    for (int x0 = 0; x0 < share; x0 += 256) {
+        const int x = x0 + threadIdx.x;
+        bool maybe = x < share;
         if (maybe && lam > 0) {
             F::lift(prm, n, base + x, c, psi, f, t);
             maybe = !replay_far<FAM>(P, levs[lam - 1], tail, f, t);
@@ -925,7 +1082,7 @@ __global__ void __launch_bounds__(256) k_replay(Problem P, const Level *levs, co
     if (threadIdx.x < 32) {
         static_assert(NS / 32 == 32, "a mask word per lane");
         const unsigned w = s_words[lane];
-        if (reach && base + 32 * lane < n) reach[(base >> 5) + lane] = w;
+        if (reach && 32 * lane < share) reach[(base >> 5) + lane] = w;
         const unsigned total = __reduce_add_sync(kFull, (unsigned)__popc(w));
         if (lane == 0 && total) atomicAdd(&sc->replay_ub, (unsigned long long)total);
         if (lane == 0 && s_lb) atomicAdd(&sc->replay_lb, (unsigned long long)s_lb);
@@ -1168,10 +1325,14 @@ void launch_chain_start(LevInfo *info, int64_t cells, int64_t recs, cudaStream_t
 // of them: 2 us saved by one launch less; at 4096 blocks it would cost more)
 constexpr unsigned kSelfScan = 512;
 
-int launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
+int launch_child_alloc(const Chunk &c, bool small, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
                        cudaStream_t st) {
     const int64_t n = (int64_t)c.nc << c.lns;
     if (n <= 0) return 0;
+    if (small) {
+        launch(k_children, 1, 256, 0, st, c);
+        return 1;
+    }
     unsigned nb = blocks_for(n, 256);
     unsigned long long *ba = bsums, *bb = bsums + nb;
     launch(k_child_mark, nb, 256, 0, st, c, keepflag, recn, ba, bb);
@@ -1185,22 +1346,19 @@ int launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsig
     return 2;
 }
 
-void launch_child_write(const Chunk &c, const uint32_t *keepflag, const uint32_t *recn, unsigned long long *bsums,
-                        unsigned stride, cudaStream_t st) {
-    const unsigned nb = blocks_for((int64_t)c.nc << c.lns, 256);
-    launch(k_child_write, nb, 256, 0, st, c, keepflag, recn, bsums, bsums + stride, 0);
-}
-
-void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, int nk, BeamSel *sel,
-                        unsigned long long *bsums, const CellView &out, uint64_t *src_rbeg, Scalars *sc,
-                        cudaStream_t st) {
+int launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, int nk, BeamSel *sel,
+                       unsigned long long *bsums, const CellView &out, uint64_t *src_rbeg, Scalars *sc, LevInfo *host,
+                       long long seq, cudaStream_t st) {
     const unsigned nb = blocks_for(ncells, 256);
     unsigned long long *ba = bsums, *bb = bsums + nb;
-    launch(k_beam_hist, nb < 1024u ? nb : 1024u, 256, 0, st, cells, ncells, sel, nk, P, sc);
-    launch(k_beam_pick, 1, 256, 0, st, sel, (unsigned long long)budget / nk);
+    launch(k_beam_hist, nb < 1024u ? nb : 1024u, 256, 0, st, cells, ncells, sel, nk, P, sc, (unsigned long long)budget / nk,
+           out, src_rbeg, host, seq);
+    if (ncells <= kBeamSmall) return 1;
     launch(k_beam_mark, nb, 256, 0, st, cells, ncells, sel, nk, P, sc, ba, bb);
-    launch(k_scan_sums, 1, 256, 0, st, ba, bb, (int)nb, sc);
-    launch(k_beam_write, nb, 256, 0, st, cells, ncells, sel, nk, P, sc, ba, bb, out, src_rbeg);
+    const int scanned = nb > kSelfScan;
+    if (scanned) launch(k_scan_sums, 1, 256, 0, st, ba, bb, (int)nb, sc);
+    launch(k_beam_write, nb, 256, 0, st, cells, ncells, sel, nk, P, sc, ba, bb, scanned, out, src_rbeg, host, seq);
+    return 3 + scanned;
 }
 
 void launch_beam_gather(const RecView &in, const RecView &out, const CellView &sel, const uint64_t *src_rbeg,
@@ -1239,7 +1397,9 @@ void launch_path_geo(const Problem &P, const Level *levs_dev, int lam, uint64_t 
 void launch_replay(const Problem &P, const Level *levs_dev, const PathStep *path, int lam, const double *prm,
                    int64_t n, uint32_t *reach, Scalars *sc, cudaStream_t st) {
     if (n <= 0) return;
-    GV_DISPATCH(P.fam, (launch(k_replay<FAMV>, blocks_for(n, 256 * kReplayPer), 256, 0, st, P, levs_dev, path, lam, prm, n,
+    const int64_t share = (n + 2 * sm_count() - 1) / (2 * sm_count());
+    const int per = share >= 1024 ? 1024 : (int)((share + 31) & ~31);
+    GV_DISPATCH(P.fam, (launch(k_replay<FAMV>, blocks_for(n, per), 256, 0, st, P, levs_dev, path, lam, prm, n, per,
                                                                             reach, sc)));
 }
 

@@ -170,8 +170,10 @@ constexpr int kBeamBins = 2048;
 struct BeamSel {
     unsigned long long hist[2][kBeamBins];  // record slots per bin
     unsigned long long best[2];      // (value << 32) | ~index of the cell with the largest value
+    unsigned long long top[2];       // the same, of the finished histogram
     int border[2];                   // bins above are selected whole
     unsigned share[2];               // selected share of the border bin (2^32 = all)
+    unsigned ticket;
 };
 
 // Path geometry for replaying surfaces along the root-to-cell path.
@@ -207,21 +209,18 @@ void launch_tile_scan(const Chunk &c, cudaStream_t st);
 bool launch_emit_wide(const Chunk &c, cudaStream_t st);
 // false if the level's record formats have no emit pass (never chosen by the engine)
 bool launch_emit(const Chunk &c, cudaStream_t st);
-// keepflag, recn: [nc * ns]; bsums: 2 * ceil(nc * ns / 256)
 // sizes of the level that a chain starts from, or goes on from
 void launch_chain_start(LevInfo *info, int64_t cells, int64_t recs, cudaStream_t st);
-// returns the kernels launched
-int launch_child_alloc(const Chunk &c, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
+// keepflag, recn: [nc * ns]; bsums: 2 * ceil(nc * ns / 256); returns the kernels launched
+// (small: by one block)
+int launch_child_alloc(const Chunk &c, bool small, uint32_t *keepflag, uint32_t *recn, unsigned long long *bsums,
                        cudaStream_t st);
-// the last of them again (after a chain found no room in the next level)
-void launch_child_write(const Chunk &c, const uint32_t *keepflag, const uint32_t *recn, unsigned long long *bsums,
-                        unsigned stride, cudaStream_t st);
 // the cells of a level (whose sum of record slots exceeds budget) with the largest UBs (nk = 2: and LBs):
-// out and src_rbeg receive them ([ncells] at most), sc->n_cells / n_recs their number
-// and slots; bsums: 2 * ceil(ncells / 256); then their records
-void launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, int nk, BeamSel *sel,
+// out and src_rbeg receive them ([ncells] at most), host their number and slots; bsums:
+// 2 * ceil(ncells / 256); returns the kernels launched; then their records
+int launch_beam_select(const Problem &P, const CellView &cells, int64_t ncells, int64_t budget, int nk, BeamSel *sel,
                         unsigned long long *bsums, const CellView &out, uint64_t *src_rbeg, Scalars *sc,
-                        cudaStream_t st);
+                       LevInfo *host, long long seq, cudaStream_t st);
 void launch_beam_gather(const RecView &in, const RecView &out, const CellView &sel, const uint64_t *src_rbeg,
                         int64_t ncells, int64_t ntiles, int rec_bytes, cudaStream_t st);
 // the path to cell `key` at level lam, or to the best leaf of sc when sc is not NULL

@@ -415,11 +415,12 @@ __device__ __forceinline__ int test64(const Level &lev, const double *f, const d
 template <int FAM>
 using SlotMask = typename std::conditional<((1 << Fam<FAM>::D) > 32), unsigned long long, unsigned>::type;
 
-// UB/LB pass masks of one record (integer fields) against every child slot, exactly
+// UB/LB pass masks of one record (integer fields) against the child slots of free slots
+// [fs0, fs1), exactly
 // as the definition evaluates them.
 template <int FAM>
-__device__ __forceinline__ void eval64(const Chunk &c, int cell, const int *qf, const int *qt, SlotMask<FAM> &ubm,
-                                       SlotMask<FAM> &lbm) {
+__device__ __forceinline__ void eval64(const Chunk &c, int cell, const int *qf, const int *qt, int fs0, int fs1,
+                                       SlotMask<FAM> &ubm, SlotMask<FAM> &lbm) {
     using F = Fam<FAM>;
     const Problem &P = c.P;
     const Level &lev = c.lev;
@@ -435,7 +436,7 @@ __device__ __forceinline__ void eval64(const Chunk &c, int cell, const int *qf, 
     ubm = 0;
     lbm = 0;
 #pragma unroll 1
-    for (int fs = 0; fs < (1 << kf); ++fs) {
+    for (int fs = fs0; fs < fs1; ++fs) {
         double pr[F::ND], d[F::NB];
         chunk_change<FAM>(c, cell, fs, d);
         F::partial64(f, t, d, pr);
