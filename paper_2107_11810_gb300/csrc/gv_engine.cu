@@ -802,7 +802,7 @@ static void fill_chunk(vote_ctx *c, int l, const LevelStore &S, const StepDims &
 static vote_status wait_report(vote_ctx *c, const LevInfo *v, long long seq) {
     for (unsigned i = 1;; ++i) {
         if (__atomic_load_n(&v->seq, __ATOMIC_ACQUIRE) == seq) return VOTE_OK;
-        if (i & 1023u) continue;
+        if (i & 0xffffu) continue;           // some 100 us: queries take the lock that other threads launch under
         const cudaError_t e = cudaStreamQuery(c->stream);
         if (e == cudaErrorNotReady) {
             cudaGetLastError();
