@@ -297,6 +297,7 @@ __device__ __forceinline__ float trunc32(double x, bool &ok) {
 
 template <int FAM, bool BWD>
 __global__ void __launch_bounds__(kSsThreads, 4) k_softscore(SoftArgs a) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // k_softscore_final waits for this kernel
     using S = SoftFam<FAM>;
     __shared__ double sm[kSsThreads / 32];
     __shared__ typename S::Pre s_pre;
@@ -408,6 +409,7 @@ __global__ void __launch_bounds__(kSsThreads, 4) k_softscore(SoftArgs a) {
 // out[q] = sum over blocks of partial[b * width + q]: block q, a fixed tree (one thread
 // adding 1024 partials one after the other took 30 us)
 __global__ void __launch_bounds__(kSsThreads) k_softscore_final(const double *partial, int nb, int width, double *out) {
+    grid_start();
     __shared__ double sm[kSsThreads / 32];
     double t = 0.0;
     for (int b = threadIdx.x; b < nb; b += kSsThreads) t += partial[b * width + blockIdx.x];
@@ -464,7 +466,7 @@ void launch_softscore(int fam, bool bwd, const double *prm, int64_t n, const uin
         else k_softscore<FAM_POSE6DOF, false><<<nb, kSsThreads, 0, st>>>(a);
         break;
     }
-    k_softscore_final<<<bwd ? d : 1, kSsThreads, 0, st>>>(partial, nb, bwd ? d : 1, out);
+    launch(k_softscore_final, bwd ? d : 1, kSsThreads, 0, st, partial, nb, bwd ? d : 1, out);
 }
 
 int softscore_partial_doubles() { return kSsBlocks * GV_MAXD; }

@@ -35,12 +35,12 @@ class SoftScore(torch.autograd.Function):
         surfaces = surfaces.contiguous()
         n = surfaces.shape[1]
         tl = _tol_arg(tol, solver.d - solver.k)
-        score = torch.empty(1, dtype=torch.float64, device=point.device)
+        score = point.new_empty(())
         vote._check(solver.lib.vote_softscore_fwd(solver.h, vote._ptr(surfaces), n, vote._ptr(mask),
                                                   vote._ptr(point), vote._ptr(tl), vote._ptr(score)))
         ctx.solver, ctx.tol, ctx.mask = solver, tl, mask
         ctx.save_for_backward(point, surfaces)
-        return score[0]
+        return score
 
     @staticmethod
     @once_differentiable
@@ -48,7 +48,7 @@ class SoftScore(torch.autograd.Function):
         point, surfaces = ctx.saved_tensors
         s = ctx.solver
         n = surfaces.shape[1]
-        g = grad.reshape(1).to(torch.float64).contiguous()
+        g = grad if grad.dtype == torch.float64 else grad.to(torch.float64)    # one element
         gp = torch.empty_like(point) if ctx.needs_input_grad[0] else None
         gs = torch.empty_like(surfaces) if ctx.needs_input_grad[1] else None
         if gp is not None or gs is not None:
