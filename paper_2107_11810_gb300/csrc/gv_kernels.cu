@@ -995,9 +995,12 @@ __global__ void __launch_bounds__(64) k_path_geo(Problem P, const Level *levs, i
 // Screen of the replay: whether a surface certainly fails the last step's test.  Its
 // residual at the target cell's centre is taken from the root in one jump, without
 // snapping: the steps' residual differs from it by at most the accumulated canonization
-// error, which the radius contains; the essential parameters differ by at most one step of
-// the last level (half of each coarser grid they are snapped to on the way).  The FP64 rounding of either way is far below one snap step (fields
-// below 2^30 steps), that of the FP32 radius and conversions below the 1e-4 added.
+// error A.  The radius contains A once, so that no surface within reach is missed; a surface
+// beyond reach can pass the steps' test by it once more, so the screen's limit is the radius
+// plus A.  The essential parameters differ by at most one step of the last level (half of
+// each grid they are snapped to on the way).  The FP64 rounding of either way is far below
+// one snap step (fields below 2^30 steps), that of the FP32 radius and conversions below
+// the 1e-4 added.
 template <int FAM>
 __device__ __forceinline__ bool replay_far(const Problem &P, const Level &lev, const PathStep *tail, const double *f,
                                            const double *t) {
@@ -1021,7 +1024,7 @@ __device__ __forceinline__ bool replay_far(const Problem &P, const Level &lev, c
     for (int j = 0; j < F::ND; ++j) {
         const float s = (float)P.inv_s_f[j];
         in &= fabsf((float)f[j] * s) < 1073741824.0f;
-        far |= fabsf((float)fo[j] * s) > __fmaf_rn(R[j], 1.0001f, 2.0f);
+        far |= fabsf((float)fo[j] * s) > __fmaf_rn(__fmaf_rn((float)lev.A1[j], s, R[j]), 1.0001f, 2.0f);
     }
     return in && far;
 }

@@ -52,3 +52,50 @@ def test_replay_equals_oracle_along_the_best_path(name):
                 oub, olb, oreach = oracle.cell_counts(p.family, p.eps, p.bounds, prm, level, coords, want_reach=True)
                 assert (ub, lb) == (oub, olb)
                 assert np.array_equal(v.mask_words_to_numpy(reach), oreach)
+
+
+# residuals at x of the dependent coordinates, the parameter row each moves one to one with
+# (of its opposite sign), and the essential parameters' part of the radius per half-width
+RESIDUAL = {
+    "line2d": lambda q, x: ([x[1] - (q[1] - q[0] * x[0])], [1], [np.abs(q[0])]),
+    "rays3d": lambda q, x: ([x[1] - (q[0] * x[0] + q[1]), x[2] - (q[2] * x[0] + q[3])], [1, 3],
+                            [np.abs(q[0]), np.abs(q[2])]),
+    "pose3dof": lambda q, x: ([x[1] - (q[0] - (q[2] * np.cos(x[0]) - q[3] * np.sin(x[0]))),
+                               x[2] - (q[1] - (q[2] * np.sin(x[0]) + q[3] * np.cos(x[0])))], [0, 1],
+                              [np.hypot(q[2], q[3])] * 2),
+}
+
+
+def surfaces_beyond_reach(name, p, leaf, n, rng):
+    """Surfaces whose residual at the leaf's centre exceeds its whole radius (canonization
+    error included) by 2 to 6 snap steps in the first dependent coordinate."""
+    from paper_2107_11810_gb300 import vote as v
+    k = v.level_constants(p.family, p.eps, p.bounds)
+    lo, hi = np.asarray(p.bounds, dtype=float).reshape(-1, 2).T
+    h = (hi - lo) * 2.0 ** -(k["Lj"] + 1.0)
+    x = lo + (2 * np.asarray(leaf) + 1) * h
+    q = p.params[:, rng.integers(0, p.params.shape[1], n)]
+    r, rows, lam = RESIDUAL[name](q, x)
+    nd = len(rows)
+    R = p.eps[-nd] + h[-nd] + lam[0] * h[0] + k["A"][-1][0]
+    for j in range(nd):
+        want = (R + k["s_f"][0] * rng.uniform(2.0, 6.0, n)) * rng.choice([-1.0, 1.0], n) if j == 0 else 0.0
+        q[rows[j]] += r[j] - want
+    return np.ascontiguousarray(q)
+
+
+@pytest.mark.parametrize("name", sorted(RESIDUAL))
+def test_replay_keeps_surfaces_that_pass_by_the_canonization_error(name):
+    """The snaps on the way move a residual by up to the accumulated canonization error, so
+    some surfaces just beyond a leaf's radius pass every step, and count."""
+    from paper_2107_11810_gb300 import vote as v
+    p = MAKE[name]()
+    s = v.Solver(p.family, p.eps, p.bounds)
+    leaf = s.solve(torch.from_numpy(np.ascontiguousarray(p.params)).cuda())["best_leaf"]
+    prm = surfaces_beyond_reach(name, p, leaf, 400_000, np.random.default_rng(9))
+    L, _ = s.levels()
+    oub, olb, oreach = oracle.cell_counts(p.family, p.eps, p.bounds, prm, L, leaf, want_reach=True)
+    assert oub > 0                               # some do pass
+    ub, lb, reach = s.cell_counts(torch.from_numpy(prm).cuda(), L, leaf, want_reach=True)
+    assert (ub, lb) == (oub, olb)
+    assert np.array_equal(v.mask_words_to_numpy(reach), oreach)
