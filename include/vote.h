@@ -108,10 +108,10 @@ typedef enum {
     VOTE_OPT_CHUNK_RECORDS = 3, /* records processed per expansion step; default 2^27
                                  for planes (their pruning hardly depends on the
                                  step size, so larger steps only save per-step
-                                 overhead), 2^25 for the other families with d = 2
-                                 or 3 (finer depth-first steps keep their pruning
-                                 effective), 2^23 for d = 4 or 5 and 2^21 for d = 6
-                                 (a step's children can hold 2^d times its records) */
+                                 overhead), 2^25 for the other families with d <= 5
+                                 (finer depth-first steps keep their pruning
+                                 effective) and 2^23 for d = 6 (a step's children
+                                 can hold 2^d times its records)                     */
     VOTE_OPT_TRACE_CAP = 4,   /* >0: record (level, coords, UB, LB) of every tested
                                  child, up to this many entries (debug; default 0)   */
     VOTE_OPT_GROUP = 5,       /* merging of identical canonical surfaces:
@@ -147,8 +147,10 @@ enum {
 typedef struct {
     int64_t levels;          /* L                                                 */
     int64_t cells;           /* cells expanded (canonized and tested)            */
-    int64_t records;         /* (cell, canonical surface) records tested          */
-    int64_t tests;           /* (child cell, canonical surface) predicate calls   */
+    int64_t records;         /* (cell, canonical surface) records of those cells  */
+    int64_t tests;           /* (child cell, canonical surface) pairs decided: some
+                                without a predicate call, where a cell is left
+                                because none of its children can survive          */
     int64_t rechecks;        /* tests re-evaluated in FP64 because the FP32 screen
                                 could not decide them (whole records: every child
                                 of a record with one uncertain test), plus child

@@ -14,16 +14,20 @@
 // multiply-add, one compare and one ballot, and the band of a record is checked once,
 // from the smallest |y^2 - R^2| of its children.  Records are read with plain coalesced
 // loads one tile ahead, so nothing waits at a block barrier.
+//
+// Cells are left as soon as no child can reach the threshold (CellWatch).  Staging the
+// ballots and the batches for that cost 10 to 15 % of a pass that leaves no cell (unrolled
+// batches as much: their registers spill); planes of 1e6 points: 237 -> 193 ms of count
+// passes (35 % of the records are not tested), of 1e4 points 7.7 -> 6.3.
 #include "gv_tile.cuh"
 
 namespace gv {
 
 // KF: free coordinates that split, DM: dependent coordinates that split (bit mask).
-// Each warp takes a contiguous range of the chunk's tiles (runs of tiles of one cell
-// stay together: the cell's coefficients are spread from one register per lane only
-// when the cell changes).  Loads run one tile ahead of the tests and tile information
-// two: records and tile information are padded past their ends, so the loop has no
-// boundary case.
+// Warps take units of consecutive tiles (the cell's coefficients are spread from one register
+// per lane only when the cell changes).  Loads run one tile ahead of the tests and tile
+// information two: records and tile information are padded past their ends, so the loop has
+// no boundary case.
 template <int FAM, bool Q16, int KF, int DM, bool LB>
 __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk c) {
     grid_start();
@@ -34,9 +38,16 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
     const int lane = threadIdx.x & 31;
     const Level &lev = c.lev;
     const int64_t nt = chunk_tiles(c);
-    const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
-    if (ta >= tb) return;
+    using W = CellWatch<1, LB>;
+    __shared__ __align__(16) uint32_t s_watch[8][W::WORDS];          // whole 16 bytes per warp
+    W watch;
+    watch.s = s_watch[threadIdx.x >> 5];
+    watch.run(make_int2(-1, -1));
+    uint32_t *row = watch.s;
+    constexpr int BT = 32 / NS;                                     // tiles of a batch of ballots
+    if (nt == 0) return;                                            // the chain has stopped
+    unsigned tt, tb;
+    watch.split(c, (unsigned)nt, blockIdx.x * 8u + (threadIdx.x >> 5), lane, tt, tb);
     float hs[ND];
     f2 negL2[ND];
 #pragma unroll
@@ -63,96 +74,131 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
                         G[j][m][p] = f2_make(coef32<FAM>(lev, j, m, lin_change<FAM>(c, F::cb(j, m), 2 * p, false)),
                                              coef32<FAM>(lev, j, m, lin_change<FAM>(c, F::cb(j, m), NFS > 1 ? 2 * p + 1 : 0, false)));
             }
-    unsigned nrec = 0;
-    const uint32_t *rp = c.in.rec + ((c.t0 + ta) * 32 + lane) * NW;
-    const int2 *tp = c.tinfo + ta;
-    uint32_t *bp = c.ballot + ta * NS, *lp = c.lballot + ta * NS;
-    int2 ti1 = tp[0], ti2 = tp[1];
-    uint32_t w1[NW];
-    load_words<NW>(rp, 0, w1);
-    float g1 = load_g(ti1.x);
-    unsigned tt = (unsigned)ta;
+    unsigned next;
+    do {
+        next = watch.next(c, lane);
+        bool head = true;
+        run = -1;
+        while (tt < tb) {
+            // the first tile of the unit, or after those skipped
+            const uint32_t *rp = c.in.rec + ((c.t0 + tt) * 32 + lane) * NW;
+            const int2 *tp = c.tinfo + tt;
+            int2 ti, ti1 = tp[0], ti2 = tp[1];
+            uint32_t w1[NW];
+            load_words<NW>(rp, 0, w1);
+            float g1 = load_g(ti1.x);
+            if (head) {
+                const unsigned skip = watch.begin(c, NS, ti1, lane);
+                if (skip) {
+                    tt += skip;
+                    head = false;
+                    continue;
+                }
+                head = false;
+            }
+            for (;;) {
+                const int bt = tb - tt < BT ? (int)(tb - tt) : BT;
+                int rs = 0;                                         // first row of the last run
 #pragma unroll 1
-    for (int k = (int)(tb - ta); k > 0; --k, ++tt, bp += NS, lp += NS) {
-        const int2 ti = ti1;
-        const float g = g1;
-        uint32_t w[NW];
+                for (int b = 0; b < bt; ++b) {
+                    ti = ti1;
+                    const float g = g1;
+                    uint32_t w[NW];
 #pragma unroll
-        for (int i = 0; i < NW; ++i) w[i] = w1[i];
-        rp += 32 * NW;
-        ++tp;
-        load_words<NW>(rp, 0, w1);
-        ti1 = ti2;
-        g1 = load_g(ti1.x);
-        ti2 = tp[1];
-        if (ti.x < 0) continue;                                     // uniform: the cell was pruned
-        if constexpr (NG > 0) {
-            if (ti.x != run) {                                      // uniform: a new cell
-                run = ti.x;
-                float d[F::NBG ? F::NBG : 1][NFS];
+                    for (int i = 0; i < NW; ++i) w[i] = w1[i];
+                    rp += 32 * NW;
+                    ++tp;
+                    load_words<NW>(rp, 0, w1);
+                    ti1 = ti2;
+                    g1 = load_g(ti1.x);
+                    ti2 = tp[1];
+                    if (ti.x < 0) continue;                         // uniform: the cell was pruned
+                    if (ti.x != run) {                                          // uniform: a new cell
+                        run = ti.x;
+                        rs = b;
+                        watch.run(ti);
+                        if constexpr (NG > 0) {
+                            float d[F::NBG ? F::NBG : 1][NFS];
 #pragma unroll
-                for (int x = 0; x < F::NBG; ++x)
+                            for (int x = 0; x < F::NBG; ++x)
 #pragma unroll
-                    for (int f = 0; f < NFS; ++f) d[x][f] = __shfl_sync(kFull, g, x * NFS + f);
+                                for (int f = 0; f < NFS; ++f) d[x][f] = __shfl_sync(kFull, g, x * NFS + f);
 #pragma unroll
-                for (int j = 0; j < ND; ++j)
+                            for (int j = 0; j < ND; ++j)
 #pragma unroll
-                    for (int m = 0; m < LE; ++m)
+                                for (int m = 0; m < LE; ++m)
 #pragma unroll
-                        for (int p = 0; p < NP; ++p)                // one free slot: the pair holds it twice
-                            if (F::uses(j, m))
-                                G[j][m][p] = f2_make(coef32<FAM>(lev, j, m, d[F::cb(j, m)][2 * p]),
-                                                     coef32<FAM>(lev, j, m, d[F::cb(j, m)][NFS > 1 ? 2 * p + 1 : 0]));
+                                    for (int p = 0; p < NP; ++p)                // one free slot: the pair holds it twice
+                                        if (F::uses(j, m))
+                                            G[j][m][p] = f2_make(coef32<FAM>(lev, j, m, d[F::cb(j, m)][2 * p]),
+                                                                 coef32<FAM>(lev, j, m, d[F::cb(j, m)][NFS > 1 ? 2 * p + 1 : 0]));
+                        }
+                    }
+                    const int nvalid = ti.y & 63;
+                    watch.cnt += (unsigned)nvalid;
+                    float qf[ND], qt[LE], R[ND], near[ND], nearL[ND];
+                    f2 negR2[ND], u[ND][NP];
+#pragma unroll
+                    for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
+#pragma unroll
+                    for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
+                    F::radius32(lev, qt, R);
+                    // a lane without a record fails every test (its residual is out of reach)
+                    if (lane >= nvalid) qf[0] = 1.0e15f;
+#pragma unroll
+                    for (int j = 0; j < ND; ++j) {
+                        negR2[j] = f2_dup(-R[j] * R[j]);
+                        near[j] = nearL[j] = 3.0e38f;
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) u[j][p] = f2_dup(qf[j]);
+                    }
+#pragma unroll
+                    for (int m = 0; m < LE; ++m) {
+                        const f2 q2 = f2_dup(qt[m]);
+#pragma unroll
+                        for (int j = 0; j < ND; ++j)
+#pragma unroll
+                            for (int p = 0; p < NP; ++p)
+                                if (F::uses(j, m)) u[j][p] = f2_fma(q2, G[j][m][p], u[j][p]);
+                    }
+                    unsigned bu[NS], bl[NS];
+                    test_children<ND, NFS, DM, LB>(u, hs, negR2, negL2, near, nearL, bu, bl);
+                    if (lane == 0) {
+                        store_row<NS>(row + b * NS, bu);
+                        if constexpr (LB) store_row<NS>(row + 32 + b * NS, bl);
+                    }
+                    const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
+                    const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, near, nearL)) & act;
+                    if (unsb) {                                                 // rare: left to the definition
+                        __syncwarp();                                           // lane 0's stores
+                        if (lane < NS) {
+                            row[b * NS + lane] &= ~unsb;
+                            if constexpr (LB) row[32 + b * NS + lane] &= ~unsb;
+                        }
+                        watch.cnt -= (unsigned)__popc(unsb);
+                        if (lane == 0) c.uns[atomicAdd(&c.sc->n_uns, 1u)] = make_uint2(tt + b, unsb);
+                    }
+                }
+                __syncwarp();
+                unsigned word = 0u;
+                if (lane < bt * NS) {
+                    const size_t at = (size_t)tt * NS + lane;
+                    word = row[lane];
+                    c.ballot[at] = word;
+                    if constexpr (LB) c.lballot[at] = row[32 + lane];
+                }
+                __syncwarp();
+                tt += (unsigned)bt;
+                watch.add(NS, NS == 8 ? 3 : (NS == 4 ? 2 : 1), &word, rs, lane);
+                const unsigned skip = watch.cnt > watch.lim || tt >= tb ? watch.look(c, NS, ti, tt, tb, lane) : 0u;
+                if (skip) {
+                    tt += skip;
+                    break;
+                }
+                if (tt >= tb) break;
             }
         }
-        const int nvalid = ti.y & 63;
-        nrec += (unsigned)nvalid;
-        float qf[ND], qt[LE], R[ND], near[ND], nearL[ND];
-        f2 negR2[ND], u[ND][NP];
-#pragma unroll
-        for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
-#pragma unroll
-        for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
-        F::radius32(lev, qt, R);
-        // a lane without a record fails every test (its residual is out of reach)
-        if (lane >= nvalid) qf[0] = 1.0e15f;
-#pragma unroll
-        for (int j = 0; j < ND; ++j) {
-            negR2[j] = f2_dup(-R[j] * R[j]);
-            near[j] = nearL[j] = 3.0e38f;
-#pragma unroll
-            for (int p = 0; p < NP; ++p) u[j][p] = f2_dup(qf[j]);
-        }
-#pragma unroll
-        for (int m = 0; m < LE; ++m) {
-            const f2 q2 = f2_dup(qt[m]);
-#pragma unroll
-            for (int j = 0; j < ND; ++j)
-#pragma unroll
-                for (int p = 0; p < NP; ++p)
-                    if (F::uses(j, m)) u[j][p] = f2_fma(q2, G[j][m][p], u[j][p]);
-        }
-        unsigned bu[NS], bl[NS];
-        test_children<ND, NFS, DM, LB>(u, hs, negR2, negL2, near, nearL, bu, bl);
-        if (lane == 0) {
-            store_row<NS>(bp, bu);
-            if constexpr (LB) store_row<NS>(lp, bl);
-        }
-        const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
-        const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, near, nearL)) & act;
-        if (unsb) {                                                 // rare: left to the definition
-            __syncwarp();                                           // lane 0's stores
-            if (lane < NS) {
-                bp[lane] &= ~unsb;
-                if constexpr (LB) lp[lane] &= ~unsb;
-            }
-            if (lane == 0) c.uns[atomicAdd(&c.sc->n_uns, 1u)] = make_uint2(tt, unsb);
-        }
-    }
-    if (lane == 0 && nrec) {
-        atomicAdd(&c.sc->records, (unsigned long long)nrec);
-        atomicAdd(&c.sc->tests, (unsigned long long)nrec * NS);
-    }
+    } while (watch.unit(__shfl_sync(kFull, next, 0), (unsigned)nt, tt, tb));
 }
 
 // a persistent grid: as many blocks as are resident (4 per SM), fewer when there are not

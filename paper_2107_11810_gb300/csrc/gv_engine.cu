@@ -783,6 +783,12 @@ static void fill_chunk(vote_ctx *c, int l, const LevelStore &S, const StepDims &
     ch.prune = c->prune;
     ch.precision = c->precision;
     ch.lb = lb;
+    // a trace lists every child's counts; with multiplicities they are not the records'
+    if (c->prune && c->precision == 1 && !c->group && c->trace_cap == 0) {
+        const int64_t per = nt / (sm_count() * 32);         // tiles per warp, about
+        ch.early = per >= 64 ? 64 : (per >= 32 ? 32 : (per >= 16 ? 16 : 1));
+    }
+    ch.cfail = (uint32_t *)c->child_idx.p;
     ch.spin = c->spin_limit;
     ch.tinfo = (int2 *)c->tinfo.p;
     ch.ballot = (uint32_t *)c->ballot.p;
@@ -1109,6 +1115,7 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
             }
             fill_chunk(c, l, c->ls[l], dims, 0, cb, 0, tb, lb, need64, ch);
             ch.dyn = di + l;
+            ch.early = 0;                    // small steps: nothing to gain
             ch.host = c->h_info + l + 1;
             ch.seq = ++c->steps;
             ch.fit_recs = fit;
@@ -1390,10 +1397,11 @@ vote_status vote_create(int family, int d, int k, const double *eps, const doubl
     // step size measured fastest on GB300 (1e6-surface workloads): planes keep almost
     // every cell above the bound, so larger steps only remove per-step overhead;
     // 3DoF prunes well and needs fine depth-first steps
-    // a step's children can hold 2^d times its records: 64-child families take
-    // smaller steps so that the next level's records stay within a few GB
-    c->chunk_records = family == VOTE_PLANE3D_SPH ? (int64_t)1 << 27
-                       : (d >= 6 ? (int64_t)1 << 21 : (d >= 4 ? (int64_t)1 << 23 : (int64_t)1 << 25));
+    // a step's children can hold 2^d times its records: 13 GB at most with these (planes 9).
+    // The count pass needs tens of tiles per warp to share what it knows of a cell: steps of
+    // 2^23, 2^24, 2^25, 2^26 records, affine 4-space 37.5, 33.3, 30.1, 30.3 ms, radial 9.6, 9.1,
+    // 8.7, 8.4, point sets 7.6, 6.6, 6.4, 6.4; 2^21 to 2^24, 6DoF 6.0, 5.2, 4.7, 4.8.
+    c->chunk_records = family == VOTE_PLANE3D_SPH ? (int64_t)1 << 27 : (d >= 6 ? (int64_t)1 << 23 : (int64_t)1 << 25);
     c->family = family;
     if (const char *lg = std::getenv("VOTE_LOG")) c->log = std::atoi(lg) > 0 ? std::atoi(lg) : 0;
     for (int j = 0; j < d; ++j) {

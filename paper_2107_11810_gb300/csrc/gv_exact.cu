@@ -62,12 +62,10 @@ __global__ void __launch_bounds__(256) k_count_exact(const __grid_constant__ Chu
     grid_start();
     const int lane = threadIdx.x & 31;
     const int64_t nwarp = (int64_t)gridDim.x * 8, nt = chunk_tiles(c);
-    unsigned nrec = 0;
     for (int64_t tt = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); tt < nt; tt += nwarp) {
         const int2 ti = c.tinfo[tt];
         if (ti.x < 0) continue;                                     // uniform: the cell was pruned
         const int nvalid = ti.y & 63;
-        nrec += (unsigned)nvalid;
         SlotMask<FAM> ubm = 0, lbm = 0;
         if (lane < nvalid) eval_record<FAM, Q16>(c, (c.t0 + tt) * 32 + lane, ti.x, 0, c.nfs, ubm, lbm);
         uint32_t *bp = c.ballot + (size_t)tt * c.ns, *lp = c.lballot + (size_t)tt * c.ns;
@@ -78,10 +76,6 @@ __global__ void __launch_bounds__(256) k_count_exact(const __grid_constant__ Chu
                 if (c.lb) lp[s] = bl;
             }
         }
-    }
-    if (lane == 0 && nrec) {
-        atomicAdd(&c.sc->records, (unsigned long long)nrec);
-        atomicAdd(&c.sc->tests, (unsigned long long)nrec * c.ns);
     }
 }
 

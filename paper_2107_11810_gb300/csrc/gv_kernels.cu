@@ -205,7 +205,9 @@ __global__ void __launch_bounds__(256) k_rot_fill(const __grid_constant__ Chunk 
 // of two; the screen's coefficient is the rounded change times that power), and per basis
 // value the largest magnitude (rounded up), which bounds the snap's band; in plain FP64
 // mode, and where there are no tables, the FP64 changes too.  Per tile its cell (-1: pruned), how many of its 32 lanes
-// hold records, and whether it is its cell's first or last tile.
+// hold records, whether it is its cell's first or last tile, and the cell's allowance: of N
+// records all but the threshold may fail a child's test.  Of cells with more than four times
+// the threshold the count pass could leave a tenth untested at most: they are counted whole.
 __device__ __forceinline__ void tile_info(const Chunk &c, int64_t i, unsigned thr) {
     const int64_t nt = chunk_tiles(c);
     if (i >= nt + 2) return;
@@ -215,10 +217,16 @@ __device__ __forceinline__ void tile_info(const Chunk &c, int64_t i, unsigned th
     if (i < nt && !(c.sc->err & kErrTimeout)) {
         const int64_t t = c.t0 + i, cell = (int64_t)c.in.tile_cell[t];
         const int cl = (int)(cell - c.in_c0);
-        const int64_t r0 = (int64_t)c.in_rbeg[cell], left = r0 + (int64_t)c.in_rcnt[cell] - 32 * t;
-        ti = make_int2(c.cells.ub[c.c0 + cl] >= thr ? cl : -1, (left < 32 ? (int)left : 32) |
-                                                                   (32 * t == r0 ? kTileFirst : 0) |
-                                                                   (left <= 32 ? kTileLast : 0));
+        const unsigned N = c.in_rcnt[cell];
+        const int64_t r0 = (int64_t)c.in_rbeg[cell], left = r0 + (int64_t)N - 32 * t;
+        const unsigned allow = c.early && N >= thr && N / 4 <= thr && N - thr < 8u * (kAllowNone - 1u)
+                                   ? (N - thr + 7u) / 8u : kAllowNone;
+        const int64_t after = (left - 1) >> 5;
+        ti = make_int2(c.cells.ub[c.c0 + cl] >= thr ? cl : -1,
+                       (left < 32 ? (int)left : 32) | (32 * t == r0 ? kTileFirst : 0) |
+                           (left <= 32 ? kTileLast : 0) |
+                           (int)(after < kLeftMax ? after : kLeftMax) << kLeftShift |
+                           ((N + 31u) / 32u <= (unsigned)c.early ? kTileOwned : 0) | (int)(allow << kAllowShift));
     }
     c.tinfo[i] = ti;
 }
@@ -232,12 +240,21 @@ __global__ void __launch_bounds__(256) k_prep(const __grid_constant__ Chunk c) {
     const unsigned thr = prune_threshold(c.P, c.sc, c.prune);
     const int nc = chunk_cells(c);
     if (c.dyn && nc == 0) return;                    // the chain has stopped: the last step's scratch stays
-    if (gid == 0) c.sc->n_uns = 0u;                  // this step's recheck queue
-    if (gid < nc) c.alive[gid] = c.cells.ub[c.c0 + gid] >= thr ? 1 : 0;
+    if (gid == 0) c.sc->n_uns = c.sc->ticket = 0u;   // this step's recheck queue and tile units
+    if ((gid & ~31ll) < nc) {                        // uniform: a warp's cells
+        const bool live = gid < nc && c.cells.ub[c.c0 + gid] >= thr;
+        if (gid < nc) c.alive[gid] = live ? 1 : 0;
+        // (a cell's records and tests count whether or not the count pass leaves it early)
+        const unsigned n = live ? c.in_rcnt[c.in_c0 + gid] : 0u;
+        const unsigned long long r = __reduce_add_sync(kFull, n & 0xffffu) +
+                                     ((unsigned long long)__reduce_add_sync(kFull, n >> 16) << 16);
+        if ((gid & 31) < 2 && r) atomicAdd((gid & 31) ? &c.sc->tests : &c.sc->records, (gid & 31) ? r << c.lns : r);
+    }
     for (int64_t x = gid, nch = (int64_t)nc << c.lns; x < nch; x += gridDim.x * 256ll) {
         c.crec[x] = 0u;                              // the children's counters
         c.clb[x] = 0u;
         if (c.weighted) c.cub[x] = 0u;
+        if (c.early) c.cfail[x] = 0u;
     }
     tile_info(c, gid, thr);
     if (c.geo64) {
@@ -833,7 +850,7 @@ __global__ void __launch_bounds__(256) k_tile_scan(const __grid_constant__ Chunk
     const int64_t t = (blockIdx.x * 8ll + (threadIdx.x >> 5)) * 32 + lane;
     if (t - lane >= nt) return;                                          // uniform
     const int2 ti = t < nt ? c.tinfo[t] : make_int2(-1, 0);
-    const int cl = ti.x;
+    const int cl = ti.x >= 0 && c.early && !c.alive[ti.x] ? -1 : ti.x;   // left by the count pass: no child survives
     const int prev = __shfl_up_sync(kFull, cl, 1);
     const unsigned heads = __ballot_sync(kFull, lane == 0 || prev != cl);
     const int next = __shfl_down_sync(kFull, cl, 1);

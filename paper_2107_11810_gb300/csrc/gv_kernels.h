@@ -43,7 +43,7 @@ struct Scalars {
     unsigned long long replay_ub;    // replay: surfaces reaching the target cell
     unsigned long long replay_lb;    // replay: ... passing its lower-bound test
     unsigned int err;                // nonzero: input out of range
-    unsigned int pad2;
+    unsigned int ticket;             // units of tiles handed out by the step's count pass
     unsigned int qmax[GV_MAXD + GV_MAXT];  // lift: largest |q_f,j|, |q_t,m| of the root records
     unsigned long long rechecks_df;  // snaps the double-float tier decided (FP32 screen undecided)
 };
@@ -86,8 +86,8 @@ struct Chunk {
     const uint32_t *in_rcnt; // its record count
     int64_t in_c0;
     int64_t t0, t1;          // tile range of the chunk
-    uint8_t *alive;          // [nc]   bit 0: cell still above the pruning threshold; bit 1: it has a
-                             //        surviving child
+    uint8_t *alive;          // [nc]   bit 0: cell still above the pruning threshold, and not left by the count
+                             //        pass; bit 1: it has a surviving child
     // cell geometry: the changes of the cell-dependent basis values (Fam::NBG) from the
     // cell centre to the child centres, one per geometry slot (the free slots without a
     // linear tail coordinate's bit)
@@ -103,7 +103,7 @@ struct Chunk {
     uint32_t *crec, *clb;    // [nc][ns]  records (UB-passing) and LB sum per child
     uint32_t *cub;           // [nc][ns]  UB sum per child (= crec without multiplicities)
     int2 *tinfo;             // [t1 - t0 + 2] per tile: chunk-local cell (-1: pruned), valid lanes | kTileFirst |
-                             //           kTileLast
+                             //           kTileLast | tiles left << kLeftShift | allowance << kAllowShift
     uint32_t *ballot;        // [t1 - t0][ns] per tile and child: UB-passing lanes
     uint32_t *lballot;       // [t1 - t0][ns] the same for the LB test
     uint2 *uns;              // queue of (tile, lanes) the FP32 screen left undecided, sc->n_uns entries
@@ -123,6 +123,10 @@ struct Chunk {
     int prune;
     int precision;           // 0 = FP64, 1 = FP32 screen + FP64 recheck
     int lb;                  // lower bounds are wanted (lballot, clb)
+    int early;               // the count pass leaves cells whose children all fall below the threshold; it
+                             // takes cells of at most this many tiles (>= 1) whole, a warp each
+    uint32_t *cfail;         // [nc][ns] early: records that certainly fail each child's UB test, of cells that
+                             //          several warps count (child_idx's memory, which is written after)
     unsigned spin;           // polls of a bounded wait for a bulk copy before giving up
 };
 // The kernels of a step depend on one another and most are short: each is launched while
@@ -161,6 +165,12 @@ inline void launch(void (*kernel)(P...), unsigned blocks, unsigned threads, size
 __device__ __forceinline__ int64_t chunk_tiles(const Chunk &c) { return c.dyn ? c.dyn->nrecs >> 5 : c.t1 - c.t0; }
 __device__ __forceinline__ int chunk_cells(const Chunk &c) { return c.dyn ? (int)c.dyn->ncells : c.nc; }
 constexpr int kTileFirst = 64, kTileLast = 128;   // flags in tinfo.y: first / last tile of its cell
+// the cell's tiles after it, at most kLeftMax (more are not skipped at once); kTileOwned: one
+// warp of the count pass takes the whole cell; and how many of the
+// cell's records may fail a child's UB test while the child can still reach the threshold, in
+// eights rounded up (kAllowNone: the cell is counted in any case)
+constexpr int kLeftShift = 8, kLeftMax = 127, kTileOwned = 1 << 15, kAllowShift = 16;
+constexpr unsigned kAllowNone = 0xffffu;
 
 constexpr int kNoExp = -1000;
 

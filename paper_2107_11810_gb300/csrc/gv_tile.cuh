@@ -212,6 +212,138 @@ __device__ __forceinline__ int32_t resnap_half(int32_t q) {
 }
 
 // ---------------------------------------------------------------------------
+// The count pass's way through a step's tiles, and cells it leaves early.
+//
+// A child whose records can no longer reach the threshold is pruned whatever the rest of
+// its cell's records give, so a cell is left once that is certain of all its children: once
+// each has more certain failures than the cell's allowance (records minus threshold).  A
+// share (1 - threshold / N) / (1 - largest child / N) of a cell's N records settles that,
+// and the levels that hold most records are those whose cells lie just above the
+// threshold: of all records a search opens, planes of 1e4 points need 0.50, of 1e6 points
+// 0.59, affine 4-space 0.36, point sets 0.66, radial 0.42; with whole batches and units
+// 0.65, 0.70, 0.48, 0.79 and 0.64 are tested.  The surviving children's counts, and with
+// them the search, are the same.  GB300, count passes and tile scans: planes of 1e6 points
+// 275 -> 225 ms, of 1e4 points 9.9 -> 8.3, affine 25.8 -> 20.4, radial 6.1 -> 5.1 (steps of
+// 2^23 records in the last two).
+// ---------------------------------------------------------------------------
+
+// Warps take units of consecutive tiles: the first tickets, one per warp, are the first
+// units of equal parts of the step, the next ones the second units, and so on.  So few
+// warps are in one cell at a time, and those that leave cells early take more tickets.
+// Few tiles, or no early leaving: one unit per warp.
+//
+// Ballots are staged in shared memory, a batch of 32 / ns tiles at a time (one tile with 32 or
+// more child slots), and stored from there by all lanes; a batch's words are also counted
+// there, lane s of every ns for child slot s (and 32 + s).  Most of this work is a batch's, and
+// little a tile's: the pass is bound by instruction issue.
+template <int V, bool LB>
+struct CellWatch {
+    // a warp's shared memory: rows of a batch (with LB those of the lower bounds after them), the
+    // step's units and their size
+    static constexpr int UNITS = LB ? 64 * V : 32 * V, SIZE = UNITS + 1, WORDS = UNITS + 4;
+    uint32_t *s;
+    // the run of tiles at hand: its decided records, those of them that passed (per lane), both
+    // since it began or since they were added up; more decided records than lim are looked at
+    unsigned cnt, pass[V], lim;
+
+    __device__ __forceinline__ static unsigned allowance(int2 ti) { return ((unsigned)ti.y >> kAllowShift) * 8u; }
+    __device__ __forceinline__ static bool watched(int2 ti) { return (unsigned)ti.y >> kAllowShift != kAllowNone; }
+    __device__ __forceinline__ static int after(int2 ti) { return (ti.y >> kLeftShift) & kLeftMax; }
+
+    // The step's units of nt tiles, and this warp's first (its ticket is the warp's number):
+    // tiles [tt, tb), none if tt >= tb.
+    __device__ __forceinline__ void split(const Chunk &c, unsigned nt, unsigned warp, int lane, unsigned &tt,
+                                          unsigned &tb) {
+        const unsigned W = gridDim.x * 8u, per = (nt + W - 1u) / W;
+        unsigned size = per, S = 1u;
+        if (c.early && per >= 16u) {
+            size = per >= 512u ? 64u : (per >= 256u ? 32u : (per >= 32u ? 16u : 8u));
+            S = (per + size - 1u) / size;
+        }
+        if (lane == 0) {
+            s[UNITS] = S;
+            s[SIZE] = size;
+        }
+        const unsigned long long at = (unsigned long long)warp * S * size;
+        tt = at < nt ? (unsigned)at : nt;
+        tb = nt - tt < size ? nt : tt + size;
+        __syncwarp();
+    }
+    // tiles of a later ticket's unit; false: there is none
+    __device__ __forceinline__ bool unit(unsigned ticket, unsigned nt, unsigned &tt, unsigned &tb) const {
+        const unsigned W = gridDim.x * 8u, S = s[UNITS], size = s[SIZE];
+        if (S <= 1u || ticket / W >= S) return false;
+        const unsigned long long at = ((unsigned long long)(ticket % W) * S + ticket / W) * size;
+        tt = at < nt ? (unsigned)at : nt;
+        tb = nt - tt < size ? nt : tt + size;
+        return true;
+    }
+    // asks for the next ticket (lane 0 has it)
+    __device__ __forceinline__ unsigned next(const Chunk &c, int lane) const {
+        const unsigned W = gridDim.x * 8u;
+        return s[UNITS] > 1u && lane == 0 ? W + atomicAdd(&c.sc->ticket, 1u) : 0xffffffffu;
+    }
+
+    // a run of tiles begins with tile ti
+    __device__ __forceinline__ void run(int2 ti) {
+        cnt = 0u;
+#pragma unroll
+        for (int v = 0; v < V; ++v) pass[v] = 0u;
+        lim = !watched(ti) ? 0xffffffffu : ((ti.y & kTileOwned) ? allowance(ti) : 511u);
+    }
+    // A unit begins with tile ti: how many tiles of its cell are not this unit's (all, if the
+    // cell is the warp's that has its first tile, or if others know that it can be left).
+    __device__ __forceinline__ unsigned begin(const Chunk &c, int ns, int2 ti, int lane) const {
+        if (ti.x < 0 || (ti.y & kTileFirst)) return 0u;
+        if (ti.y & kTileOwned) return 1u + after(ti);
+        if (!watched(ti)) return 0u;
+        const uint32_t *p = c.cfail + (size_t)ti.x * ns + (lane & (ns - 1));
+        bool d = true;
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+            if (v == 0 || ns > 32) d &= __ldcg(p + 32 * v) > allowance(ti);
+        if (!__all_sync(kFull, d)) return 0u;
+        if (lane == 0) c.alive[ti.x] = 0;
+        return 1u + after(ti);
+    }
+    // A batch's ballots (word[v]: the lane's, 0 past its end) have been stored; its rows from
+    // `first` on belong to the last run.
+    __device__ __forceinline__ void add(int ns, int lns, const unsigned *word, int first, int lane) {
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+            if ((v == 0 || ns > 32) && lane >> lns >= first) pass[v] += (unsigned)__popc(word[v]);
+    }
+    // After the batch whose last tile ti is tile tt - 1, when cnt exceeds lim or the unit ends
+    // (tb; a cell that is this warp's moves it): how many of the tiles from tt on need not be
+    // counted.
+    __device__ __forceinline__ unsigned look(const Chunk &c, int ns, int2 ti, unsigned tt, unsigned &tb, int lane) {
+        if (ti.x < 0) return 0u;
+        const unsigned rest = after(ti), allow = allowance(ti);
+        const bool owned = ti.y & kTileOwned;
+        if (owned && tt >= tb) tb = tt + rest;
+        if (!watched(ti)) return 0u;
+        bool d = true;
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+            if (v > 0 && ns <= 32) continue;
+            unsigned f = pass[v];
+            for (int o = ns; o < 32; o <<= 1) f += __shfl_xor_sync(kFull, f, o);
+            f = cnt - f;
+            if (!owned) {                                // others count the cell too: all failures are added up
+                if (lane < ns) f += atomicAdd(c.cfail + (size_t)ti.x * ns + lane + 32 * v, f);
+                f = __shfl_sync(kFull, f, lane & (ns - 1));             // modulo 32
+                pass[v] = 0u;
+            }
+            d &= f > allow;
+        }
+        if (!owned) cnt = 0u;
+        if (!__all_sync(kFull, d)) return 0u;
+        if (lane == 0) c.alive[ti.x] = 0;
+        return rest;
+    }
+};
+
+// ---------------------------------------------------------------------------
 // Cell geometry: the changes of the basis values from a cell's centre to its children's.
 // ---------------------------------------------------------------------------
 

@@ -7,9 +7,9 @@
 // warp's part of shared memory once per run of tiles of one cell, transposed so that
 // one load serves the coefficients of a whole group.
 //
-// Each warp takes a contiguous range of the chunk's tiles (so runs of tiles of one
-// cell stay together) and reads its records with plain loads; there are no
-// device-side waits.
+// Warps of the count pass take units of consecutive tiles and leave cells early (CellWatch);
+// those of the emit pass a contiguous range of tiles.  Both read their records with plain
+// loads; there are no device-side waits.
 #include "gv_tile.cuh"
 
 namespace gv {
@@ -36,9 +36,15 @@ __device__ __forceinline__ void stage_coefs(const Chunk &c, int cell, float *sg,
         }
 }
 
+// Blocks per SM that the registers have to leave room for: as many as the tests alone need
+// (affine 4-space 40 registers), whatever the rare paths would like (56).
+constexpr int wide_residents(int fam, bool lb) {
+    return fam == FAM_AFFINE4D ? (lb ? 5 : 6) : (fam == FAM_POSE6DOF ? 2 : (lb ? 3 : 4));
+}
+
 // FG: free slots per group (4, or all of them when fewer split)
 template <int FAM, bool Q16, int FG, int DM, bool LB>
-__global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chunk c) {
+__global__ void __launch_bounds__(256, wide_residents(FAM, LB)) k_count_wide(const __grid_constant__ Chunk c) {
     grid_start();
     using F = Fam<FAM>;
     constexpr int ND = F::ND, LE = F::LE, NDS = dep_slots(DM), NX = ND * LE;
@@ -50,8 +56,17 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
     const int nfs = c.nfs;
     int run = -1;
     const int64_t nt = chunk_tiles(c);
-    const int64_t nwarp = (int64_t)gridDim.x * 8, gw = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int64_t ta = gw * nt / nwarp, tb = (gw + 1) * nt / nwarp;
+    constexpr int V = (1 << F::D) > 32 ? 2 : 1, ROW = 32 * V;       // a batch: BT tiles' rows of ns ballots
+    const int ns = c.ns, BT = ns < 32 ? 32 >> c.lns : 1;
+    using W = CellWatch<V, LB>;
+    __shared__ __align__(16) uint32_t s_watch[8][W::WORDS];          // whole 16 bytes per warp
+    W watch;
+    watch.s = s_watch[threadIdx.x >> 5];
+    watch.run(make_int2(-1, -1));
+    uint32_t *rows = watch.s;
+    if (nt == 0) return;                                            // the chain has stopped
+    unsigned tt, tb;
+    watch.split(c, (unsigned)nt, blockIdx.x * 8u + (threadIdx.x >> 5), lane, tt, tb);
     const Level &lev = c.lev;
     float hs[ND];
     f2 negL2[ND];
@@ -60,96 +75,133 @@ __global__ void __launch_bounds__(256) k_count_wide(const __grid_constant__ Chun
         hs[j] = lev.Hs[j];
         negL2[j] = f2_dup(-lev.Lc[j] * lev.Lc[j]);
     }
-    unsigned nrec = 0;
-
-#pragma unroll 1
-    for (int64_t tt = ta; tt < tb; ++tt) {
-        const int2 ti = c.tinfo[tt];
-        const int cell = ti.x;
-        if (cell < 0) continue;                                     // uniform: the cell was pruned
-        uint32_t w[NW];
-        load_words<NW>(c.in.rec, (c.t0 + tt) * 32 + lane, w);       // whole tiles are allocated
-        if (F::NBG > 0 ? cell != run : run < 0) {                   // uniform: a new cell (linear bases: once)
-            __syncwarp();                                           // the old cell's reads are done
-            stage_coefs<FAM, false>(c, cell, sg, lane);
-            __syncwarp();
-            run = cell;
-        }
-        const int nvalid = ti.y & 63;
-        nrec += (unsigned)nvalid;
-        float qf[ND], qt[LE], R[ND], near[ND], nearL[ND];
-        f2 negR2[ND];
-#pragma unroll
-        for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
-#pragma unroll
-        for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
-        F::radius32(lev, qt, R);
-#pragma unroll
-        for (int j = 0; j < ND; ++j) {
-            negR2[j] = f2_dup(-R[j] * R[j]);
-            near[j] = nearL[j] = 3.0e38f;
-        }
-        // a lane without a record fails every test (its residual is out of reach)
-        if (lane >= nvalid) qf[0] = 1.0e15f;
-        uint32_t *bp = c.ballot + (size_t)tt * c.ns, *lp = c.lballot + (size_t)tt * c.ns;
-#pragma unroll 1
-        for (int fs = 0; fs < nfs; fs += FG) {
-            f2 u[ND][(FG + 1) / 2];
-#pragma unroll
-            for (int j = 0; j < ND; ++j) {
-#pragma unroll
-                for (int p = 0; p < (FG + 1) / 2; ++p) u[j][p] = f2_dup(qf[j]);
-#pragma unroll
-                for (int m = 0; m < LE; ++m) {
-                    if (!F::uses(j, m)) continue;
-                    const float *g = sg + (j * LE + m) * nfs + fs;
-                    const f2 q2 = f2_dup(qt[m]);
-                    if constexpr (FG == 4) {
-                        const ulonglong2 g4 = *reinterpret_cast<const ulonglong2 *>(g);
-                        u[j][0] = f2_fma(q2, g4.x, u[j][0]);
-                        u[j][1] = f2_fma(q2, g4.y, u[j][1]);
-                    } else if constexpr (FG == 2) {
-                        u[j][0] = f2_fma(q2, *reinterpret_cast<const f2 *>(g), u[j][0]);
-                    } else {
-                        u[j][0] = f2_fma(q2, f2_dup(g[0]), u[j][0]);
-                    }
+    bool staged = false;
+    unsigned next;
+    do {
+        next = watch.next(c, lane);
+        bool head = true;
+        run = -1;
+        while (tt < tb) {
+            int2 ti;
+            if (head && c.early) {
+                ti = c.tinfo[tt];
+                const unsigned skip = watch.begin(c, ns, ti, lane);
+                if (skip) {
+                    tt += skip;
+                    head = false;
+                    continue;
                 }
             }
-            unsigned bu[FG * NDS], bl[FG * NDS];
-            test_children<ND, FG, DM, LB>(u, hs, negR2, negL2, near, nearL, bu, bl);
-            if (lane == 0) {
+            head = false;
+            const int bt = tb - tt < (unsigned)BT ? (int)(tb - tt) : BT;
+            int rs = 0;                                             // first row of the last run
+#pragma unroll 1
+            for (int b = 0; b < bt; ++b) {
+                ti = c.tinfo[tt + b];
+                const int cell = ti.x;
+                if (cell < 0) continue;                                     // uniform: the cell was pruned
+                uint32_t w[NW];
+                load_words<NW>(c.in.rec, (c.t0 + (tt + b)) * 32 + lane, w);       // whole tiles are allocated
+                if (cell != run) {                                          // uniform: a new cell
+                    rs = b;
+                    watch.run(ti);
+                    if (F::NBG > 0 || !staged) {                            // linear bases: once
+                        __syncwarp();                                       // the old cell's reads are done
+                        stage_coefs<FAM, false>(c, cell, sg, lane);
+                        __syncwarp();
+                        staged = true;
+                    }
+                    run = cell;
+                }
+                const int nvalid = ti.y & 63;
+                watch.cnt += (unsigned)nvalid;
+                float qf[ND], qt[LE], R[ND], near[ND], nearL[ND];
+                f2 negR2[ND];
 #pragma unroll
-                for (int x = 0; x < NDS; ++x) {
-                    uint32_t *b = bp + x * nfs + fs, *l = lp + x * nfs + fs;
-                    if constexpr (FG == 4) {
-                        *reinterpret_cast<uint4 *>(b) = make_uint4(bu[4 * x], bu[4 * x + 1], bu[4 * x + 2], bu[4 * x + 3]);
-                        if constexpr (LB)
-                            *reinterpret_cast<uint4 *>(l) = make_uint4(bl[4 * x], bl[4 * x + 1], bl[4 * x + 2], bl[4 * x + 3]);
-                    } else {
+                for (int j = 0; j < ND; ++j) qf[j] = field_f<Q16>(w, j);
 #pragma unroll
-                        for (int f = 0; f < FG; ++f) {
-                            b[f] = bu[FG * x + f];
-                            if constexpr (LB) l[f] = bl[FG * x + f];
+                for (int m = 0; m < LE; ++m) qt[m] = field_f<Q16>(w, ND + m);
+                F::radius32(lev, qt, R);
+#pragma unroll
+                for (int j = 0; j < ND; ++j) {
+                    negR2[j] = f2_dup(-R[j] * R[j]);
+                    near[j] = nearL[j] = 3.0e38f;
+                }
+                // a lane without a record fails every test (its residual is out of reach)
+                if (lane >= nvalid) qf[0] = 1.0e15f;
+                uint32_t *bp = rows + b * ns, *lp = rows + ROW + b * ns;
+#pragma unroll 1
+                for (int fs = 0; fs < nfs; fs += FG) {
+                    f2 u[ND][(FG + 1) / 2];
+#pragma unroll
+                    for (int j = 0; j < ND; ++j) {
+#pragma unroll
+                        for (int p = 0; p < (FG + 1) / 2; ++p) u[j][p] = f2_dup(qf[j]);
+#pragma unroll
+                        for (int m = 0; m < LE; ++m) {
+                            if (!F::uses(j, m)) continue;
+                            const float *g = sg + (j * LE + m) * nfs + fs;
+                            const f2 q2 = f2_dup(qt[m]);
+                            if constexpr (FG == 4) {
+                                const ulonglong2 g4 = *reinterpret_cast<const ulonglong2 *>(g);
+                                u[j][0] = f2_fma(q2, g4.x, u[j][0]);
+                                u[j][1] = f2_fma(q2, g4.y, u[j][1]);
+                            } else if constexpr (FG == 2) {
+                                u[j][0] = f2_fma(q2, *reinterpret_cast<const f2 *>(g), u[j][0]);
+                            } else {
+                                u[j][0] = f2_fma(q2, f2_dup(g[0]), u[j][0]);
+                            }
+                        }
+                    }
+                    unsigned bu[FG * NDS], bl[FG * NDS];
+                    test_children<ND, FG, DM, LB>(u, hs, negR2, negL2, near, nearL, bu, bl);
+                    if (lane == 0) {
+#pragma unroll
+                        for (int x = 0; x < NDS; ++x) {
+                            uint32_t *b = bp + x * nfs + fs, *l = lp + x * nfs + fs;
+                            if constexpr (FG == 4) {
+                                *reinterpret_cast<uint4 *>(b) = make_uint4(bu[4 * x], bu[4 * x + 1], bu[4 * x + 2], bu[4 * x + 3]);
+                                if constexpr (LB)
+                                    *reinterpret_cast<uint4 *>(l) = make_uint4(bl[4 * x], bl[4 * x + 1], bl[4 * x + 2], bl[4 * x + 3]);
+                            } else {
+#pragma unroll
+                                for (int f = 0; f < FG; ++f) {
+                                    b[f] = bu[FG * x + f];
+                                    if constexpr (LB) l[f] = bl[FG * x + f];
+                                }
+                            }
                         }
                     }
                 }
+                const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
+                const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, near, nearL)) & act;
+                if (unsb) {                                                 // rare: left to the definition
+                    __syncwarp();                                           // lane 0's stores
+                    for (int s = lane; s < ns; s += 32) {
+                        bp[s] &= ~unsb;
+                        if constexpr (LB) lp[s] &= ~unsb;
+                    }
+                    watch.cnt -= (unsigned)__popc(unsb);
+                    if (lane == 0) c.uns[atomicAdd(&c.sc->n_uns, 1u)] = make_uint2(tt + b, unsb);
+                }
             }
-        }
-        const unsigned act = nvalid >= 32 ? kFull : (1u << nvalid) - 1u;
-        const unsigned unsb = __ballot_sync(kFull, undecided<FAM, LB>(lev, R, near, nearL)) & act;
-        if (unsb) {                                                 // rare: left to the definition
-            __syncwarp();                                           // lane 0's stores
-            for (int s = lane; s < c.ns; s += 32) {
-                bp[s] &= ~unsb;
-                if constexpr (LB) lp[s] &= ~unsb;
+            __syncwarp();
+            unsigned word[V];
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                word[v] = 0u;
+                if (lane + 32 * v < bt * ns) {
+                    word[v] = rows[lane + 32 * v];
+                    c.ballot[(size_t)tt * ns + lane + 32 * v] = word[v];
+                    if constexpr (LB) c.lballot[(size_t)tt * ns + lane + 32 * v] = rows[ROW + lane + 32 * v];
+                }
             }
-            if (lane == 0) c.uns[atomicAdd(&c.sc->n_uns, 1u)] = make_uint2((unsigned)tt, unsb);
+            __syncwarp();
+            tt += (unsigned)bt;
+            watch.add(ns, c.lns, word, rs, lane);
+            if (watch.cnt > watch.lim || tt >= tb) tt += watch.look(c, ns, ti, tt, tb, lane);
         }
-    }
-    if (lane == 0 && nrec) {
-        atomicAdd(&c.sc->records, (unsigned long long)nrec);
-        atomicAdd(&c.sc->tests, (unsigned long long)nrec * c.ns);
-    }
+    } while (watch.unit(__shfl_sync(kFull, next, 0), (unsigned)nt, tt, tb));
 }
 
 // The emit pass (see gv_emit.cu): slot rows of a tile (output address, passing lanes)
@@ -371,7 +423,11 @@ template <int FAM, bool Q16, int FG, int DM>
 static void launch_wide(const Chunk &c, cudaStream_t st) {
     if constexpr (DM < (1 << Fam<FAM>::ND) && (FG > 1 || DM)) {
         const unsigned g = wide_blocks(c.t1 - c.t0);
-        if (c.lb) launch(k_count_wide<FAM, Q16, FG, DM, true>, g, 256, 0, st, c);
+        if (c.early)                                    // resident warps only: they share the units
+            launch_persistent(c.lb ? (const void *)k_count_wide<FAM, Q16, FG, DM, true>
+                                   : (const void *)k_count_wide<FAM, Q16, FG, DM, false>,
+                              0, g, c, st);
+        else if (c.lb) launch(k_count_wide<FAM, Q16, FG, DM, true>, g, 256, 0, st, c);
         else launch(k_count_wide<FAM, Q16, FG, DM, false>, g, 256, 0, st, c);
     }
 }
