@@ -109,9 +109,9 @@ typedef enum {
                                  for planes (their pruning hardly depends on the
                                  step size, so larger steps only save per-step
                                  overhead), 2^25 for the other families with d <= 5
-                                 (finer depth-first steps keep their pruning
-                                 effective) and 2^23 for d = 6 (a step's children
-                                 can hold 2^d times its records)                     */
+                                 and 2^23 for d = 6 (a step's children can hold 2^d
+                                 times its records); half of these for d >= 4 when
+                                 the search goes depth first (VOTE_OPT_DIVE 0)       */
     VOTE_OPT_TRACE_CAP = 4,   /* >0: record (level, coords, UB, LB) of every tested
                                  child, up to this many entries (debug; default 0)   */
     VOTE_OPT_GROUP = 5,       /* merging of identical canonical surfaces:
@@ -129,8 +129,9 @@ typedef enum {
     VOTE_OPT_DIVE = 11,       /* 1 or 2 (default): first follow the cells with the largest
                                  UBs and LBs down to the leaves, so pruning starts from
                                  a leaf's count, and again from levels that grow large;
-                                 0: off.  Results do not depend on it (Sec. 3.3: any
-                                 valid bound may prune)                              */
+                                 0: off, the search goes depth first.  Results do
+                                 not depend on it (Sec. 3.3: any valid bound may
+                                 prune)                                              */
     VOTE_OPT_SPIN_LIMIT = 12, /* polls of a bounded device-side wait (the proximity
                                  passes' wait for their bulk copies) before the kernel
                                  gives up and the solve returns VOTE_ETIMEOUT;

@@ -9,7 +9,8 @@
 // (emit pass, canonization of Sec. 3.2).  The order (search(), dive()) follows the
 // cells with the largest bounds down to the leaves first, which raises the pruning
 // bound to about its final value, then opens the rest level by level while the next
-// level has room, else the deepest level first.  The result does not depend on it.
+// level has room, else (and without dives) the deepest level first.  The result does
+// not depend on it.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -75,6 +76,7 @@ struct vote_ctx {
     cudaStream_t stream = 0;
     int precision = 1, prune = 1, group = 0;
     int64_t chunk_records = 1 << 25;
+    bool chunk_set = false;            // VOTE_OPT_CHUNK_RECORDS was given
     uint32_t initial_lb = 0;
     int kernel_timing = 0;
     int log = 0;               // VOTE_LOG=1: per-level counters on stderr after each solve;
@@ -647,6 +649,19 @@ static const int kRotBits = 21;
 // angular coordinates of at most this many splits have a (sin, cos) table (2 MB)
 static const int kSincosBits = 16;
 
+// Without dives the search goes depth first: the leaves below its first steps are then the
+// only ones that raise the pruning bound.  Level by level as with dives, point sets (150 x
+// 150, dives off) took 15.4 ms and 7.2 GB, 6.5 ms and 4.1 GB depth first.
+static bool depth_first(const vote_ctx *c) { return !(c->dive && c->prune); }
+
+// Records of an expansion step.  Depth first every step starts from the bounds that the one
+// before found, so with 16 and more children a default step is half as large: steps of 1 / 2
+// / 4 times 2^23 records (6DoF 2^21), dives off, ms: point sets 4.8 / 6.5 / 9.8, radial 23 /
+// 13 / 16, affine 4-space 88 / 75 / 68 and 178 / 146 / 130, 6DoF 37 / 34 / 39.
+static int64_t step_records(const vote_ctx *c) {
+    return depth_first(c) && !c->chunk_set && c->P.d >= 4 ? c->chunk_records / 2 : c->chunk_records;
+}
+
 // records expanded with lower bounds outside dives
 static int64_t lb_records(int d) { return d <= 3 ? (int64_t)1 << 28 : (int64_t)1 << 22; }
 
@@ -839,17 +854,18 @@ static const int64_t kSmallStep = 2048, kSmallChain = 8192;
 static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     LevelStore &S = beam ? c->beam : c->ls[l];
     const Level &lev = c->lev[l];
-    // chunk: cells [c0, c1) from the top of the stack, about chunk_records records
+    // chunk: cells [c0, c1) from the top of the stack, about step_records(c) records
     const int64_t c1 = S.ncells, r1 = S.nrecs;
     int64_t avg = S.nrecs / (S.ncells > 0 ? S.ncells : 1);
-    int64_t K = c->chunk_records / (avg > 0 ? avg : 1);
+    const int64_t step = step_records(c);
+    int64_t K = step / (avg > 0 ? avg : 1);
     if (K < 1) K = 1;
     if (K > (1 << 22)) K = 1 << 22;
     int64_t c0, r0;
     for (;;) {
         c0 = c1 - K > 0 ? c1 - K : 0;
         if (beam) c0 = 0;
-        if (c0 == 0 && !c->kernel_timing && (beam || K == 1 || r1 <= 2 * c->chunk_records)) {
+        if (c0 == 0 && !c->kernel_timing && (beam || K == 1 || r1 <= 2 * step)) {
             r0 = 0;                                  // the level's first record: nothing to read back
             break;
         }
@@ -857,7 +873,7 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
         CK(cudaStreamSynchronize(c->stream));
         ev_collect(c);
         r0 = (int64_t)c->h_tmp[0];
-        if (beam || r1 - r0 <= 2 * c->chunk_records || K == 1) break;
+        if (beam || r1 - r0 <= 2 * step || K == 1) break;
         K = K / 2;
     }
     nvtxRangePushA("expand_chunk");
@@ -1028,7 +1044,7 @@ static vote_status dive(vote_ctx *c, int l0) {
         LevelStore &S = c->ls[l];
         if (S.ncells <= 0) return VOTE_OK;
         int64_t budget = std::max(kBeamRecords, S.nrecs / beam_divisor(c->P.d));
-        if (budget > c->chunk_records) budget = c->chunk_records;
+        if (budget > step_records(c)) budget = step_records(c);
         if (S.nrecs <= budget || S.ncells == 1) {
             TRY(expand_chunk(c, l));
             continue;
@@ -1078,7 +1094,7 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
     const Problem &P = c->P;
     const int L = P.L;
     *replayed = false;
-    const int64_t slots0 = c->ls[0].nrecs, fit = std::min(kBeamRecords, c->chunk_records) & ~(int64_t)31;
+    const int64_t slots0 = c->ls[0].nrecs, fit = std::min(kBeamRecords, step_records(c)) & ~(int64_t)31;
     if (slots0 > fit || c->group || c->kernel_timing || c->log >= 2) return VOTE_OK;
     TRY(ensure(c, c->linfo, sizeof(LevInfo) * (GV_MAXL + 1)));
     LevInfo *di = (LevInfo *)c->linfo.p;
@@ -1203,7 +1219,8 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
 // level's bounds are raised by all of its cells before its children are opened, while
 // the next level holds less than one step's records; when every level below is full,
 // the deepest first, which bounds the memory (room for 4 steps: a first solve of planes
-// with 1e6 points took 1564 ms instead of 1430 ms, more memory being mapped).  Whenever
+// with 1e6 points took 1564 ms instead of 1430 ms, more memory being mapped).  Without
+// dives: the deepest level first throughout (depth_first()).  Whenever
 // a level has grown large, another dive starts from it: its own UBs and LBs point better
 // than those of the levels above.  Measured against one root-to-leaf path of the largest
 // UB for n >= 2^17 and the deepest level first: point sets 132 -> 17 ms, 6DoF 47 -> 13,
@@ -1213,7 +1230,7 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
 static vote_status search(vote_ctx *c, const double *surfaces, int64_t n, uint32_t *mask, bool *replayed) {
     const int L = c->P.L;
     const bool dives = c->dive && c->prune;
-    const int64_t full = std::min(c->chunk_records, (int64_t)1 << 34);
+    const int64_t full = depth_first(c) ? 0 : std::min(step_records(c), (int64_t)1 << 34);   // records of a full level
     int64_t since[GV_MAXL + 1];          // records expanded into the level since its last dive
     for (int l = 0; l <= L; ++l) since[l] = -1;
     TRY(chain(c, surfaces, n, mask, replayed));
@@ -1460,6 +1477,7 @@ vote_status vote_set_option(vote_ctx *c, int key, double v) {
     case VOTE_OPT_CHUNK_RECORDS:
         if (!(v >= 1 && v <= 1e10)) break;
         c->chunk_records = (int64_t)v;
+        c->chunk_set = true;
         return VOTE_OK;
     case VOTE_OPT_TRACE_CAP: {
         if (!(v >= 0 && v <= 1e9)) break;
@@ -1569,6 +1587,7 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
         w->precision = c->precision;
         w->prune = c->prune;
         w->chunk_records = c->chunk_records;
+        w->chunk_set = c->chunk_set;
         w->dive = c->dive;
         w->group = c->group;
         w->spin_limit = c->spin_limit;
