@@ -820,20 +820,37 @@ static void fill_chunk(vote_ctx *c, int l, const LevelStore &S, const StepDims &
 
 // Waits until step number seq has reported into v (every step's report is its last but one
 // or last kernel; the stream's state is looked at now and then, so a failed launch ends it).
+// It polls for as long as a short step takes; after that it waits as the process has chosen
+// for the device (cudaSetDeviceFlags): blocked, or polling, with the core given up between
+// polls unless spinning was asked for.  A search that only polled took 442 ms of CPU time in
+// 495 ms under cudaDeviceScheduleBlockingSync (planes, 1e6 points, eps 0.03).
 static vote_status wait_report(vote_ctx *c, const LevInfo *v, long long seq) {
-    for (unsigned i = 1;; ++i) {
-        if (__atomic_load_n(&v->seq, __ATOMIC_ACQUIRE) == seq) return VOTE_OK;
-        if (i & 0xffffu) continue;           // some 100 us: queries take the lock that other threads launch under
-        const cudaError_t e = cudaStreamQuery(c->stream);
-        if (e == cudaErrorNotReady) {
-            cudaGetLastError();
-            continue;
+    auto reported = [&] { return __atomic_load_n(&v->seq, __ATOMIC_ACQUIRE) == seq; };
+    for (unsigned i = 0; i < 0x4000; ++i)    // some 20 us
+        if (reported()) return VOTE_OK;
+    unsigned flags = 0;
+    CK(cudaGetDeviceFlags(&flags));
+    const unsigned how = flags & cudaDeviceScheduleMask;
+    if (how == cudaDeviceScheduleBlockingSync) {
+        CK(cudaStreamSynchronize(c->stream));
+    } else {
+        // some 100 us between looks at the stream: they take the lock that other threads launch under
+        const unsigned every = how == cudaDeviceScheduleSpin ? 0xffffu : 0xffu;
+        for (unsigned i = 1; !reported(); ++i) {
+            if (how != cudaDeviceScheduleSpin) std::this_thread::yield();
+            if (i & every) continue;
+            const cudaError_t e = cudaStreamQuery(c->stream);
+            if (e == cudaErrorNotReady) {
+                cudaGetLastError();
+                continue;
+            }
+            CK(e);
+            break;
         }
-        CK(e);
-        if (__atomic_load_n(&v->seq, __ATOMIC_ACQUIRE) == seq) return VOTE_OK;
-        set_err("internal: an expansion step ended without its report");
-        return VOTE_EINTERNAL;
     }
+    if (reported()) return VOTE_OK;
+    set_err("internal: an expansion step ended without its report");
+    return VOTE_EINTERNAL;
 }
 
 // Lower bounds cost a third of the count pass.  Leaves need none (their own counts are
