@@ -111,7 +111,10 @@ typedef enum {
                                  overhead), 2^25 for the other families with d <= 5
                                  and 2^23 for d = 6 (a step's children can hold 2^d
                                  times its records); half of these for d >= 4 when
-                                 the search goes depth first (VOTE_OPT_DIVE 0)       */
+                                 the search goes depth first (VOTE_OPT_DIVE 0).  A
+                                 solve that runs out of device memory is repeated
+                                 depth first in steps of at most 2^23 records (d = 6:
+                                 2^21) before it returns VOTE_ENOMEM                 */
     VOTE_OPT_TRACE_CAP = 4,   /* >0: record (level, coords, UB, LB) of every tested
                                  child, up to this many entries (debug; default 0)   */
     VOTE_OPT_GROUP = 5,       /* merging of identical canonical surfaces:
@@ -212,7 +215,8 @@ vote_status vote_solve_host(vote_ctx *ctx, const double *surfaces, int64_t n, do
  *               the start of the call.
  * Problems are taken from a shared queue by VOTE_OPT_BATCH_WORKERS host workers,
  * each with its own stream and working memory, so small problems overlap on the
- * GPU.  Each problem's results equal those of vote_solve on it alone. */
+ * GPU; where memory is short, problems that found none are solved by fewer workers
+ * after the others.  Each problem's results equal those of vote_solve on it alone. */
 vote_status vote_solve_batched(vote_ctx *ctx, const double *surfaces, const int64_t *offsets, int B,
                                double *best_points, int64_t *best_leaves, int64_t *depths, uint32_t *masks,
                                double *latency_ms);

@@ -77,6 +77,8 @@ struct vote_ctx {
     int precision = 1, prune = 1, group = 0;
     int64_t chunk_records = 1 << 25;
     bool chunk_set = false;            // VOTE_OPT_CHUNK_RECORDS was given
+    bool lean = false;                 // the solve at hand is repeated with less memory (solve_device)
+    bool fault_hit = false;            // an allocation failed because the test hook asked for it
     uint32_t initial_lb = 0;
     int kernel_timing = 0;
     int log = 0;               // VOTE_LOG=1: per-level counters on stderr after each solve;
@@ -494,6 +496,7 @@ static vote_status ensure(vote_ctx *c, DevBuf &b, size_t bytes, size_t keep = 0)
     ++c->alloc_count;
     if (c->fault_alloc_at && c->alloc_count == c->fault_alloc_at) {
         set_err("injected allocation failure (allocation %lld)", (long long)c->alloc_count);
+        c->fault_hit = true;
         return VOTE_ENOMEM;
     }
     cudaError_t e = cudaMallocAsync(&b.p, want, c->stream);
@@ -515,6 +518,24 @@ static void release(vote_ctx *c, DevBuf &b) {
     if (b.p) cudaFreeAsync(b.p, c->stream);
     b.p = nullptr;
     b.bytes = 0;
+}
+
+// Gives back what solves have grown: the levels, the beam, the steps' scratch, the grouping's
+// tables, here and in the workers of batches (no solve of this context is running).
+static void release_working(vote_ctx *c) {
+    for (vote_ctx *w : c->workers) release_working(w);
+    for (int l = 0; l <= GV_MAXL + 1; ++l) {
+        LevelStore &s = l <= GV_MAXL ? c->ls[l] : c->beam;
+        DevBuf *bufs[] = {&s.rec, &s.mult, &s.tile_cell, &s.key, &s.rbeg, &s.rcnt, &s.ub, &s.lb};
+        for (DevBuf *b : bufs) release(c, *b);
+        s.ncells = s.nrecs = 0;
+    }
+    DevBuf *bufs[] = {&c->alive, &c->geo64, &c->geo32, &c->geo32lo, &c->cnt, &c->tinfo, &c->ballot, &c->lballot,
+                      &c->uns, &c->off, &c->cbase, &c->child_idx, &c->keepflag, &c->recn, &c->bsums, &c->g_table,
+                      &c->g_owner, &c->g_newpos, &c->g_ccount, &c->g_ccur, &c->g_rbeg, &c->g_rec, &c->g_mult,
+                      &c->g_tile, &c->beam_src};
+    for (DevBuf *b : bufs) release(c, *b);
+    cudaStreamSynchronize(c->stream);                      // free for others
 }
 
 // record fields and basis values of a family, from its device definition
@@ -651,14 +672,21 @@ static const int kSincosBits = 16;
 
 // Without dives the search goes depth first: the leaves below its first steps are then the
 // only ones that raise the pruning bound.  Level by level as with dives, point sets (150 x
-// 150, dives off) took 15.4 ms and 7.2 GB, 6.5 ms and 4.1 GB depth first.
-static bool depth_first(const vote_ctx *c) { return !(c->dive && c->prune); }
+// 150, dives off) took 15.4 ms and 7.2 GB, 6.5 ms and 4.1 GB depth first.  So it does where
+// memory is short: a level then holds what one step has left.
+static bool depth_first(const vote_ctx *c) { return c->lean || !(c->dive && c->prune); }
+
+// records of a step where memory is short
+static int64_t lean_records(const vote_ctx *c) {
+    return std::min(c->chunk_records, (int64_t)1 << (c->P.d >= 6 ? 21 : 23));
+}
 
 // Records of an expansion step.  Depth first every step starts from the bounds that the one
 // before found, so with 16 and more children a default step is half as large: steps of 1 / 2
 // / 4 times 2^23 records (6DoF 2^21), dives off, ms: point sets 4.8 / 6.5 / 9.8, radial 23 /
 // 13 / 16, affine 4-space 88 / 75 / 68 and 178 / 146 / 130, 6DoF 37 / 34 / 39.
 static int64_t step_records(const vote_ctx *c) {
+    if (c->lean) return lean_records(c);
     return depth_first(c) && !c->chunk_set && c->P.d >= 4 ? c->chunk_records / 2 : c->chunk_records;
 }
 
@@ -1237,7 +1265,7 @@ static vote_status chain(vote_ctx *c, const double *surfaces, int64_t n, uint32_
 // the next level holds less than one step's records; when every level below is full,
 // the deepest first, which bounds the memory (room for 4 steps: a first solve of planes
 // with 1e6 points took 1564 ms instead of 1430 ms, more memory being mapped).  Without
-// dives: the deepest level first throughout (depth_first()).  Whenever
+// dives, and where memory is short: the deepest level first throughout (depth_first()).  Whenever
 // a level has grown large, another dive starts from it: its own UBs and LBs point better
 // than those of the levels above.  Measured against one root-to-leaf path of the largest
 // UB for n >= 2^17 and the deepest level first: point sets 132 -> 17 ms, 6DoF 47 -> 13,
@@ -1297,11 +1325,26 @@ static void log_solve(const vote_ctx *c, vote_status st) {
     }
 }
 
+// One solve.  When device memory runs out, what the solve holds is given back and, where no
+// other solve of the same call holds memory (alone), it is repeated once depth first in small
+// steps, which need the least.  Measured, as a rule and so: 6DoF +-30 deg 39 GB, 48 ms and 6 GB,
+// 221 ms; planes of 1e6 points, eps 0.005, 106 GB, 13.0 s and 6 GB, 25.8 s; affine 4-space
+// 10 GB, 25 ms and 3.5 GB, 31 ms.
 static vote_status solve_device(vote_ctx *c, const double *surfaces, int64_t n, double *best_point,
-                                int64_t *best_leaf, int64_t *depth, uint32_t *mask) {
+                                int64_t *best_leaf, int64_t *depth, uint32_t *mask, bool alone = true) {
     nvtxRangePushA("vote_solve");
+    c->fault_hit = false;
     vote_status st = solve_inner(c, surfaces, n, best_point, best_leaf, depth, mask);
     if (st != VOTE_OK) cudaStreamSynchronize(c->stream);   // steps in flight report into this context
+    if (st == VOTE_ENOMEM && !c->fault_hit) {
+        release_working(c);
+        if (alone) {
+            c->lean = true;
+            st = solve_inner(c, surfaces, n, best_point, best_leaf, depth, mask);
+            if (st != VOTE_OK) cudaStreamSynchronize(c->stream);
+            c->lean = false;
+        }
+    }
     nvtxRangePop();
     if (c->log) log_solve(c, st);
     return st;
@@ -1431,8 +1474,9 @@ vote_status vote_create(int family, int d, int k, const double *eps, const doubl
     // step size measured fastest on GB300 (1e6-surface workloads): planes keep almost
     // every cell above the bound, so larger steps only remove per-step overhead;
     // 3DoF prunes well and needs fine depth-first steps
-    // a step's children can hold 2^d times its records: 13 GB at most with these (planes 9).
-    // The count pass needs tens of tiles per warp to share what it knows of a cell: steps of
+    // a step's children can hold 2^d times its records: of a step of just this size, with
+    // 16-bit fields, 9 GB (planes), 4 GB (16 children), 17 GB (radial camera, 6DoF).  A step
+    // can be twice as large; what whole solves held is at solve_device().  The count pass needs tens of tiles per warp to share what it knows of a cell: steps of
     // 2^23, 2^24, 2^25, 2^26 records, affine 4-space 37.5, 33.3, 30.1, 30.3 ms, radial 9.6, 9.1,
     // 8.7, 8.4, point sets 7.6, 6.6, 6.4, 6.4; 2^21 to 2^24, 6DoF 6.0, 5.2, 4.7, 4.8.
     c->chunk_records = family == VOTE_PLANE3D_SPH ? (int64_t)1 << 27 : (d >= 6 ? (int64_t)1 << 23 : (int64_t)1 << 25);
@@ -1615,6 +1659,11 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
     CK(cudaStreamSynchronize(c->stream));     // inputs written on the caller's stream are visible
     std::atomic<int> next(0);
     std::atomic<int> failed(0);
+    std::vector<int> todo(B), again;          // problems of this turn; those that found no memory in it
+    std::mutex again_mutex;
+    again.reserve(B);
+    for (int b = 0; b < B; ++b) todo[b] = b;
+    bool alone = false;                       // this context's other solves hold no memory
     std::vector<vote_status> wst(nw, VOTE_OK);
     std::vector<std::string> wmsg(nw);
     std::vector<vote_stats> wsum((size_t)nw);   // per worker: totals over its problems
@@ -1624,12 +1673,19 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
         vote_ctx *w = c->workers[wi];
         cudaSetDevice(c->device);
         for (;;) {
-            int b = next.fetch_add(1);
-            if (b >= B || failed.load()) break;
+            if (failed.load()) break;
+            const int i = next.fetch_add(1);
+            if (i >= (int)todo.size()) break;
+            const int b = todo[i];
             int64_t n = offsets[b + 1] - offsets[b];
             vote_status st = solve_device(w, surfaces + np * offsets[b], n, best_points + (size_t)b * d,
                                           best_leaves ? best_leaves + (size_t)b * d : nullptr, depths + b,
-                                          masks ? masks + wordoff[b] : nullptr);
+                                          masks ? masks + wordoff[b] : nullptr, alone);
+            if (st == VOTE_ENOMEM && !alone) {   // the other workers go on without this one
+                std::lock_guard<std::mutex> lock(again_mutex);
+                again.push_back(b);
+                break;
+            }
             if (st != VOTE_OK) {
                 wst[wi] = st;
                 wmsg[wi] = g_err;
@@ -1651,10 +1707,23 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
             a.launches += e.launches;
         }
     };
-    std::vector<std::thread> th;
-    for (int i = 1; i < nw; ++i) th.emplace_back(work, i);
-    work(0);
-    for (auto &t : th) t.join();
+    for (int k = nw;;) {
+        std::vector<std::thread> th;
+        for (int i = 1; i < k; ++i) th.emplace_back(work, i);
+        work(0);
+        for (auto &t : th) t.join();
+        const int done = std::min(next.load(), (int)todo.size());
+        again.insert(again.end(), todo.begin() + done, todo.end());
+        if (again.empty() || failed.load()) break;
+        // memory was short: what is left by half as many workers, at last by one, with what
+        // this context's solves hold given back
+        k = k / 2 > 1 ? k / 2 : 1;
+        alone = k == 1;
+        todo.swap(again);
+        again.clear();
+        next.store(0);
+        release_working(c);
+    }
     std::memset(&c->stats, 0, sizeof(c->stats));
     for (int i = 0; i < nw; ++i) {
         if (wst[i] != VOTE_OK) {
@@ -1898,16 +1967,9 @@ void vote_destroy(vote_ctx *c) {
         if (ws) cudaStreamDestroy(ws);
     }
     c->workers.clear();
-    for (int l = 0; l <= GV_MAXL + 1; ++l) {
-        LevelStore &s = l <= GV_MAXL ? c->ls[l] : c->beam;
-        release(c, s.rec); release(c, s.mult); release(c, s.tile_cell);
-        release(c, s.key); release(c, s.rbeg); release(c, s.rcnt); release(c, s.ub); release(c, s.lb);
-    }
-    DevBuf *bufs[] = {&c->levs_dev, &c->path, &c->scal, &c->alive, &c->geo64, &c->geo32, &c->geo32lo, &c->cnt, &c->tinfo,
-                      &c->ballot, &c->lballot, &c->uns, &c->off, &c->cbase, &c->child_idx, &c->keepflag, &c->recn, &c->bsums, &c->tr_level, &c->tr_key,
-                      &c->tr_ub, &c->tr_lb, &c->surf_tmp, &c->mask_tmp, &c->ss_partial,
-                      &c->ss_io, &c->g_table, &c->g_owner, &c->g_newpos, &c->g_ccount, &c->g_ccur,
-                      &c->g_rbeg, &c->g_rec, &c->g_mult, &c->g_tile, &c->beam_sel, &c->beam_src, &c->linfo};
+    release_working(c);
+    DevBuf *bufs[] = {&c->levs_dev, &c->path, &c->scal, &c->tr_level, &c->tr_key, &c->tr_ub, &c->tr_lb, &c->surf_tmp,
+                      &c->mask_tmp, &c->ss_partial, &c->ss_io, &c->beam_sel, &c->linfo};
     for (DevBuf *b : bufs) release(c, *b);
     for (DevBuf &b : c->sctab) release(c, b);
     release(c, c->psi0);
