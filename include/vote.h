@@ -154,11 +154,13 @@ typedef struct {
     int64_t records;         /* (cell, canonical surface) records of those cells  */
     int64_t tests;           /* (child cell, canonical surface) pairs decided: some
                                 without a predicate call, where a cell is left
-                                because none of its children can survive          */
+                                because none of its children can survive (see
+                                vote_get_evaluated)                               */
     int64_t rechecks;        /* tests re-evaluated in FP64 because the FP32 screen
                                 could not decide them (whole records: every child
                                 of a record with one uncertain test), plus child
-                                snaps taken in FP64                               */
+                                snaps taken in FP64; varies from run to run, by
+                                where cells that several warps share are left     */
     int64_t chunks;          /* expansion steps                                   */
     int64_t leaves;          /* leaves evaluated                                  */
     int64_t peak_records;    /* largest record count held at one level            */
@@ -289,6 +291,13 @@ vote_status vote_get_trace(vote_ctx *ctx, int64_t cap, int32_t *level, int64_t *
  * batch (levels and peak_records: the largest over its problems). */
 vote_status vote_get_stats(vote_ctx *ctx, vote_stats *out);
 
+/* The (child cell, canonical surface) pairs whose test the last solve evaluated (after
+ * vote_solve_batched, the batch): vote_stats.tests without the pairs of cells that were
+ * left because none of their children could survive.  Several warps may share a cell and
+ * leave it at different records, so this varies a little from run to run.  Counted when
+ * VOTE_OPT_KERNEL_TIMING is 1, else -1. */
+vote_status vote_get_evaluated(vote_ctx *ctx, int64_t *tests);
+
 /* Per kernel class (VOTE_K_*): summed device milliseconds, launches and
  * algorithmic bytes (records read/written, as defined per class) of the last
  * solve, measured with CUDA events when VOTE_OPT_KERNEL_TIMING is 1.  Arrays of
@@ -296,8 +305,8 @@ vote_status vote_get_stats(vote_ctx *ctx, vote_stats *out);
 vote_status vote_get_kernel_times(vote_ctx *ctx, double *ms, int64_t *launches, double *bytes);
 
 /* Per-level work of the last solve, for l in [0, L) (host arrays of at least L
- * entries, each may be NULL): cells[l] expanded and record slots[l] tested at
- * level l; with VOTE_OPT_GROUP on, grouped_in[l] records entered the grouping of
+ * entries, each may be NULL): cells[l] expanded at level l and their record
+ * slots[l]; with VOTE_OPT_GROUP on, grouped_in[l] records entered the grouping of
  * level l (the canonization's merge of equal canonical surfaces, Sec. 3.2) and
  * grouped_out[l] canonical records left it (both 0 with grouping off), so
  * 1 - grouped_out/grouped_in is the level's merge fraction. */

@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
             load_words<NW>(rp, 0, w1);
             float g1 = load_g(ti1.x);
             if (head) {
-                const unsigned skip = watch.begin(c, NS, ti1, lane);
+                const unsigned skip = watch.begin(c, NS, ti1, tt, tb, lane);
                 if (skip) {
                     tt += skip;
                     head = false;
@@ -199,6 +199,7 @@ __global__ void __launch_bounds__(256, 4) k_count(const __grid_constant__ Chunk 
             }
         }
     } while (watch.unit(__shfl_sync(kFull, next, 0), (unsigned)nt, tt, tb));
+    watch.report(c, NW, lane);
 }
 
 // a persistent grid: as many blocks as are resident (4 per SM), fewer when there are not

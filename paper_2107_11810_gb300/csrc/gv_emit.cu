@@ -161,8 +161,9 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
     int t1, cells1, nfail = -1;                                     // copy that did not arrive
     next_group(t1, cells1);
     if (t1 >= 0 && lane == 0) issue(0, t1);
+    int n = 0;                                                      // groups read
 #pragma unroll 1
-    for (int n = 0; t1 >= 0; ++n) {
+    for (; t1 >= 0; ++n) {
         const int b = n & 1, t0 = t1, cells = cells1;
         next_group(t1, cells1);
         if (t1 >= 0 && lane == 0) issue(n + 1, t1);
@@ -364,13 +365,15 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
     if (nfail >= 0 && lane == 0) {
         // the copies nfail and nfail + 1 (no later one was issued) may still be in flight:
         // wait for them, bounded, before the block's shared memory is released
-        for (int n = nfail; n < nfail + (t1 >= 0 ? 2 : 1); ++n)
-            if (!mbar_wait(&s_bar[n & 1], (unsigned)(n >> 1) & 1u, GV_SPIN_LIMIT, &c.sc->err)) break;
+        for (int k = nfail; k < nfail + (t1 >= 0 ? 2 : 1); ++k)
+            if (!mbar_wait(&s_bar[k & 1], (unsigned)(k >> 1) & 1u, GV_SPIN_LIMIT, &c.sc->err)) break;
     }
     nrechk = __reduce_add_sync(kFull, nrechk);
     ndf = __reduce_add_sync(kFull, ndf);
     bad = __reduce_or_sync(kFull, bad);
     if (lane == 0) {
+        // whole groups (the step's last may hold fewer tiles)
+        if (c.work && n) atomicAdd(&c.sc->emit_bytes, (unsigned long long)n * (GT * 4 * (RW + NS)));
         if (nrechk) atomicAdd(&c.sc->rechecks, (unsigned long long)nrechk);
         if (ndf) atomicAdd(&c.sc->rechecks_df, (unsigned long long)ndf);
         if (bad) atomicOr(&c.sc->err, bad << 1);

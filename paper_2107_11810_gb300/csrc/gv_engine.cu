@@ -81,6 +81,7 @@ struct vote_ctx {
     bool fault_hit = false;            // an allocation failed because the test hook asked for it
     uint32_t initial_lb = 0;
     int kernel_timing = 0;
+    int count_work = 0;        // count what the passes leave out (with kernel timing, here or in the batch)
     int log = 0;               // VOTE_LOG=1: per-level counters on stderr after each solve;
                                // 2: also one line per expansion step
     unsigned spin_limit = GV_SPIN_LIMIT;   // VOTE_OPT_SPIN_LIMIT
@@ -119,6 +120,7 @@ struct vote_ctx {
     void *h_tmp_dev() { return (char *)scal.p + ((sizeof(Scalars) + 63) / 64) * 64; }
     int64_t trace_written = 0;
     int64_t expanded = 0;      // record slots expanded in this solve
+    int64_t evaluated = 0;     // tests that the solve evaluated (stats.tests without those of cells left early), -1: not counted
     bool trace_overflow = false;
     vote_stats stats;
 };
@@ -831,6 +833,7 @@ static void fill_chunk(vote_ctx *c, int l, const LevelStore &S, const StepDims &
         const int64_t per = nt / (sm_count() * 32);         // tiles per warp, about
         ch.early = per >= 64 ? 64 : (per >= 32 ? 32 : (per >= 16 ? 16 : 1));
     }
+    ch.work = c->count_work || c->log >= 2;
     ch.cfail = (uint32_t *)c->child_idx.p;
     ch.spin = c->spin_limit;
     ch.tinfo = (int2 *)c->tinfo.p;
@@ -992,7 +995,8 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     const int nchild = launch_child_alloc(ch, small, (uint32_t *)c->keepflag.p, (uint32_t *)c->recn.p,
                                                       (unsigned long long *)c->bsums.p, c->stream);
     ev_mark(c, VOTE_K_CHILDREN);
-    // algorithmic bytes: the records of whole tiles read, the ballots written
+    // algorithmic bytes: the records of whole tiles read, the ballots written (those of the
+    // tiles that the count pass leaves out, and what the emit pass reads: at the solve's end)
     c->kbytes[VOTE_K_TEST_COUNT] += (double)nt * 32 * rb + (double)nt * ns * 4;
     c->kbytes[VOTE_K_CELL_GEO] += (double)nc * (8 + 4);
     CK(cudaGetLastError());
@@ -1004,10 +1008,13 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     S.ncells = c0;
     S.nrecs = r0;
     if (lev.leaf_children) {
-        if (c->log >= 2)
+        if (c->log >= 2) {
+            const double left0 = (double)c->h_sc->left_bytes;
+            TRY(read_scalars(c));
             std::fprintf(stderr, "[vote] step %lld level %d: %lld cells, %lld tiles, count %.0f B, leaves\n",
                          (long long)c->stats.chunks - 1, l, (long long)nc, (long long)nt,
-                         (double)nt * 32 * rb + (double)nt * ns * 4);
+                         (double)nt * 32 * rb + (double)nt * ns * 4 - ((double)c->h_sc->left_bytes - left0));
+        }
         c->stats.leaves += (int64_t)nch;
         nvtxRangePop();
         return VOTE_OK;
@@ -1025,21 +1032,18 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
         }
         c->stats.launches += 1;
         ev_mark(c, VOTE_K_TEST_EMIT);
-        c->kbytes[VOTE_K_TEST_EMIT] += (double)nt * 32 * rb + (double)nt * ns * 4 +
-                                       (double)new_slots * rec_bytes_at(c, l + 1);
+        c->kbytes[VOTE_K_TEST_EMIT] += (double)new_slots * rec_bytes_at(c, l + 1);
     }
     CK(cudaGetLastError());
     if (c->log >= 2) {
-        // the running FP64 recheck and test counters (a synchronisation per step: logging only)
-        CK(cudaMemcpyAsync(&c->h_sc->tests, &dsc(c)->tests, 24, cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaMemcpyAsync(&c->h_sc->rechecks_df, &dsc(c)->rechecks_df, 8, cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
+        // the running counters (a synchronisation per step: logging only)
+        const double left0 = (double)c->h_sc->left_bytes, read0 = (double)c->h_sc->emit_bytes;
+        TRY(read_scalars(c));
+        const double left = (double)c->h_sc->left_bytes - left0, read = (double)c->h_sc->emit_bytes - read0;
         std::fprintf(stderr, "[vote] step %lld level %d: %lld cells, %lld tiles, count %.0f B, emit %.0f B, "
                      "%lld child cells, %llu tests, %llu FP64 and %llu double-float rechecks so far\n",
                      (long long)c->stats.chunks - 1, l, (long long)nc, (long long)nt,
-                     (double)nt * 32 * rb + (double)nt * ns * 4,
-                     new_slots > 0 ? (double)nt * 32 * rb + (double)nt * ns * 4 +
-                                         (double)new_slots * rec_bytes_at(c, l + 1) : 0.0,
+                     (double)nt * 32 * rb + (double)nt * ns * 4 - left, read + (double)new_slots * rec_bytes_at(c, l + 1),
                      (long long)new_cells, c->h_sc->tests, c->h_sc->rechecks, c->h_sc->rechecks_df);
     }
     N.ncells += new_cells;
@@ -1357,6 +1361,7 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
     std::memset(&c->stats, 0, sizeof(c->stats));
     for (int l = 0; l < GV_MAXL; ++l) c->lv_cells[l] = c->lv_recs[l] = c->lv_gin[l] = c->lv_gout[l] = 0;
     c->stats.levels = P.L;
+    c->evaluated = c->count_work ? 0 : -1;
     if (n < 0 || !best_point || !depth || (n > 0 && !surfaces)) {
         set_err("invalid arguments");
         return VOTE_EINVAL;
@@ -1417,6 +1422,9 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
         c->stats.tests = (int64_t)c->h_sc->tests;
         c->stats.records = (int64_t)c->h_sc->records;
         c->stats.rechecks = (int64_t)c->h_sc->rechecks;
+        if (c->count_work) c->evaluated = (int64_t)(c->h_sc->tests - c->h_sc->left_tests);
+        c->kbytes[VOTE_K_TEST_COUNT] -= (double)c->h_sc->left_bytes;
+        c->kbytes[VOTE_K_TEST_EMIT] += (double)c->h_sc->emit_bytes;
         c->trace_written = (int64_t)c->h_sc->trace_n;
         if (c->trace_cap && c->trace_written > c->trace_cap) c->trace_overflow = true;
     }
@@ -1569,7 +1577,7 @@ vote_status vote_set_option(vote_ctx *c, int key, double v) {
         if (v != 0 && v != 1) break;
         if (v == 1 && !c->ev[0])
             for (int i = 0; i < vote_ctx::kEv; ++i) CK(cudaEventCreate(&c->ev[i]));
-        c->kernel_timing = (int)v;
+        c->kernel_timing = c->count_work = (int)v;
         return VOTE_OK;
     case VOTE_OPT_BATCH_WORKERS:
         if (!(v >= 1 && v <= 32)) break;
@@ -1626,6 +1634,7 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
                                double *latency_ms) {
     if (!c || !offsets || B < 0 || !best_points || !depths) { set_err("invalid arguments"); return VOTE_EINVAL; }
     std::memset(&c->stats, 0, sizeof(c->stats));     // this batch's counters, even when it is empty
+    c->evaluated = c->count_work ? 0 : -1;
     if (offsets[0] != 0) { set_err("offsets[0] must be 0"); return VOTE_EINVAL; }
     for (int b = 0; b < B; ++b)
         if (offsets[b + 1] < offsets[b]) { set_err("offsets must be non-decreasing"); return VOTE_EINVAL; }
@@ -1650,6 +1659,7 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
         w->chunk_records = c->chunk_records;
         w->chunk_set = c->chunk_set;
         w->dive = c->dive;
+        w->count_work = c->count_work;
         w->group = c->group;
         w->spin_limit = c->spin_limit;
         w->fault_alloc_at = 0;
@@ -1667,6 +1677,7 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
     std::vector<vote_status> wst(nw, VOTE_OK);
     std::vector<std::string> wmsg(nw);
     std::vector<vote_stats> wsum((size_t)nw);   // per worker: totals over its problems
+    std::vector<int64_t> wevaluated(nw, 0);
     for (auto &x : wsum) std::memset(&x, 0, sizeof(x));
     auto t0 = std::chrono::steady_clock::now();
     auto work = [&](int wi) {
@@ -1700,6 +1711,7 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
             a.cells += e.cells;
             a.records += e.records;
             a.tests += e.tests;
+            wevaluated[wi] += w->evaluated;
             a.rechecks += e.rechecks;
             a.chunks += e.chunks;
             a.leaves += e.leaves;
@@ -1737,6 +1749,7 @@ vote_status vote_solve_batched(vote_ctx *c, const double *surfaces, const int64_
         c->stats.cells += a.cells;
         c->stats.records += a.records;
         c->stats.tests += a.tests;
+        if (c->count_work) c->evaluated += wevaluated[i];
         c->stats.rechecks += a.rechecks;
         c->stats.chunks += a.chunks;
         c->stats.leaves += a.leaves;
@@ -1956,6 +1969,12 @@ vote_status vote_get_level_stats(vote_ctx *c, int64_t *cells, int64_t *records, 
 vote_status vote_get_stats(vote_ctx *c, vote_stats *out) {
     if (!c || !out) { set_err("invalid arguments"); return VOTE_EINVAL; }
     *out = c->stats;
+    return VOTE_OK;
+}
+
+vote_status vote_get_evaluated(vote_ctx *c, int64_t *tests) {
+    if (!c || !tests) { set_err("invalid arguments"); return VOTE_EINVAL; }
+    *tests = c->evaluated;
     return VOTE_OK;
 }
 

@@ -36,8 +36,8 @@ struct Scalars {
     unsigned long long best_key;     // (UB << coord_bits) | ~leaf key (max = best leaf)
     unsigned long long n_cells;      // cells written to the next level
     unsigned long long n_recs;       // record slots (32-aligned per cell) of the next level
-    unsigned long long tests;        // predicate calls
-    unsigned long long records;      // records tested
+    unsigned long long tests;        // (child, record) pairs decided
+    unsigned long long records;      // records of the cells expanded
     unsigned long long rechecks;     // FP64 rechecks of the FP32 screen
     unsigned long long trace_n;      // trace entries
     unsigned long long replay_ub;    // replay: surfaces reaching the target cell
@@ -46,6 +46,10 @@ struct Scalars {
     unsigned int ticket;             // units of tiles handed out by the step's count pass
     unsigned int qmax[GV_MAXD + GV_MAXT];  // lift: largest |q_f,j|, |q_t,m| of the root records
     unsigned long long rechecks_df;  // snaps the double-float tier decided (FP32 screen undecided)
+    // counted on request (Chunk::work):
+    unsigned long long left_tests;   // tests not evaluated: of cells that the count pass left
+    unsigned long long left_bytes;   // and the bytes it did not move for them
+    unsigned long long emit_bytes;   // records and ballots of the tiles that the emit pass read
 };
 
 struct Trace {
@@ -123,6 +127,7 @@ struct Chunk {
     int prune;
     int precision;           // 0 = FP64, 1 = FP32 screen + FP64 recheck
     int lb;                  // lower bounds are wanted (lballot, clb)
+    int work;                // count the work that is left out (adding it up costs a step of affine 4-space 1 %)
     int early;               // the count pass leaves cells whose children all fall below the threshold; it
                              // takes cells of at most this many tiles (>= 1) whole, a warp each
     uint32_t *cfail;         // [nc][ns] early: records that certainly fail each child's UB test, of cells that

@@ -239,8 +239,9 @@ __device__ __forceinline__ int32_t resnap_half(int32_t q) {
 template <int V, bool LB>
 struct CellWatch {
     // a warp's shared memory: rows of a batch (with LB those of the lower bounds after them), the
-    // step's units and their size
-    static constexpr int UNITS = LB ? 64 * V : 32 * V, SIZE = UNITS + 1, WORDS = UNITS + 4;
+    // step's units and their size, the tiles and records that it has left
+    static constexpr int UNITS = LB ? 64 * V : 32 * V, SIZE = UNITS + 1, TILES = UNITS + 2, RECORDS = UNITS + 3,
+                         WORDS = UNITS + 4;
     uint32_t *s;
     // the run of tiles at hand: its decided records, those of them that passed (per lane), both
     // since it began or since they were added up; more decided records than lim are looked at
@@ -263,6 +264,7 @@ struct CellWatch {
         if (lane == 0) {
             s[UNITS] = S;
             s[SIZE] = size;
+            s[TILES] = s[RECORDS] = 0u;
         }
         const unsigned long long at = (unsigned long long)warp * S * size;
         tt = at < nt ? (unsigned)at : nt;
@@ -291,9 +293,24 @@ struct CellWatch {
         for (int v = 0; v < V; ++v) pass[v] = 0u;
         lim = !watched(ti) ? 0xffffffffu : ((ti.y & kTileOwned) ? allowance(ti) : 511u);
     }
-    // A unit begins with tile ti: how many tiles of its cell are not this unit's (all, if the
-    // cell is the warp's that has its first tile, or if others know that it can be left).
-    __device__ __forceinline__ unsigned begin(const Chunk &c, int ns, int2 ti, int lane) const {
+    // lane 0: n tiles of ti's cell from tile tt on are left (none: ti is its last)
+    __device__ __forceinline__ void leave(const Chunk &c, int2 ti, unsigned tt, unsigned n) {
+        c.alive[ti.x] = 0;
+        if (!c.work || n == 0u) return;
+        const int64_t cell = c.in_c0 + ti.x;
+        const int64_t rest = (int64_t)c.in_rbeg[cell] + c.in_rcnt[cell] - 32 * (c.t0 + tt);
+        s[TILES] += n;
+        s[RECORDS] += rest < 32ll * n ? (unsigned)rest : 32u * n;
+    }
+    // The warp is done: what it has left (nw: words of a record).
+    __device__ __forceinline__ void report(const Chunk &c, int nw, int lane) const {
+        if (!c.work || lane != 0 || s[TILES] == 0u) return;
+        atomicAdd(&c.sc->left_tests, (unsigned long long)s[RECORDS] << c.lns);
+        atomicAdd(&c.sc->left_bytes, (unsigned long long)s[TILES] * 4u * (unsigned)(32 * nw + c.ns));
+    }
+    // A unit [tt, tb) begins with tile ti: how many tiles of its cell are not this unit's (all, if
+    // the cell is the warp's that has its first tile, or if others know that it can be left).
+    __device__ __forceinline__ unsigned begin(const Chunk &c, int ns, int2 ti, unsigned tt, unsigned tb, int lane) {
         if (ti.x < 0 || (ti.y & kTileFirst)) return 0u;
         if (ti.y & kTileOwned) return 1u + after(ti);
         if (!watched(ti)) return 0u;
@@ -303,8 +320,9 @@ struct CellWatch {
         for (int v = 0; v < V; ++v)
             if (v == 0 || ns > 32) d &= __ldcg(p + 32 * v) > allowance(ti);
         if (!__all_sync(kFull, d)) return 0u;
-        if (lane == 0) c.alive[ti.x] = 0;
-        return 1u + after(ti);
+        const unsigned n = 1u + after(ti);
+        if (lane == 0) leave(c, ti, tt, n < tb - tt ? n : tb - tt);
+        return n;
     }
     // A batch's ballots (word[v]: the lane's, 0 past its end) have been stored; its rows from
     // `first` on belong to the last run.
@@ -338,7 +356,7 @@ struct CellWatch {
         }
         if (!owned) cnt = 0u;
         if (!__all_sync(kFull, d)) return 0u;
-        if (lane == 0) c.alive[ti.x] = 0;
+        if (lane == 0) leave(c, ti, tt, owned || rest < tb - tt ? rest : tb - tt);
         return rest;
     }
 };

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256, wide_residents(FAM, LB)) k_count_wide(con
             int2 ti;
             if (head && c.early) {
                 ti = c.tinfo[tt];
-                const unsigned skip = watch.begin(c, ns, ti, lane);
+                const unsigned skip = watch.begin(c, ns, ti, tt, tb, lane);
                 if (skip) {
                     tt += skip;
                     head = false;
@@ -202,6 +202,7 @@ __global__ void __launch_bounds__(256, wide_residents(FAM, LB)) k_count_wide(con
             if (watch.cnt > watch.lim || tt >= tb) tt += watch.look(c, ns, ti, tt, tb, lane);
         }
     } while (watch.unit(__shfl_sync(kFull, next, 0), (unsigned)nt, tt, tb));
+    watch.report(c, NW, lane);
 }
 
 // The emit pass (see gv_emit.cu): slot rows of a tile (output address, passing lanes)
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
     float hs[ND];
 #pragma unroll
     for (int j = 0; j < ND; ++j) hs[j] = ((c.dm >> j) & 1) ? lev.Hs[j] : 0.0f;
-    unsigned nrechk = 0, ndf = 0, bad = 0;
+    unsigned nrechk = 0, ndf = 0, bad = 0, nread = 0;               // nread: tiles read
 
 #pragma unroll 1
     for (int64_t tt = ta; tt < tb; ++tt) {
@@ -259,6 +260,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
             v[h] = __ballot_sync(kFull, bal != 0u);
         }
         if (!(v[0] | v[1])) continue;                               // uniform: nothing to write
+        ++nread;
         const int64_t r = (c.t0 + tt) * 32 + lane;
         uint32_t w[NWI];
         load_words<NWI>(c.in.rec, r, w);
@@ -398,6 +400,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
     ndf = __reduce_add_sync(kFull, ndf);
     bad = __reduce_or_sync(kFull, bad);
     if (lane == 0) {
+        if (c.work && nread) atomicAdd(&c.sc->emit_bytes, (unsigned long long)nread * 4u * (unsigned)(32 * NWI + NS));
         if (nrechk) atomicAdd(&c.sc->rechecks, (unsigned long long)nrechk);
         if (ndf) atomicAdd(&c.sc->rechecks_df, (unsigned long long)ndf);
         if (bad) atomicOr(&c.sc->err, bad << 1);

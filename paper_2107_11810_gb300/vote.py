@@ -34,8 +34,8 @@ NESSENTIAL = {LINE2D: 1, PLANE3D_SPH: 3, POSE3DOF: 2, POSE6DOF: 11, RAYS3D: 2, P
               RADIAL5DOF: 7}
 EXPORTS = ["vote_create", "vote_set_option", "vote_set_stream", "vote_solve", "vote_solve_host",
            "vote_cell_counts", "vote_levels", "vote_get_trace", "vote_get_stats", "vote_get_kernel_times",
-           "vote_get_level_stats", "vote_cell_counts_noalloc", "vote_softscore_fwd", "vote_softscore_bwd",
-           "vote_refine", "vote_solve_batched", "vote_leaf_box", "vote_level_constants",
+           "vote_get_level_stats", "vote_get_evaluated", "vote_cell_counts_noalloc", "vote_softscore_fwd",
+           "vote_softscore_bwd", "vote_refine", "vote_solve_batched", "vote_leaf_box", "vote_level_constants",
            "vote_last_error", "vote_destroy"]
 
 
@@ -76,6 +76,7 @@ def load(path: str | None = None):
             lib.vote_level_constants.argtypes = [i32, i32, i32, P, P, P, P, P, P, P]
             lib.vote_get_trace.argtypes = [P, i64, P, P, P, P, P]
             lib.vote_get_stats.argtypes = [P, ctypes.POINTER(Stats)]
+            lib.vote_get_evaluated.argtypes = [P, P]
             lib.vote_get_kernel_times.argtypes = [P, P, P, P]
             lib.vote_get_level_stats.argtypes = [P, P, P, P, P]
             lib.vote_cell_counts_noalloc.argtypes = [i32, i32, i32, P, P, P, i64, i32, P, P, P, P, P]
@@ -261,6 +262,14 @@ class Solver:
         s = Stats()
         _check(self.lib.vote_get_stats(self.h, ctypes.byref(s)))
         return s.as_dict()
+
+    def evaluated_tests(self) -> int:
+        """(child cell, surface) pairs whose test the last solve or batch evaluated: those
+        of ``stats()["tests"]`` without the pairs of cells left early.  Counted with
+        VOTE_OPT_KERNEL_TIMING, else -1."""
+        t = np.zeros(1, np.int64)
+        _check(self.lib.vote_get_evaluated(self.h, _ptr(t)))
+        return int(t[0])
 
     def solve_batched(self, blocks, want_mask: bool = True):
         """Solve independent problems.  ``blocks``: CUDA float64 tensor holding the
