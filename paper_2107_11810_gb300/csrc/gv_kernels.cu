@@ -50,7 +50,7 @@ __global__ void k_root_basis(Problem P, Level lev0, double *psi) {
 __device__ __forceinline__ int lift_q(double x, double inv_s, bool &bad) {
     const double v = dmul(x, inv_s);
     const int q = __double2int_rn(v);                // saturates
-    bad |= (__double2hiint(v) & 0x7ff00000) == 0x7ff00000 || (unsigned)(q + 0x3fffffff) > 0x7ffffffeu;
+    bad |= (__double2hiint(v) & 0x7ff00000) == 0x7ff00000 || (unsigned)q + 0x3fffffffu > 0x7ffffffeu;
     return bad ? 0 : q;
 }
 
