@@ -18,11 +18,7 @@ SOURCES = ["gv_kernels.cu", "gv_count.cu", "gv_emit.cu", "gv_wide.cu", "gv_exact
 HEADERS = ["gv_device.cuh", "gv_kernels.h", "gv_tile.cuh"]
 NVCC = os.environ.get("NVCC", "nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-# -prec-sqrt=false: FP32 sqrtf (only used by the FP32 screen, whose error margin
-# covers it) maps to the hardware approximation; FP64 operations are explicit
-# IEEE intrinsics and are not affected.
-FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-prec-sqrt=false", "-Xcompiler", "-fPIC",
-         "-Xcompiler", "-ffp-contract=off",
+FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",
          "-I", os.path.join(ROOT, "include"), "-I", CSRC]
 
 

@@ -66,7 +66,6 @@ struct Level {                 // tests of the children of a level-l cell
     // set per solve, once the input's parameter ranges are known: the screen's band
     float kappa[GV_MAXD];      // undecided by the radius: |y^2 - R^2| < kappa R^2
     float bandL[GV_MAXD], bandL0[GV_MAXD];  // undecided by the lower-bound radius: | |y| - Lc | < bandL R + bandL0
-    float qt_max[GV_MAXT];     // bound on |q_t,m| of this level's records
     int q16;                   // this level's records hold 16-bit fields
     int q16_next;              // the next level's records hold 16-bit fields
 };

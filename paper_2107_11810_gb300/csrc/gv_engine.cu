@@ -449,7 +449,6 @@ static void finalize_levels(vote_ctx *c, const unsigned *qmax) {
             double ratio = v.s_t[m] / c->lev[0].s_t[m];                 // a power of two >= 1
             qtb[m] = std::floor((double)qmax[P.nd + m] / ratio) + 1.0;
             T[m] = (qtb[m] + 1.0) * v.s_t[m];
-            v.qt_max[m] = (float)qtb[m];
             fits &= qtb[m] <= 32000.0;
         }
         lambda_max(P.fam, T, lam);

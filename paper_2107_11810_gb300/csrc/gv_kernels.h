@@ -180,7 +180,7 @@ constexpr unsigned kAllowNone = 0xffffu;
 constexpr int kNoExp = -1000;
 
 // Selection of a level's cells with the largest UBs (index 0) and LBs (index 1)
-// (k_beam_*); zeroed before each use.
+// (k_beam_*); zeroed once, and every selection leaves it cleared for the next.
 constexpr int kBeamBins = 2048;
 struct BeamSel {
     unsigned long long hist[2][kBeamBins];  // record slots per bin
@@ -207,10 +207,10 @@ void launch_root_basis(const Problem &P, const Level &lev0, double *psi, cudaStr
 void launch_sincos_table(const Problem &P, int j, double2 *tab, cudaStream_t st);
 // cells (alive, geometry) and tiles (tinfo) of the chunk; returns the kernels launched
 int launch_prep(const Chunk &c, cudaStream_t st);
-// launch a persistent kernel taking one Chunk: one block per resident slot on the
-// device, at most `groups` blocks, 256 threads, smem bytes of dynamic shared memory
 // SMs of the device (read once)
 int sm_count();
+// launch a persistent kernel taking one Chunk: one block per resident slot on the
+// device, at most `groups` blocks, 256 threads, smem bytes of dynamic shared memory
 void launch_persistent(const void *kern, size_t smem, int64_t groups, const Chunk &c, cudaStream_t st);
 // the ballots of every tile and child, by the FP32 screen (undecided records queued)
 // or, in plain FP64 mode, by the definition

@@ -2,11 +2,9 @@
 // test (the surface-box test of Sec. 3.2, "eps plus the cell radius", over every
 // (canonical record, child cell) pair).
 //
-// Work unit: a tile of 32 consecutive records of one cell, one record per lane of
-// a warp.  A block of kWarps warps takes groups of kBlockTiles consecutive tiles,
-// warp w the kTW consecutive tiles w kTW .. w kTW + kTW - 1 of each group (so that
-// a warp's run of tiles of one cell stays together and its counters are flushed
-// once per run).
+// A tile is 32 consecutive records of one cell, one record per lane of a warp; warps take
+// runs of consecutive tiles (CellWatch in the count pass, units by turns in the emit pass),
+// so that most of a run lies in one cell.
 #pragma once
 #include <type_traits>
 
@@ -15,20 +13,12 @@
 namespace gv {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kWarps = 8;
-#ifndef GV_TILES_PER_WARP
-#define GV_TILES_PER_WARP 4
-#endif
-constexpr int kTW = GV_TILES_PER_WARP;           // tiles per warp
-constexpr int kBlockTiles = kWarps * kTW;        // tiles per block
-static_assert(32 * kTW < 256, "byte-packed per-slot counters would overflow");
 
 // ---------------------------------------------------------------------------
-// Bulk asynchronous copies (global -> shared) completing on an mbarrier: the
-// count and emit passes stream their records through shared memory, two groups
-// of kBlockTiles tiles per block in flight.  Every wait is bounded: after
-// kSpinLimit unsuccessful polls the kernel records VOTE_ETIMEOUT's error bit and
-// stops (the host maps it to VOTE_ETIMEOUT).
+// Bulk asynchronous copies (global -> shared) completing on an mbarrier: the emit
+// pass streams its records through shared memory, two groups of tiles per warp in
+// flight.  Every wait is bounded: after Chunk::spin unsuccessful polls the kernel
+// records kErrTimeout and stops (the host maps it to VOTE_ETIMEOUT).
 // ---------------------------------------------------------------------------
 constexpr unsigned kErrTimeout = 0x100u;
 #ifndef GV_SPIN_LIMIT
@@ -848,8 +838,9 @@ __device__ __forceinline__ void test_children(const f2 (&u)[ND][(FG + 1) / 2], c
     }
 }
 
-// Whether the screen leaves a record undecided.  The band is proportional to the radius (Level::bandR, bandL: see finalize_levels): a
-// residual is within bandR R of the radius only if |y^2 - R^2| < bandR (2 + bandR) R^2.
+// Whether the screen leaves a record undecided.  Its band is proportional to the radius
+// (bandR, in finalize_levels): a residual is within bandR R of the radius only if
+// |y^2 - R^2| < bandR (2 + bandR) R^2 = kappa R^2.
 template <int FAM, bool LB>
 __device__ __forceinline__ bool undecided(const Level &lev, const float *R, const float *near, const float *nearL) {
     using F = Fam<FAM>;
