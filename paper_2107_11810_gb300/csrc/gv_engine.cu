@@ -1075,9 +1075,13 @@ static vote_status replay(vote_ctx *c, const double *surfaces, int64_t n, int la
 // Measured (GB300, three instances per family, ms): 2^17, 2^19 and 2^20 records give
 // 13.6, 12.5 and 13.9 on the batch of 24 3DoF problems (a larger beam opens more than
 // it must) and 1.23, 0.70 and 0.70 on 10,000 lines (a smaller one takes more dependent
-// steps than a level that is opened whole).  Divisors 8 / 16 / 32: point sets 17 / 16 to
-// 84 / 54 to 87 (the best leaf's ancestor is often outside the top sixteenth), planes of
-// 1e4 points 60 / 54 / 52, 6DoF 25 / 21 / 15, radial 27 / 22 / 21.
+// steps than a level that is opened whole).  Divisors 4 / 8 / 16 / 32 / 64, mean of four
+// instances, ms: point sets (300 x 300) 12.1 / 10.7 / 10.3 / 10.4 / 10.4, affine 4-space (1e4
+// points) 33.1 / 28.5 / 27.2 / 26.4 / 26.1, radial 19.8 / 15.9 / 12.6 / 12.4 / 11.4, 6DoF 14.2 /
+// 11.3 / 7.2 / 5.5 / 5.5, planes of 1e4 points 21.2 / 16.5 / 14.7 / 14.0 / 13.5, 3DoF of 1e6
+// 4.8 / 4.4 / 4.4 / 4.4 / 4.4.  A smaller share can miss the best leaf's ancestor: with d = 4 it
+// is 8 because point sets took 16 to 84 and 54 to 87 ms with 16 and 32 instead of 17 while the
+// levels after the dive were opened in small steps, as they are where memory is short.
 static const int64_t kBeamRecords = (int64_t)1 << 19;
 static int64_t beam_divisor(int d) { return d == 4 ? 8 : (d > 4 ? 32 : 16); }
 
