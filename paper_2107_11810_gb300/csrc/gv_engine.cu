@@ -75,6 +75,7 @@ struct vote_ctx {
     int device = 0;
     cudaStream_t stream = 0;
     int precision = 1, prune = 1, group = 0;
+    unsigned sched = 0;        // how the process wants its threads to wait (cudaDeviceSchedule*)
     int64_t chunk_records = 1 << 25;
     bool chunk_set = false;            // VOTE_OPT_CHUNK_RECORDS was given
     bool lean = false;                 // the solve at hand is repeated with less memory (solve_device)
@@ -850,25 +851,22 @@ static void fill_chunk(vote_ctx *c, int l, const LevelStore &S, const StepDims &
 
 // Waits until step number seq has reported into v (every step's report is its last but one
 // or last kernel; the stream's state is looked at now and then, so a failed launch ends it).
-// It polls for as long as a short step takes; after that it waits as the process has chosen
-// for the device (cudaSetDeviceFlags): blocked, or polling, with the core given up between
-// polls unless spinning was asked for.  A search that only polled took 442 ms of CPU time in
-// 495 ms under cudaDeviceScheduleBlockingSync (planes, 1e6 points, eps 0.03).
+// It waits as the process has chosen for the device (cudaSetDeviceFlags, read once per solve):
+// blocked after polling for as long as the shortest steps take; or polling, with the core given
+// up every microsecond or so from 100 us on unless spinning was asked for (a yield after every
+// poll from 20 us on took 5 of 427 us on 10,000 lines).  A search that only polled took 442 ms of
+// CPU time in 495 ms under cudaDeviceScheduleBlockingSync (planes, 1e6 points, eps 0.03).
 static vote_status wait_report(vote_ctx *c, const LevInfo *v, long long seq) {
     auto reported = [&] { return __atomic_load_n(&v->seq, __ATOMIC_ACQUIRE) == seq; };
-    for (unsigned i = 0; i < 0x4000; ++i)    // some 20 us
+    const unsigned how = c->sched;
+    for (unsigned i = how == cudaDeviceScheduleBlockingSync ? 0x4000u : 0x20000u; i > 0; --i)
         if (reported()) return VOTE_OK;
-    unsigned flags = 0;
-    CK(cudaGetDeviceFlags(&flags));
-    const unsigned how = flags & cudaDeviceScheduleMask;
     if (how == cudaDeviceScheduleBlockingSync) {
         CK(cudaStreamSynchronize(c->stream));
     } else {
-        // some 100 us between looks at the stream: they take the lock that other threads launch under
-        const unsigned every = how == cudaDeviceScheduleSpin ? 0xffffu : 0xffu;
         for (unsigned i = 1; !reported(); ++i) {
-            if (how != cudaDeviceScheduleSpin) std::this_thread::yield();
-            if (i & every) continue;
+            if (how != cudaDeviceScheduleSpin && !(i & 0x3ffu)) std::this_thread::yield();
+            if (i & 0xffffu) continue;           // looking at the stream takes the lock that other threads launch under
             const cudaError_t e = cudaStreamQuery(c->stream);
             if (e == cudaErrorNotReady) {
                 cudaGetLastError();
@@ -1373,6 +1371,9 @@ static vote_status solve_inner(vote_ctx *c, const double *surfaces, int64_t n, d
         set_err("n = %lld too large", (long long)n);
         return VOTE_EUNSUPPORTED;
     }
+    unsigned flags = 0;
+    CK(cudaGetDeviceFlags(&flags));
+    c->sched = flags & cudaDeviceScheduleMask;
     CK(cudaMemsetAsync(c->scal.p, 0, sizeof(Scalars), c->stream));
     if (c->initial_lb) CK(cudaMemcpyAsync(&dsc(c)->best_lb, &c->initial_lb, 4, cudaMemcpyHostToDevice, c->stream));
     for (int i = 0; i < VOTE_K_CLASSES; ++i) c->kms[i] = c->kbytes[i] = 0, c->klaunch[i] = 0;
