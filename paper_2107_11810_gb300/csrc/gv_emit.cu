@@ -161,9 +161,8 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
     int t1, cells1, nfail = -1;                                     // copy that did not arrive
     next_group(t1, cells1);
     if (t1 >= 0 && lane == 0) issue(0, t1);
-    int n = 0;                                                      // groups read
 #pragma unroll 1
-    for (; t1 >= 0; ++n) {
+    for (int n = 0; t1 >= 0; ++n) {
         const int b = n & 1, t0 = t1, cells = cells1;
         next_group(t1, cells1);
         if (t1 >= 0 && lane == 0) issue(n + 1, t1);
@@ -365,19 +364,44 @@ __global__ void __launch_bounds__(256, 3) k_emit(const __grid_constant__ Chunk c
     if (nfail >= 0 && lane == 0) {
         // the copies nfail and nfail + 1 (no later one was issued) may still be in flight:
         // wait for them, bounded, before the block's shared memory is released
-        for (int k = nfail; k < nfail + (t1 >= 0 ? 2 : 1); ++k)
-            if (!mbar_wait(&s_bar[k & 1], (unsigned)(k >> 1) & 1u, GV_SPIN_LIMIT, &c.sc->err)) break;
+        for (int n = nfail; n < nfail + (t1 >= 0 ? 2 : 1); ++n)
+            if (!mbar_wait(&s_bar[n & 1], (unsigned)(n >> 1) & 1u, GV_SPIN_LIMIT, &c.sc->err)) break;
     }
     nrechk = __reduce_add_sync(kFull, nrechk);
     ndf = __reduce_add_sync(kFull, ndf);
     bad = __reduce_or_sync(kFull, bad);
     if (lane == 0) {
-        // whole groups (the step's last may hold fewer tiles)
-        if (c.work && n) atomicAdd(&c.sc->emit_bytes, (unsigned long long)n * (GT * 4 * (RW + NS)));
         if (nrechk) atomicAdd(&c.sc->rechecks, (unsigned long long)nrechk);
         if (ndf) atomicAdd(&c.sc->rechecks_df, (unsigned long long)ndf);
         if (bad) atomicOr(&c.sc->err, bad << 1);
     }
+}
+
+// The tiles whose records the emit pass is going to read, counted apart from it (on request;
+// in k_emit_wide itself the count took 0.3 % of a search of affine 4-space): groups of
+// kEmitTiles with a cell that has surviving children, or (wide) tiles with something to write.
+__global__ void __launch_bounds__(256) k_emit_work(const __grid_constant__ Chunk c, int wide, int tile_bytes) {
+    grid_start();
+    const int64_t nt = chunk_tiles(c), t = blockIdx.x * 256ll + threadIdx.x;
+    const int cell = t < nt ? c.tinfo[t].x : -1;
+    bool read = cell >= 0 && (c.alive[cell] & 2);
+    if (wide) {
+        bool any = false;
+        for (int s = 0; read && s < c.ns; ++s)
+            any |= c.cbase[(size_t)cell * c.ns + s] != ~0ull && c.ballot[(size_t)t * c.ns + s];
+        read &= any;
+    } else {
+        const unsigned b = __ballot_sync(kFull, read);
+        read = t < nt && ((b >> (threadIdx.x & 31u & ~(kEmitTiles - 1u))) & ((1u << kEmitTiles) - 1u));
+    }
+    const unsigned n = (unsigned)__popc(__ballot_sync(kFull, read));
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&c.sc->emit_bytes, (unsigned long long)n * (unsigned)tile_bytes);
+}
+
+void launch_emit_work(const Chunk &c, int rec_bytes, cudaStream_t st) {
+    const int64_t nt = c.t1 - c.t0;
+    if (nt > 0)
+        launch(k_emit_work, (unsigned)((nt + 255) / 256), 256, 0, st, c, c.P.d > 3, 32 * rec_bytes + 4 * c.ns);
 }
 
 template <int FAM, bool QI, bool QO, int KF, int DM>

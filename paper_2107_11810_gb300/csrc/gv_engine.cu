@@ -1022,6 +1022,10 @@ static vote_status expand_chunk(vote_ctx *c, int l, bool beam = false) {
     if (new_slots > 0) {
         TRY(ensure_level(c, N, l + 1, (size_t)(N.nrecs + new_slots), 0));
         ch.out = rec_view(c, N);
+        if (ch.work) {
+            launch_emit_work(ch, rb, c->stream);
+            c->stats.launches += 1;
+        }
         ev_mark(c, -1);
         if (!launch_emit(ch, c->stream)) {
             set_err("internal: no emit pass for record formats %d -> %d", lev.q16, lev.q16_next);

@@ -127,7 +127,7 @@ struct Chunk {
     int prune;
     int precision;           // 0 = FP64, 1 = FP32 screen + FP64 recheck
     int lb;                  // lower bounds are wanted (lballot, clb)
-    int work;                // count the work that is left out (adding it up costs a step of affine 4-space 1 %)
+    int work;                // count the work that is done and left out
     int early;               // the count pass leaves cells whose children all fall below the threshold; it
                              // takes cells of at most this many tiles (>= 1) whole, a warp each
     uint32_t *cfail;         // [nc][ns] early: records that certainly fail each child's UB test, of cells that
@@ -222,6 +222,8 @@ void launch_count_exact(const Chunk &c, cudaStream_t st);
 // per child its counts, per tile and child its records' place in the child, best LB
 void launch_tile_scan(const Chunk &c, cudaStream_t st);
 bool launch_emit_wide(const Chunk &c, cudaStream_t st);
+// adds the bytes of records and ballots that the emit pass will read to sc->emit_bytes
+void launch_emit_work(const Chunk &c, int rec_bytes, cudaStream_t st);
 // false if the level's record formats have no emit pass (never chosen by the engine)
 bool launch_emit(const Chunk &c, cudaStream_t st);
 // sizes of the level that a chain starts from, or goes on from

@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
     float hs[ND];
 #pragma unroll
     for (int j = 0; j < ND; ++j) hs[j] = ((c.dm >> j) & 1) ? lev.Hs[j] : 0.0f;
-    unsigned nrechk = 0, ndf = 0, bad = 0, nread = 0;               // nread: tiles read
+    unsigned nrechk = 0, ndf = 0, bad = 0;
 
 #pragma unroll 1
     for (int64_t tt = ta; tt < tb; ++tt) {
@@ -260,7 +260,6 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
             v[h] = __ballot_sync(kFull, bal != 0u);
         }
         if (!(v[0] | v[1])) continue;                               // uniform: nothing to write
-        ++nread;
         const int64_t r = (c.t0 + tt) * 32 + lane;
         uint32_t w[NWI];
         load_words<NWI>(c.in.rec, r, w);
@@ -400,7 +399,6 @@ __global__ void __launch_bounds__(256) k_emit_wide(const __grid_constant__ Chunk
     ndf = __reduce_add_sync(kFull, ndf);
     bad = __reduce_or_sync(kFull, bad);
     if (lane == 0) {
-        if (c.work && nread) atomicAdd(&c.sc->emit_bytes, (unsigned long long)nread * 4u * (unsigned)(32 * NWI + NS));
         if (nrechk) atomicAdd(&c.sc->rechecks, (unsigned long long)nrechk);
         if (ndf) atomicAdd(&c.sc->rechecks_df, (unsigned long long)ndf);
         if (bad) atomicOr(&c.sc->err, bad << 1);
