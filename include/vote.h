@@ -126,7 +126,10 @@ typedef enum {
                                  the B&B bound, e.g. from a previous frame); must not
                                  exceed the true maximum depth; default 0            */
     VOTE_OPT_KERNEL_TIMING = 8, /* 1 = time each kernel class with CUDA events on the
-                                 context's stream (see vote_get_kernel_times)        */
+                                 context's stream (see vote_get_kernel_times) and
+                                 count evaluated tests (vote_get_evaluated); small
+                                 searches then take a slower path, so time whole
+                                 solves without it                                   */
     VOTE_OPT_BATCH_WORKERS = 10, /* host workers (streams) of vote_solve_batched, 1..32,
                                  default 4                                           */
     VOTE_OPT_DIVE = 11,       /* 1 or 2 (default): first follow the cells with the largest
