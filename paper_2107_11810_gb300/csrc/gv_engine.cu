@@ -522,8 +522,9 @@ static void release(vote_ctx *c, DevBuf &b) {
     b.bytes = 0;
 }
 
-// Gives back what solves have grown: the levels, the beam, the steps' scratch, the grouping's
-// tables, here and in the workers of batches (no solve of this context is running).
+// Gives back what solves have grown: the levels, the beam, the steps' scratch, the rotations'
+// and the grouping's tables, here and in the workers of batches (no solve of this context is
+// running).
 static void release_working(vote_ctx *c) {
     for (vote_ctx *w : c->workers) release_working(w);
     for (int l = 0; l <= GV_MAXL + 1; ++l) {
@@ -531,6 +532,7 @@ static void release_working(vote_ctx *c) {
         DevBuf *bufs[] = {&s.rec, &s.mult, &s.tile_cell, &s.key, &s.rbeg, &s.rcnt, &s.ub, &s.lb};
         for (DevBuf *b : bufs) release(c, *b);
         s.ncells = s.nrecs = 0;
+        if (l <= GV_MAXL) release(c, c->rot[l]), release(c, c->rotflag[l]);
     }
     DevBuf *bufs[] = {&c->alive, &c->geo64, &c->geo32, &c->geo32lo, &c->cnt, &c->tinfo, &c->ballot, &c->lballot,
                       &c->uns, &c->off, &c->cbase, &c->child_idx, &c->keepflag, &c->recn, &c->bsums, &c->g_table,
@@ -2000,7 +2002,6 @@ void vote_destroy(vote_ctx *c) {
     for (DevBuf *b : bufs) release(c, *b);
     for (DevBuf &b : c->sctab) release(c, b);
     release(c, c->psi0);
-    for (int l = 0; l <= GV_MAXL; ++l) release(c, c->rot[l]), release(c, c->rotflag[l]);
     cudaStreamSynchronize(c->stream);
     for (int i = 0; i < vote_ctx::kEv; ++i)
         if (c->ev[i]) cudaEventDestroy(c->ev[i]);
